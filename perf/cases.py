@@ -190,3 +190,72 @@ def tolerance(case):
         return {"rel": 1e-6, "max": 4e-6}
     # codes and shared exponents are exact; two fp32 roundings of the exact scale are at most 2 ulp apart
     return {"rel": 2.5e-7, "max": 5e-7}
+
+
+def _base_matrix(n):
+    """The +-1 base matrix of order n = 2 (q + 1), q = 1 (mod 4) a prime: Paley's second construction."""
+    q = n // 2 - 1
+    squares = {(a * a) % q for a in range(1, q)}
+    core = torch.ones(q + 1, q + 1, dtype=torch.float64)
+    for i in range(1, q + 1):
+        for j in range(1, q + 1):
+            core[i, j] = 0 if i == j else (1 if (i - j) % q in squares else -1)
+    core[0, 0] = 0
+    core[0, 1:] = core[1:, 0] = 1
+    # a zero becomes [[1, -1], [-1, -1]], an entry s becomes s [[1, 1], [1, -1]]
+    one = torch.tensor([[1.0, 1.0], [1.0, -1.0]], dtype=torch.float64)
+    zero = torch.tensor([[1.0, -1.0], [-1.0, -1.0]], dtype=torch.float64)
+    return torch.kron(core, one) + torch.kron((core == 0).to(torch.float64), zero)
+
+
+def _rotated(x, b):
+    """Rows of x rotated by I (x) H_b / sqrt(b), in 64 bits."""
+    T, d = x.shape
+    base = 1
+    if b & (b - 1):
+        base = b
+        while base % 2 == 0:
+            base //= 2
+        base *= 4
+    v = x.to(torch.float64).reshape(T, d // base, base)
+    if base > 1:
+        v = v @ _base_matrix(base).to(x.device)
+    v = v.reshape(T, d)
+    h = base
+    while h < b:
+        v = v.reshape(T, d // (2 * h), 2, h)
+        v = torch.stack((v[:, :, 0] + v[:, :, 1], v[:, :, 0] - v[:, :, 1]), 2).reshape(T, d)
+        h *= 2
+    return v / math.sqrt(b)
+
+
+def exact(case, seed):
+    """The fp32 outputs of `run` in 64 bits: scales and statistics.  Codes and shared exponents have no such value."""
+    if case["call"] == "massdiff" or case.get("fmt") == "mxfp4":
+        return None
+    s = prepare(case, seed)
+    b = case["b"]
+    if case["call"] == "stats":
+        x = s["x"] if s["perm"] is None else s["x"][:, s["perm"].long()]
+        chan, block, token = torch.zeros(case["d"], dtype=torch.float64, device="cuda"), 0, []
+        for x_raw, x_perm in zip(s["x"].split(1024), x.split(1024)):
+            norms = x_perm.abs().to(torch.float64).reshape(x_perm.shape[0], -1, b).sum(2)
+            chan, block = chan + x_raw.abs().to(torch.float64).sum(0), block + norms.sum(0)
+            token.append(norms.max(1).values)
+        return chan, block / case["T"], torch.cat(token)
+    scales = []
+    rows = zip(s["gate"].split(1024), s["up"].split(1024)) if case["call"] == "swiglu" else s["x"].split(1024)
+    for x in rows:
+        if case["call"] == "swiglu":
+            g = x[0].to(torch.float64)
+            x = (g / (1 + torch.exp(-g)) * x[1].to(torch.float64)).to(torch.bfloat16)
+        elif s["perm"] is not None:
+            x = x[:, s["perm"].long()]
+        y = _rotated(x, b)
+        if case["fmt"] == "int4_asym":
+            lo = y.min(1).values
+            step = (y.max(1).values - lo) / 15
+            scales.append(torch.stack((step, torch.where(step > 0, torch.round(lo / step), torch.zeros_like(lo))), 1))
+        else:
+            scales.append(y.abs().reshape(y.shape[0], -1, case["group"] or case["d"]).max(2).values / 7)
+    return None, torch.cat(scales)
