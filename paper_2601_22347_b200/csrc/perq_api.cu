@@ -871,11 +871,23 @@ int perq_massdiff_perm_device(const float *chan_abs_sum, int32_t d, int32_t b, i
         (reinterpret_cast<uintptr_t>(workspace) & 3u) != 0)
         return PERQ_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int32_t *order = static_cast<int32_t *>(workspace);
-    perq::perq_massdiff_rank_kernel<<<(d + perq::MD_THREADS - 1) / perq::MD_THREADS, perq::MD_THREADS, 0, st>>>(chan_abs_sum, d, order);
-    if (cudaGetLastError() != cudaSuccess) return PERQ_ERR_CUDA;
-    perq::perq_massdiff_greedy_kernel<<<1, 32, 0, st>>>(chan_abs_sum, order, d, b, perm);
-    return cudaGetLastError() == cudaSuccess ? PERQ_OK : PERQ_ERR_CUDA;
+    perq::MassdiffParams p;
+    p.a = chan_abs_sum;
+    p.order = static_cast<int32_t *>(workspace);
+    p.perm = perm;
+    p.d = d;
+    p.b = b;
+    const int n = d / b;
+    const perq::MdSmem lay(n);
+    if (int rc = allow_smem(perq::perq_massdiff_greedy_kernel, lay.total)) return rc;
+    const int ctas = (d + perq::MD_RANK_CHANNELS - 1) / perq::MD_RANK_CHANNELS;
+    const int threads = std::min(perq::MD_MAX_THREADS, (n + 31) / 32 * 64);      // two threads per list entry up to 512 blocks
+    if (launch_overlapped(perq::perq_massdiff_rank_kernel, ctas, perq::MD_RANK_THREADS, 0, st, p) != cudaSuccess ||
+        launch_overlapped(perq::perq_massdiff_greedy_kernel, 1, threads, lay.total, st, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return PERQ_ERR_CUDA;
+    }
+    return PERQ_OK;
 }
 
 int perq_chan_abs_max(const void *x, int64_t T, int32_t d, float *chan_abs_max, void *stream)

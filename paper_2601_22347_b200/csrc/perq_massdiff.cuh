@@ -3,80 +3,287 @@
 // (equal masses: lower channel first), each to the open block with the smallest running sum (equal sums:
 // lower block first), running sums in double, perm = the blocks concatenated.
 //
-// Two kernels: ranks by counting (every CTA ranks 256 channels against all d: d^2 comparisons spread over the
-// grid), then the greedy itself, which is sequential in the channels: one warp scans the open blocks for the
-// minimum (lanes over blocks, integer warp reductions), d times.
+// Two kernels.  Ranks by counting: d^2 comparisons spread over the grid (32 channels per CTA, its eight warps
+// share the d comparisons of a channel), two instructions each.  Then the greedy itself, one CTA, in BATCHES:
+//
+//   The open blocks are kept in a list sorted by (running sum, block).  If the next channels were handed to
+//   the blocks of the list in order, block i would reach new_i = s_i + c_i.  That is what the one-by-one
+//   greedy does as long as no block that has received a channel has become the lightest again.  Let M be the
+//   smallest (new_i, block).  new_i >= s_i, so every list entry above M comes after M's own entry: the entries
+//   up to M are exactly the prefix that the greedy serves before it returns to a block.  That prefix is served
+//   at once, and its new sums are merged into the list.
+//
+// The greedy is a serial chain: one channel at a time (a scan of all running sums per channel) it took 2316 us, in
+// batches it takes 164 us
+// for 8192 channels in 256 blocks.  Sums differ by about one channel mass, so a batch serves most of the
+// blocks: 64 batches there, 31 to 157 for 8 to 512 blocks of real statistics.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "perq_fast.cuh"
+
 namespace perq {
 
-constexpr int MD_THREADS = 256;
-constexpr int MD_TILE = 1024;
-constexpr int MD_MAX_BLOCKS = 4096;      // running sums and fill counts live in shared memory
+constexpr int MD_RANK_THREADS = 256;
+constexpr int MD_RANK_CHANNELS = 32;     // channels per CTA of the ranking
+constexpr int MD_TILE = 8192;            // masses staged at a time
+constexpr int MD_MAX_BLOCKS = 4096;      // the list lives in shared memory
+constexpr int MD_MAX_THREADS = 1024;
+constexpr int MD_WINDOW = 2048;          // ordered channels staged at a time by the greedy
 
-// order[r] = the channel of rank r (rank = number of channels that come before it)
-__global__ void __launch_bounds__(MD_THREADS) perq_massdiff_rank_kernel(const float *a, int d, int32_t *order)
+struct MassdiffParams {
+    const float *a;          // [d] channel masses
+    int32_t *order;          // [d] channels by rank
+    int32_t *perm;           // [d]
+    int d, b;
+};
+
+// Shared memory of the greedy: two lists (sum, block), the new sums, fill counts, the channel window, and a
+// few words of reduction space.
+struct MdSmem {
+    size_t sum0, sum1, fresh, key, key_old, id0, id1, fill, place, shared_place, doubtful, chan, mass, red, total;
+    __host__ __device__ explicit MdSmem(int n)
+    {
+        const size_t m = ((size_t)n + 3) & ~(size_t)3;
+        size_t o = 0;
+        sum0 = o;  o += m * 8;
+        sum1 = o;  o += m * 8;
+        fresh = o; o += m * 8;
+        key = o;   o += m * 4;
+        key_old = o; o += m * 4;
+        id0 = o;   o += m * 4;
+        id1 = o;   o += m * 4;
+        fill = o;  o += m * 4;
+        place = o; o += m * 4;
+        shared_place = o; o += m;
+        doubtful = o; o += m * 2;
+        o = (o + 15) & ~(size_t)15;
+        chan = o;  o += (size_t)MD_WINDOW * 4;
+        mass = o;  o += (size_t)MD_WINDOW * 4;
+        red = o;   o += 32 * 16;
+        total = o;
+    }
+};
+
+// Counting by packed fp32 adds: 1.0 for every comparison that holds, two per add (1.5 instructions a comparison
+// where an integer count took 3; counts stay below 2^24, so they are exact).
+__device__ __forceinline__ float md_gt(float a, float b) { float r; asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ float md_ge(float a, float b) { float r; asm("set.ge.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+
+// order[r] = the channel of rank r (rank = number of channels that come before it).  A lane counts for one
+// channel; the staged masses are read four at a time, the same ones by every lane.  Before the CTA's own 32
+// channels an equal mass comes first, after them it does not: one comparison per mass except among the 32.
+__global__ void __launch_bounds__(MD_RANK_THREADS) perq_massdiff_rank_kernel(MassdiffParams p)
 {
-    __shared__ float tile[MD_TILE];
-    const int i = blockIdx.x * MD_THREADS + threadIdx.x;
-    const float ai = (i < d) ? a[i] : 0.0f;
+    __shared__ __align__(16) float tile[MD_TILE];
+    __shared__ int part[MD_RANK_THREADS];
+    griddep_wait();
+    griddep_launch();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * MD_RANK_CHANNELS, i = i0 + lane;
+    const float ai = (i < p.d) ? p.a[i] : 0.0f;
+    const float nan = __int_as_float(0x7fffffff);        // padding: no comparison holds
     int rank = 0;
-    for (int k0 = 0; k0 < d; k0 += MD_TILE) {
+    f32x2 c0 = pack2(0.0f, 0.0f), c1 = c0;
+    for (int k0 = 0; k0 < p.d; k0 += MD_TILE) {
+        const int kn = min(MD_TILE, p.d - k0);
+        const int per = ((kn + 255) / 256) * 32;         // masses per warp: a multiple of 32
         __syncthreads();
-        for (int k = threadIdx.x; k < MD_TILE; k += MD_THREADS) tile[k] = (k0 + k < d) ? a[k0 + k] : 0.0f;
+        for (int k = threadIdx.x; k < per * 8; k += MD_RANK_THREADS) tile[k] = (k < kn) ? p.a[k0 + k] : nan;
         __syncthreads();
-        const int kn = min(MD_TILE, d - k0);
-        for (int k = 0; k < kn; ++k) {
-            const float ak = tile[k];
-            rank += (ak > ai || (ak == ai && k0 + k < i)) ? 1 : 0;
+        const int lo = warp * per, hi = lo + per, own = i0 - k0;       // all multiples of 32
+        const float4 *t4 = reinterpret_cast<const float4 *>(tile);
+        const int before = min(hi, own);
+#pragma unroll 8
+        for (int k = lo; k < before; k += 4) {
+            const float4 v = t4[k >> 2];
+            c0 = add2(c0, pack2(md_ge(v.x, ai), md_ge(v.y, ai)));
+            c1 = add2(c1, pack2(md_ge(v.z, ai), md_ge(v.w, ai)));
+        }
+        if (own >= lo && own < hi) {
+            for (int k = own; k < own + 32; ++k) {
+                const float ak = tile[k];
+                rank += (ak > ai || (ak == ai && k0 + k < i)) ? 1 : 0;
+            }
+        }
+#pragma unroll 8
+        for (int k = max(lo, own + 32); k < hi; k += 4) {
+            const float4 v = t4[k >> 2];
+            c0 = add2(c0, pack2(md_gt(v.x, ai), md_gt(v.y, ai)));
+            c1 = add2(c1, pack2(md_gt(v.z, ai), md_gt(v.w, ai)));
         }
     }
-    if (i < d) order[rank] = i;
+    rank += (int)((c0.x + c0.y) + (c1.x + c1.y));
+    part[threadIdx.x] = rank;
+    __syncthreads();
+    if (warp == 0 && i < p.d) {
+#pragma unroll
+        for (int w = 1; w < MD_RANK_THREADS / 32; ++w) rank += part[w * 32 + lane];
+        p.order[min(rank, p.d - 1)] = i;
+    }
 }
 
-// one warp; n = d / b <= MD_MAX_BLOCKS.  Running sums are non-negative doubles, so their bit patterns order
-// like the values: the minimum over the warp is three integer warp reductions (high word, low word among
-// the lanes that hold the minimal high word, block index among the lanes that hold the minimal sum).  A full
-// block's sum is replaced by +infinity.
-__global__ void __launch_bounds__(32) perq_massdiff_greedy_kernel(const float *a, const int32_t *order, int d, int b,
-                                                                  int32_t *perm)
+// Running sums are non-negative doubles, so their bit patterns order like the values.
+__device__ __forceinline__ bool md_less(unsigned long long s, int i, unsigned long long t, int j) { return s < t || (s == t && i < j); }
+
+__global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel(MassdiffParams p)
 {
-    __shared__ unsigned long long sum[MD_MAX_BLOCKS];      // bit patterns of the doubles
-    __shared__ int fill[MD_MAX_BLOCKS];
-    const int lane = threadIdx.x, n = d / b;
-    for (int j = lane; j < n; j += 32) { sum[j] = 0ull; fill[j] = 0; }
-    __syncwarp();
+    extern __shared__ __align__(16) unsigned char md_smem[];
+    const int d = p.d, b = p.b, n = d / b;
+    const MdSmem lay(n);
+    unsigned long long *sum = (unsigned long long *)(md_smem + lay.sum0), *sum_next = (unsigned long long *)(md_smem + lay.sum1);
+    unsigned long long *fresh = (unsigned long long *)(md_smem + lay.fresh);
+    float *key = (float *)(md_smem + lay.key), *key_old = (float *)(md_smem + lay.key_old);
+    int *id = (int *)(md_smem + lay.id0), *id_next = (int *)(md_smem + lay.id1);
+    int *fill = (int *)(md_smem + lay.fill), *place = (int *)(md_smem + lay.place);
+    unsigned char *shared_place = md_smem + lay.shared_place;
+    unsigned short *doubtful = (unsigned short *)(md_smem + lay.doubtful);
+    int *chan = (int *)(md_smem + lay.chan);
+    float *mass = (float *)(md_smem + lay.mass);
+    unsigned long long *red_sum = (unsigned long long *)(md_smem + lay.red);
+    int *red_id = (int *)(md_smem + lay.red + 32 * 8), *red_open = (int *)(md_smem + lay.red + 32 * 12);
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const unsigned long long INF = 0x7ff0000000000000ull;
-    for (int s0 = 0; s0 < d; s0 += 32) {
-        // the next 32 channels and their masses, one per lane
-        const int cl = (s0 + lane < d) ? order[s0 + lane] : 0;
-        const float al = (s0 + lane < d) ? a[cl] : 0.0f;
-        const int steps = min(32, d - s0);
-        for (int t = 0; t < steps; ++t) {
-            const int c = __shfl_sync(0xffffffffu, cl, t);
-            const float ac = __shfl_sync(0xffffffffu, al, t);
-            unsigned long long best = ~0ull;
-            int bj = 0x7fffffff;
-#pragma unroll 4
-            for (int j = lane; j < n; j += 32) {
-                const unsigned long long v = sum[j];
-                if (v < best) { best = v; bj = j; }          // ascending j: equal sums keep the lower block
+
+    for (int j = tid; j < n; j += nthr) { sum[j] = 0ull; id[j] = j; fill[j] = 0; shared_place[j] = 0; }
+    if (tid < 32) { red_sum[tid] = INF; red_id[tid] = 0x7fffffff; red_open[tid] = 0; }
+    griddep_wait();             // nothing above reads or writes global memory
+    griddep_launch();
+    int split = 0;              // log2 of the threads that count for one entry
+    while (split < 1 && (n << (split + 1)) <= nthr) ++split;
+    int m = n;                  // open blocks: list entries [0, m)
+    int s = 0, w0 = 0, w1 = 0;  // next rank; staged window of ranks [w0, w1)
+    uint32_t batch = 0;
+    while (s < d) {
+        if (s >= w1) {
+            __syncthreads();    // everybody has read the last window
+            w0 = s;
+            w1 = min(d, s + MD_WINDOW);
+            for (int k = tid; k < w1 - w0; k += nthr) {
+                const int c = min(max(p.order[w0 + k], 0), d - 1);
+                chan[k] = c;
+                mass[k] = p.a[c];
             }
+            __syncthreads();
+        }
+        // ---- the sums that the next q blocks of the list would reach, and the smallest of them
+        const int q = min(m, w1 - s);
+        unsigned long long best = INF;
+        int best_id = 0x7fffffff;
+        for (int j = tid; j < q; j += nthr) {
+            const double ns = __longlong_as_double((long long)sum[j]) + (double)mass[s - w0 + j];
+            const unsigned long long v = (fill[id[j]] + 1 < b) ? (unsigned long long)__double_as_longlong(ns) : INF;
+            fresh[j] = v;
+            if (v != INF && md_less(v, id[j], best, best_id)) { best = v; best_id = id[j]; }
+        }
+        {
             const uint32_t hi = (uint32_t)(best >> 32), lo = (uint32_t)best;
             const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
             const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-            const int mj = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)bj : 0x7fffffffu);
-            if (lane == 0) {
-                const int f = fill[mj];
-                perm[(size_t)mj * b + f] = c;
-                fill[mj] = f + 1;
-                const double ns = __longlong_as_double((long long)(((unsigned long long)mhi << 32) | mlo)) + (double)ac;
-                sum[mj] = (f + 1 < b) ? (unsigned long long)__double_as_longlong(ns) : INF;
-            }
-            __syncwarp();
+            const int mid = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)best_id : 0x7fffffffu);
+            if (lane == 0) { red_sum[warp] = ((unsigned long long)mhi << 32) | mlo; red_id[warp] = mid; }
         }
+        __syncthreads();
+        unsigned long long M;
+        int M_id;
+        {
+            const unsigned long long v = red_sum[lane];
+            const int vi = red_id[lane];
+            const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
+            const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
+            const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
+            M_id = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)vi : 0x7fffffffu);
+            M = ((unsigned long long)mhi << 32) | mlo;
+        }
+        // ---- K: the list entries up to M.  Distances of all sums to M in fp32 (sums within a batch are close
+        // to each other: the difference, not the sum, is what fp32 resolves)
+        const double m64 = __longlong_as_double((long long)M);
+        for (int j = tid; j < m; j += nthr) {
+            key_old[j] = (float)(__longlong_as_double((long long)sum[j]) - m64);
+            if (j < q) key[j] = (fresh[j] != INF) ? (float)(__longlong_as_double((long long)fresh[j]) - m64) : __int_as_float(0x7f800000);
+        }
+        int K = 0;
+        for (int j0 = 0; j0 < q; j0 += nthr) {
+            const int j = j0 + tid;
+            K += __syncthreads_count(j < q && !md_less(M, M_id, sum[min(j, q - 1)], id[min(j, q - 1)]));
+        }
+        K = max(K, 1);
+        // ---- serve them; every entry's place in the merged list: new sums below it (counted, 2^split threads
+        // to an entry), and for a new sum the untouched entries below it (searched).  fp32 distances to M
+        // decide; equal ones show below as two entries that took one place.
+        int *closed = red_open + (batch & 1u), *closed_next = red_open + ((batch + 1) & 1u);
+        for (int j0 = 0; j0 < m; j0 += nthr >> split) {
+            const int j = j0 + (tid >> split), sub = tid & ((1 << split) - 1);
+            const bool in = j < m, served = in && j < K;
+            const float v = in ? (served ? key[j] : key_old[j]) : 0.0f;
+            f32x2 c0 = pack2(0.0f, 0.0f), c1 = c0;
+            const int k4 = K >> 2;
+#pragma unroll 4
+            for (int k = sub; k < k4; k += 1 << split) {
+                const float4 x = reinterpret_cast<const float4 *>(key)[k];
+                c0 = add2(c0, pack2(md_gt(v, x.x), md_gt(v, x.y)));
+                c1 = add2(c1, pack2(md_gt(v, x.z), md_gt(v, x.w)));
+            }
+            float c = (c0.x + c0.y) + (c1.x + c1.y);
+            if (sub == 0) {
+                for (int k = 4 * k4; k < K; ++k) c += md_gt(v, key[k]);
+            }
+            for (int o = 1; o < (1 << split); o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+            if (!in || sub != 0) continue;
+            const int blk = id[j];
+            if (served) {
+                const int f = fill[blk];
+                p.perm[(size_t)blk * b + f] = chan[s - w0 + j];
+                fill[blk] = f + 1;
+                if (fresh[j] == INF) { place[j] = -1; atomicAdd(closed, 1); continue; }
+            }
+            int lo = K, hi = served ? m : j;
+            if (served || (j > K && !(key_old[j - 1] < v))) {
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (key_old[mid] < v) lo = mid + 1; else hi = mid;
+                }
+            } else {
+                lo = j;
+            }
+            const int pos = (int)c + lo - K;
+            sum_next[pos] = served ? fresh[j] : sum[j];
+            id_next[pos] = blk;
+            place[j] = pos;
+        }
+        __syncthreads();
+        const int m_next = m - *closed;
+        if (tid == 0) *closed_next = 0;
+        // ---- equal sums (masses are sums of bf16: a few per batch): entries that took one place are put in their
+        // order by (sum, block), one warp to an entry
+        int clash = 0;
+        for (int j = tid; j < m; j += nthr) {
+            if (place[j] >= 0 && id_next[place[j]] != id[j]) { shared_place[place[j]] = 1; clash = 1; }
+        }
+        if (__syncthreads_or(clash)) {
+            for (int j = tid; j < m; j += nthr)
+                if (place[j] >= 0 && shared_place[place[j]]) doubtful[atomicAdd(&red_open[2], 1)] = (unsigned short)j;
+            __syncthreads();
+            const int nd = red_open[2];
+            for (int e = warp; e < nd; e += nthr >> 5) {
+                const int j = doubtful[e], pj = place[j], blk = id[j];
+                const unsigned long long v = j < K ? fresh[j] : sum[j];
+                int before = 0;
+                for (int k = lane; k < m; k += 32)
+                    before += (place[k] == pj && md_less(k < K ? fresh[k] : sum[k], id[k], v, blk)) ? 1 : 0;
+                before = __reduce_add_sync(0xffffffffu, before);
+                if (lane == 0) { sum_next[pj + before] = v; id_next[pj + before] = blk; }
+            }
+            __syncthreads();
+            for (int e = tid; e < nd; e += nthr) shared_place[place[doubtful[e]]] = 0;
+            if (tid == 0) red_open[2] = 0;
+            __syncthreads();
+        }
+        ++batch;
+        { unsigned long long *t = sum; sum = sum_next; sum_next = t; int *u = id; id = id_next; id_next = u; }
+        m = m_next;
+        s += K;
     }
 }
 

@@ -776,6 +776,21 @@ def test_massdiff_on_the_device_matches_the_oracle(B, oracle, d, b):
     assert np.array_equal(got.cpu().numpy(), ref)
 
 
+@pytest.mark.parametrize("kind", ["equal", "two_values", "geometric", "zeros", "few_large"])
+@pytest.mark.parametrize("d,b", [(1024, 32), (2080, 32), (4096, 2), (8192, 16), (16384, 4), (32768, 128)])
+def test_massdiff_batches_match_the_host_function(B, kind, d, b):
+    """Equal running sums, batches of one, batches that end at a staged window, more blocks than threads."""
+    rng = np.random.default_rng(77 + d + b)
+    a = {"equal": np.ones(d), "two_values": rng.integers(1, 3, d), "geometric": 1.01 ** -np.arange(d).clip(0, 5000),
+         "zeros": np.zeros(d), "few_large": rng.exponential(size=d) * np.where(rng.random(d) < 0.002, 1e4, 1.0)}[kind]
+    a = rng.permutation(a.astype(np.float32))
+    dev = torch.empty(d + 1, device="cuda")[1:]          # 4-byte alignment is all the entry point asks for
+    dev.copy_(torch.from_numpy(a))
+    got = B.perq_massdiff_perm_device(dev, b)
+    torch.cuda.synchronize()
+    assert np.array_equal(got.cpu().numpy(), B.perq_massdiff_perm(a, b))
+
+
 def test_calibration_pass_stays_on_the_device(B, oracle):
     """statistic -> permutation -> permuted rotate+quantize without a host copy, against the oracle's chain."""
     w = inputs.config3(T=96)
