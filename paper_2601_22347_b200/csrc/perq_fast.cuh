@@ -319,13 +319,14 @@ __device__ __forceinline__ uint32_t hadamard_bf16(int k, int n) { return (__popc
 
 // ---------------------------------------------------------------- exact re-evaluation
 
-// bf16 bit pattern (low 16 bits of h) -> double, exactly, with integer operations (the
-// fp32->fp64 conversion instruction is slow); zero and subnormals take the conversion.
+// bf16 bit pattern (low 16 bits of h) -> double, exactly.  The pattern's exponent and mantissa fields, placed in
+// a double's, make the value times 2^-896 -- zeros and subnormals included, which become fp64 subnormals -- so one
+// exact product (part of a fused multiply-add where the value is added to a sum) completes the conversion.  (The
+// fp32 -> fp64 conversion instruction is slow, and compiled as a predicated alternative it cost every element of an
+// exact sum: 5400 cycles for one 14336-term sum by 14 warps, 1100 without it.)
 __device__ __forceinline__ double bf16_bits_to_f64(uint32_t h)
 {
-    const uint32_t mag = h & 0x7fffu;
-    if (mag < 0x80u) return (double)__uint_as_float(h << 16);
-    return __hiloint2double((int)(((mag << 13) + 0x38000000u) | ((h & 0x8000u) << 16)), 0);
+    return __hiloint2double((int)(((h & 0x7fffu) << 13) | ((h & 0x8000u) << 16)), 0) * 0x1p896;
 }
 
 // Exact unnormalised output i of the block starting at `blk` (bf16 in shared memory), evaluated
