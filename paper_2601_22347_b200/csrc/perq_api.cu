@@ -24,6 +24,7 @@
 #include "perq_stats.cuh"
 #include "perq_diag.cuh"
 #include "perq_massdiff.cuh"
+#include "perq_row.cuh"
 
 namespace {
 
@@ -192,6 +193,139 @@ int launch_generic(const void *x, const int32_t *perm, int64_t T, int32_t d, int
     return cudaGetLastError() == cudaSuccess ? PERQ_OK : PERQ_ERR_CUDA;
 }
 
+// Row kernel: a warp per 1024 channels, one CTA per row (short rows share one).  It takes every call that the
+// segment kernels do not and that it can hold (below); it was 1.1 to 17 times faster than the general kernel over all
+// of them (widths 768 .. 14336, 1 .. 4096 rows, all formats), which keeps the rest: other widths and ranges, fp32 output.
+template <int ROT, int MODE>
+int launch_row_inst(const perq::RowParams &p, int grid, int threads, size_t smem, cudaStream_t st)
+{
+    auto kernel = perq::perq_row_kernel<ROT, MODE>;
+    if (int rc = allow_smem(kernel, smem)) return rc;
+    if (launch_overlapped(kernel, grid, threads, smem, st, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return PERQ_ERR_CUDA;
+    }
+    return PERQ_OK;
+}
+
+template <int MODE>
+int launch_row_token(int rot, const perq::RowParams &p, int grid, int threads, size_t smem, cudaStream_t st)
+{
+    switch (rot) {
+    case perq::ROT_LOCAL: return launch_row_inst<perq::ROT_LOCAL, MODE>(p, grid, threads, smem, st);
+    case perq::ROT_WIDE: return launch_row_inst<perq::ROT_WIDE, MODE>(p, grid, threads, smem, st);
+    case perq::ROT_COL1: return launch_row_inst<perq::ROT_COL1, MODE>(p, grid, threads, smem, st);
+    case perq::ROT_COL2: return launch_row_inst<perq::ROT_COL2, MODE>(p, grid, threads, smem, st);
+    default: return launch_row_inst<perq::ROT_NP2, MODE>(p, grid, threads, smem, st);
+    }
+}
+
+int launch_row_mode(int rot, int mode, const perq::RowParams &p, int grid, int threads, size_t smem, cudaStream_t st)
+{
+    switch (mode) {
+    case perq::ROW_TOKEN: return launch_row_token<perq::ROW_TOKEN>(rot, p, grid, threads, smem, st);
+    case perq::ROW_FP4: return launch_row_token<perq::ROW_FP4>(rot, p, grid, threads, smem, st);
+    case perq::ROW_ASYM: return launch_row_token<perq::ROW_ASYM>(rot, p, grid, threads, smem, st);
+    case perq::ROW_MX:
+        if (rot == perq::ROT_LOCAL) return launch_row_inst<perq::ROT_LOCAL, perq::ROW_MX>(p, grid, threads, smem, st);
+        if (rot == perq::ROT_WIDE) return launch_row_inst<perq::ROT_WIDE, perq::ROW_MX>(p, grid, threads, smem, st);
+        return launch_row_inst<perq::ROT_NP2, perq::ROW_MX>(p, grid, threads, smem, st);
+    default:
+        if (rot == perq::ROT_LOCAL) return launch_row_inst<perq::ROT_LOCAL, perq::ROW_GROUP>(p, grid, threads, smem, st);
+        if (rot == perq::ROT_NP2) return launch_row_inst<perq::ROT_NP2, perq::ROW_GROUP>(p, grid, threads, smem, st);
+        return -1;                            // (ranges inside long blocks: the fp64 rotation)
+    }
+}
+
+// Returns -1 if the row kernel does not cover the call.
+int try_launch_row(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t b, int32_t fmt, int g,
+                   void *out_codes, void *out_scales, cudaStream_t st)
+{
+    const int n0 = base_order(b);
+    if (d > perq::ROW_MAX_D || T >= (1ll << 31)) return -1;
+    perq::RowParams p;
+    std::memset(&p, 0, sizeof(p));
+    if (n0 > 0) {
+        const int k = ilog2(b / n0);
+        if (b != d || k < 6 || k > 10) return -1;
+        p.log2b = k;
+        p.n0 = n0;
+        p.pad = perq::row_pad(n0);
+        base_matrix_rows(n0, p.hrow);
+        // stages: k on fp32 values, and the sum of n0 products on the tensor cores in steps of 16
+        p.err_rel = perq::FAST_ERR_K_FULL * (float)(k + 2 * ((n0 + 15) / 16)) * perq::TWO_M24;
+    } else {
+        if (n0 < 0 || d % 128 != 0 || b < 16) return -1;
+        p.log2b = ilog2(b);
+        const float per_stage = p.log2b <= 7 ? perq::FAST_ERR_K : p.log2b <= 9 ? perq::FAST_ERR_K_LONG : perq::FAST_ERR_K_FULL;
+        p.err_rel = per_stage * (float)p.log2b * perq::TWO_M24;
+    }
+    int mode;
+    if (fmt == PERQ_FMT_MXFP4) mode = perq::ROW_MX;
+    else if (fmt == PERQ_FMT_FP4) mode = perq::ROW_FP4;
+    else if (fmt == PERQ_FMT_INT4_ASYM) mode = perq::ROW_ASYM;
+    else if (fmt == PERQ_FMT_INT4 && g == d) mode = perq::ROW_TOKEN;
+    else if (fmt == PERQ_FMT_INT4 && is_pow2(g) && g >= 32 && g <= 1024) mode = perq::ROW_GROUP;
+    else return -1;
+    p.log2g = ilog2(g);
+    p.x = static_cast<const uint16_t *>(x);
+    p.perm = perm;
+    p.out_codes = static_cast<uint8_t *>(out_codes);
+    p.out_scales = out_scales;
+    p.T = (uint32_t)T;
+    p.d = d;
+    p.sqrt_b = std::sqrt((double)b);
+    p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);
+    p.inv_15_sqrt_b = 1.0 / (15.0 * p.sqrt_b);
+    const int segs = (d + perq::SEG_ELEMS - 1) / perq::SEG_ELEMS;
+    // per-range scales inside blocks of 256 and more: rotated in fp64, where every output is exact
+    const bool wide_ranges = mode == perq::ROW_GROUP && n0 == 0 && b >= 256 && g <= b;
+    // 2^k * 4t: the first pass has one task per output tile and quarter of the groups (two tiles up to k = 8)
+    const int tasks = n0 > 0 ? 4 * ((n0 + 7) / 8 + (p.log2b <= 8 ? 1 : 0)) / (p.log2b <= 8 ? 2 : 1) : 0;
+    p.row_warps = tasks > segs && tasks <= perq::ROW_MAX_WARPS ? tasks : segs;
+    size_t o = 0;
+    auto take = [&o](size_t bytes) { const size_t at = o; o += (bytes + 127) & ~(size_t)127; return (uint32_t)at; };
+    p.off_perm = perm ? take((size_t)d * 2) : 0;
+    if (n0 > 0) {
+        p.off_quad = take((size_t)d / 4 * 2);
+        p.off_bmat = take((size_t)perq::row_base_np(n0) * perq::gen_base_ldk(n0) * 2);
+        p.off_hrow = take((size_t)n0 * 12);
+    }
+    o = (o + 1023) & ~(size_t)1023;
+    p.off_group = (uint32_t)o;
+    o = (size_t)perq::ROW_NSTAGE * segs * perq::SEG_BYTES;
+    p.off_xs = perm ? take((size_t)segs * perq::SEG_BYTES) : 0;
+    p.off_tile = wide_ranges ? take((size_t)segs * perq::ROW64_TILE)
+                             : take((size_t)d * 4 + (n0 > 0 ? (size_t)p.pad * 4 * (size_t)(d / n0 / 8) : 0));
+    p.off_misc = take(wide_ranges ? (size_t)perq::ROW_NSTAGE * 8 : sizeof(perq::RowMisc));
+    p.group_bytes = (uint32_t)((o + 1023) & ~(size_t)1023);
+    const size_t fixed = p.off_group + 1024;             // tables, and room to align the base
+    if (fixed + p.group_bytes > kMaxSmem) return -1;
+    const int sms = sm_count();
+    if (sms <= 0) return PERQ_ERR_CUDA;
+    // rows in flight per SM: what registers and shared memory allow, but few rows are spread over the SMs first
+    int groups = (wide_ranges ? perq::ROW64_CTA_WARPS : perq::ROW_CTA_WARPS) / p.row_warps;
+    groups = std::min<int>(std::max(groups, 1), (int)((kMaxSmem - fixed) / p.group_bytes));
+    groups = (int)std::min<long long>(groups, (T + sms - 1) / sms);
+    const int per_sm = std::max(1, std::min((wide_ranges ? perq::ROW64_SM_WARPS : perq::ROW_SM_WARPS) / (groups * p.row_warps),
+                                            (int)(kMaxSmem / (fixed + (size_t)groups * p.group_bytes + 1024))));
+    const int grid = (int)std::min<long long>((T + groups - 1) / groups, (long long)sms * per_sm);
+    const int threads = groups * p.row_warps * 32;
+    const size_t smem = fixed + (size_t)groups * p.group_bytes;
+    if (wide_ranges) {
+        if (int rc = allow_smem(perq::perq_row64_kernel, smem)) return rc;
+        if (launch_overlapped(perq::perq_row64_kernel, grid, threads, smem, st, p) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return PERQ_ERR_CUDA;
+        }
+        return PERQ_OK;
+    }
+    const bool columns = mode == perq::ROW_TOKEN || mode == perq::ROW_FP4 || mode == perq::ROW_ASYM;
+    const int rot = n0 > 0 ? perq::ROT_NP2 : p.log2b <= perq::ROW_WARP_LOG2B ? perq::ROT_LOCAL
+                  : columns && b == 4096 ? perq::ROT_COL1 : columns && b == 2048 ? perq::ROT_COL2 : perq::ROT_WIDE;
+    return launch_row_mode(rot, mode, p, grid, threads, smem, st);
+}
+
 template <int LOG2B, int MODE, int LOG2G, bool PERM, int XB>
 int launch_fast_inst(const perq::FastParams &p, int grid, cudaStream_t st)
 {
@@ -243,18 +377,6 @@ int launch_fast_mode(int mode, int G, int log2b, const perq::FastParams &p, int 
     case 4: return launch_fast_b<perq::MODE_TOKEN, 2, PERM>(log2b, p, grid, st);
     case 8: return launch_fast_b<perq::MODE_TOKEN, 3, PERM>(log2b, p, grid, st);
     default: return launch_fast_b<perq::MODE_TOKEN, -1, PERM>(log2b, p, grid, st);   // any other row length: G at run time
-    }
-}
-
-// full-vector block (b == d): unpermuted, per-token INT4 or MXFP4
-template <int MODE>
-int launch_fast_full(int G, const perq::FastParams &p, int grid, cudaStream_t st)
-{
-    switch (G) {
-    case 1: return launch_fast_inst<7, MODE, 0, false, 3>(p, grid, st);
-    case 2: return launch_fast_inst<7, MODE, 1, false, 4>(p, grid, st);
-    case 4: return launch_fast_inst<7, MODE, 2, false, 5>(p, grid, st);
-    default: return launch_fast_inst<7, MODE, 3, false, 6>(p, grid, st);
     }
 }
 
@@ -361,9 +483,9 @@ int launch_tok(int segs, int log2b, const perq::FastParams &p, int grid, cudaStr
     }
 }
 
-// The fast kernel covers d % 1024 == 0 with b <= 128 and scales per token (d / 1024 in {1,2,4,8}),
-// per 128 (INT4) or per 32 (MXFP4), with a permutation also d <= 16384; and b == d in {1024 .. 8192}
-// without a permutation, per token or MXFP4.  Returns -1 if it does not apply.
+// The segment kernels cover d % 1024 == 0 with b <= 128 and scales per token (up to 15 segments), per 128 (INT4) or
+// per 32 (MXFP4), with a permutation also d <= 16384; blocks of 256 .. 1024 inside a longer row and b == d (MXFP4: up
+// to 8192, per token: 1024) without a permutation.  Returns -1 if they do not apply.
 int try_launch_fast(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t b, int32_t fmt, int g,
                     void *out_codes, void *out_scales, cudaStream_t st)
 {
@@ -374,6 +496,9 @@ int try_launch_fast(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     const bool longb = !full && b > 128;                  // 256, 512 or 1024 inside a longer row
     if (longb && (b > perq::SEG_ELEMS || permuted)) return -1;
     if (full && (permuted || (segs != 1 && segs != 2 && segs != 4 && segs != 8))) return -1;
+    // whole-row blocks with one INT4 scale: one warp per row keeps them in registers; from two warps on the row
+    // kernel's exchange is the better one (4096 rows: 13.0 us here, 16.7 there at 1024; 57.0 and 31.2 at 4096)
+    if (full && fmt == PERQ_FMT_INT4 && segs > 1) return -1;
     if (permuted && (d > perq::FastSmem::PERM_MAX_D || segs > perq::FAST_WARPS)) return -1;
     int mode, G = 1;
     if (fmt == PERQ_FMT_MXFP4) {
@@ -430,9 +555,8 @@ int try_launch_fast(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     }
     if (full && mode == perq::MODE_MX && segs <= 4)          // (units are rows; grid as computed above)
         return launch_full<perq::MODE_MX>(segs, p, grid, st);
-    if (full)
-        return mode == perq::MODE_MX ? launch_fast_full<perq::MODE_MX>(G, p, grid, st)
-                                     : launch_fast_full<perq::MODE_TOKEN>(G, p, grid, st);
+    if (full && mode == perq::MODE_MX) return launch_fast_inst<7, perq::MODE_MX, 3, false, 6>(p, grid, st);
+    if (full) return launch_fast_inst<7, perq::MODE_TOKEN, 0, false, 3>(p, grid, st);
     if (longb)
         return mode == perq::MODE_MX ? launch_fast_long<perq::MODE_MX>(ilog2(b) - 7, G, p, grid, st)
                                      : launch_fast_long<perq::MODE_TOKEN>(ilog2(b) - 7, G, p, grid, st);
@@ -472,6 +596,8 @@ int launch_any(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t
         const int rc = try_launch_fast(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
         if (rc >= 0) return rc;
     }
+    const int rc = try_launch_row(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
+    if (rc >= 0) return rc;
     return launch_generic(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
 }
 

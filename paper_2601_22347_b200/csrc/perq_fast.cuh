@@ -2,7 +2,7 @@
 //   b <= 128              every scale mode (INT4 per token / per 128, MXFP4, FP4 per token, asymmetric
 //                         INT4 per token), with or without a permutation (permuted: d <= 16384);
 //   b in {256, 512, 1024} unpermuted, INT4 per token or MXFP4;
-//   b == d <= 8192        unpermuted, INT4 per token or MXFP4 (full-vector rotation).
+//   b == d                unpermuted (full-vector rotation): 1024 INT4 per token, 8192 MXFP4.
 // Per-token scales need G <= 15 (one named barrier per group of G warps).
 //
 // Data path (HBM-bound, one pass):

@@ -16,7 +16,9 @@
 // The greedy is a serial chain: one channel at a time (a scan of all running sums per channel) it took 2316 us, in
 // batches it takes 164 us
 // for 8192 channels in 256 blocks.  Sums differ by about one channel mass, so a batch serves most of the
-// blocks: 64 batches there, 31 to 157 for 8 to 512 blocks of real statistics.
+// blocks: 64 batches there, 31 to 157 for 8 to 512 blocks of real statistics.  Masses that fall steeply make small
+// batches; then channels are served one by one for a while, each an insertion into the list by all threads at one
+// barrier.  Zero masses (padded channels) change no sum: what is left of them fills the blocks in list order.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -39,10 +41,10 @@ struct MassdiffParams {
     int d, b;
 };
 
-// Shared memory of the greedy: two lists (sum, block), the new sums, fill counts, the channel window, and a
-// few words of reduction space.
+// Shared memory of the greedy: two lists (sum; block and its fill count in one word), the new sums, fp32 distances,
+// the channel window, and a few words of reduction space.
 struct MdSmem {
-    size_t sum0, sum1, fresh, key, key_old, id0, id1, fill, place, shared_place, doubtful, chan, mass, red, total;
+    size_t sum0, sum1, fresh, key, key_old, id0, id1, place, crowded, doubtful, chan, mass, red, total;
     __host__ __device__ explicit MdSmem(int n)
     {
         const size_t m = ((size_t)n + 3) & ~(size_t)3;
@@ -54,9 +56,8 @@ struct MdSmem {
         key_old = o; o += m * 4;
         id0 = o;   o += m * 4;
         id1 = o;   o += m * 4;
-        fill = o;  o += m * 4;
         place = o; o += m * 4;
-        shared_place = o; o += m;
+        crowded = o; o += m;
         doubtful = o; o += m * 2;
         o = (o + 15) & ~(size_t)15;
         chan = o;  o += (size_t)MD_WINDOW * 4;
@@ -124,8 +125,17 @@ __global__ void __launch_bounds__(MD_RANK_THREADS) perq_massdiff_rank_kernel(Mas
     }
 }
 
-// Running sums are non-negative doubles, so their bit patterns order like the values.
-__device__ __forceinline__ bool md_less(unsigned long long s, int i, unsigned long long t, int j) { return s < t || (s == t && i < j); }
+// Running sums are non-negative doubles, so their bit patterns order like the values.  An entry's second word:
+// block in the low MD_ID_BITS bits, channels it has received above them.
+constexpr int MD_ID_BITS = 13;
+constexpr int MD_ID_MASK = (1 << MD_ID_BITS) - 1;
+__device__ __forceinline__ bool md_less(unsigned long long s, int i, unsigned long long t, int j)
+{
+    return s < t || (s == t && (i & MD_ID_MASK) < (j & MD_ID_MASK));
+}
+
+constexpr int MD_SERIAL_K = 6;           // batches below this are followed by MD_SERIAL_STEPS channels one by one
+constexpr int MD_SERIAL_STEPS = 32;
 
 __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel(MassdiffParams p)
 {
@@ -136,24 +146,28 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
     unsigned long long *fresh = (unsigned long long *)(md_smem + lay.fresh);
     float *key = (float *)(md_smem + lay.key), *key_old = (float *)(md_smem + lay.key_old);
     int *id = (int *)(md_smem + lay.id0), *id_next = (int *)(md_smem + lay.id1);
-    int *fill = (int *)(md_smem + lay.fill), *place = (int *)(md_smem + lay.place);
-    unsigned char *shared_place = md_smem + lay.shared_place;
+    int *place = (int *)(md_smem + lay.place), *chan = (int *)(md_smem + lay.chan);
+    unsigned char *crowded = md_smem + lay.crowded;
     unsigned short *doubtful = (unsigned short *)(md_smem + lay.doubtful);
-    int *chan = (int *)(md_smem + lay.chan);
     float *mass = (float *)(md_smem + lay.mass);
     unsigned long long *red_sum = (unsigned long long *)(md_smem + lay.red);
     int *red_id = (int *)(md_smem + lay.red + 32 * 8), *red_open = (int *)(md_smem + lay.red + 32 * 12);
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const unsigned long long INF = 0x7ff0000000000000ull;
+    auto swap_lists = [&]() {
+        unsigned long long *t = sum; sum = sum_next; sum_next = t;
+        int *u = id; id = id_next; id_next = u;
+    };
 
-    for (int j = tid; j < n; j += nthr) { sum[j] = 0ull; id[j] = j; fill[j] = 0; shared_place[j] = 0; }
-    if (tid < 32) { red_sum[tid] = INF; red_id[tid] = 0x7fffffff; red_open[tid] = 0; }
+    for (int j = tid; j < n; j += nthr) { sum[j] = 0ull; id[j] = j; crowded[j] = 0; }
+    if (tid < 32) { red_sum[tid] = INF; red_id[tid] = MD_ID_MASK; red_open[tid] = 0; }
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();
     int split = 0;              // log2 of the threads that count for one entry
     while (split < 1 && (n << (split + 1)) <= nthr) ++split;
     int m = n;                  // open blocks: list entries [0, m)
     int s = 0, w0 = 0, w1 = 0;  // next rank; staged window of ranks [w0, w1)
+    int serial = 0;             // channels still to be served one by one
     uint32_t batch = 0;
     while (s < d) {
         if (s >= w1) {
@@ -167,21 +181,46 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             }
             __syncthreads();
         }
+        if (mass[s - w0] == 0.0f) break;          // (only zero masses are left: below)
+        if (serial > 0) {
+            // ---- one channel: the first entry takes it and moves to its new place (one barrier)
+            --serial;
+            const unsigned long long s0 = sum[0];
+            const int e0 = id[0], f = e0 >> MD_ID_BITS;
+            const bool full = f + 1 == b;
+            const double ns = __longlong_as_double((long long)s0) + (double)mass[s - w0];
+            const unsigned long long v = (unsigned long long)__double_as_longlong(ns);
+            const int e1 = e0 + (1 << MD_ID_BITS);
+            for (int j = tid; j < m; j += nthr) {
+                if (j == 0) p.perm[(size_t)(e0 & MD_ID_MASK) * b + f] = chan[s - w0];
+                // entries 1 .. below the new sum move up by one place; the new sum goes behind them
+                const bool below = j > 0 && (full || md_less(sum[j], id[j], v, e1));
+                const bool next_below = j + 1 < m && (full || md_less(sum[j + 1], id[j + 1], v, e1));
+                if (below) { sum_next[j - 1] = sum[j]; id_next[j - 1] = id[j]; }
+                else if (j > 0) { sum_next[j] = sum[j]; id_next[j] = id[j]; }
+                if (!full && (below || j == 0) && !next_below) { sum_next[j] = v; id_next[j] = e1; }
+            }
+            if (full) --m;
+            ++s;
+            __syncthreads();
+            swap_lists();
+            continue;
+        }
         // ---- the sums that the next q blocks of the list would reach, and the smallest of them
         const int q = min(m, w1 - s);
         unsigned long long best = INF;
-        int best_id = 0x7fffffff;
+        int best_id = MD_ID_MASK;
         for (int j = tid; j < q; j += nthr) {
             const double ns = __longlong_as_double((long long)sum[j]) + (double)mass[s - w0 + j];
-            const unsigned long long v = (fill[id[j]] + 1 < b) ? (unsigned long long)__double_as_longlong(ns) : INF;
+            const unsigned long long v = ((id[j] >> MD_ID_BITS) + 1 < b) ? (unsigned long long)__double_as_longlong(ns) : INF;
             fresh[j] = v;
-            if (v != INF && md_less(v, id[j], best, best_id)) { best = v; best_id = id[j]; }
+            if (v != INF && md_less(v, id[j], best, best_id)) { best = v; best_id = id[j] & MD_ID_MASK; }
         }
         {
             const uint32_t hi = (uint32_t)(best >> 32), lo = (uint32_t)best;
             const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
             const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-            const int mid = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)best_id : 0x7fffffffu);
+            const int mid = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)best_id : (uint32_t)MD_ID_MASK);
             if (lane == 0) { red_sum[warp] = ((unsigned long long)mhi << 32) | mlo; red_id[warp] = mid; }
         }
         __syncthreads();
@@ -193,7 +232,7 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
             const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
             const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-            M_id = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)vi : 0x7fffffffu);
+            M_id = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)vi : (uint32_t)MD_ID_MASK);
             M = ((unsigned long long)mhi << 32) | mlo;
         }
         // ---- K: the list entries up to M.  Distances of all sums to M in fp32 (sums within a batch are close
@@ -211,7 +250,8 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
         K = max(K, 1);
         // ---- serve them; every entry's place in the merged list: new sums below it (counted, 2^split threads
         // to an entry), and for a new sum the untouched entries below it (searched).  fp32 distances to M
-        // decide; equal ones show below as two entries that took one place.
+        // decide; equal ones (masses are sums of bf16: equal sums do occur, a few per batch) show as entries that
+        // took one place.
         int *closed = red_open + (batch & 1u), *closed_next = red_open + ((batch + 1) & 1u);
         for (int j0 = 0; j0 < m; j0 += nthr >> split) {
             const int j = j0 + (tid >> split), sub = tid & ((1 << split) - 1);
@@ -231,13 +271,14 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             }
             for (int o = 1; o < (1 << split); o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
             if (!in || sub != 0) continue;
-            const int blk = id[j];
+            int blk = id[j];
+            const unsigned long long v64 = served ? fresh[j] : sum[j];
             if (served) {
-                const int f = fill[blk];
-                p.perm[(size_t)blk * b + f] = chan[s - w0 + j];
-                fill[blk] = f + 1;
-                if (fresh[j] == INF) { place[j] = -1; atomicAdd(closed, 1); continue; }
+                p.perm[(size_t)(blk & MD_ID_MASK) * b + (blk >> MD_ID_BITS)] = chan[s - w0 + j];
+                blk += 1 << MD_ID_BITS;
+                if (v64 == INF) { place[j] = -1; atomicAdd(closed, 1); continue; }
             }
+            // (untouched entries are in order; equal distances among them share the first one's place)
             int lo = K, hi = served ? m : j;
             if (served || (j > K && !(key_old[j - 1] < v))) {
                 while (lo < hi) {
@@ -248,42 +289,51 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
                 lo = j;
             }
             const int pos = (int)c + lo - K;
-            sum_next[pos] = served ? fresh[j] : sum[j];
+            sum_next[pos] = v64;
             id_next[pos] = blk;
             place[j] = pos;
         }
         __syncthreads();
-        const int m_next = m - *closed;
-        if (tid == 0) *closed_next = 0;
-        // ---- equal sums (masses are sums of bf16: a few per batch): entries that took one place are put in their
-        // order by (sum, block), one warp to an entry
+        // ---- entries that took one place are put in their order by (sum, block), one warp to an entry
         int clash = 0;
         for (int j = tid; j < m; j += nthr) {
-            if (place[j] >= 0 && id_next[place[j]] != id[j]) { shared_place[place[j]] = 1; clash = 1; }
+            const int pj = place[j];
+            if (pj >= 0 && ((id_next[pj] ^ id[j]) & MD_ID_MASK) != 0) { crowded[pj] = 1; clash = 1; }
         }
         if (__syncthreads_or(clash)) {
             for (int j = tid; j < m; j += nthr)
-                if (place[j] >= 0 && shared_place[place[j]]) doubtful[atomicAdd(&red_open[2], 1)] = (unsigned short)j;
+                if (place[j] >= 0 && crowded[place[j]]) doubtful[atomicAdd(&red_open[2], 1)] = (unsigned short)j;
             __syncthreads();
             const int nd = red_open[2];
             for (int e = warp; e < nd; e += nthr >> 5) {
                 const int j = doubtful[e], pj = place[j], blk = id[j];
-                const unsigned long long v = j < K ? fresh[j] : sum[j];
+                const unsigned long long v64 = j < K ? fresh[j] : sum[j];
                 int before = 0;
                 for (int k = lane; k < m; k += 32)
-                    before += (place[k] == pj && md_less(k < K ? fresh[k] : sum[k], id[k], v, blk)) ? 1 : 0;
+                    before += (place[k] == pj && md_less(k < K ? fresh[k] : sum[k], id[k], v64, blk)) ? 1 : 0;
                 before = __reduce_add_sync(0xffffffffu, before);
-                if (lane == 0) { sum_next[pj + before] = v; id_next[pj + before] = blk; }
+                if (lane == 0) { sum_next[pj + before] = v64; id_next[pj + before] = blk + (j < K ? 1 << MD_ID_BITS : 0); }
             }
             __syncthreads();
-            for (int e = tid; e < nd; e += nthr) shared_place[place[doubtful[e]]] = 0;
+            for (int e = tid; e < nd; e += nthr) crowded[place[doubtful[e]]] = 0;
             if (tid == 0) red_open[2] = 0;
-            __syncthreads();
         }
-        ++batch;
-        { unsigned long long *t = sum; sum = sum_next; sum_next = t; int *u = id; id = id_next; id_next = u; }
-        m = m_next;
+        if (tid == 0) *closed_next = 0;
+        __syncthreads();
+        m -= *closed;
         s += K;
+        ++batch;
+        if (K < MD_SERIAL_K && K < q) serial = MD_SERIAL_STEPS;
+        swap_lists();
+    }
+    // ---- zero masses change no sum: the blocks of the list take what they have room for, one after the other
+    if (s < d) {
+        for (int r = s + tid; r < d; r += nthr) {
+            const int c = min(max(p.order[r], 0), d - 1);
+            int left = r - s, j = 0;
+            while (j < m && left >= b - (id[j] >> MD_ID_BITS)) { left -= b - (id[j] >> MD_ID_BITS); ++j; }
+            if (j < m) p.perm[(size_t)(id[j] & MD_ID_MASK) * b + (id[j] >> MD_ID_BITS) + left] = c;
+        }
     }
 }
 

@@ -818,3 +818,53 @@ def test_chan_abs_max_and_the_comparison_permutations(B, oracle, T, d):
     b = 32
     assert np.array_equal(B.perq_zigzag_perm(got.cpu().numpy(), b), oracle.zigzag_perm(ref, b))
     assert np.array_equal(B.perq_absmax_perm(got.cpu().numpy()), oracle.absmax_perm(ref))
+
+
+# ------------------------------------------------------------------ row kernel: ragged widths, long blocks, 2^k * 4t
+
+def _row_inputs(T, d, seed):
+    """Ordinary rows, a zero row, a row with one nonzero (every output of its block is a candidate for the maximum),
+    a constant row, a row of +-1, rows at the ends of the exponent range."""
+    bits, _ = inputs.laplace_outliers(T, d, 3, 200.0, seed)
+    x = inputs.bf16_bits_to_f32(bits)
+    x[0] = 0.0
+    if T > 6:
+        x[1] = 0.0
+        x[1, d // 3] = 2.5
+        x[2] = 1.0
+        x[3] = np.where(np.random.default_rng(seed).random(d) < 0.5, -1.0, 1.0)
+        x[4] *= 2.0 ** -120
+        x[5] *= 2.0 ** 90
+    return inputs.f32_to_bf16_bits(x)
+
+
+ROW_FORMATS = [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0), ("int4_asym", 0)]
+
+
+@pytest.mark.parametrize("fmt,group", ROW_FORMATS)
+@pytest.mark.parametrize("d,b,T,perm", [(128, 16, 9, False), (128, 128, 7, True), (1152, 32, 400, True), (1920, 64, 8, False),
+                                        (3200, 128, 2000, False), (9728, 16, 9, True), (16256, 128, 8, True),
+                                        (1536, 512, 9, False), (2048, 1024, 700, True), (16384, 256, 7, True)])
+def test_row_kernel_ragged_widths_and_blocks_inside_a_segment(B, oracle, d, b, T, perm, fmt, group):
+    bits = _row_inputs(T, d, 7000 + d + b)
+    w = inputs.Workload("row", bits, inputs.random_perm(d, 71) if perm else None, b, fmt, group, 0)
+    check(B, oracle, w, rows=np.unique(np.r_[0:min(T, 8), T - 1]))
+
+
+@pytest.mark.parametrize("fmt,group", ROW_FORMATS)
+@pytest.mark.parametrize("d,b,T,perm", [(2048, 2048, 300, False), (4096, 4096, 750, False), (8192, 4096, 9, True), (6144, 2048, 8, False),
+                                        (8192, 8192, 8, True), (16384, 16384, 7, False), (14336, 2048, 7, True),
+                                        (768, 768, 12, True), (2304, 2304, 9, False), (3840, 3840, 300, False), (12288, 12288, 8, False)])
+def test_row_kernel_blocks_over_several_warps(B, oracle, d, b, T, perm, fmt, group):
+    bits = _row_inputs(T, d, 7100 + d + b)
+    w = inputs.Workload("row-wide", bits, inputs.random_perm(d, 72) if perm else None, b, fmt, group, 0)
+    check(B, oracle, w, rows=np.unique(np.r_[0:min(T, 8), T - 1]))
+
+
+@pytest.mark.parametrize("group", [32, 64, 256, 512, 1024])
+@pytest.mark.parametrize("d,b", [(1024, 32), (3072, 1024), (4096, 2048), (5120, 512)])
+def test_row_kernel_scale_ranges(B, oracle, d, b, group):
+    if group % b and b % group:
+        pytest.skip("ranges are parts or multiples of a block")
+    bits = _row_inputs(40, d, 7200 + d + b)
+    check(B, oracle, inputs.Workload("row-range", bits, inputs.random_perm(d, 73), b, "int4", group, 0))
