@@ -329,6 +329,9 @@ __device__ __forceinline__ double bf16_bits_to_f64(uint32_t h)
     return __hiloint2double((int)(((h & 0x7fffu) << 13) | ((h & 0x8000u) << 16)), 0) * 0x1p896;
 }
 
+// The value times 2^-896 of the bf16 pattern in the high half of w (the low half is ignored).
+__device__ __forceinline__ double bf16_raw_f64(uint32_t w) { return __hiloint2double((int)((uint32_t)((int)w >> 3) & 0x8fffe000u), 0); }
+
 // Exact unnormalised output i of the block starting at `blk` (bf16 in shared memory), evaluated
 // by the 4 lanes of a quad: each lane reduces a quarter of the block with a signed pairwise
 // tree in fp64, then the quarters are combined.  q = lane % 4, qmask = the quad's lanes.
@@ -341,8 +344,8 @@ __device__ __forceinline__ double exact_coord_quad(const uint16_t *blk, int i, i
 #pragma unroll
     for (int r = 0; r < PER / 2; ++r) {
         const uint32_t w = src[r];
-        v[2 * r] = bf16_bits_to_f64(w);
-        v[2 * r + 1] = bf16_bits_to_f64(w >> 16);
+        v[2 * r] = bf16_raw_f64(w << 16);
+        v[2 * r + 1] = bf16_raw_f64(w);
     }
 #pragma unroll
     for (int t = 0; (1 << t) < PER; ++t) {
@@ -353,7 +356,49 @@ __device__ __forceinline__ double exact_coord_quad(const uint16_t *blk, int i, i
     double part = (__popc(i & (q << (LOG2B - 2))) & 1) ? -v[0] : v[0];
     part += __shfl_xor_sync(qmask, part, 1);
     part += __shfl_xor_sync(qmask, part, 2);
-    return part;
+    return part * 0x1p896;
+}
+
+// Largest magnitude of the exact unnormalised outputs i0 .. i0+3 (i0 a multiple of 4) of the block starting at blk,
+// by the 4 lanes of a quad, every quad with a slot of its own (all lanes of the warp call; the same value in the
+// four lanes).  A lane adds its quarter of the inputs, signed by the high bits of i0, in four sums by k & 3; summed
+// over the quad, a 4-point butterfly gives the four outputs.  Inputs enter as their fields in a double (times
+// 2^-896, see bf16_bits_to_f64), the sums are scaled at the end.  No element of the slot has to be singled out, and
+// it costs what one output costs (16-byte loads: 8 inputs 64 bytes apart per lane, the odd lane groups one step
+// ahead, so that the two quads of a quarter warp read different banks).
+template <int LOG2B>
+__device__ __forceinline__ double exact_slot_max_quad(const uint16_t *blk, int i0, int lane)
+{
+    const int q = lane & 3;
+    double S[4] = {0.0, 0.0, 0.0, 0.0};
+    if (LOG2B == 4) {
+        const uint2 w2 = *reinterpret_cast<const uint2 *>(blk + 4 * q);
+        const uint32_t flip = (__popc(i0 & (4 * q)) & 1) ? 0x80008000u : 0u, w[2] = {w2.x ^ flip, w2.y ^ flip};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) S[e] = bf16_raw_f64((e & 1) ? w[e >> 1] : w[e >> 1] << 16);
+    } else {
+        constexpr int STEPS = LOG2B >= 5 ? (1 << LOG2B) / 32 : 1;
+#pragma unroll
+        for (int t = 0; t < STEPS; ++t) {
+            const int c = 4 * (t ^ ((lane >> 2) & (STEPS > 1 ? 1 : 0))) + q;
+            const uint4 w4 = reinterpret_cast<const uint4 *>(blk)[c];
+            const uint32_t base = (__popc(i0 & (8 * c)) & 1) ? 0x80008000u : 0u, high = (i0 & 4) ? base ^ 0x80008000u : base;
+            const uint32_t w[4] = {w4.x ^ base, w4.y ^ base, w4.z ^ high, w4.w ^ high};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                S[2 * (j & 1)] += bf16_raw_f64(w[j] << 16);
+                S[2 * (j & 1) + 1] += bf16_raw_f64(w[j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) S[e] += __shfl_xor_sync(0xffffffffu, S[e], o);
+    }
+    const double a0 = S[0] + S[1], a1 = S[0] - S[1], a2 = S[2] + S[3], a3 = S[2] - S[3];
+    // |a +- b| is largest as |a| + |b|
+    return fmax(fabs(a0) + fabs(a2), fabs(a1) + fabs(a3)) * 0x1p896;
 }
 
 // Exact unnormalised output i of the B-element block at blk, by a whole warp.
@@ -471,24 +516,6 @@ __device__ __forceinline__ void locate(int g, int q, int e, int &blk_elem, int &
     elem = p * 16 + 4 * q + j;
     blk_elem = (p >> CB) << LOG2B;
     i = elem - blk_elem;
-}
-
-// Bit mask of the lane's 32 held values (bit s*4+j) whose magnitude reaches thr; ms[s] is the
-// magnitude maximum of slot s, used to skip slots.
-__device__ __forceinline__ uint32_t candidate_mask(const f32x2 (&v)[8][2], const float (&ms)[8], float thr)
-{
-    uint32_t cm = 0u;
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-        if (ms[s] >= thr) {
-            const float a = v[s][0].x, b = v[s][0].y, c = v[s][1].x, d = v[s][1].y;
-            cm |= (fabsf(a) >= thr ? 1u : 0u) << (4 * s);
-            cm |= (fabsf(b) >= thr ? 2u : 0u) << (4 * s);
-            cm |= (fabsf(c) >= thr ? 4u : 0u) << (4 * s);
-            cm |= (fabsf(d) >= thr ? 8u : 0u) << (4 * s);
-        }
-    }
-    return cm;
 }
 
 // Exact maximum magnitude (bit pattern of a non-negative double, the same in every lane) over the
@@ -1475,26 +1502,23 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                     wreq[nreq + __popc(enq & ((1u << lane) - 1u))] = ((unsigned long long)seg_index << 32) | my_pos;
                 nreq += __popc(enq);
                 if (!(a32 > 0.0f) && q == 0) reinterpret_cast<float *>(p.out_scales)[seg_index * 8 + g] = 0.0f;
-                // rare: several candidates in a quad are evaluated now, by the quad
-                const bool has_cand = !simple && (a32 > 0.0f) && (lane_max >= thr);
-                unsigned cq = __ballot_sync(0xffffffffu, has_cand) & qmask;
-                if (__any_sync(0xffffffffu, cq != 0u)) {
+                // otherwise: the candidate slots are evaluated now, every quad taking its slots in turn
+                uint32_t todo = simple ? 0u : slot_mask;
+                if (__any_sync(0xffffffffu, todo != 0u)) {
                     double a_exact = 0.0;
-                    while (cq) {
-                        const int src = __ffs(cq) - 1;
-                        cq &= cq - 1;
-                        uint32_t cm = 0u;
-                        if (lane == src) cm = candidate_mask(v, ms, thr);
-                        cm = __shfl_sync(qmask, cm, src);
-                        while (cm) {
-                            const int e = __ffs(cm) - 1;
-                            cm &= cm - 1;
-                            int blk_elem, i, elem;
-                            locate<LOG2B>(src >> 2, src & 3, e, blk_elem, i, elem);
-                            a_exact = fmax(a_exact, fabs(exact_coord_quad<LOG2B>(seg + blk_elem, i, q, qmask)));
-                        }
+                    unsigned cl = __ballot_sync(0xffffffffu, todo != 0u);
+                    while (cl) {                                   // (warp-uniform: quads without a slot repeat their first)
+                        const unsigned mine = (cl >> (lane & 28)) & 0xFu;
+                        const int src = (lane & 28) | ((__ffs(mine) - 1) & 3);
+                        const uint32_t sm = __shfl_sync(0xffffffffu, todo, src);
+                        const int sl = (__ffs(sm) - 1) & 7;
+                        const int pch = g * 8 + (sl ^ (f_g & ~PM)), blk_elem = (pch >> CB) << LOG2B;
+                        const double val = exact_slot_max_quad<LOG2B>(seg + blk_elem, pch * 16 - blk_elem + 4 * (src & 3), lane);
+                        if (sm != 0u) a_exact = fmax(a_exact, val);
+                        if (lane == src) todo &= todo - 1;
+                        cl = __ballot_sync(0xffffffffu, todo != 0u);
                     }
-                    if (has_cand || (!simple && (a32 > 0.0f))) {
+                    if (!simple && a32 > 0.0f) {
                         if (q == 0)
                             reinterpret_cast<float *>(p.out_scales)[seg_index * 8 + g] =
                                 (a_exact == 0.0) ? 0.0f : (float)(a_exact * p.inv_7_sqrt_b);
