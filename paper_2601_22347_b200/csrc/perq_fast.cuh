@@ -877,6 +877,10 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     const int GROUPS = FAST_WARPS / G;
     const uint32_t UNIT_BYTES = (uint32_t)G * SEG_BYTES;
     constexpr float MAGIC = 12582920.0f;          // 1.5 * 2^23 + 8: low nibble of the sum = code + 8
+    // per token: a pinned maximum is recorded and evaluated later (not where the inputs in global memory are not the
+    // row's: gated rows; nor where one lane's evaluation reads much more than the row's warp has at hand: 64 and 128
+    // inputs through a permutation, or for both extremes of an asymmetric row)
+    constexpr bool DEFER_TOK = !SWIGLU && !(LOG2B > 5 && (PERM || MODE == MODE_ASYM));
     static_assert(TOK || LOG2G == 0 || WBITS > 0, "only per-token scales or a full-vector block couple the warps of a row");
     extern __shared__ __align__(128) unsigned char fsmem_raw[];
     // 1024-byte aligned base: the ldmatrix and code-store addresses below are formed with XOR
@@ -1299,8 +1303,8 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                 const bool mine_hi = (cand_hi >> w_in_g) & 1u, mine_lo = (cand_lo >> w_in_g) & 1u;
                 if (one_each) {
                     unsigned long long e_hi = 0ull, e_lo = 0ull;
-                    if (mine_hi) e_hi = side_entry(true, true);
-                    if (mine_lo) e_lo = side_entry(false, true);
+                    if (mine_hi) e_hi = side_entry(true, DEFER_TOK);
+                    if (mine_lo) e_lo = side_entry(false, DEFER_TOK);
                     if (lane == 0) {
                         if (mine_hi) wpub[pidx] = e_hi;
                         if (mine_lo) wpub2[pidx] = e_lo;
@@ -1562,7 +1566,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                 const unsigned cl = __ballot_sync(0xffffffffu, slot_mask != 0u);
                 const int src = __ffs(cl) - 1;
                 const uint32_t sm = __shfl_sync(0xffffffffu, slot_mask, src);
-                if (!SWIGLU && ncand == 1 && (cl & (cl - 1)) == 0u && (sm & (sm - 1)) == 0u) {
+                if (DEFER_TOK && ncand == 1 && (cl & (cl - 1)) == 0u && (sm & (sm - 1)) == 0u) {
                     // one slot holds the maximum: record it, the scale is stored later
                     const int sl = __ffs(sm) - 1, sg = src >> 2;
                     const int pch = sg * 8 + (sl ^ ((sg & 3) & ~PM));

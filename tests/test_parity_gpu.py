@@ -868,3 +868,10 @@ def test_row_kernel_scale_ranges(B, oracle, d, b, group):
         pytest.skip("ranges are parts or multiples of a block")
     bits = _row_inputs(40, d, 7200 + d + b)
     check(B, oracle, inputs.Workload("row-range", bits, inputs.random_perm(d, 73), b, "int4", group, 0))
+
+
+@pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
+@pytest.mark.parametrize("T,d,b", [(1, 4096, 128), (300, 2048, 64), (40, 14336, 128)])
+def test_permuted_rows_with_scales_formed_at_once(B, oracle, T, d, b, fmt):
+    bits = _row_inputs(T, d, 7400 + d)
+    check(B, oracle, inputs.Workload("at-once", bits, inputs.random_perm(d, 75), b, fmt, 0, 0))
