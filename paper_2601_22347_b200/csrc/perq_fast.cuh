@@ -738,8 +738,9 @@ __device__ __forceinline__ void serve_asym_requests(const FastParams &p, const u
 // range: exp2 of a compensated argument (2^-22 for the approximation, 2^-24 each for the correction factor and
 // its product; weighted by e / (1 + e) <= 1), the sum 1 + e (2^-24), one approximate reciprocal (2^-23), two
 // products (2^-24 each).  A result whose low half-word lies in
-// [0x7fe0, 0x801f] -- within 31 fp32 ulps, at least 1.8e-6 relative, of the halfway pattern 0x8000 -- could
-// round to either neighbour and is evaluated again in fp64; so is every result that is zero, below 2^-100 or
+// [0x7ff0, 0x800f] -- within 15 fp32 ulps, at least 8.9e-7 relative, of the halfway pattern 0x8000 -- could
+// round to either neighbour and is evaluated again in fp64 (one element in 2048; with 31 ulps every fifth piece of a
+// warp went there); so is every result that is zero, below 2^-100 or
 // not finite, which covers the arguments whose exponential or reciprocal left the normal range (they give a
 // zero or an infinity here) and the subnormal results, where the relative bound does not hold.
 __device__ __forceinline__ float ex2_ftz(float x)
@@ -768,8 +769,8 @@ __device__ __forceinline__ f32x2 swish_mul2(f32x2 g, f32x2 u)
     const f32x2 rc = pack2(rcp_ftz(den.x), rcp_ftz(den.y));
     return mul2(mul2(g, rc), u);                                     // (finite inputs never give a NaN in this order)
 }
-// zero if and only if the low half-word of an fp32 pattern lies in [0x7fe0, 0x801f]
-__device__ __forceinline__ uint32_t swiglu_midpoint_key(float h) { return ((__float_as_uint(h) + 0x20u) & 0xffc0u) ^ 0x8000u; }
+// zero if and only if the low half-word of an fp32 pattern lies in [0x7ff0, 0x800f]
+__device__ __forceinline__ uint32_t swiglu_midpoint_key(float h) { return ((__float_as_uint(h) + 0x10u) & 0xffe0u) ^ 0x8000u; }
 __device__ __forceinline__ bool swiglu_needs_fp64(float h)
 {
     return swiglu_midpoint_key(h) == 0u || !(fabsf(h) >= 0x1p-100f) || !(fabsf(h) <= 3.4028234663852886e38f);
