@@ -147,10 +147,10 @@ int allow_smem(K kernel, size_t bytes)
 // is still running (its prologue overlaps the predecessor's tail); every kernel launched this way calls
 // griddep_wait() before its first global memory access, so stream order is kept for all data.
 template <typename P>
-cudaError_t launch_overlapped(void (*kernel)(P), int grid, int block, size_t smem, cudaStream_t st, const P &params)
+cudaError_t launch_overlapped(void (*kernel)(P), int grid, int block, size_t smem, cudaStream_t st, const P &params, int grid_y = 1)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)grid, (unsigned)grid_y);
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -332,7 +332,8 @@ int launch_fast_inst(const perq::FastParams &p, int grid, cudaStream_t st)
     auto kernel = perq::perq_fast_kernel<LOG2B, MODE, LOG2G, PERM, XB>;
     const size_t smem = PERM ? perq::FastSmem::total_perm : XB > 3 ? perq::FastSmem::total_full : perq::FastSmem::total;
     if (int rc = allow_smem(kernel, smem)) return rc;
-    if (launch_overlapped(kernel, grid, perq::FAST_THREADS, smem, st, p) != cudaSuccess) {
+    const int parts = PERM && !perq::per_token_mode(MODE) ? (p.segs + p.G - 1) / p.G : 1;
+    if (launch_overlapped(kernel, grid, perq::FAST_THREADS, smem, st, p, parts) != cudaSuccess) {
         (void)cudaGetLastError();
         return PERQ_ERR_CUDA;
     }
@@ -532,11 +533,18 @@ int try_launch_fast(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     p.x2 = nullptr;
     p.perm = perm;
     p.G = G;
+    p.segs = segs;
     p.d = d;
     p.sqrt_b = std::sqrt((double)b);
     p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);
     const int sms = sm_count();
     if (sms <= 0) return PERQ_ERR_CUDA;
+    if (permuted && !perq::per_token_mode(mode) && T * 2 <= sms) {
+        // few permuted rows: as many CTAs per row as there are SMs for it
+        const int parts = (int)std::min<long long>(segs, sms / T);
+        p.G = (segs + parts - 1) / parts;
+        return launch_fast_mode<true>(mode, p.G, ilog2(b), p, (int)T, st);
+    }
     const int groups_per_cta = perq::FAST_WARPS / G;
     const long long want = (units + groups_per_cta - 1) / groups_per_cta;
     const int grid = (int)std::min<long long>(want, sms);
@@ -785,6 +793,7 @@ int perq_swiglu_rotate_quantize(const void *gate, const void *up, const int32_t 
     p.units_total = (uint32_t)units;
     p.perm = nullptr;
     p.G = G;
+    p.segs = segs;
     p.d = d;
     p.sqrt_b = std::sqrt((double)b);
     p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);

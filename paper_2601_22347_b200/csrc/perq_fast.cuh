@@ -84,7 +84,8 @@ struct FastParams {
     uint32_t units_total;    // units of G segments (fewer than 2^31); rows when G = d / 1024
     const uint16_t *x2;      // gated-activation variants only: the second projection ("up"), same shape as x
     const int32_t *perm;     // permuted variants only: perm[d] (device)
-    int G;                   // permuted variants: segments per row
+    int G;                   // permuted variants: warps per unit
+    int segs;                // segments per row (permuted rows that are split over CTAs: more than G)
     int d;
     double sqrt_b;
     double inv_7_sqrt_b;     // 1 / (7 sqrt(b)): INT4 scale = exact |u|max times this
@@ -874,9 +875,15 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     constexpr bool TOK = per_token_mode(MODE);
     constexpr bool RUNTIME_G = (PERM && !TOK) || LOG2G < 0;
     constexpr int NST = (PERM || WBITS > 0) ? 3 : SWIGLU ? 2 : FAST_NSTAGE;
-    const int G = RUNTIME_G ? p.G : (1 << (LOG2G < 0 ? 0 : LOG2G));   // warps (segments) per unit
-    const int GROUPS = FAST_WARPS / G;
-    const uint32_t UNIT_BYTES = (uint32_t)G * SEG_BYTES;
+    // Permuted rows whose scale ranges lie inside a segment may be split over gridDim.y CTAs: each stages the whole row
+    // and gathers, rotates and stores its p.G segments (few rows: the copy of the permutation into shared memory, 14336
+    // entries by one SM, was most of a call).
+    constexpr bool SPLIT = PERM && !TOK;
+    const int seg0 = SPLIT ? (int)blockIdx.y * p.G : 0;
+    const int G = SPLIT ? min(p.G, p.segs - seg0) : RUNTIME_G ? p.G : (1 << (LOG2G < 0 ? 0 : LOG2G));   // warps (segments) per unit
+    const int GROUPS = (SPLIT && gridDim.y > 1) ? 1 : FAST_WARPS / G;
+    const int ROW_SEGS = SPLIT ? p.segs : G;
+    const uint32_t UNIT_BYTES = (uint32_t)ROW_SEGS * SEG_BYTES;
     constexpr float MAGIC = 12582920.0f;          // 1.5 * 2^23 + 8: low nibble of the sum = code + 8
     // per token: a pinned maximum is recorded and evaluated later (not where the inputs in global memory are not the
     // row's: gated rows; nor where one lane's evaluation reads much more than the row's warp has at hand: 64 and 128
@@ -935,16 +942,17 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     if (PERM) {     // the permutation as byte offsets into a staged row; out-of-range entries are clamped
         uint16_t *pt = reinterpret_cast<uint16_t *>(fsmem + FastSmem::perm_tab);
         if ((reinterpret_cast<uintptr_t>(p.perm) & 15u) == 0) {      // four entries per load, all loads independent
-            const int4 *p4 = reinterpret_cast<const int4 *>(p.perm);
+            const int4 *p4 = reinterpret_cast<const int4 *>(p.perm) + seg0 * (SEG_ELEMS / 4);
 #pragma unroll 8
-            for (int i = tid; i < p.d / 4; i += FAST_THREADS) {
+            for (int i = tid; i < G * (SEG_ELEMS / 4); i += FAST_THREADS) {
                 const int4 e = __ldg(p4 + i);
                 const uint32_t o0 = (uint32_t)(2 * min(max(e.x, 0), p.d - 1)), o1 = (uint32_t)(2 * min(max(e.y, 0), p.d - 1));
                 const uint32_t o2 = (uint32_t)(2 * min(max(e.z, 0), p.d - 1)), o3 = (uint32_t)(2 * min(max(e.w, 0), p.d - 1));
                 reinterpret_cast<uint2 *>(pt)[i] = make_uint2(o0 | (o1 << 16), o2 | (o3 << 16));
             }
         } else {
-            for (int i = tid; i < p.d; i += FAST_THREADS) pt[i] = (uint16_t)(2 * min(max(__ldg(p.perm + i), 0), p.d - 1));
+            for (int i = tid; i < G * SEG_ELEMS; i += FAST_THREADS)
+                pt[i] = (uint16_t)(2 * min(max(__ldg(p.perm + seg0 * SEG_ELEMS + i), 0), p.d - 1));
         }
     }
     if (tid < 2 * FAST_WARPS) { wacc[tid] = 0ull; wacc2[tid] = ~0ull; wcnt[tid] = 0u; wflag[tid] = 0u; }
@@ -988,9 +996,9 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     // (the loop is bound by the number of instructions it issues).
     const uint32_t n_units = (p.units_total - first + stride - 1) / stride;
     const uint32_t refill_end = n_units > (uint32_t)NST ? n_units - NST : 0u;      // iterations 1 .. refill_end load a unit
-    const size_t unit_step = (size_t)stride * ((size_t)G * SEG_ELEMS);
-    const uint16_t *xload = p.x + (size_t)first * ((size_t)G * SEG_ELEMS);         // leader: the next unit to load
-    const uint16_t *xload2 = (SWIGLU ? p.x2 : p.x) + (size_t)first * ((size_t)G * SEG_ELEMS);
+    const size_t unit_step = (size_t)stride * ((size_t)ROW_SEGS * SEG_ELEMS);
+    const uint16_t *xload = p.x + (size_t)first * ((size_t)ROW_SEGS * SEG_ELEMS);         // leader: the next unit to load
+    const uint16_t *xload2 = (SWIGLU ? p.x2 : p.x) + (size_t)first * ((size_t)ROW_SEGS * SEG_ELEMS);
     // prologue: fill the ring
     if (leader) {
 #pragma unroll
@@ -1011,8 +1019,8 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
 #pragma unroll
     for (int k = 0; k < NCLS; ++k) { q_cp[k] = qsgn(k) * (1.0f + q_delta); q_cm[k] = qsgn(k) * (1.0f - q_delta); }
 
-    uint8_t *code_out = p.out_codes + ((size_t)first * G + w_in_g) * SEG_CODE_BYTES;   // this warp's codes of the current unit
-    const size_t code_out_step = (size_t)stride * G * SEG_CODE_BYTES;
+    uint8_t *code_out = p.out_codes + ((size_t)first * ROW_SEGS + seg0 + w_in_g) * SEG_CODE_BYTES;   // this warp's codes of the current unit
+    const size_t code_out_step = (size_t)stride * ROW_SEGS * SEG_CODE_BYTES;
     uint32_t unit = first;
     for (uint32_t it = 0; it < n_units; ++it, unit += stride, code_out += code_out_step) {
         const uint32_t stage = it % NST;
@@ -1027,7 +1035,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
         }
         // the staged row (or, unpermuted, the staged unit) and this warp's 1024 elements of it
         const uint16_t *raw_row = reinterpret_cast<const uint16_t *>(fsmem + FastSmem::stages) +
-                                  ((size_t)group * NST + stage) * ((size_t)G * SEG_ELEMS);
+                                  ((size_t)group * NST + stage) * ((size_t)ROW_SEGS * SEG_ELEMS);
         uint32_t seg_addr = stage_base + stage * UNIT_BYTES + (uint32_t)w_in_g * SEG_BYTES;
         const uint16_t *seg = raw_row + (size_t)w_in_g * SEG_ELEMS;
         if (SWIGLU) swiglu_segment(seg_addr, up_base + stage * UNIT_BYTES + (uint32_t)w_in_g * SEG_BYTES, lane);
@@ -1050,7 +1058,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
             seg_addr = pbuf_addr;
             seg = reinterpret_cast<const uint16_t *>(fsmem + FastSmem::pbuf) + (size_t)warp * SEG_ELEMS;
         }
-        const size_t seg_index = (size_t)unit * G + w_in_g;
+        const size_t seg_index = (size_t)unit * ROW_SEGS + seg0 + w_in_g;
         // Hadamard block of the element at offset e of this warp's segment: its bf16 inputs and the
         // element's index inside the block
         auto block_of = [&](int e, const uint16_t *&bp, int &i) {

@@ -870,6 +870,15 @@ def test_row_kernel_scale_ranges(B, oracle, d, b, group):
     check(B, oracle, inputs.Workload("row-range", bits, inputs.random_perm(d, 73), b, "int4", group, 0))
 
 
+@pytest.mark.parametrize("fmt,group", [("int4", 128), ("mxfp4", 32)])
+@pytest.mark.parametrize("T,d,b", [(1, 14336, 128), (1, 1024, 16), (3, 9216, 64), (10, 14336, 32), (15, 16384, 128), (37, 5120, 32),
+                                   (74, 3072, 16), (75, 3072, 16)])
+def test_few_permuted_rows_are_split_over_ctas(B, oracle, T, d, b, fmt, group):
+    """Every split of a row into parts, the last one shorter; the first row count that is not split."""
+    bits, _ = inputs.gaussian_outliers(T, d, 5, 50.0, seed=7300 + d + T)
+    check(B, oracle, inputs.Workload("split", bits, inputs.random_perm(d, 74), b, fmt, group, 0))
+
+
 @pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
 @pytest.mark.parametrize("T,d,b", [(1, 4096, 128), (300, 2048, 64), (40, 14336, 128)])
 def test_permuted_rows_with_scales_formed_at_once(B, oracle, T, d, b, fmt):
