@@ -214,6 +214,23 @@ __device__ __forceinline__ void sts_u16_at(uint32_t addr, uint32_t v)
 {
     asm volatile("st.shared.u16 [%0+%2], %1;" ::"r"(addr), "h"((uint16_t)v), "n"(OFF) : "memory");
 }
+// A quad's codes of a segment without a trip through shared memory.  Lane q holds the 16-bit pieces 4 q .. 4 q + 3 of
+// its lane group's eight chunks (c[s]: slot s, low half); after two exchanges inside the quad it holds all four pieces
+// of slots 2 q and 2 q + 1, 16 adjacent bytes; odd: the slots' chunks lie the other way round.
+__device__ __forceinline__ uint4 quad_codes(const uint32_t (&c)[8], int q, bool odd)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) w[m] = __byte_perm(c[2 * m], c[2 * m + 1], 0x5410);
+    const bool b2 = (q & 2) != 0, b1 = (q & 1) != 0;
+    const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b2 ? w[0] : w[2], 2), r1 = __shfl_xor_sync(0xffffffffu, b2 ? w[1] : w[3], 2);
+    const uint32_t l0 = b2 ? r0 : w[0], l1 = b2 ? r1 : w[1], h0 = b2 ? w[2] : r0, h1 = b2 ? w[3] : r1;
+    const uint32_t lr = __shfl_xor_sync(0xffffffffu, b1 ? l0 : l1, 1), hr = __shfl_xor_sync(0xffffffffu, b1 ? h0 : h1, 1);
+    const uint32_t t0 = b1 ? lr : l0, t1 = b1 ? l1 : lr, t2 = b1 ? hr : h0, t3 = b1 ? h1 : hr;
+    const uint32_t x0 = __byte_perm(t0, t1, 0x5410), x1 = __byte_perm(t2, t3, 0x5410);
+    const uint32_t y0 = __byte_perm(t0, t1, 0x7632), y1 = __byte_perm(t2, t3, 0x7632);
+    return odd ? make_uint4(y0, y1, x0, x1) : make_uint4(x0, x1, y0, y1);
+}
 // Store of the 16-bit code piece of slot s (a constant once the slot loop is unrolled) at base ^ (s * 8),
 // for a base whose offset bits 3..5 lie inside XV: the slot bits in XV are XORed into the address, the
 // others are added as an immediate offset (no instruction).
@@ -879,6 +896,9 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     // and gathers, rotates and stores its p.G segments (few rows: the copy of the permutation into shared memory, 14336
     // entries by one SM, was most of a call).
     constexpr bool SPLIT = PERM && !TOK;
+    // Permuted rows are bound by shared-memory wavefronts (the gather): their codes go from registers straight to
+    // global memory, and through the staging buffer only where a fix-up has to rewrite some.
+    constexpr bool DIRECT = PERM && !TOK;
     const int seg0 = SPLIT ? (int)blockIdx.y * p.G : 0;
     const int G = SPLIT ? min(p.G, p.segs - seg0) : RUNTIME_G ? p.G : (1 << (LOG2G < 0 ? 0 : LOG2G));   // warps (segments) per unit
     const int GROUPS = (SPLIT && gridDim.y > 1) ? 1 : FAST_WARPS / G;
@@ -1201,8 +1221,10 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
         const uint32_t code_buf = code_base + par2 * SEG_CODE_BYTES;
         const uint32_t code_addr0 = code_buf + code_lane;
         uint8_t *code_gen = fsmem + FastSmem::codes + (size_t)warp * (2 * SEG_CODE_BYTES) + (size_t)par2 * SEG_CODE_BYTES;
-        bulk_store_wait_read<1>();           // the store that last read this staging buffer has drained
+        if (!DIRECT) bulk_store_wait_read<1>();           // the store that last read this staging buffer has drained
         __syncwarp();
+        uint32_t cw[8];                      // DIRECT: the lane's code pieces
+        bool staged = false;                 // DIRECT: (warp-uniform) the codes are in the staging buffer
 
         if (MODE == MODE_ASYM) {
             // ---------------------------------------------------------------- asymmetric INT4 per token
@@ -1664,12 +1686,18 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                 const uint32_t pm = ((__float_as_uint(tm1.y) * 16u + __float_as_uint(tm1.x)) * 16u + __float_as_uint(tm0.y)) * 16u
                                     + __float_as_uint(tm0.x);
                 tie_any |= pp ^ pm;          // low 16 bits: the four codes (offset by 8) under either multiplier
-                sts_code<(3 & ~PM)>(code_addr0, s, pp ^ 0x8888u);
+                if (DIRECT) cw[s] = pp ^ 0x8888u;
+                else sts_code<(3 & ~PM)>(code_addr0, s, pp ^ 0x8888u);
             }
             tie_any &= 0xffffu;
 
             // ---- exact resolution of near ties (rare)
             if (__any_sync(0xffffffffu, tie_any != 0u)) {
+                if (DIRECT) {
+                    staged = true;
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) sts_code<(3 & ~PM)>(code_addr0, s, cw[s]);
+                }
                 // flagged elements; FP4: from the kept difference words, and zm marks those whose two codes differ
                 // in the sign alone (both magnitudes are zero: they need the sign of the exact value, not the scale
                 // and none of its fp64 divisions)
@@ -1954,9 +1982,15 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                 const uint32_t pu = cvt_e2m1x4(up0.x, up0.y, up1.x, up1.y);
                 const uint32_t pd = cvt_e2m1x4(dn0.x, dn0.y, dn1.x, dn1.y);
                 tie_any |= pu ^ pd;
-                sts_code<(3 & ~PM)>(code_addr0, s, pu);
+                if (DIRECT) cw[s] = pu;
+                else sts_code<(3 & ~PM)>(code_addr0, s, pu);
             }
             if (__any_sync(0xffffffffu, tie_any != 0u)) {
+                if (DIRECT) {
+                    staged = true;
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) sts_code<(3 & ~PM)>(code_addr0, s, cw[s]);
+                }
                 uint32_t fm = 0u;
                 if (tie_any != 0u) {
 #pragma unroll
@@ -1998,6 +2032,21 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
             }
         }
 
+        if (DIRECT) {
+            // ---- packed codes: registers (or, after a fix-up, the staging buffer) -> global
+            const int fx = f_g & ~PM, at = (g * 8 + ((2 * q ^ fx) & ~1)) * 8;
+            uint4 v16;
+            __syncwarp();
+            if (staged) {
+                asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v16.x), "=r"(v16.y), "=r"(v16.z), "=r"(v16.w) : "r"(code_buf + (uint32_t)at) : "memory");
+                __syncwarp();
+            } else {
+                v16 = quad_codes(cw, q, (fx & 1) != 0);
+            }
+            *reinterpret_cast<uint4 *>(code_out + at) = v16;
+            if (lane == 0) mbar_arrive(empty_base + stage * 8);            // this warp no longer reads the staged row
+            continue;
+        }
         // ---- packed codes: shared staging -> global
         fence_async_smem();
         __syncwarp();
