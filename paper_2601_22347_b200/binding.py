@@ -92,14 +92,16 @@ def _check(rc: int, where: str):
         raise PerqError(rc, where)
 
 
+# Addresses and stream handles go to ctypes as plain integers (the functions' argtypes convert them): small calls
+# are bound by the host, and wrapper objects, the torch.cuda.Stream object among them, were a third of its time.
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> C.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return int(getattr(stream, "cuda_stream", stream))
 
 
 def perq_out_sizes(T: int, d: int, fmt: int, group: int):
@@ -133,9 +135,10 @@ def perq_rotate_quantize(x: torch.Tensor, perm: Optional[torch.Tensor], b: int, 
     T, d = x.shape
     if out_codes is None:
         out_codes, out_scales = alloc_outputs(T, d, fmt, group, x.device)
-    rc = load().perq_rotate_quantize(_ptr(x), _ptr(perm), T, d, b, fmt, group, _ptr(out_codes), _ptr(out_scales),
-                                     _stream(stream))
-    _check(rc, "perq_rotate_quantize")
+    rc = (_lib or load()).perq_rotate_quantize(x.data_ptr(), _ptr(perm), T, d, b, fmt, group, _ptr(out_codes),
+                                               _ptr(out_scales), _stream(stream))
+    if rc != PERQ_OK:
+        _check(rc, "perq_rotate_quantize")
     return out_codes, out_scales
 
 
