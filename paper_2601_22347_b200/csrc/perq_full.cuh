@@ -172,7 +172,7 @@ __device__ __noinline__ void full_mx_fix_ties(uint32_t t_lane, const uint16_t *r
     }
 }
 
-// MODE_MX only (for now): template parameter kept for the per-token formats.
+// MODE_MX only: per-token scales of whole-row blocks are the row kernel's.
 template <int LOG2D, int MODE>
 __global__ void __launch_bounds__(FAST_THREADS, 1) perq_full_kernel(FastParams p)
 {

@@ -21,7 +21,7 @@
 // What bounds it: shared-memory passes (4 bytes per element and trip) and, for per-token scales of whole-row
 // blocks, the exact row maximum, a d-term fp64 sum that all warps of the row share.  The general kernel, which
 // these shapes ran on, made a trip per three stages with eight warps per row and left each exact sum to one warp:
-// 1024 x 14336 with b = d took 928 us there and takes 57 here, 1531 x 9728 with b = 128 asymmetric 94 and 34,
+// 1024 x 14336 with b = d took 928 us there and takes 57 here, 1531 x 9728 with b = 128 asymmetric 94 and 32,
 // 16384 x 4096 with b = d (group kernel) 228 and 114.
 //
 // Exactness rules as in perq_generic.cuh: |u32 - u| <= err_rel * (largest |u32| of the block); every value that
@@ -87,21 +87,22 @@ __host__ __device__ constexpr int row_base_np(int n0) { return (n0 + 15) / 16 * 
 
 // -------------------------------------------------------------------------------------------- exact sums
 
-// (-1)^{popcount(i & k)} terms: flips the sign of v where s is odd.
-__device__ __forceinline__ double row_signed(double v, uint32_t s)
-{
-    return __hiloint2double(__double2hiint(v) ^ (int)(s << 31), __double2loint(v));
-}
-
 // Exact unnormalised output at row position pos of a power-of-two block of up to 1024, by one warp.
 __device__ __noinline__ double row_exact_warp(const uint16_t *xs, uint32_t pos, int log2b, int lane)
 {
     const uint32_t b = 1u << log2b, blk = (pos >> log2b) << log2b, i = pos - blk;
-    double acc = 0.0;
-    for (uint32_t k = lane; k < b; k += 32) acc += row_signed(bf16_bits_to_f64(xs[blk + k]), (uint32_t)__popc(i & k) & 1u);
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(xs + blk);
+    double e = 0.0, o = 0.0;                 // even and odd inputs (times 2^-896, see bf16_bits_to_f64)
+#pragma unroll 2
+    for (uint32_t w = lane; w < b / 2; w += 32) {
+        const uint32_t v = src[w] ^ ((__popc(i & (2 * w)) & 1) ? 0x80008000u : 0u);
+        e += bf16_raw_f64(v << 16);
+        o += bf16_raw_f64(v);
+    }
+    double acc = (i & 1u) ? e - o : e + o;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    return __shfl_sync(0xffffffffu, acc, 0);
+    for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+    return __shfl_sync(0xffffffffu, acc, 0) * 0x1p896;
 }
 
 // The same by the four lanes of a quad, every quad with a position of its own (all 32 lanes call; quads
@@ -113,15 +114,14 @@ __device__ __forceinline__ double row_exact_quad(const uint16_t *xs, uint32_t po
     double e = 0.0, o = 0.0;
 #pragma unroll 4
     for (uint32_t w = 0; w < per / 2; ++w) {
-        const uint32_t v = src[w];
-        const uint32_t s = (uint32_t)__popc(i & (k0 + 2 * w)) & 1u;
-        e += row_signed(bf16_bits_to_f64(v), s);
-        o += row_signed(bf16_bits_to_f64(v >> 16), s);
+        const uint32_t v = src[w] ^ ((__popc(i & (k0 + 2 * w)) & 1) ? 0x80008000u : 0u);
+        e += bf16_raw_f64(v << 16);
+        o += bf16_raw_f64(v);
     }
     double acc = (i & 1u) ? e - o : e + o;
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    return __shfl_sync(0xffffffffu, acc, lane & 28);
+    return __shfl_sync(0xffffffffu, acc, lane & 28) * 0x1p896;
 }
 
 // Signs of eight adjacent inputs (bit j set: input k + j is subtracted) of the output at position i, in blocks of a
@@ -1208,7 +1208,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
 // outputs, each of which is a sum over the whole block.  For b = 2048 and ranges of 128 that is 16 terms per
 // element of the row (157 us for 4096 x 2048 in the general kernel, 87 with the sums shared by a CTA, two thirds of it
 // these sums); the butterfly itself in fp64 is 11 additions per element and makes EVERY output exact, so this kernel
-// rotates in fp64 and rounds its outputs to fp32 for the quantiser (32 us).  Maxima come from the fp64 values; the rounding window is the rounding to fp32 alone.
+// rotates in fp64 and rounds its outputs to fp32 for the quantiser (31.5 us).  Maxima come from the fp64 values; the rounding window is the rounding to fp32 alone.
 //
 // A warp owns 1024 positions.  Lane l starts with the values at 32 m + l, combined over the block's segments while
 // they are converted (2^896 completes the conversion, see bf16_bits_to_f64, and carries the sign), rotates index
@@ -1289,11 +1289,11 @@ __global__ void __maxnreg__(ROW64_REGS) perq_row64_kernel(const __grid_constant_
         for (int m = 0; m < 32; ++m) v[m] = 0.0;
         for (int w = 0; w < (1 << log2r); ++w) {
             const double c = (__popc(w & wl) & 1) ? -0x1p896 : 0x1p896;
-            const uint16_t *src = xs + (wb + w) * SEG_ELEMS + lane;
+            const int16_t *src = reinterpret_cast<const int16_t *>(xs) + (wb + w) * SEG_ELEMS + lane;
 #pragma unroll
             for (int m = 0; m < 32; ++m) {
-                const uint32_t h = src[32 * m];
-                v[m] = fma(__hiloint2double((int)(((h & 0x7fffu) << 13) | ((h & 0x8000u) << 16)), 0), c, v[m]);
+                const uint32_t h = (uint32_t)(int)src[32 * m];          // (sign-extended: the shift puts the sign into bit 31)
+                v[m] = fma(__hiloint2double((int)((h << 13) & 0x8fffffffu), 0), c, v[m]);
             }
         }
         row64_stage(v, 1);
