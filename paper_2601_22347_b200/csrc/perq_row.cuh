@@ -514,9 +514,13 @@ __device__ __noinline__ uint32_t row_exact_code(double u, double sqrt_b, double 
 // Symmetric INT4: exact code of a doubtful element, u its exact value, a the exact maximum of its range.  The tie
 // is between |y / s| = n and n + 1, y / s = 7 u / a: the sign of 14 |u| - (2 n + 1) a decides (two products whose
 // rounding errors are far below the margin), the definition's divisions only an all but exact tie.
+// n from the fp32 multiplier where that is 7 / a to a few ulp (scales of whole rows, or from exact values).  In a range
+// that is small beside its block (PINNED false) the fp32 maximum is partly rounding noise: its multiplier can be off by
+// any factor and every element of the range comes here, so n is formed from the exact values.
+template <bool PINNED>
 __device__ __forceinline__ uint32_t row_int4_code(double u, double a, float mul, double sqrt_b)
 {
-    const int n = (int)(fabsf((float)u) * mul);
+    const int n = PINNED ? (int)(fabsf((float)u) * mul) : (int)(7.0 * fabs(u) / a);
     const double diff = 14.0 * fabs(u) - (double)(2 * n + 1) * a;
     if (!(fabs(diff) > a * 1.0e-12)) return row_exact_code<ROW_TOKEN>(u, sqrt_b, a / sqrt_b / 7.0, 0.0, 0);
     const int k = n + (diff > 0.0 ? 1 : 0);
@@ -999,7 +1003,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
                             const int e = __ffs(tie) - 1;
                             tie &= tie - 1;
                             const double v = row_sum_parts(ms, tslot + t);
-                            row_patch(cw, e, rot, MODE == ROW_TOKEN ? row_int4_code(v, a_ex, Q.mul, p.sqrt_b)
+                            row_patch(cw, e, rot, MODE == ROW_TOKEN ? row_int4_code<true>(v, a_ex, Q.mul, p.sqrt_b)
                                                                     : row_exact_code<MODE>(v, p.sqrt_b, s64, 0.0, 0));
                         }
                     }
@@ -1167,7 +1171,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
                         const int e = __ffs(tie) - 1;
                         tie &= tie - 1;
                         const double v = row_sum_parts(ms, slot + t);
-                        row_patch(cw, e, rot, MODE == ROW_GROUP ? row_int4_code(v, a_ex, Q.mul, p.sqrt_b)
+                        row_patch(cw, e, rot, MODE == ROW_GROUP ? row_int4_code<false>(v, a_ex, Q.mul, p.sqrt_b)
                                                                 : row_exact_code<MODE>(v, p.sqrt_b, s64, z64, Eb - 127));
                     }
                     if (more) __syncthreads();
@@ -1185,7 +1189,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
                         ts &= ts - 1;
                         const double v = row_exact_warp(xs, row_position(is, rs, 0, e), p.log2b, lane);
                         if (lane == src)
-                            row_patch(cw, e, rot, MODE == ROW_TOKEN || MODE == ROW_GROUP ? row_int4_code(v, a_ex, Q.mul, p.sqrt_b)
+                            row_patch(cw, e, rot, MODE == ROW_TOKEN || MODE == ROW_GROUP ? row_int4_code<MODE == ROW_TOKEN>(v, a_ex, Q.mul, p.sqrt_b)
                                                                                        : row_exact_code<MODE>(v, p.sqrt_b, s64, z64, Eb - 127));
                     }
                 }
@@ -1358,7 +1362,7 @@ __global__ void __maxnreg__(ROW64_REGS) perq_row64_kernel(const __grid_constant_
                 const int e = __ffs(ts) - 1;
                 ts &= ts - 1;
                 const double x = row_exact_warp(xs, is + e, p.log2b, lane);
-                if (lane == src) row_patch(cw, e, 0, row_int4_code(x, a_ex, Q.mul, p.sqrt_b));
+                if (lane == src) row_patch(cw, e, 0, row_int4_code<true>(x, a_ex, Q.mul, p.sqrt_b));
             }
         }
         if (live) *reinterpret_cast<uint4 *>(p.out_codes + (size_t)row * (d / 2) + (size_t)tid * 16) = make_uint4(cw[0], cw[1], cw[2], cw[3]);

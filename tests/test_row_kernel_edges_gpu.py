@@ -1,0 +1,78 @@
+"""Parity of the row kernel with the oracle on inputs at the edges of its fp32 arithmetic: scale ranges that hold
+small outputs of a block with large ones."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_22347_b200 import inputs
+
+from parity import compare_quantized
+
+pytestmark = pytest.mark.gpu
+
+FMT = {"int4": 0, "mxfp4": 1, "fp4": 3, "int4_asym": 4}
+
+
+@pytest.fixture(scope="module")
+def B():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_22347_b200 import binding, build
+    build.build()
+    binding.load()
+    return binding
+
+
+@pytest.fixture(autouse=True)
+def clean_error_word(B):
+    B.perq_device_error_clear()
+    yield
+    assert B.perq_device_error() == 0
+
+
+def run(B, bits, perm, b, fmt, group):
+    x = torch.from_numpy(bits.view(np.int16).copy()).cuda().view(torch.bfloat16)
+    p = None if perm is None else torch.from_numpy(perm).cuda()
+    codes, scales = B.perq_rotate_quantize(x, p, b, FMT[fmt], group)
+    torch.cuda.synchronize()
+    return codes.cpu().numpy(), scales.cpu().numpy()
+
+
+def check(B, oracle, bits, perm, b, fmt, group):
+    codes, scales = run(B, bits, perm, b, fmt, group)
+    return compare_quantized(fmt, codes, scales, oracle.rotate_quantize(bits, perm, b, FMT[fmt], group, want_pre=True))
+
+
+def through(bits, perm):
+    """The rows whose gather through perm gives `bits`."""
+    if perm is None:
+        return bits
+    out = np.empty_like(bits)
+    out[:, perm] = bits
+    return out
+
+
+# ------------------------------------------------------------------ small outputs of a block with large ones
+
+def _cancelling_rows(T, d, b, log2_ratio, seed):
+    """Blocks whose upper half of outputs holds values 2^-log2_ratio of the lower half's: 16 large channels that occur
+    in both halves of the block (and cancel in the upper outputs), 16 ordinary ones."""
+    rng = np.random.default_rng(seed)
+    x = np.zeros((T, d // b, b))
+    for t in range(T):
+        for j in range(d // b):
+            k = rng.choice(b // 2, 16, replace=False)
+            x[t, j, k] = x[t, j, k + b // 2] = rng.standard_normal(16) * 2.0 ** log2_ratio
+            free = np.setdiff1d(np.arange(b), np.r_[k, k + b // 2])
+            x[t, j, rng.choice(free, 16, replace=False)] = rng.standard_normal(16)
+    return inputs.f32_to_bf16_bits(x.reshape(T, d).astype(np.float32))
+
+
+@pytest.mark.parametrize("log2_ratio", [18, 20, 21])
+@pytest.mark.parametrize("T,d,b,group,perm", [(40, 1024, 128, 32, False), (40, 1152, 128, 64, True), (60, 640, 64, 32, False),
+                                              (9, 14336, 14336, 128, False), (20, 3072, 3072, 128, True), (20, 3072, 3072, 32, False),
+                                              (20, 1024, 256, 64, True), (10, 4096, 2048, 128, True)])
+def test_ranges_far_below_their_block(B, oracle, T, d, b, group, perm, log2_ratio):
+    """The fp32 maximum of such a range is partly rounding noise: it does not pin a code to two neighbours."""
+    p = inputs.random_perm(d, 81) if perm else None
+    bits = through(_cancelling_rows(T, d, b, log2_ratio, 8000 + d + b + log2_ratio), p)
+    check(B, oracle, bits, p, b, "int4", group)
