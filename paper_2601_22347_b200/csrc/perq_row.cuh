@@ -906,7 +906,8 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
             Q.mul = inv;
             const float eb = (MODE == ROW_GROUP) ? bm : a32;             // error reference of the range's maximum
             thr = a32 - 2.0f * err * eb - a32 * 2.4e-7f;
-            if (a32 > 0.0f && lm >= thr) cand = row_reach(u, fmaxf(thr, 1.0e-45f));
+            // (a threshold at or below zero, a range within the error of its block: a value that is zero in fp32 can be the largest)
+            if (a32 > 0.0f && lm >= thr) cand = row_reach(u, thr);
             // error of an element and of the fp32 maximum, in code units
             Q.tau = 7.0f * err * (bm + eb) * fminf(inv * (1.0f / 7.0f), 3.0e38f) + 4.0e-6f;
             if (MODE == ROW_FP4 && !(bm > 0.0f)) Q.tau = 0.0f;            // an all-zero block is exact
@@ -934,7 +935,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
             const float tol = 2.0f * err * bm + lm * 4.8e-7f;
             near = lm > 0.0f && (dist <= tol || e8 == 0);
             thr = lm - tol;
-            if (near) cand = row_reach(u, fmaxf(thr, 1.0e-45f));
+            if (near) cand = row_reach(u, thr);
         } else {
             const float e_abs = a_row * (2.0f * err + 2.4e-7f);
             const bool some = a_row > 0.0f;
