@@ -894,7 +894,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
         uint32_t cand = 0u;
         int Eb = 0;
         float a32 = a_row, thr = 0.0f;
-        bool near = false;
+        bool near = false, zero = false;
         float z32 = 0.0f, vmin = 0.0f, inv = 0.0f;
         if (MODE == ROW_GROUP) {
             a32 = lm;
@@ -1074,7 +1074,8 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
             }
             for (int o = 1; o < (1 << (p.log2g - 5)); o <<= 1) a_ex = fmax(a_ex, __shfl_xor_sync(0xffffffffu, a_ex, o));
         } else {
-            // MX: exact exponents of the groups near a boundary
+            // MX: exact exponents of the groups near a boundary; a group whose exact values are all zero
+            zero = !(lm > 0.0f);
             if (wide ? __syncthreads_or(near) : __any_sync(0xffffffffu, near)) {
                 uint32_t want = cand;
                 if (wide) {
@@ -1106,6 +1107,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
                     int ex;
                     (void)frexp(a_ex / p.sqrt_b, &ex);
                     Eb = ex - 3 + 127;
+                    zero = a_ex == 0.0;       // (the fp32 values of a group that cancels exactly are rounding noise)
                 }
             }
         }
@@ -1141,8 +1143,9 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
             if (NP2) Q.mul = (float)(scalbn(1.0, 127 - Eb) / p.sqrt_b);
             else if ((p.log2b & 1) == 0) Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - p.log2b / 2, 1), 254) << 23);
             else Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - (p.log2b - 1) / 2, 1), 254) << 23) * 0.70710678118654752f;
-            if (!(lm > 0.0f)) { Q.mul = 0.0f; byte = 0u; }
-            Q.tau = (bm > 0.0f) ? 2.0f * err * bm * Q.mul + 2.0e-6f : 0.0f;       // (an all-zero block is exact)
+            if (zero) { Eb = 0; Q.mul = 0.0f; byte = 0u; }
+            // (an all-zero block is exact, and so is a group whose candidates were all zero: no window, codes 0)
+            Q.tau = (bm > 0.0f && !(near && zero)) ? 2.0f * err * bm * Q.mul + 2.0e-6f : 0.0f;
             if (live) (reinterpret_cast<uint8_t *>(p.out_scales))[(size_t)row * (d >> 5) + tid] = (uint8_t)byte;
             if (row_quantise<MODE>(u, Q, cw)) tie = row_tie_bits<MODE>(u, Q);
         }

@@ -1,5 +1,5 @@
 """Parity of the row kernel with the oracle on inputs at the edges of its fp32 arithmetic: scale ranges that hold
-small outputs of a block with large ones."""
+small outputs of a block with large ones, MX groups that cancel exactly."""
 import numpy as np
 import pytest
 import torch
@@ -78,3 +78,32 @@ def test_ranges_far_below_their_block(B, oracle, T, d, b, group, perm, log2_rati
     p = inputs.random_perm(d, 81) if perm else None
     bits = through(_cancelling_rows(T, d, b, log2_ratio, 8000 + d + b + log2_ratio), p)
     check(B, oracle, bits, p, b, "int4", group)
+
+
+# ------------------------------------------------------------------ MX groups that are exactly zero in a block that is not
+
+def _zero_quarter_rows(T, d, b, seed):
+    """Blocks of four runs 3v, 4v, 5v, 4v: the second quarter of the outputs is (3 - 4 + 5 - 4) H v = 0 exactly.  v spans
+    29 binades, so that fp32 leaves noise there; the products are exact in bf16, all sums exact in fp64 (50 bits)."""
+    rng = np.random.default_rng(seed)
+    shape = (T, d // b, 1, b // 4)
+    v = rng.integers(1, 16, size=shape) * np.exp2(rng.integers(-14, 15, size=shape)) * rng.choice([-1.0, 1.0], size=shape)
+    x = (v * np.array([3.0, 4.0, 5.0, 4.0])[None, None, :, None]).reshape(T, d)
+    bits = inputs.f32_to_bf16_bits(x.astype(np.float32))
+    assert np.array_equal(inputs.bf16_to_f64(bits), x)
+    return bits
+
+
+def check_zero_groups(B, oracle, T, d, b, perm):
+    p = inputs.random_perm(d, 82) if perm else None
+    bits = through(_zero_quarter_rows(T, d, b, 8100 + d + b), p)
+    zero = oracle.rotate_quantize(bits, p, b, FMT["mxfp4"], 32)["scales"] == 0
+    assert zero.sum() * 4 == zero.size
+    check(B, oracle, bits, p, b, "mxfp4", 32)
+
+
+@pytest.mark.parametrize("T,d,b,perm", [(20, 1024, 256, True), (20, 1152, 128, False), (20, 1152, 128, True), (9, 3072, 3072, False),
+                                        (6, 14336, 14336, True), (9, 2048, 2048, True), (7, 6144, 2048, False),
+                                        (5, 16384, 16384, False), (9, 8192, 4096, True)])
+def test_row_kernel_mx_groups_that_cancel(B, oracle, T, d, b, perm):
+    check_zero_groups(B, oracle, T, d, b, perm)
