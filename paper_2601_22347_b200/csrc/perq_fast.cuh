@@ -1906,6 +1906,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                         int ex;
                         (void)frexp(over_sqrt_b(best), &ex);
                         Eb = ex - 3 + 127;
+                        if (best == 0.0) a32 = bref = 0.0f;        // the fp32 maximum is rounding noise: scale byte 0, no window
                     }
                 }
             } else if (near_w != 0u) {   // rare: exact maximum of the group from every element that could attain it
@@ -1942,6 +1943,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
                             int ex;
                             (void)frexp(over_sqrt_b(best), &ex);
                             Eb = ex - 3 + 127;
+                            if (best == 0.0) a32 = bref = 0.0f;    // scale byte 0, no window
                         }
                     }
                 }

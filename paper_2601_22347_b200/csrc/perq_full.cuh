@@ -129,7 +129,7 @@ __device__ __noinline__ int full_mx_exact_exponents(uint32_t t_lane, const uint1
         if (lane == owner) {
             int ex;
             (void)frexp(full_over_sqrt_d<LOG2D>(best, sqrt_d), &ex);
-            Eb = ex - 3 + 127;
+            Eb = best == 0.0 ? MX_ZERO_GROUP : ex - 3 + 127;
         }
     }
     return Eb;
@@ -352,7 +352,10 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_full_kernel(FastParams p
         int Eb = mx_exponent_fp32<LOG2D>(a32, dist);
         const float tol = 2.0f * err_rel * bref + a32 * 2.4e-7f;
         const bool near = (a32 > 0.0f) && (dist <= tol || (__float_as_uint(a32) >> 23) == 0u);
-        if (__any_sync(0xffffffffu, near)) Eb = full_mx_exact_exponents<LOG2D>(t_lane, raw_row, a32, tol, near, Eb, i0, p.sqrt_b, lane);
+        if (__any_sync(0xffffffffu, near)) {
+            Eb = full_mx_exact_exponents<LOG2D>(t_lane, raw_row, a32, tol, near, Eb, i0, p.sqrt_b, lane);
+            if (Eb == MX_ZERO_GROUP) a32 = bref = 0.0f;
+        }
         Eb = min(max(Eb, 0), 254);
         float c;
         if ((LOG2D & 1) == 0) c = __uint_as_float((uint32_t)min(max(254 - Eb - LOG2D / 2, 1), 254) << 23);

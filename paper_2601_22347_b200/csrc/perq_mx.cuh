@@ -26,6 +26,10 @@ struct MxSmem {
     static constexpr size_t total = used + 1024;                                                  // room to align the base
 };
 
+// Returned for a group whose exact values are all zero (its fp32 maximum is rounding noise): scale byte 0 and, since
+// its zeros are exact, no rounding window.
+constexpr int MX_ZERO_GROUP = -0x10000;
+
 // Shared exponent E + 127 (before clamping) of the 32-value group that lane q of a quad owns, from the fp32
 // group maximum a32: E = floor(log2(a / sqrt(b))) - 2.  dist is the distance of a32 to the nearest value at
 // which that floor changes.
@@ -120,7 +124,7 @@ __device__ __noinline__ int mx_exact_exponents(uint32_t seg_addr, const uint16_t
             if (q == m) {
                 int ex;
                 (void)frexp(over_sqrt_b(best), &ex);
-                Eb = ex - 3 + 127;
+                Eb = best == 0.0 ? MX_ZERO_GROUP : ex - 3 + 127;
             }
         }
     }
@@ -270,7 +274,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_mx_kernel(FastParams p)
             f32x2 v[8][2];
             tok_rotate<LOG2B>(seg_addr, L, v);
             float gm[4];
-            const float a32 = mx_group_max(v, q, gm);
+            float a32 = mx_group_max(v, q, gm);
             // error reference: the largest |u| of the Hadamard block (it may span several groups)
             float bref = a32;
             if (CB >= 2) bref = fmaxf(bref, __shfl_xor_sync(0xffffffffu, bref, 1));
@@ -282,6 +286,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_mx_kernel(FastParams p)
             if (__any_sync(0xffffffffu, near)) {
                 const uint16_t *seg = stage_gen + (seg_addr - smem_base - (uint32_t)MxSmem::stages) / 2;
                 Eb = mx_exact_exponents<LOG2B>(seg_addr, seg, a32, tol, near, Eb, p.sqrt_b, lane);
+                if (Eb == MX_ZERO_GROUP) a32 = bref = 0.0f;
             }
             Eb = min(max(Eb, 0), 254);
             // multiplier 2^-E / sqrt(b) and the additive rounding window, in scaled units

@@ -1,4 +1,4 @@
-"""Parity of the row kernel with the oracle on inputs at the edges of its fp32 arithmetic: scale ranges that hold
+"""Parity with the oracle on inputs at the edges of the kernels' fp32 arithmetic: scale ranges that hold
 small outputs of a block with large ones, MX groups that cancel exactly."""
 import numpy as np
 import pytest
@@ -106,4 +106,12 @@ def check_zero_groups(B, oracle, T, d, b, perm):
                                         (6, 14336, 14336, True), (9, 2048, 2048, True), (7, 6144, 2048, False),
                                         (5, 16384, 16384, False), (9, 8192, 4096, True)])
 def test_row_kernel_mx_groups_that_cancel(B, oracle, T, d, b, perm):
+    check_zero_groups(B, oracle, T, d, b, perm)
+
+
+@pytest.mark.parametrize("T,d,b,perm", [(20, 1024, 128, False), (20, 3072, 128, False), (20, 2048, 128, True), (20, 2048, 256, False),
+                                        (9, 2048, 512, False), (9, 2048, 1024, False), (9, 1024, 1024, False), (9, 2048, 2048, False),
+                                        (9, 4096, 4096, False), (9, 8192, 8192, False)])
+def test_segment_kernels_mx_groups_that_cancel(B, oracle, T, d, b, perm):
+    """The lean, the group (odd segment counts, permuted, blocks over lanes and warps) and the full-vector kernel."""
     check_zero_groups(B, oracle, T, d, b, perm)
