@@ -1,5 +1,5 @@
 """Parity with the oracle on inputs at the edges of the kernels' fp32 arithmetic: scale ranges that hold
-small outputs of a block with large ones, MX groups that cancel exactly."""
+small outputs of a block with large ones, MX groups that cancel exactly, rows at the upper end of the range."""
 import numpy as np
 import pytest
 import torch
@@ -115,3 +115,24 @@ def test_row_kernel_mx_groups_that_cancel(B, oracle, T, d, b, perm):
 def test_segment_kernels_mx_groups_that_cancel(B, oracle, T, d, b, perm):
     """The lean, the group (odd segment counts, permuted, blocks over lanes and warps) and the full-vector kernel."""
     check_zero_groups(B, oracle, T, d, b, perm)
+
+
+# ------------------------------------------------------------------ rows at the upper end of the fp32 range
+
+def _rows_at_the_upper_end(oracle, T, d, b, seed):
+    """Rows whose largest unnormalised output lies in (2^125.98, 2^126.98] or (2^126.98, 2^127.98], alternating."""
+    rng = np.random.default_rng(seed)
+    x = inputs.bf16_to_f64(inputs.f32_to_bf16_bits((rng.standard_normal((T, d)) + 0.2).astype(np.float32)))
+    u = np.abs(oracle.rotate(inputs.f32_to_bf16_bits(x.astype(np.float32)), None, b)).max(axis=1) * np.sqrt(b)
+    x *= np.exp2(np.floor(126.98 + np.arange(T) % 2 - np.log2(u)))[:, None]
+    bits = inputs.f32_to_bf16_bits(x.astype(np.float32))
+    assert np.array_equal(inputs.bf16_to_f64(bits), x)
+    return bits
+
+
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("int4", 64), ("fp4", 0), ("int4_asym", 0), ("mxfp4", 32)])
+@pytest.mark.parametrize("T,d,b", [(12, 1152, 128), (12, 2048, 2048), (12, 3072, 3072), (12, 4096, 4096), (6, 16384, 16384),
+                                   (6, 14336, 14336)])
+def test_rows_at_the_upper_end_of_the_range(B, oracle, T, d, b, fmt, group):
+    """Outputs whose reciprocal, range or sum of two leaves the fp32 range where they themselves do not."""
+    check(B, oracle, _rows_at_the_upper_end(oracle, T, d, b, 8200 + d + b), None, b, fmt, group)
