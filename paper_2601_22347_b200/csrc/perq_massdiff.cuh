@@ -67,6 +67,12 @@ struct MdSmem {
     }
 };
 
+// A mass as both kernels see it: NaN and negative values count as 0, infinity as the largest float.  The entry point asks
+// for finite non-negative masses; with others in the list, places would collide without being noticed (NaN compares
+// with nothing, negative sums order the wrong way round as bit patterns), and a place that nobody has written holds
+// no block.
+__device__ __forceinline__ float md_mass(float a) { return fminf(fmaxf(a, 0.0f), 3.4028234663852886e38f); }
+
 // Counting by packed fp32 adds: 1.0 for every comparison that holds, two per add (1.5 instructions a comparison
 // where an integer count took 3; counts stay below 2^24, so they are exact).
 __device__ __forceinline__ float md_gt(float a, float b) { float r; asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
@@ -83,7 +89,7 @@ __global__ void __launch_bounds__(MD_RANK_THREADS) perq_massdiff_rank_kernel(Mas
     griddep_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = blockIdx.x * MD_RANK_CHANNELS, i = i0 + lane;
-    const float ai = (i < p.d) ? p.a[i] : 0.0f;
+    const float ai = (i < p.d) ? md_mass(p.a[i]) : 0.0f;
     const float nan = __int_as_float(0x7fffffff);        // padding: no comparison holds
     int rank = 0;
     f32x2 c0 = pack2(0.0f, 0.0f), c1 = c0;
@@ -91,7 +97,7 @@ __global__ void __launch_bounds__(MD_RANK_THREADS) perq_massdiff_rank_kernel(Mas
         const int kn = min(MD_TILE, p.d - k0);
         const int per = ((kn + 255) / 256) * 32;         // masses per warp: a multiple of 32
         __syncthreads();
-        for (int k = threadIdx.x; k < per * 8; k += MD_RANK_THREADS) tile[k] = (k < kn) ? p.a[k0 + k] : nan;
+        for (int k = threadIdx.x; k < per * 8; k += MD_RANK_THREADS) tile[k] = (k < kn) ? md_mass(p.a[k0 + k]) : nan;
         __syncthreads();
         const int lo = warp * per, hi = lo + per, own = i0 - k0;       // all multiples of 32
         const float4 *t4 = reinterpret_cast<const float4 *>(tile);
@@ -177,7 +183,7 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             for (int k = tid; k < w1 - w0; k += nthr) {
                 const int c = min(max(p.order[w0 + k], 0), d - 1);
                 chan[k] = c;
-                mass[k] = p.a[c];
+                mass[k] = md_mass(p.a[c]);
             }
             __syncthreads();
         }
