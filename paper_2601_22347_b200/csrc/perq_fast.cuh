@@ -132,6 +132,9 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
+// Orders the calling thread's own initialisations before bulk copies that use the barriers: every thread that
+// initialises one calls it, before the CTA's barrier.
+__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -956,6 +959,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     if (tid < FAST_WARPS * FAST_NSTAGE) {
         mbar_init(smem_u32(fsmem + FastSmem::full) + tid * 8, 1);
         if (PERM) mbar_init(smem_u32(fsmem + FastSmem::empty) + tid * 8, (uint32_t)G);
+        mbar_init_fence();
     }
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();           // the stream's next kernel may be set up on every SM this grid has left (it waits like this one)
@@ -976,7 +980,6 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
         }
     }
     if (tid < 2 * FAST_WARPS) { wacc[tid] = 0ull; wacc2[tid] = ~0ull; wcnt[tid] = 0u; wflag[tid] = 0u; }
-    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
 
     const uint32_t first = blockIdx.x * GROUPS + group;

@@ -204,8 +204,10 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_full_kernel(FastParams p
     const uint32_t y_warp = y_group + (uint32_t)w_in_g * (8 * FULL_YS * 4);                                      // this warp's chunk rows
     const uint32_t xch_group = smem_base + (uint32_t)FullSmem::xch + (uint32_t)(group * W) * 8;
 
-    if (tid < FAST_WARPS * NST) mbar_init(smem_base + (uint32_t)FullSmem::full + tid * 8, 1);
-    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (tid < FAST_WARPS * NST) {
+        mbar_init(smem_base + (uint32_t)FullSmem::full + tid * 8, 1);
+        mbar_init_fence();
+    }
     __syncthreads();
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_mx_kernel(FastParams p)
     const uint32_t code_buf = smem_base + (uint32_t)MxSmem::codes + (uint32_t)warp * (MX_SPW * SEG_CODE_BYTES);
 
     if (lane < NST) mbar_init(full_base + lane * 8, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_init_fence();
     __syncwarp();
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();           // the stream's next kernel may be set up on every SM this grid has left (it waits like this one)

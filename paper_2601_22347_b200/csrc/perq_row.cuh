@@ -671,13 +671,15 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
     const uint32_t stage_bytes = (uint32_t)segs * SEG_BYTES, full = smem_u32(ms->full);
     const uint32_t row_bytes = (uint32_t)d * 2u;
 
-    if (tid < ROW_NSTAGE) mbar_init(full + tid * 8, 1);
+    if (tid < ROW_NSTAGE) {
+        mbar_init(full + tid * 8, 1);
+        mbar_init_fence();
+    }
     for (int e = tid; e < 2 * ROW_CAP * ROW_MAX_WARPS; e += nthr) (&ms->part[0][0])[e] = 0.0;
     if (tid == 0) {
         ms->cnt[0] = ms->cnt[1] = 0u;
         ms->amax = ms->ahi = 0ull;
         ms->alo = ~0ull;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (NP2) {
         // base matrix as bf16 +-1 (0 in the padding), [output][input]; its sign rows; (group, column) of every four inputs
@@ -1260,8 +1262,10 @@ __global__ void __maxnreg__(ROW64_REGS) perq_row64_kernel(const __grid_constant_
     const uint32_t stage_bytes = (uint32_t)segs * SEG_BYTES, row_bytes = (uint32_t)d * 2u;
     double *tile = reinterpret_cast<double *>(smem + p.off_tile + warp * ROW64_TILE);
 
-    if (tid < ROW_NSTAGE) mbar_init(full + tid * 8, 1);
-    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (tid < ROW_NSTAGE) {
+        mbar_init(full + tid * 8, 1);
+        mbar_init_fence();
+    }
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();
     if (permuted) row_load_perm(p, tabs, threadIdx.x, blockDim.x);

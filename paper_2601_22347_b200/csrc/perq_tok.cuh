@@ -433,8 +433,10 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_tok_kernel(FastParams p)
     const uint32_t xch_group = smem_base + (uint32_t)TokSmem::xch + (uint32_t)(group * W) * 8;
     unsigned long long *wreq = reinterpret_cast<unsigned long long *>(tsmem + TokSmem::wreq) + warp * TOK_MAX_RECORDS;
 
-    if (tid < FAST_WARPS * NST) mbar_init(smem_base + (uint32_t)TokSmem::full + tid * 8, 1);
-    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (tid < FAST_WARPS * NST) {
+        mbar_init(smem_base + (uint32_t)TokSmem::full + tid * 8, 1);
+        mbar_init_fence();
+    }
     __syncthreads();
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();           // the stream's next kernel may be set up on every SM this grid has left (it waits like this one)
