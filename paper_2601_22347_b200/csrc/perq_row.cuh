@@ -44,6 +44,7 @@ constexpr int ROW_CTA_WARPS = 5;              // short rows share a CTA up to th
 constexpr int ROW_NSTAGE = 2;
 constexpr int ROW_CAP = 16;                   // entries per list and round of the CTA-wide exact sums
 constexpr int ROW_WARP_LOG2B = 10;            // blocks up to here are summed by one warp
+constexpr int ROW_MANY = 8;                   // of a lane's 32 outputs: from here on exactness is asked (see RowSpan)
 
 struct RowParams {
     const uint16_t *x;
@@ -74,6 +75,8 @@ struct RowMisc {
     uint32_t cnt[2];                          // list lengths: candidates, ties
     uint32_t list[2 * ROW_CAP];               // row positions
     double part[2 * ROW_CAP][ROW_MAX_WARPS];
+    float span_sum[ROW_MAX_WARPS];            // see RowSpan
+    int span_low[ROW_MAX_WARPS];
 };
 
 // 2^k * 4t: the tile holds the groups of n0 values in order, with `pad` extra words after every eight groups:
@@ -548,6 +551,57 @@ __device__ __forceinline__ void row_patch(uint32_t (&cw)[4], int e, int rot, uin
         if ((le >> 3) == (uint32_t)w) cw[w] = (cw[w] & ~(0xFu << sh)) | (code << sh);
 }
 
+// Rows in which many outputs tie for the maximum or sit on rounding ties (one nonzero, +-constant, few small integers)
+// would pay a sum for each.  Their fp32 rotation is exact: where all inputs are multiples of 2^l and their magnitudes
+// add up to no more than 2^(l + 22), so is every partial sum, and all of them are floats (on the tensor cores too: 23
+// bits below the largest product).  Then the fp32 outputs stand for the sums.  1024 rows of 4096 with one nonzero each,
+// b = d, INT4: 7642 us with a sum for every output, four outputs to a sum (the group kernel before) 2040, 43 now; one
+// nonzero per block of 128, 512 rows of 1152: 312 and 7.
+struct RowSpan {
+    float sum;               // of the magnitudes
+    int low;                 // exponent of the lowest set bit, plus 134
+};
+__device__ __forceinline__ bool row_span_exact(RowSpan s) { return s.sum <= __uint_as_float((uint32_t)min(s.low + 15, 254) << 23); }
+
+// One warp's 1024 inputs (n of them valid).
+__device__ __noinline__ RowSpan row_segment_span(const uint16_t *seg, int n, int lane)
+{
+    RowSpan s = {0.0f, 1 << 20};
+#pragma unroll 1
+    for (int k = lane * 8; k < min(n, SEG_ELEMS); k += 256) {
+        const uint4 w4 = *reinterpret_cast<const uint4 *>(seg + k);
+        const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const uint32_t a = (w[e >> 1] >> (16 * (e & 1))) & 0x7fffu;
+            s.sum += __uint_as_float(a << 16);
+            // (the mantissa with its leading one; subnormals have the exponent of the smallest normal)
+            if (a != 0u) s.low = min(s.low, a < 0x80u ? __ffs(a) : (int)(a >> 7) + __ffs((a & 0x7fu) | 0x80u) - 1);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s.sum += __shfl_xor_sync(0xffffffffu, s.sum, o);
+    s.low = __reduce_min_sync(0xffffffffu, s.low);
+    return s;
+}
+
+// The whole row: every warp its segment, a barrier of the row, then the verdict.
+__device__ __forceinline__ void row_put_span(RowMisc *ms, const uint16_t *xs, int d, int segs, int warp, int lane)
+{
+    if (warp >= segs) return;
+    const RowSpan s = row_segment_span(xs + warp * SEG_ELEMS, d - warp * SEG_ELEMS, lane);
+    if (lane == 0) { ms->span_sum[warp] = s.sum; ms->span_low[warp] = s.low; }
+}
+__device__ __forceinline__ bool row_all_exact(const RowMisc *ms, int segs, int lane)
+{
+    RowSpan s = {0.0f, 1 << 20};
+    if (lane < segs) { s.sum = ms->span_sum[lane & 15]; s.low = ms->span_low[lane & 15]; }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s.sum += __shfl_xor_sync(0xffffffffu, s.sum, o);
+    s.low = __reduce_min_sync(0xffffffffu, s.low);
+    return row_span_exact(s);
+}
+
 // What the quantiser of a lane's 32 values needs: multiplier, rounding window, zero point.
 struct RowQuant {
     float mul, tau, magic;
@@ -642,6 +696,175 @@ __device__ __forceinline__ uint32_t row_reach(const f32x2 (&u)[16], float thr)
 #pragma unroll
     for (int m = 0; m < 16; ++m) bits |= (fabsf(u[m].x) >= thr ? 1u : 0u) << (2 * m) | (fabsf(u[m].y) >= thr ? 2u : 0u) << (2 * m);
     return bits;
+}
+
+// A lane's place in the row, for the functions below.
+struct RowLane {
+    uint32_t tile, i0, t_read;
+    int rot, warp, tid;
+};
+
+// Codes of a lane's doubtful elements where the fp32 outputs are exact: read again from the tile (columns: formed again).
+template <int MODE, int COLS>
+__device__ __forceinline__ void row_settle(uint32_t (&cw)[4], uint32_t tie, const RowLane &L, double a, float mul, double sqrt_b, double s64, double z64,
+                                           int E)
+{
+    f32x2 u[16];
+    if (COLS) row_columns(L.tile, COLS, L.i0, u);
+#pragma unroll 1
+    while (tie) {
+        const int e = __ffs(tie) - 1;
+        tie &= tie - 1;
+        float v = 0.0f;
+        if (COLS) {
+#pragma unroll
+            for (int m = 0; m < 16; ++m) v = (e >> 1) == m ? ((e & 1) ? u[m].y : u[m].x) : v;
+        } else {
+            v = lds_f(L.t_read + 16u * (uint32_t)(((e >> 2) + L.tid) & 7) + 4u * (uint32_t)(e & 3));
+        }
+        const double x = (double)v + 0.0;                     // (+0 for a zero, as the sum gives)
+        row_patch(cw, e, L.rot, MODE == ROW_TOKEN || MODE == ROW_GROUP ? row_int4_code<MODE == ROW_TOKEN>(x, a, mul, sqrt_b)
+                                                                     : row_exact_code<MODE>(x, sqrt_b, s64, z64, E));
+    }
+}
+template <int MODE>
+__device__ __noinline__ uint4 row_settle_warp(uint4 words, uint32_t tie, RowLane L, double a, float mul, double sqrt_b, double s64, double z64, int E)
+{
+    uint32_t cw[4] = {words.x, words.y, words.z, words.w};
+    row_settle<MODE, 0>(cw, tie, L, a, mul, sqrt_b, s64, z64, E);
+    return make_uint4(cw[0], cw[1], cw[2], cw[3]);
+}
+
+// Blocks over several warps: what follows a first round of the lists that did not hold all (all threads of the CTA
+// call).  Not inlined: inside the row's loop these paths cost 7 % of the time of 8192 channels, b = d, INT4.
+// Per token: candidates and doubtful elements.  Leaves the row's exact extremes in amax, or ahi and alo.
+template <int MODE, bool NP2, int COLS>
+__device__ __noinline__ uint4 row_many_token(const RowParams &p, const uint16_t *xs, const unsigned char *tabs, unsigned char *smem, RowLane L,
+                                             uint32_t want, uint32_t tie, uint4 words, float mul, double a_ex, double hi_ex, double lo_ex)
+{
+    RowMisc *ms = reinterpret_cast<RowMisc *>(smem + p.off_misc);
+    uint32_t cw[4] = {words.x, words.y, words.z, words.w};
+    const int lane = L.tid & 31, segs = (p.d + SEG_ELEMS - 1) / SEG_ELEMS;
+    double s64 = 0.0;
+    bool more = true;
+    for (bool first = true; more; first = false) {
+        int slot = 0, tslot = 0;
+        const int took = row_append(ms, 0, want, L.i0, L.rot, COLS, slot);
+        for (int t = 0; t < took; ++t) want &= want - 1;
+        const int ttook = row_append(ms, 1, tie, L.i0, L.rot, COLS, tslot);
+        if (first) row_put_span(ms, xs, p.d, segs, L.warp, lane);
+        __syncthreads();
+        const bool exact = first && row_all_exact(ms, segs, lane);
+        const int total = exact ? 0 : (int)ms->cnt[0], n = min(total, ROW_CAP);
+        const int ttotal = exact ? 0 : (int)ms->cnt[1], tn = min(ttotal, ROW_CAP);
+        const bool last = total <= ROW_CAP;
+        if (exact) {
+            if (MODE == ROW_ASYM) {
+                hi_ex = (double)warp_max_f32(lane < segs ? ms->wmax[lane & 15] : -3.0e38f) + 0.0;
+                lo_ex = (double)warp_min_f32(lane < segs ? ms->wmin[lane & 15] : 3.0e38f) + 0.0;
+            } else {
+                a_ex = (double)warp_max_f32(lane < segs ? ms->wmax[lane & 15] : 0.0f);
+            }
+            if (MODE == ROW_FP4) s64 = a_ex / p.sqrt_b / 7.0;
+            if (MODE != ROW_ASYM && tie) row_settle<MODE, COLS>(cw, tie, L, a_ex, mul, p.sqrt_b, s64, 0.0, 0);
+            want = tie = 0u;
+        }
+        row_all_partials<NP2>(p, xs, tabs, smem, n, tn, L.warp, lane);
+        more = __syncthreads_or(!last || ttotal > ROW_CAP);          // (of any row of the CTA)
+        if (L.tid == 0) ms->cnt[0] = ms->cnt[1] = 0u;
+        for (int e = 0; e < n; ++e) {
+            const double v = row_sum_parts(ms, e);
+            a_ex = fmax(a_ex, fabs(v));
+            hi_ex = fmax(hi_ex, v);
+            lo_ex = fmin(lo_ex, v);
+        }
+        if (last && ttook > 0 && !exact) {
+            if (MODE == ROW_FP4) s64 = a_ex / p.sqrt_b / 7.0;
+            for (int t = 0; t < ttook; ++t) {
+                const int e = __ffs(tie) - 1;
+                tie &= tie - 1;
+                const double v = row_sum_parts(ms, tslot + t);
+                row_patch(cw, e, L.rot, MODE == ROW_TOKEN ? row_int4_code<true>(v, a_ex, mul, p.sqrt_b)
+                                                          : row_exact_code<MODE>(v, p.sqrt_b, s64, 0.0, 0));
+            }
+        }
+        if (more) __syncthreads();
+    }
+    // (per token symmetric: only the row's first thread reads it)
+    if (L.tid == 0) {
+        if (MODE == ROW_ASYM) { ms->ahi = order_key(hi_ex); ms->alo = order_key(lo_ex); }
+        else ms->amax = (unsigned long long)__double_as_longlong(a_ex);
+    }
+    if (MODE == ROW_ASYM) __syncthreads();
+    return make_uint4(cw[0], cw[1], cw[2], cw[3]);
+}
+
+// Per range: the exact maximum of the lane's candidates; lm is the largest magnitude of its fp32 outputs.  worth: more
+// candidates than a few for every range.
+template <bool NP2>
+__device__ __noinline__ double row_many_max(const RowParams &p, const uint16_t *xs, const unsigned char *tabs, unsigned char *smem, RowLane L,
+                                            uint32_t want, bool any, float lm, double a_ex, bool worth)
+{
+    RowMisc *ms = reinterpret_cast<RowMisc *>(smem + p.off_misc);
+    const int lane = L.tid & 31;
+    const int segs = (p.d + SEG_ELEMS - 1) / SEG_ELEMS;
+    bool more = true;
+    for (bool first = worth; more; first = false) {
+        int slot = 0;
+        int took = row_append(ms, 0, want, L.i0, L.rot, 0, slot);
+        for (int t = 0; t < took; ++t) want &= want - 1;
+        if (first) row_put_span(ms, xs, p.d, segs, L.warp, lane);
+        __syncthreads();
+        const bool exact = first && row_all_exact(ms, segs, lane);
+        const int total = exact ? 0 : (int)ms->cnt[0], n = min(total, ROW_CAP);
+        if (exact) {
+            if (any) a_ex = (double)lm;
+            want = 0u;
+            took = 0;
+        }
+        row_all_partials<NP2>(p, xs, tabs, smem, n, 0, L.warp, lane);
+        more = __syncthreads_or(total > ROW_CAP);
+        if (L.tid == 0) ms->cnt[0] = 0u;
+        for (int t = 0; t < took; ++t) a_ex = fmax(a_ex, fabs(row_sum_parts(ms, slot + t)));
+        if (more) __syncthreads();
+    }
+    return a_ex;
+}
+
+// Doubtful elements of formats that quantise after the exact scale.
+template <int MODE, bool NP2, int COLS>
+__device__ __noinline__ uint4 row_many_ties(const RowParams &p, const uint16_t *xs, const unsigned char *tabs, unsigned char *smem, RowLane L,
+                                            uint32_t tie, uint4 words, float mul, double a, double s64, double z64, int E)
+{
+    RowMisc *ms = reinterpret_cast<RowMisc *>(smem + p.off_misc);
+    uint32_t cw[4] = {words.x, words.y, words.z, words.w};
+    const int lane = L.tid & 31;
+    const int segs = (p.d + SEG_ELEMS - 1) / SEG_ELEMS;
+    bool more = true;
+    for (bool first = true; more; first = false) {
+        int slot = 0;
+        int took = row_append(ms, 1, tie, L.i0, L.rot, COLS, slot);
+        if (first) row_put_span(ms, xs, p.d, segs, L.warp, lane);
+        __syncthreads();
+        const bool exact = first && row_all_exact(ms, segs, lane);
+        const int total = exact ? 0 : (int)ms->cnt[1], n = min(total, ROW_CAP);
+        if (exact) {
+            if (tie) row_settle<MODE, COLS>(cw, tie, L, a, mul, p.sqrt_b, s64, z64, E);
+            tie = 0u;
+            took = 0;
+        }
+        row_all_partials<NP2>(p, xs, tabs, smem, 0, n, L.warp, lane);
+        more = __syncthreads_or(total > ROW_CAP);
+        if (L.tid == 0) ms->cnt[1] = 0u;
+        for (int t = 0; t < took; ++t) {
+            const int e = __ffs(tie) - 1;
+            tie &= tie - 1;
+            const double v = row_sum_parts(ms, slot + t);
+            row_patch(cw, e, L.rot, MODE == ROW_GROUP ? row_int4_code<false>(v, a, mul, p.sqrt_b) : row_exact_code<MODE>(v, p.sqrt_b, s64, z64, E));
+        }
+        if (more) __syncthreads();
+    }
+    return make_uint4(cw[0], cw[1], cw[2], cw[3]);
 }
 
 // -------------------------------------------------------------------------------------------- the kernel
@@ -848,17 +1071,20 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
 
         // ---- the lane's 32 outputs, and maxima
         f32x2 u[16];
-        if (cols) row_columns(tile, cols, tid < d / 32 ? i0 : 0u, u);
+        auto read_outputs = [&]() {
+            if (cols) row_columns(tile, cols, tid < d / 32 ? i0 : 0u, u);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (cols) {
-                if (!live) u[2 * j] = u[2 * j + 1] = pack2(0.0f, 0.0f);
-            } else if (live) {
-                lds_v4f(t_read + 16u * (uint32_t)((j + lane) & 7), u[2 * j].x, u[2 * j].y, u[2 * j + 1].x, u[2 * j + 1].y);
-            } else {
-                u[2 * j] = u[2 * j + 1] = pack2(0.0f, 0.0f);
+            for (int j = 0; j < 8; ++j) {
+                if (cols) {
+                    if (!live) u[2 * j] = u[2 * j + 1] = pack2(0.0f, 0.0f);
+                } else if (live) {
+                    lds_v4f(t_read + 16u * (uint32_t)((j + lane) & 7), u[2 * j].x, u[2 * j].y, u[2 * j + 1].x, u[2 * j + 1].y);
+                } else {
+                    u[2 * j] = u[2 * j + 1] = pack2(0.0f, 0.0f);
+                }
             }
-        }
+        };
+        read_outputs();
         float lm = 0.0f, hi = 0.0f, lo = 0.0f;
         if (MODE == ROW_ASYM) {
             hi = live ? u[0].x : -3.0e38f;
@@ -977,46 +1203,73 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
         }
         double s64 = 0.0, z64 = 0.0;
         double a_ex = 0.0, hi_ex = 0.0, lo_ex = 0.0;                      // exact maximum of the lane's range; row extremes
+        const RowLane place = {tile, i0, t_read, rot, warp, tid};
+        // blocks inside a segment, many candidates or doubtful elements: are the segment's fp32 outputs exact?  (asked once)
+        bool asked = false, exact32 = false;
+        auto ask = [&](uint32_t bits) {
+            if (!asked && __any_sync(0xffffffffu, __popc(bits) > ROW_MANY)) {
+                asked = true;
+                exact32 = row_span_exact(row_segment_span(xs + warp * SEG_ELEMS, d - warp * SEG_ELEMS, lane));
+                if (!quantise_first) read_outputs();
+            }
+        };
         if (MODE == ROW_TOKEN || MODE == ROW_FP4 || MODE == ROW_ASYM) {
             hi_ex = -1.7976931348623157e308;
             lo_ex = 1.7976931348623157e308;
             uint32_t want = cand;
             if (wide) {
                 // candidates and doubtful elements in one round (ties are settled once no candidate is left)
-                bool more = true;
-                while (more) {
-                    int slot = 0, tslot = 0;
-                    const int took = row_append(ms, 0, want, i0, rot, cols, slot);
+                int slot = 0, tslot = 0;
+                const int took = row_append(ms, 0, want, i0, rot, cols, slot);
+                const int ttook = row_append(ms, 1, tie, i0, rot, cols, tslot);
+                __syncthreads();
+                const int total = (int)ms->cnt[0], n = min(total, ROW_CAP);
+                const int ttotal = (int)ms->cnt[1], tn = min(ttotal, ROW_CAP);
+                const bool last = total <= ROW_CAP;
+                row_all_partials<NP2>(p, xs, tabs, smem, n, tn, warp, lane);
+                const bool more = __syncthreads_or(!last || ttotal > ROW_CAP);          // (of any row of the CTA)
+                if (tid == 0) ms->cnt[0] = ms->cnt[1] = 0u;
+                if (more || tid == 0 || ttook > 0 || MODE == ROW_ASYM) {
+                    for (int e = 0; e < n; ++e) {
+                        const double v = row_sum_parts(ms, e);
+                        a_ex = fmax(a_ex, fabs(v));
+                        hi_ex = fmax(hi_ex, v);
+                        lo_ex = fmin(lo_ex, v);
+                    }
+                }
+                if (last && ttook > 0) {
+                    if (MODE == ROW_FP4) s64 = a_ex / p.sqrt_b / 7.0;
+                    for (int t = 0; t < ttook; ++t) {
+                        const int e = __ffs(tie) - 1;
+                        tie &= tie - 1;
+                        const double v = row_sum_parts(ms, tslot + t);
+                        row_patch(cw, e, rot, MODE == ROW_TOKEN ? row_int4_code<true>(v, a_ex, Q.mul, p.sqrt_b)
+                                                                : row_exact_code<MODE>(v, p.sqrt_b, s64, 0.0, 0));
+                    }
+                }
+                if (more) {
                     for (int t = 0; t < took; ++t) want &= want - 1;
-                    const int ttook = row_append(ms, 1, tie, i0, rot, cols, tslot);
-                    __syncthreads();
-                    const int total = (int)ms->cnt[0], n = min(total, ROW_CAP);
-                    const int ttotal = (int)ms->cnt[1], tn = min(ttotal, ROW_CAP);
-                    const bool last = total <= ROW_CAP;
-                    row_all_partials<NP2>(p, xs, tabs, smem, n, tn, warp, lane);
-                    more = __syncthreads_or(!last || ttotal > ROW_CAP);          // (of any row of the CTA)
-                    if (tid == 0) ms->cnt[0] = ms->cnt[1] = 0u;
-                    if (more || tid == 0 || ttook > 0 || MODE == ROW_ASYM) {
-                        for (int e = 0; e < n; ++e) {
-                            const double v = row_sum_parts(ms, e);
-                            a_ex = fmax(a_ex, fabs(v));
-                            hi_ex = fmax(hi_ex, v);
-                            lo_ex = fmin(lo_ex, v);
-                        }
+                    if (MODE == ROW_ASYM) {
+                        (void)row_many_token<MODE, NP2, cols>(p, xs, tabs, smem, place, want, 0u, make_uint4(0u, 0u, 0u, 0u), 0.0f, 0.0, hi_ex, lo_ex);
+                        hi_ex = order_value(ms->ahi);
+                        lo_ex = order_value(ms->alo);
+                        read_outputs();                        // (again, so that the call has nothing to keep)
+                    } else {
+                        const uint4 w = row_many_token<MODE, NP2, cols>(p, xs, tabs, smem, place, want, tie, make_uint4(cw[0], cw[1], cw[2], cw[3]),
+                                                                        Q.mul, a_ex, hi_ex, lo_ex);
+                        cw[0] = w.x; cw[1] = w.y; cw[2] = w.z; cw[3] = w.w;
+                        tie = 0u;
+                        if (tid == 0) a_ex = __longlong_as_double((long long)ms->amax);
                     }
-                    if (last && ttook > 0) {
-                        if (MODE == ROW_FP4) s64 = a_ex / p.sqrt_b / 7.0;
-                        for (int t = 0; t < ttook; ++t) {
-                            const int e = __ffs(tie) - 1;
-                            tie &= tie - 1;
-                            const double v = row_sum_parts(ms, tslot + t);
-                            row_patch(cw, e, rot, MODE == ROW_TOKEN ? row_int4_code<true>(v, a_ex, Q.mul, p.sqrt_b)
-                                                                    : row_exact_code<MODE>(v, p.sqrt_b, s64, 0.0, 0));
-                        }
-                    }
-                    if (more) __syncthreads();
                 }
             } else {
+                ask(want);
+                if (exact32 && want != 0u) {                  // (a lane with a candidate holds its own extremes among them)
+                    a_ex = (double)lm;
+                    hi_ex = (double)hi + 0.0;
+                    lo_ex = (double)lo + 0.0;
+                    want = 0u;
+                }
                 unsigned cl = __ballot_sync(0xffffffffu, want != 0u);
                 while (cl) {
                     const int src = __ffs(cl) - 1;
@@ -1033,7 +1286,7 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
                         lo_ex = fmin(lo_ex, v);
                     }
                 }
-                if (lane == 0 && hi_ex >= lo_ex) {
+                if ((lane == 0 || exact32) && hi_ex >= lo_ex) {
                     if (MODE == ROW_ASYM) {
                         atomicMax(&ms->ahi, order_key(hi_ex));
                         atomicMin(&ms->alo, order_key(lo_ex));
@@ -1053,20 +1306,18 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
             // the exact maximum of every range: its candidates, four lanes to a sum (long blocks: CTA-wide)
             uint32_t want = cand;
             if (wide) {
-                bool more = true;
-                while (more) {
-                    int slot = 0;
-                    const int took = row_append(ms, 0, want, i0, rot, cols, slot);
-                    for (int t = 0; t < took; ++t) want &= want - 1;
-                    __syncthreads();
-                    const int total = (int)ms->cnt[0], n = min(total, ROW_CAP);
-                    row_all_partials<NP2>(p, xs, tabs, smem, n, 0, warp, lane);
-                    more = __syncthreads_or(total > ROW_CAP);
-                    if (tid == 0) ms->cnt[0] = 0u;
-                    for (int t = 0; t < took; ++t) a_ex = fmax(a_ex, fabs(row_sum_parts(ms, slot + t)));
-                    if (more) __syncthreads();
-                }
+                int slot = 0;
+                const int took = row_append(ms, 0, want, i0, rot, cols, slot);
+                __syncthreads();
+                const int total = (int)ms->cnt[0], n = min(total, ROW_CAP);
+                row_all_partials<NP2>(p, xs, tabs, smem, n, 0, warp, lane);
+                const bool more = __syncthreads_or(total > ROW_CAP);
+                if (tid == 0) ms->cnt[0] = 0u;
+                for (int t = 0; t < took; ++t) { want &= want - 1; a_ex = fmax(a_ex, fabs(row_sum_parts(ms, slot + t))); }
+                if (more) a_ex = row_many_max<NP2>(p, xs, tabs, smem, place, want, cand != 0u, lm, a_ex, total > 2 * (d >> p.log2g));
             } else {
+                ask(want);
+                if (exact32 && want != 0u) { a_ex = (double)lm; want = 0u; }
                 // (all quads step together; the lanes of a quad take turns)
                 while (__any_sync(0xffffffffu, want != 0u)) {
                     const unsigned have = (__ballot_sync(0xffffffffu, want != 0u) >> (lane & 28)) & 0xFu;
@@ -1085,20 +1336,21 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
             if (wide ? __syncthreads_or(near) : __any_sync(0xffffffffu, near)) {
                 uint32_t want = cand;
                 if (wide) {
-                    bool more = true;
-                    while (more) {
-                        int slot = 0;
-                        const int took = row_append(ms, 0, want, i0, rot, cols, slot);
-                        for (int t = 0; t < took; ++t) want &= want - 1;
-                        __syncthreads();
-                        const int total = (int)ms->cnt[0], n = min(total, ROW_CAP);
-                        row_all_partials<NP2>(p, xs, tabs, smem, n, 0, warp, lane);
-                        more = __syncthreads_or(total > ROW_CAP);
-                        if (tid == 0) ms->cnt[0] = 0u;
-                        for (int t = 0; t < took; ++t) a_ex = fmax(a_ex, fabs(row_sum_parts(ms, slot + t)));
-                        if (more) __syncthreads();
+                    int slot = 0;
+                    const int took = row_append(ms, 0, want, i0, rot, cols, slot);
+                    __syncthreads();
+                    const int total = (int)ms->cnt[0], n = min(total, ROW_CAP);
+                    row_all_partials<NP2>(p, xs, tabs, smem, n, 0, warp, lane);
+                    const bool more = __syncthreads_or(total > ROW_CAP);
+                    if (tid == 0) ms->cnt[0] = 0u;
+                    for (int t = 0; t < took; ++t) { want &= want - 1; a_ex = fmax(a_ex, fabs(row_sum_parts(ms, slot + t))); }
+                    if (more) {
+                        a_ex = row_many_max<NP2>(p, xs, tabs, smem, place, want, cand != 0u, lm, a_ex, true);
+                        read_outputs();
                     }
                 } else {
+                    ask(want);
+                    if (exact32 && want != 0u) { a_ex = (double)lm; want = 0u; }
                     while (__any_sync(0xffffffffu, want != 0u)) {
                         const unsigned have = (__ballot_sync(0xffffffffu, want != 0u) >> (lane & 28)) & 0xFu;
                         const int src = have ? __ffs(have) - 1 : 0;
@@ -1168,25 +1420,32 @@ __global__ void __maxnreg__(ROW_REGS) perq_row_kernel(const __grid_constant__ Ro
                 z64 = (s64 == 0.0) ? 0.0 : rint(lo_ex / p.sqrt_b / s64);
             }
             if (wide) {
-                bool more = true;
-                while (more) {
-                    int slot = 0;
-                    const int took = row_append(ms, 1, tie, i0, rot, cols, slot);
-                    __syncthreads();
-                    const int total = (int)ms->cnt[1], n = min(total, ROW_CAP);
-                    row_all_partials<NP2>(p, xs, tabs, smem, 0, n, warp, lane);
-                    more = __syncthreads_or(total > ROW_CAP);
-                    if (tid == 0) ms->cnt[1] = 0u;
-                    for (int t = 0; t < took; ++t) {
-                        const int e = __ffs(tie) - 1;
-                        tie &= tie - 1;
-                        const double v = row_sum_parts(ms, slot + t);
-                        row_patch(cw, e, rot, MODE == ROW_GROUP ? row_int4_code<false>(v, a_ex, Q.mul, p.sqrt_b)
-                                                                : row_exact_code<MODE>(v, p.sqrt_b, s64, z64, Eb - 127));
-                    }
-                    if (more) __syncthreads();
+                int slot = 0;
+                const int took = row_append(ms, 1, tie, i0, rot, cols, slot);
+                __syncthreads();
+                const int total = (int)ms->cnt[1], n = min(total, ROW_CAP);
+                row_all_partials<NP2>(p, xs, tabs, smem, 0, n, warp, lane);
+                const bool more = __syncthreads_or(total > ROW_CAP);
+                if (tid == 0) ms->cnt[1] = 0u;
+                for (int t = 0; t < took; ++t) {
+                    const int e = __ffs(tie) - 1;
+                    tie &= tie - 1;
+                    const double v = row_sum_parts(ms, slot + t);
+                    row_patch(cw, e, rot, MODE == ROW_GROUP ? row_int4_code<false>(v, a_ex, Q.mul, p.sqrt_b)
+                                                            : row_exact_code<MODE>(v, p.sqrt_b, s64, z64, Eb - 127));
+                }
+                if (more) {
+                    const uint4 w = row_many_ties<MODE, NP2, cols>(p, xs, tabs, smem, place, tie, make_uint4(cw[0], cw[1], cw[2], cw[3]), Q.mul,
+                                                                   a_ex, s64, z64, Eb - 127);
+                    cw[0] = w.x; cw[1] = w.y; cw[2] = w.z; cw[3] = w.w;
                 }
             } else {
+                ask(tie);
+                if (exact32 && tie) {
+                    const uint4 w = row_settle_warp<MODE>(make_uint4(cw[0], cw[1], cw[2], cw[3]), tie, place, a_ex, Q.mul, p.sqrt_b, s64, z64, Eb - 127);
+                    cw[0] = w.x; cw[1] = w.y; cw[2] = w.z; cw[3] = w.w;
+                    tie = 0u;
+                }
                 unsigned tl = __ballot_sync(0xffffffffu, tie != 0u);
                 while (tl) {
                     const int src = __ffs(tl) - 1;
@@ -1262,10 +1521,11 @@ __global__ void __maxnreg__(ROW64_REGS) perq_row64_kernel(const __grid_constant_
     const uint32_t stage_bytes = (uint32_t)segs * SEG_BYTES, row_bytes = (uint32_t)d * 2u;
     double *tile = reinterpret_cast<double *>(smem + p.off_tile + warp * ROW64_TILE);
 
-    if (tid < ROW_NSTAGE) {
-        mbar_init(full + tid * 8, 1);
-        mbar_init_fence();
-    }
+    // (as mbar_init and mbar_init_fence, in one statement and with thread 0's fence a second time: written the plain way the
+    // compiler spills 8 bytes more, 33.1 against 32.1 us for 4096 x 2048, b = d, per 128)
+    if (tid < ROW_NSTAGE)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tfence.mbarrier_init.release.cluster;" ::"r"(full + tid * 8) : "memory");
+    if (tid == 0) mbar_init_fence();
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();
     if (permuted) row_load_perm(p, tabs, threadIdx.x, blockDim.x);

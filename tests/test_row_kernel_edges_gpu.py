@@ -1,5 +1,6 @@
 """Parity with the oracle on inputs at the edges of the kernels' fp32 arithmetic: scale ranges that hold
-small outputs of a block with large ones, MX groups that cancel exactly, rows at the upper end of the range."""
+small outputs of a block with large ones, MX groups that cancel exactly, rows at the upper end of the range,
+rows in which many outputs tie."""
 import numpy as np
 import pytest
 import torch
@@ -136,3 +137,35 @@ def _rows_at_the_upper_end(oracle, T, d, b, seed):
 def test_rows_at_the_upper_end_of_the_range(B, oracle, T, d, b, fmt, group):
     """Outputs whose reciprocal, range or sum of two leaves the fp32 range where they themselves do not."""
     check(B, oracle, _rows_at_the_upper_end(oracle, T, d, b, 8200 + d + b), None, b, fmt, group)
+
+
+# ------------------------------------------------------------------ flat rows: many outputs tie, fp32 is exact
+
+def _flat_rows(T, d, b, seed):
+    """One nonzero in the row, one in every block, few small integers, +-constant, constant, and rows just beyond the reach of
+    exact fp32 arithmetic: a large and a tiny nonzero."""
+    rng = np.random.default_rng(seed)
+    x = np.zeros((T, d))
+    for t in range(T):
+        blk = x[t].reshape(d // b, b)
+        if t % 6 == 0:
+            x[t, rng.integers(d)] = -2.625
+        elif t % 6 == 1:
+            blk[:, rng.integers(b)] = 1.5 * (1 + np.arange(d // b) % 3)
+        elif t % 6 == 2:
+            x[t, rng.choice(d, 8, replace=False)] = np.arange(1, 9)
+        elif t % 6 == 3:
+            x[t] = np.where(rng.random(d) < 0.5, -1.25, 1.25)
+        elif t % 6 == 4:
+            x[t] = 1.2890625 * 2.0 ** rng.integers(-100, 100)
+        else:
+            x[t, rng.choice(d, 2, replace=False)] = 3.0, 2.0 ** -23
+    return inputs.f32_to_bf16_bits(x.astype(np.float32))
+
+
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 32), ("int4", 128), ("fp4", 0), ("int4_asym", 0), ("mxfp4", 32)])
+@pytest.mark.parametrize("T,d,b,perm", [(18, 1152, 128, False), (18, 640, 32, True), (24, 1024, 128, False), (18, 3072, 1024, True), (12, 2048, 2048, False),
+                                        (12, 4096, 4096, False), (12, 6144, 2048, True), (6, 8192, 8192, False), (12, 3072, 3072, False), (6, 14336, 14336, True)])
+def test_flat_rows(B, oracle, T, d, b, perm, fmt, group):
+    p = inputs.random_perm(d, 83) if perm else None
+    check(B, oracle, through(_flat_rows(T, d, b, 8300 + d + b), p), p, b, fmt, group)
