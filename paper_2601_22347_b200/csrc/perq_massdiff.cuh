@@ -13,12 +13,14 @@
 //   up to M are exactly the prefix that the greedy serves before it returns to a block.  That prefix is served
 //   at once, and its new sums are merged into the list.
 //
-// The greedy is a serial chain: one channel at a time (a scan of all running sums per channel) it took 2316 us, in
-// batches it takes 164 us
-// for 8192 channels in 256 blocks.  Sums differ by about one channel mass, so a batch serves most of the
-// blocks: 64 batches there, 31 to 157 for 8 to 512 blocks of real statistics.  Masses that fall steeply make small
-// batches; then channels are served one by one for a while, each an insertion into the list by all threads at one
-// barrier.  Zero masses (padded channels) change no sum: what is left of them fills the blocks in list order.
+// Sums differ by about one channel mass, so a batch serves most of the blocks: 66 batches for 8192 channels of a
+// real statistic in 256 blocks, 176 us (one channel at a time, one warp scanning all running sums: 2316 us).
+// Masses that fall steeply make small batches, and few blocks small ones anyway.  Channels are then served one by one by
+// one warp: 32 channels reach no more than the first 32 entries of the list, so a lane holds one entry in registers and a
+// channel costs three warp reductions; afterwards the entries are merged back like a batch.  (By all threads, a barrier
+// and an insertion into the list per channel, 8192 steeply falling masses took 2593 us, 4096 channels in four blocks 2813;
+// this way 1030 and 594.  The scan: 2303 and 860.)
+// Zero masses (padded channels) change no sum, and a last open block takes what is left: no greedy is needed then.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -140,8 +142,22 @@ __device__ __forceinline__ bool md_less(unsigned long long s, int i, unsigned lo
     return s < t || (s == t && (i & MD_ID_MASK) < (j & MD_ID_MASK));
 }
 
-constexpr int MD_SERIAL_K = 6;           // batches below this are followed by MD_SERIAL_STEPS channels one by one
-constexpr int MD_SERIAL_STEPS = 32;
+// A batch costs as much as 16 channels one by one.  Below 6 channels it is followed by 32 of those, by two and four
+// times 32 if the next batches are small again; up to 16 blocks all channels go one by one.  (Whenever 32 blocks or
+// fewer are open: 244 against 176 us for the 8192 channels above, whose last blocks fill in large batches.)
+constexpr int MD_FEW_BLOCKS = 16;
+constexpr int MD_SERIAL_K = 6;
+constexpr int MD_SERIAL_RUNS = 4;
+
+// The smallest (sum, block) of a warp's lanes.
+__device__ __forceinline__ void md_warp_min(unsigned long long v, int blk, unsigned long long &m, int &m_blk)
+{
+    const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
+    const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
+    m_blk = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)blk : (uint32_t)MD_ID_MASK);
+    m = ((unsigned long long)mhi << 32) | mlo;
+}
 
 __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel(MassdiffParams p)
 {
@@ -173,7 +189,7 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
     while (split < 1 && (n << (split + 1)) <= nthr) ++split;
     int m = n;                  // open blocks: list entries [0, m)
     int s = 0, w0 = 0, w1 = 0;  // next rank; staged window of ranks [w0, w1)
-    int serial = 0;             // channels still to be served one by one
+    int serial = 0, runs = 1;   // runs of 32 channels still to be served one by one; after the next small batch
     uint32_t batch = 0;
     while (s < d) {
         if (s >= w1) {
@@ -187,59 +203,60 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             }
             __syncthreads();
         }
-        if (mass[s - w0] == 0.0f) break;          // (only zero masses are left: below)
-        if (serial > 0) {
-            // ---- one channel: the first entry takes it and moves to its new place (one barrier)
-            --serial;
-            const unsigned long long s0 = sum[0];
-            const int e0 = id[0], f = e0 >> MD_ID_BITS;
-            const bool full = f + 1 == b;
-            const double ns = __longlong_as_double((long long)s0) + (double)mass[s - w0];
-            const unsigned long long v = (unsigned long long)__double_as_longlong(ns);
-            const int e1 = e0 + (1 << MD_ID_BITS);
-            for (int j = tid; j < m; j += nthr) {
-                if (j == 0) p.perm[(size_t)(e0 & MD_ID_MASK) * b + f] = chan[s - w0];
-                // entries 1 .. below the new sum move up by one place; the new sum goes behind them
-                const bool below = j > 0 && (full || md_less(sum[j], id[j], v, e1));
-                const bool next_below = j + 1 < m && (full || md_less(sum[j + 1], id[j + 1], v, e1));
-                if (below) { sum_next[j - 1] = sum[j]; id_next[j - 1] = id[j]; }
-                else if (j > 0) { sum_next[j] = sum[j]; id_next[j] = id[j]; }
-                if (!full && (below || j == 0) && !next_below) { sum_next[j] = v; id_next[j] = e1; }
+        if (m == 1 || mass[s - w0] == 0.0f) break;          // one block or only zero masses are left: below
+        const bool one_by_one = n <= MD_FEW_BLOCKS || serial > 0;
+        unsigned long long M;                     // the smallest new sum
+        int M_id = MD_ID_MASK, K, q, steps, given;
+        if (one_by_one) {
+            // ---- 32 channels (few blocks: the window) one by one: lane j of warp 0 has entry j
+            if (serial > 0) --serial;
+            if (warp == 0) {
+                const int room = n <= MD_FEW_BLOCKS ? w1 - s : min(32, w1 - s);
+                unsigned long long v = lane < m ? sum[lane] : ~0ull;
+                int e = lane < m ? id[lane] : MD_ID_MASK, t = 0;
+                const int e0 = e;
+                for (; t < room; ++t) {
+                    const float a = mass[s - w0 + t];
+                    if (a == 0.0f) break;
+                    unsigned long long least;
+                    int blk;
+                    md_warp_min(v, e & MD_ID_MASK, least, blk);
+                    if (v == least && (e & MD_ID_MASK) == blk && lane < m) {
+                        const int f = e >> MD_ID_BITS;
+                        p.perm[(size_t)blk * b + f] = chan[s - w0 + t];
+                        const double ns = __longlong_as_double((long long)v) + (double)a;
+                        v = f + 1 < b ? (unsigned long long)__double_as_longlong(ns) : INF;
+                        e += 1 << MD_ID_BITS;
+                    }
+                }
+                if (lane < m) { fresh[lane] = v; id[lane] = e; }
+                // (the entries that were served are a prefix of the list)
+                const unsigned touched = __ballot_sync(0xffffffffu, e != e0);
+                md_warp_min(e != e0 ? v : INF, e & MD_ID_MASK, M, M_id);
+                if (lane == 0) { red_sum[0] = M; red_open[3] = t; red_open[4] = max(1, 32 - __clz((int)touched)); }
             }
-            if (full) --m;
-            ++s;
             __syncthreads();
-            swap_lists();
-            continue;
-        }
-        // ---- the sums that the next q blocks of the list would reach, and the smallest of them
-        const int q = min(m, w1 - s);
-        unsigned long long best = INF;
-        int best_id = MD_ID_MASK;
-        for (int j = tid; j < q; j += nthr) {
-            const double ns = __longlong_as_double((long long)sum[j]) + (double)mass[s - w0 + j];
-            const unsigned long long v = ((id[j] >> MD_ID_BITS) + 1 < b) ? (unsigned long long)__double_as_longlong(ns) : INF;
-            fresh[j] = v;
-            if (v != INF && md_less(v, id[j], best, best_id)) { best = v; best_id = id[j] & MD_ID_MASK; }
-        }
-        {
-            const uint32_t hi = (uint32_t)(best >> 32), lo = (uint32_t)best;
-            const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
-            const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-            const int mid = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)best_id : (uint32_t)MD_ID_MASK);
-            if (lane == 0) { red_sum[warp] = ((unsigned long long)mhi << 32) | mlo; red_id[warp] = mid; }
-        }
-        __syncthreads();
-        unsigned long long M;
-        int M_id;
-        {
-            const unsigned long long v = red_sum[lane];
-            const int vi = red_id[lane];
-            const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
-            const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
-            const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-            M_id = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (uint32_t)vi : (uint32_t)MD_ID_MASK);
-            M = ((unsigned long long)mhi << 32) | mlo;
+            M = red_sum[0];
+            steps = red_open[3];
+            K = q = red_open[4];
+            given = 0;                            // (the entries' fill counts and perm are written)
+        } else {
+            // ---- the sums that the next q blocks of the list would reach, and the smallest of them
+            q = min(m, w1 - s);
+            unsigned long long best = INF;
+            int best_id = MD_ID_MASK;
+            for (int j = tid; j < q; j += nthr) {
+                const double ns = __longlong_as_double((long long)sum[j]) + (double)mass[s - w0 + j];
+                const unsigned long long v = ((id[j] >> MD_ID_BITS) + 1 < b) ? (unsigned long long)__double_as_longlong(ns) : INF;
+                fresh[j] = v;
+                if (v != INF && md_less(v, id[j], best, best_id)) { best = v; best_id = id[j] & MD_ID_MASK; }
+            }
+            md_warp_min(best, best_id, M, M_id);
+            if (lane == 0) { red_sum[warp] = M; red_id[warp] = M_id; }
+            __syncthreads();
+            md_warp_min(red_sum[lane], red_id[lane], M, M_id);
+            K = steps = 0;
+            given = 1 << MD_ID_BITS;
         }
         // ---- K: the list entries up to M.  Distances of all sums to M in fp32 (sums within a batch are close
         // to each other: the difference, not the sum, is what fp32 resolves)
@@ -248,12 +265,17 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             key_old[j] = (float)(__longlong_as_double((long long)sum[j]) - m64);
             if (j < q) key[j] = (fresh[j] != INF) ? (float)(__longlong_as_double((long long)fresh[j]) - m64) : __int_as_float(0x7f800000);
         }
-        int K = 0;
-        for (int j0 = 0; j0 < q; j0 += nthr) {
-            const int j = j0 + tid;
-            K += __syncthreads_count(j < q && !md_less(M, M_id, sum[min(j, q - 1)], id[min(j, q - 1)]));
+        if (one_by_one) {
+            __syncthreads();
+        } else {
+            for (int j0 = 0; j0 < q; j0 += nthr) {
+                const int j = j0 + tid;
+                K += __syncthreads_count(j < q && !md_less(M, M_id, sum[min(j, q - 1)], id[min(j, q - 1)]));
+            }
+            K = steps = max(K, 1);
+            if (K < MD_SERIAL_K && K < q) { serial = runs; runs = min(2 * runs, MD_SERIAL_RUNS); }
+            else if (K < q) runs = 1;
         }
-        K = max(K, 1);
         // ---- serve them; every entry's place in the merged list: new sums below it (counted, 2^split threads
         // to an entry), and for a new sum the untouched entries below it (searched).  fp32 distances to M
         // decide; equal ones (masses are sums of bf16: equal sums do occur, a few per batch) show as entries that
@@ -280,8 +302,8 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             int blk = id[j];
             const unsigned long long v64 = served ? fresh[j] : sum[j];
             if (served) {
-                p.perm[(size_t)(blk & MD_ID_MASK) * b + (blk >> MD_ID_BITS)] = chan[s - w0 + j];
-                blk += 1 << MD_ID_BITS;
+                if (given) p.perm[(size_t)(blk & MD_ID_MASK) * b + (blk >> MD_ID_BITS)] = chan[s - w0 + j];
+                blk += given;
                 if (v64 == INF) { place[j] = -1; atomicAdd(closed, 1); continue; }
             }
             // (untouched entries are in order; equal distances among them share the first one's place)
@@ -318,7 +340,7 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
                 for (int k = lane; k < m; k += 32)
                     before += (place[k] == pj && md_less(k < K ? fresh[k] : sum[k], id[k], v64, blk)) ? 1 : 0;
                 before = __reduce_add_sync(0xffffffffu, before);
-                if (lane == 0) { sum_next[pj + before] = v64; id_next[pj + before] = blk + (j < K ? 1 << MD_ID_BITS : 0); }
+                if (lane == 0) { sum_next[pj + before] = v64; id_next[pj + before] = blk + (j < K ? given : 0); }
             }
             __syncthreads();
             for (int e = tid; e < nd; e += nthr) crowded[place[doubtful[e]]] = 0;
@@ -327,12 +349,12 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
         if (tid == 0) *closed_next = 0;
         __syncthreads();
         m -= *closed;
-        s += K;
+        s += steps;
         ++batch;
-        if (K < MD_SERIAL_K && K < q) serial = MD_SERIAL_STEPS;
         swap_lists();
     }
-    // ---- zero masses change no sum: the blocks of the list take what they have room for, one after the other
+    // ---- zero masses change no sum: the blocks of the list take what they have room for, one after the other (so does
+    // the last open block)
     if (s < d) {
         for (int r = s + tid; r < d; r += nthr) {
             const int c = min(max(p.order[r], 0), d - 1);

@@ -32,3 +32,16 @@ def test_masses_that_are_not_finite_and_non_negative(B, d, b):
     a[d // 2] = np.nan
     clean = np.minimum(np.where(a > 0, a, 0), np.finfo(np.float32).max).astype(np.float32)
     assert np.array_equal(device_perm(B, a, b), B.perq_massdiff_perm(clean, b))
+
+
+@pytest.mark.parametrize("kind", ["exponential", "steep", "equal", "half_zero", "few_large"])
+@pytest.mark.parametrize("d,b", [(32, 32), (64, 32), (96, 32), (1024, 32), (1056, 32), (2112, 64), (4096, 1024), (4096, 1), (8192, 8192),
+                                 (6144, 48), (32768, 1024)])
+def test_channels_one_by_one(B, kind, d, b):
+    """1 to 32 blocks (never merged inside a window of 2048 channels), 33, and masses whose batches are too small."""
+    rng = np.random.default_rng(9100 + d + b)
+    a = {"exponential": rng.exponential(size=d), "steep": 1.02 ** -np.arange(d).clip(0, 4000), "equal": np.ones(d),
+         "half_zero": rng.exponential(size=d) * (rng.random(d) < 0.5),
+         "few_large": rng.exponential(size=d) * np.where(rng.random(d) < 0.01, 1e5, 1.0)}[kind]
+    a = rng.permutation(a.astype(np.float32))
+    assert np.array_equal(device_perm(B, a, b), B.perq_massdiff_perm(a, b))
