@@ -103,9 +103,9 @@ typedef enum {
  *            paper does not print its base matrices; B is Paley's second construction for the prime
  *            q = 2t - 1 (symmetric, B B^T = 4t I), so codes need not equal those of another implementation's
  *            matrix.  Other non-power-of-two b, and such a b inside a longer row: PERQ_ERR_BLOCK.
- *            The tensor-core kernels cover d % 1024 == 0 with
- *            b <= 128 (any scale mode, with or without perm) and, unpermuted with per-token or MX
- *            scales, b <= 1024 and b == d <= 8192; everything else runs on a slower general kernel.
+ *            All of these run on tensor-core kernels when d % 128 == 0 and d <= 16384 (for 2^k' * 4t: 6 <= k' <= 10)
+ *            and an INT4 group is 0 or a power of two from 32 to 1024; other widths, groups and the F32_DEBUG
+ *            output run on a slower general kernel.
  * fmt        perq_fmt_t.
  * group      INT4: 0 (per token) or a multiple of 8 that divides d and is a multiple or a divisor of b.
  *            MXFP4: 0 or 32 (always 32).  FP4, INT4_ASYM: 0.
@@ -117,9 +117,12 @@ typedef enum {
  * Codes and scales are deterministic (bit-identical from run to run).  Which kernel serves a call depends
  * on its shape; every kernel stores the fp32 rounding of the exact scale up to one more rounding of a
  * constant factor, so scales of the same row from different shapes' kernels agree to 1 ulp, not bit for bit.
- * Range limit: a token whose largest |y| lies below about 2^-120 (every input subnormal or nearly so) gets
+ * Range limits: a token whose largest |y| lies below about 2^-120 (every input subnormal or nearly so) gets
  * the exact scale but all-zero INT4/FP4 codes from the tensor-core kernels, because the fp32 reciprocal of
- * such a scale overflows; the definition would give +-7 at the maximum.
+ * such a scale overflows; the definition would give +-7 at the maximum.  At the other end sqrt(b) |y| has to stay
+ * below 2^126 (d % 1024 == 0 with b <= 128, or unpermuted blocks of 256 to 1024: above it the codes come out 0) or
+ * below 2^128 (all other shapes).  A scale range or MX group that is part of a Hadamard block and whose outputs all
+ * cancel to zero in fp32 (below about 2^-24 of the block's largest) gets scale 0.
  */
 int perq_rotate_quantize(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t b,
                          int32_t fmt, int32_t group, void *out_codes, void *out_scales,
@@ -305,8 +308,9 @@ int perq_zigzag_perm(const float *chan_abs_max_host, int32_t d, int32_t b, int32
  *   workspace        device, at least d * 4 bytes (the channels in visiting order); caller-owned
  *   stream           cudaStream_t (0 = default); two kernels are enqueued, nothing is synchronised
  *
- * b >= 1, d % b == 0, d <= PERQ_MAX_D and at most 4096 blocks (d / b).  The greedy is sequential in the
- * channels (one warp scans the open blocks d times): about 2.3 ms for d = 8192, b = 32.
+ * b >= 1, d % b == 0, d <= PERQ_MAX_D and at most 4096 blocks (d / b).  One CTA serves the channels in batches,
+ * about 0.18 ms for a statistic of d = 8192, b = 32; masses that fall steeply are served one by one (about 1 ms
+ * there).  NaN and negative masses count as 0, infinity as the largest float.
  * Errors: NULL, SHAPE, BLOCK (also: too many blocks), WORKSPACE, ALIGN, CUDA.
  */
 int perq_massdiff_perm_device(const float *chan_abs_sum, int32_t d, int32_t b, int32_t *perm,
