@@ -194,7 +194,7 @@ int launch_generic(const void *x, const int32_t *perm, int64_t T, int32_t d, int
 }
 
 // Row kernel: a warp per 1024 channels, one CTA per row (short rows share one).  It takes every call that the
-// segment kernels do not and that it can hold (below); it was 1.1 to 17 times faster than the general kernel over all
+// segment kernels do not and that it can hold (below); it was 1.0 to 15 times faster than the general kernel over all
 // of them (widths 768 .. 14336, 1 .. 4096 rows, all formats), which keeps the rest: other widths and ranges, fp32 output.
 template <int ROT, int MODE>
 int launch_row_inst(const perq::RowParams &p, int grid, int threads, size_t smem, cudaStream_t st)
@@ -498,7 +498,8 @@ int try_launch_fast(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     if (longb && (b > perq::SEG_ELEMS || permuted)) return -1;
     if (full && (permuted || (segs != 1 && segs != 2 && segs != 4 && segs != 8))) return -1;
     // whole-row blocks with one INT4 scale: one warp per row keeps them in registers; from two warps on the row
-    // kernel's exchange is the better one (4096 rows: 13.0 us here, 16.7 there at 1024; 57.0 and 31.2 at 4096)
+    // kernel's exchange is the better one (4096 rows of 1024 channels: 13.0 us here, 16.7 there; 2048 .. 8192 channels, 1, 128
+    // and 4096 rows: 3.8 .. 8.3, 11.8 .. 27 and 31 .. 178 us here, 3.4 .. 4.9, 4.5 .. 7.1 and 20 .. 80 there)
     if (full && fmt == PERQ_FMT_INT4 && segs > 1) return -1;
     if (permuted && (d > perq::FastSmem::PERM_MAX_D || segs > perq::FAST_WARPS)) return -1;
     int mode, G = 1;
