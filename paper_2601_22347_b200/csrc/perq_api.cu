@@ -25,6 +25,8 @@
 #include "perq_diag.cuh"
 #include "perq_massdiff.cuh"
 #include "perq_row.cuh"
+#include "perq_tile.cuh"
+#include "perq_col.cuh"
 
 namespace {
 
@@ -598,11 +600,16 @@ int launch_swiglu_b(int log2b, const perq::FastParams &p, int grid, cudaStream_t
     }
 }
 
+#include "perq_tile_launch.cuh"
+
 int launch_any(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t b, int32_t fmt, int g,
                void *out_codes, void *out_scales, cudaStream_t st)
 {
     if (is_pow2(b)) {
-        const int rc = try_launch_fast(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
+        int rc = b == d && b > 128 ? try_launch_col(x, perm, T, d, b, fmt, g, out_codes, out_scales, st)
+                                   : try_launch_tile(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
+        if (rc >= 0) return rc;
+        rc = try_launch_fast(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
         if (rc >= 0) return rc;
     }
     const int rc = try_launch_row(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);

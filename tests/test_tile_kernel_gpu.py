@@ -1,0 +1,98 @@
+"""Parity of the tile and column kernels with the oracle: calls large enough to be theirs, with ragged numbers of rows, in which
+every CTA serves several tiles (ring stages, accumulators and note slots are used again and change their phase).  The GPU
+runs the whole call, the oracle the base rows it is made of; every repetition of a base row has to give the same bytes.
+
+The base rows hold what each rule of these kernels meets: rows with outliers, rows without, zeros, one nonzero (every
+output of its block ties), small integers (true rounding ties), a row of them at the lowest and one at the highest
+exponents of bf16 that the formats take.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_22347_b200 import inputs
+
+from parity import compare_quantized
+
+pytestmark = pytest.mark.gpu
+
+FMT = {"int4": 0, "mxfp4": 1, "fp4": 3, "int4_asym": 4}
+BASE = 160
+
+
+@pytest.fixture(scope="module")
+def B():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_22347_b200 import binding, build
+    build.build()
+    binding.load()
+    return binding
+
+
+@pytest.fixture(autouse=True)
+def clean_error_word(B):
+    B.perq_device_error_clear()
+    yield
+    assert B.perq_device_error() == 0
+
+
+def bf16(v):
+    return (np.ascontiguousarray(v, dtype=np.float32).view(np.uint32) >> 16).astype(np.uint16)
+
+
+def base_rows(d, seed):
+    rng = np.random.default_rng(seed)
+    x = inputs.laplace_outliers(BASE, d, max(1, d // 1024), 200.0, seed)[0]
+    x[40:80] = inputs.gaussian_outliers(40, d, 0, 1.0, seed + 1)[0]
+    x[80:120] = inputs.student_t_outliers(40, d, 3.0, max(2, d // 256), 100.0, seed + 2)[0]
+    x[7] = 0
+    x[8] = bf16(np.eye(1, d, d // 3) * 3.0)                                    # one nonzero
+    x[9] = bf16(rng.integers(-3, 4, d))                                        # small integers
+    x[10] = bf16(np.where(rng.random(d) < 8.0 / d, rng.integers(1, 9, d), 0))  # a few of them
+    x[11] = bf16(np.ones(d))
+    x[12] = bf16(rng.standard_normal(d) * 2.0 ** -80)
+    x[13] = bf16(rng.standard_normal(d) * 2.0 ** 100)
+    x[14, d // 2:] = 0
+    return x
+
+
+def check(B, oracle, T, d, b, fmt, group, seed, offset=0):
+    base = base_rows(d, seed)
+    idx = (np.arange(T) + np.arange(T) // BASE) % BASE           # a base row meets different CTAs, warps and stages
+    idx_t = torch.from_numpy(idx).cuda()
+    x = torch.from_numpy(base.view(np.int16)).cuda()[idx_t].view(torch.bfloat16)
+    codes, scales = B.alloc_outputs(T, d, FMT[fmt], group, "cuda")
+    if offset:                                                   # codes that are 16-byte but not 32-byte aligned
+        codes = torch.zeros(T * d // 2 + offset, dtype=torch.uint8, device="cuda")[offset:].view(T, d // 2)
+        assert codes.data_ptr() % 32 == 16
+    B.perq_rotate_quantize(x, None, b, FMT[fmt], group, codes, scales)
+    torch.cuda.synchronize()
+    first = torch.empty(BASE, dtype=torch.int64, device="cuda")
+    first[idx_t.flip(0)] = torch.arange(T - 1, -1, -1, device="cuda")
+    assert torch.equal(codes, codes[first[idx_t]]) and torch.equal(scales, scales[first[idx_t]])
+    rows = np.r_[np.arange(0, 16), np.random.default_rng(seed).choice(np.arange(16, BASE), 16 if b <= 128 else 6, replace=False)]
+    at = first[torch.from_numpy(rows).cuda()]
+    ora = oracle.rotate_quantize(base[rows], None, b, FMT[fmt], group, want_pre=True)
+    compare_quantized(fmt, codes[at].cpu().numpy(), scales[at].cpu().numpy(), ora)
+
+
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0), ("int4_asym", 0)])
+@pytest.mark.parametrize("b", [16, 32, 64, 128])
+def test_ragged_widths(B, oracle, b, fmt, group):
+    # pieces per row: 6 (21 rows a tile), 76 and 111 (one), 9 (14, 126 of 128 lanes)
+    for d, T in ((768, 6001), (9728, 691), (14208, 433), (1152, 5003)):
+        check(B, oracle, T, d, b, fmt, group, 30000 + d + b)
+
+
+@pytest.mark.parametrize("fmt,group,b", [("int4", 0, 64), ("int4", 0, 128), ("int4", 128, 16), ("int4", 128, 128), ("mxfp4", 32, 32),
+                                         ("mxfp4", 32, 64), ("mxfp4", 32, 128), ("fp4", 0, 16), ("fp4", 0, 128), ("int4_asym", 0, 32),
+                                         ("int4_asym", 0, 128)])
+@pytest.mark.parametrize("d", [4096, 8192, 14336])
+def test_whole_segments(B, oracle, d, fmt, group, b):
+    check(B, oracle, 17 * 2 ** 20 // d, d, b, fmt, group, 31000 + d + b, offset=16)
+
+
+@pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
+@pytest.mark.parametrize("d,T", [(4096, 4099), (2048, 16389)])
+def test_whole_row_rotations(B, oracle, d, T, fmt):
+    check(B, oracle, T, d, d, fmt, 0, 32000 + d)
