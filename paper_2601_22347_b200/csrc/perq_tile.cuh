@@ -52,12 +52,16 @@ struct TileRows {
 
 // What is left to settle of a tile: places, and what their codes depend on.
 constexpr int TILE_JOBS = 96;
-// a job: kind (2 bits), row of the tile (5, from bit 20), code as stored (4, from bit 16), column (7), piece (7)
-enum TileJob : uint32_t { JOB_MAX = 0u << 30, JOB_TIE = 1u << 30, JOB_PIECE = 2u << 30 };     // candidates in a quad; an element; a whole piece
+constexpr int TILE_TIES = 4;                  // notes of a lane and 32 columns
+// a job: kind (1 bit), row of the tile (5, from bit 20), code as stored (4, from bit 16), column (7), piece (7)
+// Pieces with more places than are worth a note each are left to their lanes (tile_put_extremes, tile_requantise).
+enum TileFlat : uint32_t { FLAT_ROWS = 1u, FLAT_CODES = 2u };          // extremes that are in ex_* only; codes
+enum TileJob : uint32_t { JOB_MAX = 0u << 30, JOB_TIE = 1u << 30 };     // candidates in a quad; an element
 struct TileNotes {
     unsigned long long ex_hi[TILE_ROW_CAP], ex_lo[TILE_ROW_CAP];       // exact: magnitude bits, or order keys of the extremes
     unsigned long long aux[TILE_PIECES];                               // per piece: exact maximum (ranges), exponents (MX)
-    uint32_t count;
+    uint32_t settled[4];                                               // pieces whose codes are exact already
+    uint32_t flat, count;                                              // (more notes than fit: count goes on)
     uint32_t job[TILE_JOBS];
 };
 // A note and what its code depends on: exponents or the exact maximum (MX, ranges), or up to two quads that hold the
@@ -258,11 +262,23 @@ __device__ __forceinline__ void tile_butterfly(uint32_t w0, uint32_t w1, int lan
         for (int e = 0; e < 4; ++e) o[e] = fma(sg, o[e], __shfl_xor_sync(0xffffffffu, o[e], 1 << t));
     }
 }
-template <int LOG2B>
-__device__ __forceinline__ void tile_exact_piece(const TileParams &p, uint32_t piece, int lane, double (&o)[4])
+// Whether the fp32 outputs of a piece are exact (see RowSpan; the products are aligned to the largest of a step and none of
+// their bits lies lower than the span), by one lane.
+__device__ __noinline__ bool tile_lane_exact(const uint16_t *x)
 {
-    const uint2 w = __ldg(reinterpret_cast<const uint2 *>(p.x + (size_t)piece * 128) + lane);
-    tile_butterfly<LOG2B>(w.x, w.y, lane, o);
+    RowSpan s = {0.0f, 1 << 20};
+#pragma unroll 4
+    for (int k = 0; k < 16; ++k) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x) + k);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const uint32_t a = (w[e >> 1] >> (16 * (e & 1))) & 0x7fffu;
+            s.sum += __uint_as_float(a << 16);
+            if (a != 0u) s.low = min(s.low, a < 0x80u ? __ffs(a) : (int)(a >> 7) + __ffs((a & 0x7fu) | 0x80u) - 1);
+        }
+    }
+    return row_span_exact(s);
 }
 
 // Largest exact magnitude among the outputs of piece r of a tile at the columns c0 + (set bits of want), by a warp.
@@ -427,10 +443,191 @@ __device__ __forceinline__ bool tile_zero_point(float hr, float lr, float err, f
     return !(fabsf(v - z) <= 0.5f - (err * ar * (1.0f + ar * (2.0f / 15.0f)) + slack));
 }
 
-__device__ __forceinline__ void tile_note(TileNotes *notes, uint32_t job)
+// false: no room
+__device__ __forceinline__ bool tile_note(TileNotes *notes, uint32_t job)
 {
     const uint32_t at = atomicAdd(&notes->count, 1u);
-    if (at < TILE_JOBS) notes->job[at] = job;                // (more than fit: every piece is settled)
+    if (at < TILE_JOBS) notes->job[at] = job;
+    return at < TILE_JOBS;
+}
+
+// ---- Flat rows, small integers: where a piece has many candidates or doubtful elements its fp32 outputs are as a rule exact,
+// which a look at its inputs shows; sums only where they are not.  A piece per lane, all lanes at work.  (2048 x 9728 of
+// integers -3 .. 3, b = 128, INT4 per token: 237 us, 856 with the pieces settled in turn by one warp, 270 in registers)
+
+// The quads of 32 columns that hold candidates for a row's extremes.
+template <int MODE>
+__device__ __forceinline__ uint32_t tile_candidates(const f32x2 (&u)[16], float thr_hi, float thr_lo)
+{
+    uint32_t quads = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const f32x2 v0 = u[2 * j], v1 = u[2 * j + 1];
+        bool r;
+        if (MODE == ROW_ASYM) r = fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= thr_hi || fminf(fminf(v0.x, v0.y), fminf(v1.x, v1.y)) <= thr_lo;
+        else r = fmaxf(max3abs(fabsf(v0.x), v0.y, v1.x), fabsf(v1.y)) >= thr_hi;
+        quads |= r ? (1u << j) : 0u;
+    }
+    return quads;
+}
+
+// Exact extremes of the lane's candidates (cmask: chunks that have some; 0: nothing to do) into its row's words.
+template <int LOG2B, int MODE>
+__device__ __noinline__ void tile_put_extremes(const TileParams &p, uint32_t tmem, uint32_t piece, uint32_t cmask, float thr_hi, float thr_lo, TileNotes *notes, int ri)
+{
+    f32x2 u[16];
+    const bool exact = cmask != 0u && tile_lane_exact(p.x + (size_t)piece * 128);
+    double hi = MODE == ROW_ASYM ? -1.7976931348623157e308 : 0.0, lo = 1.7976931348623157e308;
+    __syncwarp();
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        if (!__any_sync(0xffffffffu, (cmask >> c) & 1u)) continue;
+        tmem_load32(tmem + 32 * c, u);
+        uint32_t quads = (cmask >> c) & 1u ? tile_candidates<MODE>(u, thr_hi, thr_lo) : 0u;
+        if (exact && quads) {
+            quads = 0u;
+            if (MODE == ROW_ASYM) {
+                float h = u[0].x, l = u[0].x;
+#pragma unroll
+                for (int k = 0; k < 16; ++k) { h = fmaxf(fmaxf(h, u[k].x), u[k].y); l = fminf(fminf(l, u[k].x), u[k].y); }
+                hi = fmax(hi, (double)h);
+                lo = fmin(lo, (double)l);
+            } else {
+                hi = fmax(hi, (double)tile_max(u));
+            }
+        }
+        while (quads) {
+            double S[8], o[4];
+            const uint32_t col = (uint32_t)(32 * c) + 4u * ((uint32_t)__ffs(quads) - 1u);
+            quads &= quads - 1u;
+            tile_sums_global<LOG2B>(p, piece, col, S);
+            tile_quad_of(S, col, o);
+            hi = fmax(hi, MODE == ROW_ASYM ? tile_max_of(o) : tile_abs_max(o));
+            lo = fmin(lo, tile_min_of(o));
+        }
+        __syncwarp();
+    }
+    if (cmask != 0u) {
+        if (MODE == ROW_ASYM) {
+            atomicMax(&notes->ex_hi[ri], order_key(hi + 0.0));
+            atomicMin(&notes->ex_lo[ri], order_key(lo + 0.0));
+        } else {
+            atomicMax(&notes->ex_hi[ri], (unsigned long long)__double_as_longlong(hi));
+        }
+    }
+    __syncwarp();
+}
+
+// Exact codes of the pieces of the lanes with `mine`: quantised again, by exact scales, and their doubtful elements settled here.
+// aux: exponents (MX) or bits of the exact maximum (ranges); token rows have their extremes in the row's words.
+template <int LOG2B, int MODE>
+__device__ __noinline__ void tile_requantise(const TileParams &p, uint32_t tmem, uint32_t piece, bool mine, unsigned long long aux, TileNotes *notes, int w, int ri)
+{
+    f32x2 u[16];
+    const int lane = (int)(threadIdx.x & 31u);
+    const unsigned whose = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) notes->settled[w] = whose;
+    const bool exact = mine && tile_lane_exact(p.x + (size_t)piece * 128);
+    const float err = exact ? 1.2e-7f : p.err;               // (exact elements: the fp32 extremes of an exact range)
+    __syncwarp();
+    float ref = 0.0f;                                        // (of the piece: not less than any block's)
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) { tmem_load32(tmem + 32 * c, u); ref = fmaxf(ref, tile_max(u)); }
+    TileScale q = {0.0, 0.0, 0.0, 0.0, 0.0f, 0};
+    RowQuant Q;
+    Q.magic = 12584968.0f;
+    Q.mul = Q.tau = 0.0f;
+    if (MODE == ROW_ASYM) {
+        const double hi = order_value(notes->ex_hi[ri]), lo = order_value(notes->ex_lo[ri]);
+        float z, slack, per_ref;
+        if (mine) q = tile_scale_asym(p, hi, lo);
+        (void)tile_zero_point((float)hi, (float)lo, err, Q.mul, z, slack, per_ref);
+        Q.magic = 12582912.0f - (float)q.z64;
+        Q.tau = (float)hi > (float)lo ? per_ref * ref + slack : 3.0e38f;
+    } else if (MODE != ROW_MX) {
+        q = tile_scale_max<MODE>(p, __longlong_as_double((long long)(MODE == ROW_GROUP ? aux : notes->ex_hi[ri])));
+        Q.mul = row_inverse((float)(__longlong_as_double((long long)(MODE == ROW_GROUP ? aux : notes->ex_hi[ri]))));
+        Q.tau = (err + 5.0e-7f) * Q.mul * ref + (MODE == ROW_FP4 ? 0.0f : 2.0e-7f);
+    }
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        tmem_load32(tmem + 32 * c, u);
+        if (MODE == ROW_MX) {
+            const int Eb = (int)(((uint32_t)aux >> (8 * c)) & 0xffu);
+            q = tile_scale_mx(p, (uint32_t)Eb);
+            Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - LOG2B / 2, 1), 254) << 23) * ((LOG2B & 1) ? 0.70710678118654752f : 1.0f);
+            Q.tau = Eb == 0 ? 3.0e38f : 2.0f * err * ref * Q.mul + 2.0e-6f;          // (the lowest exponent: perhaps a group of zeros)
+        }
+        uint32_t cw[4];
+        const bool fl = tile_quantise<MODE>(u, Q, cw) && mine;
+        uint32_t tie = fl ? row_tie_bits<MODE>(u, Q) : 0u;
+        if ((MODE == ROW_MX || MODE == ROW_FP4) && exact && Q.tau < 0.2f) {           // exact zeros have code 0, as stored
+            uint32_t zero = 0u;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) zero |= (u[i].x == 0.0f ? 1u << (2 * i) : 0u) | (u[i].y == 0.0f ? 2u << (2 * i) : 0u);
+            tie &= ~zero;
+        }
+        // few lanes with many: an element per lane
+        unsigned lanes = __ballot_sync(0xffffffffu, __popc(tie) > 2);
+        if (__popc(lanes) > 4) lanes = 0u;
+        while (lanes) {
+            const int src = __ffs(lanes) - 1;
+            lanes &= lanes - 1;
+            const bool ex = __shfl_sync(0xffffffffu, (int)exact, src) != 0;
+            const uint32_t pc = __shfl_sync(0xffffffffu, piece, src), ts = __shfl_sync(0xffffffffu, tie, src);
+            float f = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float a = __shfl_sync(0xffffffffu, u[i].x, src), b = __shfl_sync(0xffffffffu, u[i].y, src);
+                f = (lane >> 1) == i ? ((lane & 1) ? b : a) : f;
+            }
+            TileScale r;
+            r.f = __shfl_sync(0xffffffffu, q.f, src);
+            r.a = __shfl_sync(0xffffffffu, q.a, src);
+            r.s64 = __shfl_sync(0xffffffffu, q.s64, src);
+            r.z64 = __shfl_sync(0xffffffffu, q.z64, src);
+            r.mul = __shfl_sync(0xffffffffu, q.mul, src);
+            r.E = __shfl_sync(0xffffffffu, q.E, src);
+            double v = (double)f + 0.0;
+            if (!ex) {
+                double S[8];
+                tile_sums_global<LOG2B>(p, pc, (uint32_t)(32 * c + lane), S);
+                v = tile_output_of(S, (uint32_t)(32 * c + lane));
+            }
+            uint32_t w = 0u, code = 0u;                        // the word of the lane's element as stored; its code
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { const uint32_t t = __shfl_sync(0xffffffffu, cw[i], src); w = (lane >> 3) == i ? t : w; }
+            const uint32_t sh = 4u * (uint32_t)(lane & 7);
+            code = ((ts >> lane) & 1u) ? tile_code<MODE>(p, v, r) : (w >> sh) & 0xFu;
+            code <<= sh;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) code |= __shfl_xor_sync(0xffffffffu, code, o);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { const uint32_t t = __shfl_sync(0xffffffffu, code, 8 * i); if (lane == src) cw[i] = t; }
+            if (lane == src) tie = 0u;
+        }
+#pragma unroll 1
+        while (tie) {
+            const uint32_t e = (uint32_t)__ffs(tie) - 1u, col = (uint32_t)(32 * c) + e;
+            tie &= tie - 1u;
+            double v;
+            if (exact) {
+                float f = 0.0f;
+#pragma unroll
+                for (uint32_t i = 0; i < 16; ++i) f = (e >> 1) == i ? ((e & 1u) ? u[i].y : u[i].x) : f;
+                v = (double)f + 0.0;                          // (+0 for a zero, as the sums give)
+            } else {
+                double S[8];
+                tile_sums_global<LOG2B>(p, piece, col, S);
+                v = tile_output_of(S, col);
+            }
+            const uint32_t sh = 4u * (e & 7u), code = tile_code<MODE>(p, v, q) << sh, keep = ~(0xFu << sh);
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) cw[i] = (e >> 3) == i ? (cw[i] & keep) | code : cw[i];
+        }
+        if (mine) *reinterpret_cast<uint4 *>(p.out_codes + (size_t)piece * 64 + 16 * c) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
+        __syncwarp();
+    }
 }
 
 // A lane's place in the tiles: the same for all of them.
@@ -457,7 +654,8 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
     float m[4] = {0.0f, 0.0f, 0.0f, 0.0f};                         // largest magnitude of each chunk of 32 columns
     float inv = 0.0f, lm = 0.0f, slack = 0.0f, per_ref = 0.0f, thr_hi = 0.0f, thr_lo = 0.0f;
     uint32_t cmask = 0u;                                           // per token: chunks with candidates for the row's extremes
-    bool many = false;                                             // more doubtful places than are worth a note each
+    bool many_max = false, many = false;                           // more candidates, doubtful elements than are worth a note each
+    unsigned long long aux = 0ull;                                 // exact maximum (ranges)
 
     tmem_issue32(tmem, ua);
     if (MODE == ROW_GROUP) {
@@ -479,15 +677,8 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
         for (int j = 0; j < 32; ++j) want |= (qm[j] >= thr) ? (1u << j) : 0u;
         if (!live || !(lm > 0.0f)) want = 0u;
         double a_ex = 0.0;
-        unsigned lanes = __ballot_sync(0xffffffffu, __popc(want) > ROW_MANY);
-        while (lanes) {                                              // many: all of the piece's outputs
-            const int src = __ffs(lanes) - 1;
-            lanes &= lanes - 1;
-            double o[4];
-            tile_exact_piece<LOG2B>(p, piece - (uint32_t)lane + (uint32_t)src, lane, o);
-            const unsigned long long a = warp_max_u64((unsigned long long)__double_as_longlong(tile_abs_max(o)));
-            if (lane == src) { a_ex = __longlong_as_double((long long)a); want = 0u; }
-        }
+        if (__popc(want) > 2 && tile_lane_exact(p.x + (size_t)piece * 128)) { a_ex = (double)lm; want = 0u; }
+        __syncwarp();
         while (__any_sync(0xffffffffu, want != 0u)) {
             const uint32_t c = want ? 4u * ((uint32_t)__ffs(want) - 1u) : 0u, c0 = c & ~((1u << LOG2B) - 1u);
             double S[8], o[4];
@@ -502,7 +693,8 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
         }
         tmem_issue32(tmem, ua);
         if (live) reinterpret_cast<float *>(p.out_scales)[piece] = row_scale(a_ex, p.inv_7_sqrt_b, p.sqrt_b, 7.0);
-        notes->aux[l] = (unsigned long long)__double_as_longlong(a_ex);
+        aux = (unsigned long long)__double_as_longlong(a_ex);
+        notes->aux[l] = aux;
         inv = row_inverse((float)a_ex);
         // the element's error and the multiplier's (three roundings); the distance's own
         per_ref = (err + 5.0e-7f) * inv;
@@ -576,36 +768,19 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
                 if (!some) inv = z = per_ref = slack = 0.0f;
                 else if (flat) per_ref = 3.0e38f;                     // (equal in fp32: everything is in doubt)
                 // the zero point of a row of the tile is in doubt: its exact extremes now (the four warps agree on this)
-                bool doubt = near;
+                // (from the row words alone: warps that share the tile but not the row must not miss the barrier)
+                bool doubt = false;
                 if (L.coupled) {
                     const uint32_t khi = rows->mx[par][lane], klo = rows->mn[par][lane];
                     float f[4];
-                    doubt = khi > klo && tile_zero_point(order_value32(khi), order_value32(klo), err, f[0], f[1], f[2], f[3]);
-                    doubt = doubt || near;
+                    if (khi >= klo) {
+                        const float h = order_value32(khi), l0 = order_value32(klo);
+                        doubt = fmaxf(fabsf(h), fabsf(l0)) > 0.0f && tile_zero_point(h, l0, err, f[0], f[1], f[2], f[3]);
+                    }
                 }
                 if (L.coupled ? __any_sync(0xffffffffu, doubt) : __any_sync(0xffffffffu, near)) {
-#pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
-                        tmem_load32(tmem + 32 * c, ub);
-                        uint32_t quads = 0u;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const f32x2 v0 = ub[2 * j], v1 = ub[2 * j + 1];
-                            const bool r = fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= thr_hi || fminf(fminf(v0.x, v0.y), fminf(v1.x, v1.y)) <= thr_lo;
-                            quads |= r ? (1u << j) : 0u;
-                        }
-                        if (!near || !((cmask >> c) & 1u)) quads = 0u;
-                        while (quads) {
-                            double S[8], o[4];
-                            const uint32_t col = (uint32_t)(32 * c) + 4u * ((uint32_t)__ffs(quads) - 1u);
-                            quads &= quads - 1u;
-                            tile_sums_global<LOG2B>(p, piece, col, S);
-                            tile_quad_of(S, col, o);
-                            atomicMax(&notes->ex_hi[L.ri], order_key(tile_max_of(o)));
-                            atomicMin(&notes->ex_lo[L.ri], order_key(tile_min_of(o)));
-                        }
-                        __syncwarp();
-                    }
+                    tmem_wait(ua);
+                    tile_put_extremes<LOG2B, MODE>(p, tmem, piece, near ? cmask : 0u, thr_hi, thr_lo, notes, L.ri);
                     if (L.coupled) named_barrier(bar, 128); else __syncwarp();
                     if (near) z = (float)tile_scale_asym(p, order_value(notes->ex_hi[L.ri]), order_value(notes->ex_lo[L.ri])).z64;
                     tmem_issue32(tmem, ua);
@@ -652,18 +827,23 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
                 bool zero = !(gm > 0.0f);
                 if (__any_sync(0xffffffffu, near)) {          // rare: the exact maximum of the group
                     uint32_t want = near ? row_reach(u, gm - tol) : 0u;
+                    auto settle = [&](double best) {
+                        int ex;
+                        (void)frexp(best / p.sqrt_b, &ex);
+                        Eb = ex - 3 + 127;
+                        zero = best == 0.0;                   // (the fp32 values of a group that cancels exactly are rounding noise)
+                    };
                     unsigned lanes = __ballot_sync(0xffffffffu, want != 0u);
+                    if (__popc(lanes) > 4) {                  // flat rows, integers
+                        if (want != 0u && tile_lane_exact(p.x + (size_t)piece * 128)) { settle((double)gm); want = 0u; }
+                        lanes = __ballot_sync(0xffffffffu, want != 0u);
+                    }
                     while (lanes) {
                         const int src = __ffs(lanes) - 1;
                         lanes &= lanes - 1;
                         const uint32_t ws = __shfl_sync(0xffffffffu, want, src);
                         const double best = tile_exact_max<LOG2B>(tile, half, (uint32_t)(L.w * 32 + src), (uint32_t)(64 * h + 32 * k), ws, lane);
-                        if (lane == src) {
-                            int ex;
-                            (void)frexp(best / p.sqrt_b, &ex);
-                            Eb = ex - 3 + 127;
-                            zero = best == 0.0;               // (the fp32 values of a group that cancels exactly are rounding noise)
-                        }
+                        if (lane == src) settle(best);
                     }
                 }
                 Eb = min(max(Eb, 0), 254);
@@ -681,33 +861,24 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
             if (TOK) {                                        // candidates for the row's extremes
                 const bool cand = (cmask >> (2 * h + k)) & 1u;
                 if (__any_sync(0xffffffffu, cand)) {
-                    uint32_t quads = 0u;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const f32x2 v0 = u[2 * j], v1 = u[2 * j + 1];
-                        bool r;
-                        if (MODE == ROW_ASYM) r = fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= thr_hi || fminf(fminf(v0.x, v0.y), fminf(v1.x, v1.y)) <= thr_lo;
-                        else r = fmaxf(max3abs(fabsf(v0.x), v0.y, v1.x), fabsf(v1.y)) >= thr_hi;
-                        quads |= r ? (1u << j) : 0u;
-                    }
-                    if (!cand) quads = 0u;
-                    if (__popc(quads) > 2) { many = true; quads = 0u; }
+                    uint32_t quads = cand ? tile_candidates<MODE>(u, thr_hi, thr_lo) : 0u;
+                    if (__popc(quads) > 2) { many_max = true; quads = 0u; }
                     while (quads) {
                         const uint32_t j = (uint32_t)__ffs(quads) - 1u;
                         quads &= quads - 1u;
-                        tile_note(notes, JOB_MAX | (uint32_t)L.ri << 20 | (place + (4u * j << 7)));
+                        if (!tile_note(notes, JOB_MAX | (uint32_t)L.ri << 20 | (place + (4u * j << 7)))) many_max = true;
                     }
                 }
             }
             const bool fl = tile_quantise<MODE>(u, Q, cw + 4 * k) && live;
             if (__any_sync(0xffffffffu, fl)) {
                 uint32_t tie = fl ? row_tie_bits<MODE>(u, Q) : 0u;
-                if (__popc(tie) > ROW_MANY) { many = true; tie = 0u; }
+                if (__popc(tie) > TILE_TIES) { many = true; tie = 0u; }
                 while (tie) {
                     const uint32_t e = (uint32_t)__ffs(tie) - 1u;
                     tie &= tie - 1u;
                     const uint32_t w = e < 16 ? (e < 8 ? cw[4 * k] : cw[4 * k + 1]) : (e < 24 ? cw[4 * k + 2] : cw[4 * k + 3]);
-                    tile_note(notes, JOB_TIE | (uint32_t)(TOK ? L.ri : 0) << 20 | ((w >> (4 * (e & 7u))) & 0xFu) << 16 | (place + (e << 7)));
+                    if (!tile_note(notes, JOB_TIE | (uint32_t)(TOK ? L.ri : 0) << 20 | ((w >> (4 * (e & 7u))) & 0xFu) << 16 | (place + (e << 7)))) { many = true; break; }
                 }
             }
         };
@@ -721,9 +892,21 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
     }
     if (MODE == ROW_MX) {
         if (live) reinterpret_cast<uint32_t *>(p.out_scales)[piece] = exps;
-        notes->aux[l] = exps;
+        aux = exps;
+        notes->aux[l] = aux;
     }
-    if (many) tile_note(notes, JOB_PIECE | (uint32_t)l);
+    bool codes = __any_sync(0xffffffffu, many);
+    if (TOK) {
+        const bool ext = codes || __any_sync(0xffffffffu, many_max);
+        if (ext && lane == 0) atomicOr(&notes->flat, codes ? FLAT_ROWS | FLAT_CODES : FLAT_ROWS);
+        if (L.coupled) {                                              // (the four warps take this way together)
+            named_barrier(bar, 128);
+            codes = (*reinterpret_cast<volatile uint32_t *>(&notes->flat) & FLAT_CODES) != 0u;
+        }
+        if (ext || codes) tile_put_extremes<LOG2B, MODE>(p, tmem, piece, many_max || codes ? cmask : 0u, thr_hi, thr_lo, notes, L.ri);
+        if (codes && L.coupled) named_barrier(bar, 128);
+    }
+    if (codes) tile_requantise<LOG2B, MODE>(p, tmem, piece, many, aux, notes, L.w, L.ri);
 }
 
 // -------------------------------------------------------------------------------------------- notes
@@ -793,26 +976,24 @@ struct TileCollector {
     __device__ __forceinline__ void make_room() { if (n > TILE_RECORDS - 32) hand_over(0u); }
 };
 
-// The notes of a tile, by a warp.  Most become records; what cannot (rows with several candidates, whole pieces, more
-// notes than fit) is settled here: exact extremes of the token rows and their scales, then the doubtful codes.
+// The notes of a tile, by a warp.  Most become records; token rows with several candidates, or with extremes that have no note,
+// are settled here: their exact extremes and scales, then the doubtful codes.
 template <int LOG2B, int MODE>
 __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, TileNotes *notes, TileCollector &to, int lane)
 {
     constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4 || MODE == ROW_ASYM;
     const uint32_t piece0 = t * (uint32_t)p.tile_pieces, rp = (uint32_t)p.row_pieces;
-    const uint32_t listed = *reinterpret_cast<volatile uint32_t *>(&notes->count);
-    const bool all = listed > TILE_JOBS;
-    const uint32_t n = all ? 0u : listed;
-    if (!TOK && listed == 0u) return;
+    const uint32_t n = min(*reinterpret_cast<volatile uint32_t *>(&notes->count), (uint32_t)TILE_JOBS);
+    if (!TOK && n == 0u) return;
     const uint32_t here = min((uint32_t)p.tile_pieces, p.pieces - piece0);              // pieces of the tile
-    if (TOK && n <= 32u && !all) {
+    if (TOK && n <= 32u && *reinterpret_cast<volatile uint32_t *>(&notes->flat) == 0u) {
         const bool has = (uint32_t)lane < n;
         const uint32_t j = has ? notes->job[lane] : 0u, row = (j >> 20) & 31u;
         const bool cand = has && (j >> 30) == (JOB_MAX >> 30);
         const unsigned cands = __ballot_sync(0xffffffffu, cand);
         const unsigned mates = __match_any_sync(0xffffffffu, has ? row : 0x100u + (uint32_t)lane) & cands;      // its row's candidates
         const bool my_row = (uint32_t)lane * rp < here;
-        const bool bad = has && ((j >> 30) == (JOB_PIECE >> 30) || __popc(mates) > (MODE == ROW_ASYM ? 2 : 1) || mates == 0u);
+        const bool bad = has && (__popc(mates) > (MODE == ROW_ASYM ? 2 : 1) || mates == 0u);
         if (!__any_sync(0xffffffffu, bad)) {
             // rows without a candidate are rows of zeros
             const uint32_t rows = __reduce_or_sync(0xffffffffu, cand ? 1u << row : 0u);
@@ -840,22 +1021,6 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
             return;
         }
     }
-    // the pieces that are settled as a whole, in turn: all of them, or the listed ones
-    auto for_pieces = [&](auto &&f) {
-        if (all) {
-            for (uint32_t r = 0; r < here; ++r) f(r);
-        } else {
-            for (uint32_t k0 = 0; k0 < n; k0 += 32) {
-                const uint32_t j = k0 + lane < n ? notes->job[k0 + lane] : 0u;
-                unsigned found = __ballot_sync(0xffffffffu, (j >> 30) == (JOB_PIECE >> 30));
-                while (found) {
-                    const int src = __ffs(found) - 1;
-                    found &= found - 1;
-                    f(__shfl_sync(0xffffffffu, j, src) & 127u);
-                }
-            }
-        }
-    };
     if (TOK) {
         for (uint32_t k = lane; k < n; k += 32) {
             const uint32_t j = notes->job[k], row = (j >> 20) & 31u, c = (j >> 7) & 127u;
@@ -872,22 +1037,6 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
             }
         }
         __syncwarp();
-        for_pieces([&](uint32_t r) {
-            double o[4];
-            tile_exact_piece<LOG2B>(p, piece0 + r, lane, o);
-            unsigned long long hi, lo = 0ull;
-            if (MODE == ROW_ASYM) {
-                hi = warp_max_u64(order_key(tile_max_of(o)));
-                lo = ~warp_max_u64(~order_key(tile_min_of(o)));
-            } else {
-                hi = warp_max_u64((unsigned long long)__double_as_longlong(tile_abs_max(o)));
-            }
-            if (lane == 0) {
-                atomicMax(&notes->ex_hi[r / rp], hi);
-                if (MODE == ROW_ASYM) atomicMin(&notes->ex_lo[r / rp], lo);
-            }
-        });
-        __syncwarp();
         // ---- scales: a row per lane
         const bool mine = (uint32_t)lane * rp < here;
         const size_t row = (size_t)(piece0 / rp) + lane;
@@ -903,28 +1052,18 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
         __syncwarp();
     }
     // ---- doubtful codes
-    auto scale_of = [&](uint32_t r, uint32_t c) -> TileScale {
-        if (MODE == ROW_MX) return tile_scale_mx(p, (uint32_t)notes->aux[r] >> (8 * (c >> 5)) & 0xffu);
-        if (MODE == ROW_GROUP) return tile_scale_max<MODE>(p, __longlong_as_double((long long)notes->aux[r]));
-        const uint32_t row = r / rp;
-        if (MODE == ROW_ASYM) return tile_scale_asym(p, order_value(notes->ex_hi[row]), order_value(notes->ex_lo[row]));
-        return tile_scale_max<MODE>(p, __longlong_as_double((long long)notes->ex_hi[row]));
-    };
-    // (not those of pieces that are settled as a whole: a correction would meet the new code)
-    uint32_t whole_pieces[4] = {0u, 0u, 0u, 0u};
-    for_pieces([&](uint32_t r) {
-#pragma unroll
-        for (int w = 0; w < 4; ++w) whole_pieces[w] |= (r >> 5) == (uint32_t)w ? 1u << (r & 31u) : 0u;
-    });
+    // (not those of pieces that were quantised again: a correction would meet the new code)
     for (uint32_t k0 = 0; k0 < n; k0 += 32) {
         const uint32_t j = k0 + lane < n ? notes->job[k0 + lane] : 0u, r = j & 127u, c = (j >> 7) & 127u;
-        const uint32_t settled = r < 64u ? (r < 32u ? whole_pieces[0] : whole_pieces[1]) : (r < 96u ? whole_pieces[2] : whole_pieces[3]);
-        const bool tie = k0 + lane < n && (j >> 30) == (JOB_TIE >> 30) && !((settled >> (r & 31u)) & 1u);
+        const bool tie = k0 + lane < n && (j >> 30) == (JOB_TIE >> 30) && !((notes->settled[r >> 5] >> (r & 31u)) & 1u);
         if (TOK) {
             if (tie) {
                 double S[8];
                 tile_sums_global<LOG2B>(p, piece0 + r, c, S);
-                tile_mend(p, piece0 + r, j, tile_code<MODE>(p, tile_output_of(S, c), scale_of(r, c)));
+                const uint32_t row = (j >> 20) & 31u;
+                const TileScale q = MODE == ROW_ASYM ? tile_scale_asym(p, order_value(notes->ex_hi[row]), order_value(notes->ex_lo[row]))
+                                                     : tile_scale_max<MODE>(p, __longlong_as_double((long long)notes->ex_hi[row]));
+                tile_mend(p, piece0 + r, j, tile_code<MODE>(p, tile_output_of(S, c), q));
             }
         } else {
             to.make_room();
@@ -940,17 +1079,6 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
             to.n += __popc(who);
         }
     }
-    __syncwarp();
-    auto whole = [&](uint32_t r) {
-        double o[4];
-        tile_exact_piece<LOG2B>(p, piece0 + r, lane, o);
-        const TileScale q = scale_of(r, 4u * (uint32_t)lane);
-        uint32_t w = 0u;
-#pragma unroll 1
-        for (int e = 0; e < 4; ++e) w |= tile_code<MODE>(p, (e == 0 ? o[0] : e == 1 ? o[1] : e == 2 ? o[2] : o[3]) + 0.0, q) << (4 * e);
-        *reinterpret_cast<volatile uint16_t *>(p.out_codes + (size_t)(piece0 + r) * 64 + 2 * lane) = (uint16_t)w;
-    };
-    for_pieces(whole);
     __syncwarp();
 }
 
@@ -985,7 +1113,8 @@ __device__ __forceinline__ void tile_clear_notes(TileNotes *notes, int lane)
 {
     notes->ex_hi[lane] = 0ull;
     notes->ex_lo[lane] = ~0ull;
-    if (lane == 0) notes->count = 0u;
+    if (lane < 4) notes->settled[lane] = 0u;
+    if (lane == 0) notes->flat = notes->count = 0u;
 }
 
 template <int LOG2B, int MODE>

@@ -56,8 +56,20 @@ def base_rows(d, seed):
     return x
 
 
-def check(B, oracle, T, d, b, fmt, group, seed, offset=0):
-    base = base_rows(d, seed)
+def flat_rows(d, seed):
+    rng = np.random.default_rng(seed)
+    x = np.empty((BASE, d), np.uint16)
+    for i in range(BASE):
+        v = (np.ones(d), rng.integers(-3, 4, d), rng.choice([-1.0, 1.0], d), np.where(np.arange(d) % 128 == i % 128, 3.0, 0),
+             np.repeat(2.0 ** rng.integers(-3, 4, d // 128), 128))[i % 5].astype(np.float64)
+        if i % 2:                                                # pieces whose fp32 outputs are not exact
+            v[(i % 128)::(128 if i % 4 == 1 else 384)] = 2.0 ** -30 * (i % 7 + 1)
+        x[i] = bf16(v)
+    return x
+
+
+def check(B, oracle, T, d, b, fmt, group, seed, offset=0, make=base_rows):
+    base = make(d, seed)
     idx = (np.arange(T) + np.arange(T) // BASE) % BASE           # a base row meets different CTAs, warps and stages
     idx_t = torch.from_numpy(idx).cuda()
     x = torch.from_numpy(base.view(np.int16)).cuda()[idx_t].view(torch.bfloat16)
@@ -96,3 +108,11 @@ def test_whole_segments(B, oracle, d, fmt, group, b):
 @pytest.mark.parametrize("d,T", [(4096, 4099), (2048, 16389)])
 def test_whole_row_rotations(B, oracle, d, T, fmt):
     check(B, oracle, T, d, d, fmt, 0, 32000 + d)
+
+
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0), ("int4_asym", 0)])
+@pytest.mark.parametrize("d,T", [(1536, 3001), (9728, 691), (4096, 4096)])
+def test_flat_rows(B, oracle, d, T, fmt, group):
+    # nearly every piece has more candidates or ties than are noted: lanes settle them, with exact fp32 outputs and without
+    for b in (16, 128):
+        check(B, oracle, T, d, b, fmt, group, 33000 + d + b, make=flat_rows)
