@@ -267,7 +267,7 @@ __device__ __forceinline__ void tile_butterfly(uint32_t w0, uint32_t w1, int lan
 __device__ __noinline__ bool tile_lane_exact(const uint16_t *x)
 {
     RowSpan s = {0.0f, 1 << 20};
-#pragma unroll 4
+#pragma unroll 8
     for (int k = 0; k < 16; ++k) {
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x) + k);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -453,7 +453,7 @@ __device__ __forceinline__ bool tile_note(TileNotes *notes, uint32_t job)
 
 // ---- Flat rows, small integers: where a piece has many candidates or doubtful elements its fp32 outputs are as a rule exact,
 // which a look at its inputs shows; sums only where they are not.  A piece per lane, all lanes at work.  (2048 x 9728 of
-// integers -3 .. 3, b = 128, INT4 per token: 237 us, 856 with the pieces settled in turn by one warp, 270 in registers)
+// integers -3 .. 3, b = 128, INT4 per token: 245 us, 856 with the pieces settled in turn by one warp, 270 in registers)
 
 // The quads of 32 columns that hold candidates for a row's extremes.
 template <int MODE>
@@ -476,7 +476,7 @@ template <int LOG2B, int MODE>
 __device__ __noinline__ void tile_put_extremes(const TileParams &p, uint32_t tmem, uint32_t piece, uint32_t cmask, float thr_hi, float thr_lo, TileNotes *notes, int ri)
 {
     f32x2 u[16];
-    const bool exact = cmask != 0u && tile_lane_exact(p.x + (size_t)piece * 128);
+    int exact = -1;                                          // (asked for when there are several: a look costs as much as a sum)
     double hi = MODE == ROW_ASYM ? -1.7976931348623157e308 : 0.0, lo = 1.7976931348623157e308;
     __syncwarp();
 #pragma unroll 1
@@ -484,7 +484,8 @@ __device__ __noinline__ void tile_put_extremes(const TileParams &p, uint32_t tme
         if (!__any_sync(0xffffffffu, (cmask >> c) & 1u)) continue;
         tmem_load32(tmem + 32 * c, u);
         uint32_t quads = (cmask >> c) & 1u ? tile_candidates<MODE>(u, thr_hi, thr_lo) : 0u;
-        if (exact && quads) {
+        if (exact < 0 && __popc(quads) > 2) exact = tile_lane_exact(p.x + (size_t)piece * 128);
+        if (exact > 0 && quads) {
             quads = 0u;
             if (MODE == ROW_ASYM) {
                 float h = u[0].x, l = u[0].x;
