@@ -10,6 +10,14 @@
 // The row kernel, which makes a trip through an fp32 tile, spends 1160 warp instructions on 1024 elements and five
 // barriers of a row's warps on a row; here two barriers serve four rows.
 //
+// Error bound.  What the tensor cores lose depends on the inputs: a step adds 16 products to the accumulator, cuts all of
+// them at 2^(e-25), e the exponent of the largest, and the sum at 2^(e-23) (measured: a model of that gives the same bits
+// on inputs of 4 to 26 binades).  Beside a large input tiny ones can be lost in every piece, to the same side: a bound that
+// covers any inputs is 900 * 2^-24 of the row's largest output, and with it a row has six doubtful codes.  But only inputs
+// 2^16 below their piece's l1 norm can be lost, and few rows have many: four warps count them (col_lost) while the tile waits
+// for its group.  (16384 x 4096, INT4: 98 us; 129 with a bound of 208 * 2^-24 for all rows; 85 with one of 12 that some
+// rows exceed.)
+//
 // Exact maxima and doubtful codes: sums over the whole row.  They are listed while the rows are quantised, and then a warp
 // takes the sums of a row (or two): 16384 terms for each of the four.  Rows in which more is listed than fits (ties:
 // one nonzero, few small integers; a zero point in doubt) are rotated again in fp64 by the four warps, where every output is
@@ -22,11 +30,15 @@ namespace perq {
 constexpr int COL_WGS = 3;
 constexpr int COL_ACCS = 4;
 constexpr int COL_STAGES = 5;
-constexpr int COL_WARPS = COL_WGS * 4 + 2;                    // one that loads, one that issues the contractions
+constexpr int COL_WARPS = COL_WGS * 4 + 4;                    // four that bound the rows' errors; one of them loads, one issues the contractions
 constexpr int COL_THREADS = COL_WARPS * 32;
 constexpr int COL_LIST = 8;                                   // listed places per row
 constexpr int COL_ROWS = 8;                                   // rows per tile at most
-constexpr float COL_ERR_K = 1.0f;                             // |u32 - u| <= K * log2(d) * 2^-24 * largest |u32| of the row
+constexpr float COL_LOST = 0x1p-12f;                          // of the largest output: where more may be lost the row is rotated in fp64
+// The stages over the C pieces of a row round to nearest.  Those of one stage add up to 2^-24 * sqrt(values that meet in an
+// output) of the row's largest output at most (Cauchy, Parseval): sqrt(C/2) + sqrt(C/4) + .. + 1.  In 2^-24 of that
+// output, a little more than that:
+__host__ __device__ constexpr float col_stage_err(int log2c) { return log2c == 5 ? 11.3f : 7.3f; }
 
 struct ColNotes {                                             // of a tile; two per group, used in turn
     float hi[COL_ROWS][4], lo[COL_ROWS][4];                   // fp32 extremes by warp (symmetric: hi is the largest magnitude)
@@ -45,8 +57,10 @@ struct ColSmem {
     static constexpr uint32_t had = stages + COL_STAGES * 2 * half;
     static constexpr uint32_t groups = had + 2 * half;
     static constexpr uint32_t bars = groups + COL_WGS * (uint32_t)sizeof(ColGroup);
-    static constexpr uint32_t n_bars = 2 * (COL_STAGES + COL_ACCS);
-    static constexpr uint32_t slot = bars + n_bars * 8;
+    // loaded, empty: of each stage; done, free: of each accumulator; scanned: of each stage
+    static constexpr uint32_t n_bars = 3 * COL_STAGES + 2 * COL_ACCS;
+    static constexpr uint32_t lost = bars + n_bars * 8;              // float[COL_ROWS] of each stage
+    static constexpr uint32_t slot = lost + COL_STAGES * COL_ROWS * 4;
     static constexpr uint32_t total = slot + 16 + 1024;
 };
 static_assert(sizeof(ColGroup) % 8 == 0 && ColSmem::total <= 227 * 1024, "shared memory of the column kernel");
@@ -58,6 +72,72 @@ __device__ __forceinline__ void col_rotate(uint32_t tmem, uint32_t tile, uint32_
 #pragma unroll
     for (int s = 0; s < 8; ++s)                               // 16 inputs a step
         tile_mma(tmem, h + (s >> 2) * (ColSmem::half / 16) + 2 * (s & 3), x + (s >> 2) * (ColSmem::half / 16) + 2 * (s & 3), tile_idesc(128), s > 0);
+}
+
+// Bound of what the contraction loses in any output of piece r of a tile, by one lane.  With g = 2^(e-23) and 2^(e+1) above
+// the sum of the piece's magnitudes, inputs of 2^7 g and more are multiples of g, every term and sum is below 2^(e+1), and
+// all grids that a step cuts at divide g.  A step without smaller inputs only moves the accumulator's part below g, and only
+// where its grid is coarser than any before: between two steps that have some, by less than g in all.  A step with n of
+// them cuts these and the accumulator, by less than g / 4 each.
+// guess: biased e of the lane's piece of the previous tile, plus one.  Inputs are counted against it while they are added
+// up, zeros as well; again where it was too low, or there are many.
+__device__ __forceinline__ void col_words(uint32_t tile, uint32_t r, uint32_t c, uint32_t (&w)[4])
+{
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(tile + tile_at(ColSmem::half, r, 8u * c)));
+}
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t above_bf16x2(uint32_t a, uint32_t b)      // all ones where a > b
+{
+    uint32_t r;
+    asm("set.gt.u32.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+// -2^(e-16), twice (biased e)
+__device__ __forceinline__ uint32_t col_limit(uint32_t e) { return ((e > 16u ? (e - 16u) << 7 : 0u) | 0x8000u) * 0x10001u; }
+// Nonzero inputs below 2^(e-16).
+__device__ __noinline__ float col_count(uint32_t tile, uint32_t r, uint32_t e)
+{
+    const uint32_t limit = col_limit(e);
+    uint32_t n = 0u;
+#pragma unroll 1
+    for (uint32_t c = 0; c < 16; ++c) {
+        uint32_t w[4];
+        col_words(tile, r, c, w);
+        // (x - 1 as bits; a zero becomes NaN)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) n += __popc(above_bf16x2((w[k] | 0x80008000u) - 0x00010001u, limit));
+    }
+    return (float)(n / 16u);
+}
+__device__ __forceinline__ float col_lost(uint32_t tile, uint32_t r, uint32_t &guess)
+{
+    constexpr float MANY = 12.0f;
+    const uint32_t limit = col_limit(guess);
+    float a = 0.0f, b = 0.0f;
+    uint32_t count = 0u;
+#pragma unroll 4
+    for (uint32_t c = 0; c < 16; ++c) {
+        uint32_t w[4];
+        col_words(tile, r, c, w);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] |= 0x80008000u;
+        const uint32_t s = add_bf16x2(add_bf16x2(w[0], w[1]), add_bf16x2(w[2], w[3]));
+        a += __uint_as_float(s);                              // (the lower half only adds to its magnitude)
+        b += __uint_as_float(s << 16);
+        count += above_bf16x2(w[0], limit) + above_bf16x2(w[1], limit);          // (each half takes off one)
+        count += above_bf16x2(w[2], limit) + above_bf16x2(w[3], limit);
+    }
+    const uint32_t e = (__float_as_uint((a + b) * -1.01f) >> 23) & 0xffu;         // (two roundings to bf16, 17 to fp32)
+    const uint32_t lo = (0u - count) & 0xffffu;                                   // (the lower halves' borrows: as many as they count)
+    float n = (float)(lo + ((((0u - count) >> 16) + lo) & 0xffffu));
+    if (e > guess || n > MANY) n = col_count(tile, r, e);
+    guess = min(e, 253u) + 1u;
+    return e >= 254u ? 3.0e38f : (n + 5.0f * fminf(n, 8.0f)) * (__uint_as_float(e << 23) * 0x1p-25f);          // (sums that might overflow)
 }
 
 // The stages over the pieces of a row: 32 values of one row (LOG2C 5), or 16 each of two (4).
@@ -193,10 +273,12 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
     const uint32_t base = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t full = base + ColSmem::bars, empty = full + COL_STAGES * 8, done = empty + COL_STAGES * 8, avail = done + COL_ACCS * 8;
+    const uint32_t scanned = avail + COL_ACCS * 8;
+    float *lost = reinterpret_cast<float *>(smem + ColSmem::lost);
 
     if (tid < (int)ColSmem::n_bars) {
         const uint32_t bar = full + tid * 8;
-        mbar_init(bar, (bar >= empty && bar < done) || bar >= avail ? 4 : 1);
+        mbar_init(bar, bar >= scanned || (bar >= empty && bar < done) || bar >= avail ? 4 : 1);
         mbar_init_fence();
     }
     for (int e = tid; e < COL_WGS * 2 * COL_ROWS; e += COL_THREADS)
@@ -218,33 +300,53 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
     auto give_up = [&]() { if (lane == 0) atomicOr(&g_perq_device_error, 8u); };
 
     // (a wait that runs out ends its warp's part; the others' waits run out too, and all meet at the end)
-    if (warp == COL_WGS * 4) {
-        if (lane == 0) {
-            uint32_t j = 0;
-            for (; j < n; ++j) {
-                const uint32_t s = j % COL_STAGES;
-                if (j >= COL_STAGES && !mbar_wait_fast(empty + s * 8, ((j / COL_STAGES) - 1u) & 1u)) { give_up(); break; }
-                mbar_expect_tx(full + s * 8, 2 * ColSmem::half);
-                const int y = (int)((first + j * gridDim.x) * (uint32_t)TILE_PIECES);
-                tma_load_2d(stage_at(s), &map, 0, y, full + s * 8);
-                tma_load_2d(stage_at(s) + ColSmem::half, &map, 64, y, full + s * 8);
+    if (warp >= COL_WGS * 4) {
+        // a quarter of every tile's pieces each, one per lane.  Tile j is looked at when tile j - 4 has been finished: the three
+        // groups are at j - 3 .. j - 1 then, and none waits for this.
+        const uint32_t q = (uint32_t)(warp - COL_WGS * 4);
+        uint32_t j = 0, loads = 0, guess = 0u;
+        bool ok = true;
+        auto load = [&]() {
+            const uint32_t s = loads % COL_STAGES;
+            mbar_expect_tx(full + s * 8, 2 * ColSmem::half);
+            const int y = (int)((first + loads * gridDim.x) * (uint32_t)TILE_PIECES);
+            tma_load_2d(stage_at(s), &map, 0, y, full + s * 8);
+            tma_load_2d(stage_at(s) + ColSmem::half, &map, 64, y, full + s * 8);
+            ++loads;
+        };
+        if (q == 0u && lane == 0) while (loads < n && loads < COL_STAGES) load();
+        for (; j < n && ok; ++j) {
+            const uint32_t s = j % COL_STAGES, b = j % COL_ACCS;
+            if (q == 0u && j >= 4u && j + 1u < n) {
+                static_assert(COL_STAGES == 5, "tile j + 1 goes where tile j - 4 was");
+                const uint32_t e = (j + 1u) % COL_STAGES;
+                ok = mbar_wait_fast(empty + e * 8, ((j + 1u) / COL_STAGES - 1u) & 1u);
+                if (ok && lane == 0) load();
             }
-            // no copy is in flight when the CTA ends, also after a wait that ran out
-            for (uint32_t k = j > COL_STAGES ? j - COL_STAGES : 0u; k < j; ++k) (void)mbar_wait_fast(full + (k % COL_STAGES) * 8, (k / COL_STAGES) & 1u);
-        }
-        __syncwarp();
-    } else if (warp == COL_WGS * 4 + 1) {
-        if (lane == 0) {
-            uint32_t j = 0;
-            for (; j < n; ++j) {
-                const uint32_t s = j % COL_STAGES, b = j % COL_ACCS;
-                bool ok = mbar_wait_fast(full + s * 8, (j / COL_STAGES) & 1u);
+            ok = mbar_wait_fast(full + s * 8, (j / COL_STAGES) & 1u) && ok;
+            if (q == 1u) {
                 if (j >= COL_ACCS) ok = mbar_wait_fast(avail + b * 8, ((j / COL_ACCS) - 1u) & 1u) && ok;
-                if (!ok) { give_up(); break; }
-                tmem_fence_after();
-                col_rotate(tmem + b * 128, stage_at(s), base + ColSmem::had);
-                tile_commit(done + b * 8);
+                if (ok && lane == 0) {
+                    tmem_fence_after();
+                    col_rotate(tmem + b * 128, stage_at(s), base + ColSmem::had);
+                    tile_commit(done + b * 8);
+                }
             }
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) { give_up(); break; }
+            const uint32_t r = 32u * q + (uint32_t)lane;
+            float e = col_lost(stage_at(s), r, guess);
+#pragma unroll
+            for (int o = 1; o < C; o <<= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+            if ((lane & (C - 1)) == 0) lost[s * COL_ROWS + r / C] = e;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(scanned + s * 8);
+        }
+        // nothing is in flight when the CTA ends, also after a wait that ran out
+        if (q == 0u && lane == 0) {
+            for (uint32_t k = loads > COL_STAGES ? loads - COL_STAGES : 0u; k < loads; ++k) (void)mbar_wait_fast(full + (k % COL_STAGES) * 8, (k / COL_STAGES) & 1u);
+        }
+        if (q == 1u && lane == 0) {
             for (uint32_t k = j > COL_ACCS ? j - COL_ACCS : 0u; k < j; ++k) (void)mbar_wait_fast(done + (k % COL_ACCS) * 8, (k / COL_ACCS) & 1u);
         }
         __syncwarp();
@@ -252,14 +354,14 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
         const int wg = warp >> 2, w = warp & 3, bar = 1 + wg;
         ColGroup *G = reinterpret_cast<ColGroup *>(smem + ColSmem::groups) + wg;
         const uint32_t rows_all = p.pieces / C;
-        const float err = p.err;
         f32x2 u[16];
         for (uint32_t j = (uint32_t)wg, it = 0; j < n; j += COL_WGS, ++it) {
             const uint32_t s = j % COL_STAGES, b = j % COL_ACCS, tile = stage_at(s), acc = tmem + b * 128 + ((uint32_t)(w * 32) << 16);
             const uint32_t row0 = (first + j * gridDim.x) * R, rows = min((uint32_t)R, rows_all - row0);
             ColNotes *N = &G->notes[it & 1u];
             // (a wait that runs out is the same for the four warps: they leave together)
-            if (!mbar_wait_fast(done + b * 8, (j / COL_ACCS) & 1u) || !mbar_wait_fast(full + s * 8, (j / COL_STAGES) & 1u)) { give_up(); break; }
+            if (!mbar_wait_fast(done + b * 8, (j / COL_ACCS) & 1u) || !mbar_wait_fast(full + s * 8, (j / COL_STAGES) & 1u) ||
+                !mbar_wait_fast(scanned + s * 8, (j / COL_STAGES) & 1u)) { give_up(); break; }
             tmem_fence_after();
             // this lane's extremes of row k of 32 columns (symmetric: the largest magnitude)
             auto extremes = [&](int k, float &hi, float &lo) {
@@ -298,6 +400,12 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
             }
             named_barrier(bar, 128);
             if (w == 0 && lane < COL_ROWS) G->notes[(it & 1u) ^ 1u].count[lane] = 0u;      // (everybody has left that tile)
+            if (w == 1 && lane < R) {                                        // (much lost: the row again, in fp64)
+                const float4 h4 = *reinterpret_cast<const float4 *>(N->hi[lane]), l4 = *reinterpret_cast<const float4 *>(N->lo[lane]);
+                float a_row = fmaxf(fmaxf(h4.x, h4.y), fmaxf(h4.z, h4.w));
+                if (MODE == ROW_ASYM) a_row = fmaxf(a_row, -fminf(fminf(l4.x, l4.y), fminf(l4.z, l4.w)));
+                if (!(lost[s * COL_ROWS + lane] <= fminf(a_row, 3.0e38f) * COL_LOST)) atomicAdd(&N->count[lane], COL_LIST + 1u);
+            }
             // ---- codes, by the fp32 extremes
 #pragma unroll 1
             for (int un = 0; un < 4; ++un) {
@@ -310,10 +418,12 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
                     const int r = un * RU + k;
                     const float4 h4 = *reinterpret_cast<const float4 *>(N->hi[r]);
                     const float hr = fmaxf(fmaxf(h4.x, h4.y), fmaxf(h4.z, h4.w));
-                    const float own_hi = N->hi[r][w];
+                    const float own_hi = N->hi[r][w], lost_r = lost[s * COL_ROWS + r];
                     if (MODE == ROW_ASYM) {
                         const float4 l4 = *reinterpret_cast<const float4 *>(N->lo[r]);
-                        const float lr = fminf(fminf(l4.x, l4.y), fminf(l4.z, l4.w)), a_row = fmaxf(fabsf(hr), fabsf(lr)), e_abs = a_row * (2.0f * err + 2.4e-7f);
+                        const float lr = fminf(fminf(l4.x, l4.y), fminf(l4.z, l4.w)), a_row = fmaxf(fabsf(hr), fabsf(lr));
+                        const float e_row = fmaf(p.err, a_row, lost_r), e_abs = 2.0f * e_row + 2.4e-7f * a_row;
+                        const float err = fminf(__fdividef(0.25f * e_row, 0.25f * a_row), 1.0f);
                         float inv, z, slack, per_ref;
                         const bool near = tile_zero_point(hr, lr, err, inv, z, slack, per_ref) && a_row > 0.0f;
                         if (!(a_row > 0.0f)) inv = z = slack = per_ref = 0.0f;
@@ -330,11 +440,11 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
                             }
                         }
                     } else {
-                        const float thr = hr - hr * (2.0f * err + 2.4e-7f), inv = row_inverse(hr);
+                        const float e_row = fmaf(p.err, hr, lost_r), thr = hr - (2.0f * e_row + 2.4e-7f * hr), inv = row_inverse(hr);
                         Q[k].mul = inv;
                         Q[k].magic = 12584968.0f;
                         // an element's error and the maximum's; integers: the distance's own
-                        Q[k].tau = (2.0f * err + 5.0e-7f) * hr * inv + (MODE == ROW_FP4 ? 0.0f : 2.0e-7f);
+                        Q[k].tau = (2.0f * e_row + 5.0e-7f * hr) * inv + (MODE == ROW_FP4 ? 0.0f : 2.0e-7f);
                         if (hr > 0.0f && own_hi >= thr) {                              // (the same for the warp)
 #pragma unroll
                             for (int m = k * (C / 2); m < (k + 1) * (C / 2); ++m)

@@ -139,14 +139,11 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     }
 }
 
-// Where the column kernel is better than the row kernel (us, CUDA graphs, row / column): 4096 channels, 1024 rows 12.2 /
-// 10.8, 4096 rows 30.8 / 26.0, 16384 rows 113 / 84; asymmetric 19.7 / 21.3, 51 / 37, 190 / 122; 2048 channels, 4096 rows 17.8 / 19.3, 16384
-// rows 57.7 / 51.0, asymmetric 28.5 / 27.1, 95 / 79.
-bool col_is_better(int mode, int d, long long pieces)
-{
-    if (d == 2048) return pieces >= 16 * 16384;
-    return pieces >= 32 * (mode == perq::ROW_ASYM ? 4096 : 1024);
-}
+// Where the column kernel is better than the row kernel (us, CUDA graphs, row / column, laplace and swiglu values): 4096
+// channels, 2048 rows 18.4 / 21.9 and 18.6 / 21.4, 4096 rows 31.3 / 30.0 and 30.9 / 29.8, 16384 rows 113 / 98 and 113 / 99;
+// FP4 33.0 / 31.0, 117 / 99; asymmetric 51 / 40, 191 / 134.  2048 channels, 8192 rows 30.8 / 31.6, 16384 rows 58.0 / 54.9;
+// FP4 59.4 / 55.8, asymmetric 95 / 80.
+bool col_is_better(int d, long long pieces) { return pieces >= (d == 2048 ? 16 * 16384 : 32 * 4096); }
 
 // Whole-row rotations of 2048 and 4096 channels with one scale per token.  Returns -1 if the column kernel does not take
 // the call.
@@ -161,7 +158,7 @@ int try_launch_col(const void *x, const int32_t *perm, int64_t T, int32_t d, int
     else return -1;
     const long long pieces = (long long)T * (d / 128);
     if (pieces >= (1ll << 31) - perq::TILE_PIECES) return -1;
-    if (!col_is_better(mode, d, pieces)) return -1;
+    if (!col_is_better(d, pieces)) return -1;
     perq::TileParams p;
     std::memset(&p, 0, sizeof(p));
     p.x = static_cast<const uint16_t *>(x);
@@ -171,7 +168,7 @@ int try_launch_col(const void *x, const int32_t *perm, int64_t T, int32_t d, int
     p.tile_pieces = perq::TILE_PIECES;
     p.tiles = (uint32_t)((pieces + perq::TILE_PIECES - 1) / perq::TILE_PIECES);
     p.row_pieces = d / 128;
-    p.err = perq::COL_ERR_K * (float)ilog2(d) * perq::TWO_M24;
+    p.err = perq::col_stage_err(ilog2(d) - 7) * perq::TWO_M24;      // (what the contraction loses is added row by row)
     p.sqrt_b = std::sqrt((double)b);
     p.inv_sqrt_b = 1.0 / p.sqrt_b;
     p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);

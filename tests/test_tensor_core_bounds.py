@@ -1,0 +1,112 @@
+"""Error bounds of the kernels that rotate by chained tensor-core steps (tile and column kernel), against the oracle, on rows
+whose fp32 outputs are as wrong as that arithmetic allows: a maximum, and a side of a rounding boundary, that fp32 hides."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_22347_b200 import inputs
+
+from mma_rows import hadamard, chained_contraction, hidden_in_every_piece, hidden_maximum, hidden_side, hidden_step, outputs, to_bf16
+from parity import compare_quantized
+
+FMT = {"int4": 0, "mxfp4": 1, "fp4": 3, "int4_asym": 4}
+
+
+@pytest.fixture(scope="module")
+def B():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_22347_b200 import binding, build
+    build.build()
+    binding.load()
+    binding.perq_device_error_clear()
+    yield binding
+    assert binding.perq_device_error() == 0
+
+
+def bits(x):
+    x = np.asarray(x, np.float32)
+    assert np.array_equal(x, to_bf16(x))
+    return inputs.f32_to_bf16_bits(x)
+
+
+def whole_rows(d, seed):
+    """Rows with one hidden output, moved to other places and magnitudes: an input's sign by a row of the Hadamard matrix
+    moves all outputs, a shift of the inputs by XOR changes only their signs."""
+    c = d // 128
+    kinds = [hidden_maximum(d, 128, 110), hidden_maximum(d, 128, 95), hidden_in_every_piece(d, 94 * c), hidden_side(d, 128, 6.5 / 7, 10),
+             hidden_side(d, 128, 5 / 7, 10), hidden_step(d, 128, 12, 10), hidden_step(d, 128, 11, 6)]
+    rng, k = np.random.default_rng(seed), np.arange(d)
+    rows = []
+    for i in range(12):
+        for x in kinds:
+            m, s = (0, 0) if i == 0 else (int(rng.integers(d)), int(rng.integers(d)) & ~15)
+            signs = 1.0 - 2.0 * (np.array([bin(v).count("1") for v in (k & m)]) & 1)
+            rows.append((x * signs)[k ^ s] * 2.0 ** int(rng.integers(-20, 20)))
+    return bits(np.array(rows))
+
+
+def run(B, oracle, base, T, b, fmt, group):
+    """T rows made of the base rows, each of which is compared, and the same bytes at every repetition."""
+    n = len(base)
+    idx = (np.arange(T) + np.arange(T) // n) % n
+    idx_t = torch.from_numpy(idx).cuda()
+    x = torch.from_numpy(base.view(np.int16)).cuda()[idx_t].view(torch.bfloat16)
+    codes, scales = B.perq_rotate_quantize(x, None, b, FMT[fmt], group)
+    torch.cuda.synchronize()
+    first = torch.empty(n, dtype=torch.int64, device="cuda")
+    first[idx_t.flip(0)] = torch.arange(T - 1, -1, -1, device="cuda")
+    assert torch.equal(codes, codes[first[idx_t]]) and torch.equal(scales, scales[first[idx_t]])
+    ora = oracle.rotate_quantize(base, None, b, FMT[fmt], group, want_pre=True)
+    compare_quantized(fmt, codes[first].cpu().numpy(), scales[first].cpu().numpy(), ora)
+
+
+def test_rows_hide_what_they_say():
+    """The model's fp32 outputs of the rows above: another maximum, another side."""
+    h = hadamard(128)
+    for d in (2048, 4096):
+        for x, wrong in ((hidden_maximum(d, 128, 110), 46), (hidden_in_every_piece(d, 94 * d // 128), 90)):
+            v = chained_contraction(x.reshape(-1, 128), h)
+            u32 = hadamard(d // 128) @ v                       # (the later stages without rounding)
+            top = np.abs(outputs(x)).max()
+            at = np.unravel_index(np.abs(outputs(x)).argmax(), u32.shape)
+            assert np.abs(u32).max() - abs(u32[at]) > (wrong - 1) * 2.0 ** -24 * top
+        x = hidden_side(d, 128, 6.5 / 7, 10)
+        v = (hadamard(d // 128) @ chained_contraction(x.reshape(-1, 128), h)).ravel()
+        u = outputs(x)
+        assert u[1] > 6.5 / 7 * u.max() and v[1] < 6.5 / 7 * v.max() * (1 - 30 * 2.0 ** -24)
+
+
+def lost_at_most(x):
+    """The column kernel's bound of what a piece of 128 loses, from its inputs."""
+    e = np.floor(np.log2(np.abs(x).sum(1) * 1.001))
+    n = ((x != 0) & (np.abs(x) < np.exp2(e - 16)[:, None])).sum(1)
+    return (n + 5 * np.minimum(n, 8)) * np.exp2(e - 25)
+
+
+@pytest.mark.parametrize("kind", ["gauss", "binades", "few", "coherent", "decreasing"])
+def test_what_the_contraction_loses(kind):
+    """No output of the model is further off than the bound (0.17 to 0.63 of it)."""
+    rng, h, worst = np.random.default_rng(41000), hadamard(128), 0.0
+    for it in range(6):
+        x = rng.standard_normal((64, 128))
+        if kind == "binades":
+            x *= np.exp2(-rng.integers(0, 40, x.shape))
+        elif kind == "few":
+            x = np.where(rng.random(x.shape) < 0.1, x, 0.0) * np.exp2(-rng.integers(0, 26, x.shape))
+        elif kind == "coherent":
+            x = np.where(rng.random(x.shape) < 0.02, x, np.abs(x) * np.exp2(-rng.integers(14, 28, (64, 1))) * h[rng.integers(0, 128, 64)])
+        elif kind == "decreasing":
+            x *= np.exp2(-np.arange(128) / rng.integers(2, 12, (64, 1)))
+        x = to_bf16(x)
+        off = np.abs(chained_contraction(x, h) - x @ h).max(1)
+        bound = lost_at_most(x)
+        assert (off <= bound).all()
+        worst = max(worst, (off / np.where(bound > 0, bound, 1)).max())
+    assert worst > 0.1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
+@pytest.mark.parametrize("d,T", [(4096, 4099), (2048, 16389)])
+def test_whole_row_rotations(B, oracle, d, T, fmt):
+    run(B, oracle, whole_rows(d, 40000 + d), T, d, fmt, 0)
