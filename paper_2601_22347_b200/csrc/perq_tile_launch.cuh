@@ -68,26 +68,35 @@ int launch_tile_b(int log2b, const CUtensorMap &map, const perq::TileParams &p, 
 }
 
 // Where the tile kernel is the better one.  It pays 3 to 5 us more than the kernels that rotate in registers (tensor
-// memory, operand, the last tile and batch), so calls have to be large; how large depends on what those kernels need.  Both
-// sides in us (CUDA graphs, others / tile), 2^20 elements unless stated:
-//   widths that are no multiple of 1024 (row kernel), 9728, b = 32, 4 / 16: MXFP4 9.4 / 7.3, 22 / 12; per 128 12 / 7.5, 30 / 13;
-//     INT4 per token 9.4 / 8.5, 24 / 16; FP4 11 / 8.6, 29 / 16; asymmetric 12 / 10, 31 / 23.  (2: 0.8 .. 1.1 of the others' rate.)
-//   MXFP4, 4096, 16: b = 32 13.9 / 12.4, 64 14.5 / 13.9, 128 15.1 / 14.8; b = 16 13.7 / 14.1, at 32 21.5 / 21.0
-//   per 128, 4096, 16 (8): b = 16 15.0 / 13.1 (9.5 / 9.3), b = 128 20.1 / 18.0 (12.7 / 12.7)
-//   INT4 per token, 4096, 8: b = 32 9.2 / 9.5, 64 11.4 / 10.0, 128 12.5 / 11.4; 2048, 16: 64 15.9 / 13.2, but 64: 38.7 / 44.2;
-//     14336, 16 (4): b = 16 13.9 / 12.5 (6.0 / 7.5), 128 22.1 / 15.3 (8.8 / 9.4)
-//   FP4, 4096, 1: b = 32 8.6 / 6.7, 64 9.4 / 7.0; 128 7.3 / 8.1, at 8 14.2 / 11.5; 14336, 8: 12.4 / 9.4, 14.8 / 11.6
-//   asymmetric, 4096, 16: b = 32 21.5 / 17.9, 64 24 / 18.4, 128 26.8 / 22.2, b = 16 20.7 / 18.4, but 64: 52.4 / 54.6
+// memory, operand, the last tile and batch), so calls have to be large; how large depends on what those kernels need, on how
+// many lanes of a tile whole rows fill, and on the doubtful codes, which grow with the error bound of b (tile_err).  Both
+// sides in us (CUDA graphs, others / tile; laplace and, after a comma, swiglu values), 2^20 elements unless stated:
+//   widths that are no multiple of 1024 (row kernel), 9728, 4 / 16: MXFP4 b = 32 10.6 / 8.5, 24 / 13, b = 128 12.1 / 10.7, 27 / 19; per
+//     128 b = 32 13 / 8.7, 31 / 15 (2: 8.4 / 7.8); INT4 per token b = 32 10.0 / 9.7, 23 / 18, b = 128 11.9 / 12.7, 27 / 23; FP4 b = 64
+//     13.0 / 11.4, 32 / 23, b = 128 12.8 / 13.9, 32 / 26; 8320, whose rows fill half a tile: INT4 b = 64 10.7 / 10.8, 27 / 21
+//   MXFP4, 4096, 16: b = 32 13.9 / 12.4, b = 64 15.2 / 14.6; 64: 40 / 34, 42 / 38; b = 128 46 / 55; b = 16 45 / 41, but 8 x 2^22 values of
+//     four significant bits 84 / 227
+//   per 128, 4096, 16: b = 16 15.9 / 13.9, b = 64 18.6 / 16.0; b = 128 21.2 / 20.7, at 24 28.9 / 27.2
+//   INT4 per token, 8 (64): 4096, b = 64 12.7 / 11.9 (43 / 38); b = 128 13.1 / 15.0 (53 / 57); 2048, b = 64 (39 / 48)
+//     other widths, 32: b = 32 6144 25.1 / 24.9, 29 / 25, 14336 26 / 22; b = 16 6144 22.4 / 25.2, 14336 23.3 / 21.5; 16: b = 64 3072 17.0 / 16.7,
+//     14336 18 / 16; b = 128 12288 22.5 / 20.8, 6144 21.8 / 22.1 (61 / 64)
+//   FP4, 1 (16): 4096, b = 32 9.4 / 8.0 (21 / 15), b = 64 10.9 / 8.8 (25 / 18), at 200 161 / 142, 154 / 161; 2048, b = 32 at 32 29.9 / 23.6, at 64
+//     51 / 45, 48 / 48, b = 64 at 24 27 / 25, at 48 45 / 50; b = 128, 4096, 64: 60 / 71
+//     other widths, 8: b = 32 3072 11.8 / 11.2, 14336 12.5 / 11.7; 16: b = 64 6144 20 / 19, 3072 at 64 56 / 62; b = 128 12288 27 / 23, 6144 25.2 / 24.6 (73 / 81)
 bool tile_is_better(int mode, int d, int b, long long pieces)
 {
     const long long M = 8192;                                // pieces of 2^20 elements
-    if (d % perq::SEG_ELEMS != 0) return pieces >= (mode == perq::ROW_GROUP ? 2 : 4) * M;
-    const bool lean = d == 2048 || d == 4096 || d == 8192;  // (per token: these have a kernel of their own up to b = 64)
+    if (d % perq::SEG_ELEMS != 0) return pieces >= (mode == perq::ROW_GROUP ? 2 : b == 128 && mode != perq::ROW_MX ? 16 : 4) * M;
+    const bool lean = d == 2048 || d == 4096 || d == 8192;  // (per token: these have a kernel of their own up to b = 128)
     switch (mode) {
-    case perq::ROW_MX: return pieces >= (b == 16 ? 32 : 16) * M;
-    case perq::ROW_GROUP: return pieces >= 16 * M;
-    case perq::ROW_TOKEN: return lean ? d >= 4096 && b >= 64 && pieces >= 8 * M : d >= 3072 && pieces >= 16 * M;
-    case perq::ROW_FP4: return lean && b <= 64 ? pieces >= M : d >= 3072 && pieces >= 8 * M;
+    case perq::ROW_MX: return (b == 32 || b == 64) && pieces >= 16 * M;
+    case perq::ROW_GROUP: return pieces >= (b == 128 ? 24 : 16) * M;
+    case perq::ROW_TOKEN:
+        if (lean) return d >= 4096 && b == 64 && pieces >= 8 * M;
+        return b >= 64 ? d >= (b == 128 ? 12288 : 3072) && pieces >= 16 * M : d > (b == 16 ? 12288 : 2048) && pieces >= 32 * M;
+    case perq::ROW_FP4:
+        if (lean) return b <= 64 && pieces >= M && pieces <= (d == 2048 ? b == 64 ? 24 : 32 : d == 4096 && b == 64 ? 128 : 1 << 17) * M;
+        return b >= 64 ? d >= (b == 128 ? 12288 : 6144) && pieces >= 16 * M : d >= 3072 && pieces >= 8 * M;
     default: return d >= 3072 && (b >= 32 || !lean) && pieces >= 16 * M;
     }
 }
@@ -121,7 +130,7 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     p.row_pieces = row_pieces;
     p.wide_store = (reinterpret_cast<uintptr_t>(out_codes) & 31u) == 0;
     const int log2b = ilog2(b);
-    p.err = perq::FAST_ERR_K * (float)log2b * perq::TWO_M24;
+    p.err = perq::tile_err(log2b);
     p.sqrt_b = std::sqrt((double)b);
     p.inv_sqrt_b = 1.0 / p.sqrt_b;
     p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);
@@ -140,10 +149,13 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
 }
 
 // Where the column kernel is better than the row kernel (us, CUDA graphs, row / column, laplace and swiglu values): 4096
-// channels, 2048 rows 18.4 / 21.9 and 18.6 / 21.4, 4096 rows 31.3 / 30.0 and 30.9 / 29.8, 16384 rows 113 / 98 and 113 / 99;
-// FP4 33.0 / 31.0, 117 / 99; asymmetric 51 / 40, 191 / 134.  2048 channels, 8192 rows 30.8 / 31.6, 16384 rows 58.0 / 54.9;
-// FP4 59.4 / 55.8, asymmetric 95 / 80.
-bool col_is_better(int d, long long pieces) { return pieces >= (d == 2048 ? 16 * 16384 : 32 * 4096); }
+// channels, 2048 rows 18.4 / 21.9, 18.6 / 21.4, 4096 rows 31.3 / 30.0, 30.9 / 29.8, 8192 rows 58.5 / 53.0, 58.9 / 53.7, 16384 rows 113 / 98,
+// 113 / 99; FP4 62.0 / 56.1 and 117 / 99; asymmetric, 4096 rows 51 / 40, 16384 rows 191 / 134.  2048 channels, 8192 rows 30.8 / 31.6, 16384
+// rows 58.0 / 54.9; FP4 59.4 / 55.8, asymmetric 95 / 80.
+bool col_is_better(int mode, int d, long long pieces)
+{
+    return pieces >= (d == 2048 ? 16 * 16384 : 32 * (mode == perq::ROW_ASYM ? 4096 : 8192));
+}
 
 // Whole-row rotations of 2048 and 4096 channels with one scale per token.  Returns -1 if the column kernel does not take
 // the call.
@@ -158,7 +170,7 @@ int try_launch_col(const void *x, const int32_t *perm, int64_t T, int32_t d, int
     else return -1;
     const long long pieces = (long long)T * (d / 128);
     if (pieces >= (1ll << 31) - perq::TILE_PIECES) return -1;
-    if (!col_is_better(d, pieces)) return -1;
+    if (!col_is_better(mode, d, pieces)) return -1;
     perq::TileParams p;
     std::memset(&p, 0, sizeof(p));
     p.x = static_cast<const uint16_t *>(x);

@@ -45,6 +45,23 @@ def whole_rows(d, seed):
     return bits(np.array(rows))
 
 
+def block_rows(d, b, seed):
+    """Rows of one block that hides an output and others, at a quarter of its size and less, that do."""
+    gap = 124 if b == 128 else 62
+    kinds = [hidden_maximum(b, b, gap), hidden_maximum(b, b, gap - 8), hidden_side(b, b, 6.5 / 7, 10), hidden_side(b, b, 5 / 7, 10),
+             hidden_side(b, b, 3.5 / 7, 10), hidden_step(b, b, 12, 10)]
+    rng, k = np.random.default_rng(seed), np.arange(b)
+    x = np.zeros((96, d // b, b))
+    for i in range(len(x)):
+        top = rng.integers(d // b)
+        for j in range(d // b):
+            signs = 1.0 - 2.0 * (np.array([bin(v).count("1") for v in (k & int(rng.integers(b)))]) & 1)
+            size = 0 if j == top else int(rng.integers(-30, -2))
+            x[i, j] = (kinds[(i + j) % 6 if j != top else i % 6] * signs)[k ^ (int(rng.integers(b)) & ~15)] * 2.0 ** size
+        x[i] *= 2.0 ** int(rng.integers(-20, 20))
+    return bits(x.reshape(len(x), d))
+
+
 def run(B, oracle, base, T, b, fmt, group):
     """T rows made of the base rows, each of which is compared, and the same bytes at every repetition."""
     n = len(base)
@@ -107,6 +124,31 @@ def test_what_the_contraction_loses(kind):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
-@pytest.mark.parametrize("d,T", [(4096, 4099), (2048, 16389)])
+@pytest.mark.parametrize("d,T", [(4096, 8195), (2048, 16389)])
 def test_whole_row_rotations(B, oracle, d, T, fmt):
     run(B, oracle, whole_rows(d, 40000 + d), T, d, fmt, 0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("fp4", 0), ("mxfp4", 32)])
+@pytest.mark.parametrize("b", [64, 128])
+def test_blocks(B, oracle, b, fmt, group):
+    run(B, oracle, block_rows(1152, b, 42000 + b), 16 * 2 ** 20 // 1152 + 3, b, fmt, group)
+
+
+def test_tile_err_covers_the_model():
+    """|u32 - u| of the model against the tile kernel's constants (16, 20, 45 and 103 * 2^-24 of the block's largest output)."""
+    rng = np.random.default_rng(43000)
+    for b, err in ((16, 16), (32, 20), (64, 45), (128, 103)):
+        h, worst = hadamard(b), 0.0
+        rows = [rng.standard_normal((64, b)) * np.exp2(-rng.integers(0, 1 + 8 * t, (64, b))) for t in range(5)]
+        if b >= 64:
+            rows.append(np.array([hidden_maximum(b, b, 62), hidden_side(b, b, 6.5 / 7, 10), hidden_step(b, b, 12, 10)]))
+        # one large input, and every other one just below what is kept beside it, agreeing in sign
+        rows.append(np.where(np.arange(b) == 0, 1.0, h[rng.integers(0, b, 64)] * 1.9921875 * 2.0 ** -rng.integers(20, 26, (64, 1)).astype(float)))
+        for x in rows:
+            x = to_bf16(x)
+            off = np.abs(chained_contraction(x, h) - x @ h).max(1) / np.abs(x @ h).max(1)
+            worst = max(worst, off.max() * 2 ** 24)
+        assert worst < err
+        assert worst > (3 if b == 16 else 6 if b == 32 else 24 if b == 64 else 56)
