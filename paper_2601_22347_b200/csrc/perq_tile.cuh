@@ -50,35 +50,33 @@ struct TileParams {
     double sqrt_b, inv_sqrt_b, inv_7_sqrt_b;
 };
 
-// fp32 maxima of token rows that lie in several warps: magnitude bits, or order keys of the extremes; two tiles' worth,
-// used in turn.
+// fp32 maxima (bits) of token rows that lie in several warps; two tiles' worth, used in turn.
 struct TileRows {
-    uint32_t mx[2][TILE_ROW_CAP], mn[2][TILE_ROW_CAP];
+    uint32_t mx[2][TILE_ROW_CAP];
 };
 
 // What is left to settle of a tile: places, and what their codes depend on.
 constexpr int TILE_JOBS = 96;
 constexpr int TILE_TIES = 4;                  // notes of a lane and 32 columns
 // a job: kind (1 bit), row of the tile (5, from bit 20), code as stored (4, from bit 16), column (7), piece (7)
-// Pieces with more places than are worth a note each are left to their lanes (tile_put_extremes, tile_requantise).
-enum TileFlat : uint32_t { FLAT_ROWS = 1u, FLAT_CODES = 2u };          // extremes that are in ex_* only; codes
+// Pieces with more places than are worth a note each are left to their lanes (tile_put_maximum, tile_requantise).
+enum TileFlat : uint32_t { FLAT_ROWS = 1u, FLAT_CODES = 2u };          // maxima that are in `ex` only; codes
 enum TileJob : uint32_t { JOB_MAX = 0u << 30, JOB_TIE = 1u << 30 };     // candidates in a quad; an element
 struct TileNotes {
-    unsigned long long ex_hi[TILE_ROW_CAP], ex_lo[TILE_ROW_CAP];       // exact: magnitude bits, or order keys of the extremes
+    unsigned long long ex[TILE_ROW_CAP];                               // exact maxima of token rows (bits)
     unsigned long long aux[TILE_PIECES];                               // per piece: exact maximum (ranges), exponents (MX)
     uint32_t settled[4];                                               // pieces whose codes are exact already
     uint32_t flat, count;                                              // (more notes than fit: count goes on)
     uint32_t job[TILE_JOBS];
 };
-// A note and what its code depends on: exponents or the exact maximum (MX, ranges), or up to two quads that hold the
-// extremes of the element's row (piece and column each; the second may be missing).
+// A note and what its code depends on: exponents or the exact maximum (MX, ranges), or the quad that holds the maximum of
+// the element's row (piece and column).
 struct TileRecord {
     uint32_t job, piece;
-    uint32_t aux[4];
-    uint32_t pad[2];
+    uint32_t aux[2];
 };
 constexpr int TILE_RECORDS = 64;              // per batch
-constexpr uint32_t TILE_NONE = 0xffffffffu, TILE_LAST = 1u << 30;
+constexpr uint32_t TILE_LAST = 1u << 30;
 
 // -------------------------------------------------------------------------------------------- tensor core and TMA
 
@@ -250,8 +248,6 @@ __device__ __forceinline__ double tile_output_of(double (&S)[8], uint32_t c)
     return fma(s2, fma(s1, S[3], S[2]), fma(s1, S[1], S[0])) + 0.0;        // (+0 for a sum of zeros of either sign)
 }
 __device__ __forceinline__ double tile_abs_max(const double (&o)[4]) { return fmax(fmax(fabs(o[0]), fabs(o[1])), fmax(fabs(o[2]), fabs(o[3]))); }
-__device__ __forceinline__ double tile_max_of(const double (&o)[4]) { return fmax(fmax(o[0], o[1]), fmax(o[2], o[3])); }
-__device__ __forceinline__ double tile_min_of(const double (&o)[4]) { return fmin(fmin(o[0], o[1]), fmin(o[2], o[3])); }
 
 // All exact outputs of a piece, by a warp: lane l brings the inputs of columns 4 l .. 4 l + 3 and gets the outputs there
 // (the butterfly in fp64).
@@ -362,13 +358,6 @@ __device__ __forceinline__ void tile_mend(const TileParams &p, uint32_t piece, u
 
 // -------------------------------------------------------------------------------------------- quantising
 
-__device__ __forceinline__ uint32_t order_key32(float f)
-{
-    const uint32_t u = __float_as_uint(f);
-    return (u >> 31) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float order_value32(uint32_t k) { return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k); }
-
 // Codes of the lane's 32 values, and whether any of them is within the window of a tie (as row_quantise; integers are
 // packed on the fp32 side: magic + k0 + 256 k2 and magic + k1 + 256 k3 are one packed fma).  TWO: the second half of the
 // values by B.
@@ -461,47 +450,32 @@ __device__ __forceinline__ bool tile_note(TileNotes *notes, uint32_t job)
 // which a look at its inputs shows; sums only where they are not.  A piece per lane, all lanes at work.  (2048 x 9728 of
 // integers -3 .. 3, b = 128, INT4 per token: 245 us, 856 with the pieces settled in turn by one warp, 270 in registers)
 
-// The quads of 32 columns that hold candidates for a row's extremes.
-template <int MODE>
-__device__ __forceinline__ uint32_t tile_candidates(const f32x2 (&u)[16], float thr_hi, float thr_lo)
+// The quads of 32 columns that hold candidates for a row's maximum.
+__device__ __forceinline__ uint32_t tile_candidates(const f32x2 (&u)[16], float thr)
 {
     uint32_t quads = 0u;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const f32x2 v0 = u[2 * j], v1 = u[2 * j + 1];
-        bool r;
-        if (MODE == ROW_ASYM) r = fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)) >= thr_hi || fminf(fminf(v0.x, v0.y), fminf(v1.x, v1.y)) <= thr_lo;
-        else r = fmaxf(max3abs(fabsf(v0.x), v0.y, v1.x), fabsf(v1.y)) >= thr_hi;
-        quads |= r ? (1u << j) : 0u;
-    }
+    for (int j = 0; j < 8; ++j) quads |= fmaxf(max3abs(fabsf(u[2 * j].x), u[2 * j].y, u[2 * j + 1].x), fabsf(u[2 * j + 1].y)) >= thr ? (1u << j) : 0u;
     return quads;
 }
 
-// Exact extremes of the lane's candidates (cmask: chunks that have some; 0: nothing to do) into its row's words.
-template <int LOG2B, int MODE>
-__device__ __noinline__ void tile_put_extremes(const TileParams &p, uint32_t tmem, uint32_t piece, uint32_t cmask, float thr_hi, float thr_lo, TileNotes *notes, int ri)
+// Exact maximum of the lane's candidates (cmask: chunks that have some; 0: nothing to do) into its row's word.
+template <int LOG2B>
+__device__ __noinline__ void tile_put_maximum(const TileParams &p, uint32_t tmem, uint32_t piece, uint32_t cmask, float thr, TileNotes *notes, int ri)
 {
     f32x2 u[16];
     int exact = -1;                                          // (asked for when there are several: a look costs as much as a sum)
-    double hi = MODE == ROW_ASYM ? -1.7976931348623157e308 : 0.0, lo = 1.7976931348623157e308;
+    double a = 0.0;
     __syncwarp();
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
         if (!__any_sync(0xffffffffu, (cmask >> c) & 1u)) continue;
         tmem_load32(tmem + 32 * c, u);
-        uint32_t quads = (cmask >> c) & 1u ? tile_candidates<MODE>(u, thr_hi, thr_lo) : 0u;
+        uint32_t quads = (cmask >> c) & 1u ? tile_candidates(u, thr) : 0u;
         if (exact < 0 && __popc(quads) > 2) exact = tile_lane_exact(p.x + (size_t)piece * 128);
         if (exact > 0 && quads) {
             quads = 0u;
-            if (MODE == ROW_ASYM) {
-                float h = u[0].x, l = u[0].x;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) { h = fmaxf(fmaxf(h, u[k].x), u[k].y); l = fminf(fminf(l, u[k].x), u[k].y); }
-                hi = fmax(hi, (double)h);
-                lo = fmin(lo, (double)l);
-            } else {
-                hi = fmax(hi, (double)tile_max(u));
-            }
+            a = fmax(a, (double)tile_max(u));
         }
         while (quads) {
             double S[8], o[4];
@@ -509,24 +483,16 @@ __device__ __noinline__ void tile_put_extremes(const TileParams &p, uint32_t tme
             quads &= quads - 1u;
             tile_sums_global<LOG2B>(p, piece, col, S);
             tile_quad_of(S, col, o);
-            hi = fmax(hi, MODE == ROW_ASYM ? tile_max_of(o) : tile_abs_max(o));
-            lo = fmin(lo, tile_min_of(o));
+            a = fmax(a, tile_abs_max(o));
         }
         __syncwarp();
     }
-    if (cmask != 0u) {
-        if (MODE == ROW_ASYM) {
-            atomicMax(&notes->ex_hi[ri], order_key(hi + 0.0));
-            atomicMin(&notes->ex_lo[ri], order_key(lo + 0.0));
-        } else {
-            atomicMax(&notes->ex_hi[ri], (unsigned long long)__double_as_longlong(hi));
-        }
-    }
+    if (cmask != 0u) atomicMax(&notes->ex[ri], (unsigned long long)__double_as_longlong(a));
     __syncwarp();
 }
 
 // Exact codes of the pieces of the lanes with `mine`: quantised again, by exact scales, and their doubtful elements settled here.
-// aux: exponents (MX) or bits of the exact maximum (ranges); token rows have their extremes in the row's words.
+// aux: exponents (MX) or bits of the exact maximum (ranges); token rows have their maxima in the row's words.
 template <int LOG2B, int MODE>
 __device__ __noinline__ void tile_requantise(const TileParams &p, uint32_t tmem, uint32_t piece, bool mine, unsigned long long aux, TileNotes *notes, int w, int ri)
 {
@@ -535,7 +501,7 @@ __device__ __noinline__ void tile_requantise(const TileParams &p, uint32_t tmem,
     const unsigned whose = __ballot_sync(0xffffffffu, mine);
     if (lane == 0) notes->settled[w] = whose;
     const bool exact = mine && tile_lane_exact(p.x + (size_t)piece * 128);
-    const float err = exact ? 1.2e-7f : p.err;               // (exact elements: the fp32 extremes of an exact range)
+    const float err = exact ? 1.2e-7f : p.err;               // (exact elements: the fp32 maximum of an exact range)
     __syncwarp();
     float ref = 0.0f;                                        // (of the piece: not less than any block's)
 #pragma unroll 1
@@ -544,16 +510,9 @@ __device__ __noinline__ void tile_requantise(const TileParams &p, uint32_t tmem,
     RowQuant Q;
     Q.magic = 12584968.0f;
     Q.mul = Q.tau = 0.0f;
-    if (MODE == ROW_ASYM) {
-        const double hi = order_value(notes->ex_hi[ri]), lo = order_value(notes->ex_lo[ri]);
-        float z, slack, per_ref;
-        if (mine) q = tile_scale_asym(p, hi, lo);
-        (void)tile_zero_point((float)hi, (float)lo, err, Q.mul, z, slack, per_ref);
-        Q.magic = 12582912.0f - (float)q.z64;
-        Q.tau = (float)hi > (float)lo ? per_ref * ref + slack : 3.0e38f;
-    } else if (MODE != ROW_MX) {
-        q = tile_scale_max<MODE>(p, __longlong_as_double((long long)(MODE == ROW_GROUP ? aux : notes->ex_hi[ri])));
-        Q.mul = row_inverse((float)(__longlong_as_double((long long)(MODE == ROW_GROUP ? aux : notes->ex_hi[ri]))));
+    if (MODE != ROW_MX) {
+        q = tile_scale_max<MODE>(p, __longlong_as_double((long long)(MODE == ROW_GROUP ? aux : notes->ex[ri])));
+        Q.mul = row_inverse((float)q.a);
         Q.tau = (err + 5.0e-7f) * Q.mul * ref + (MODE == ROW_FP4 ? 0.0f : 2.0e-7f);
     }
 #pragma unroll 1
@@ -649,7 +608,7 @@ template <int LOG2B, int MODE>
 __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLane &L, uint32_t tmem, uint32_t tile, uint32_t half, uint32_t t, TileRows *rows,
                                               uint32_t par, int bar, TileNotes *notes)
 {
-    constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4 || MODE == ROW_ASYM;
+    constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4;
     const int lane = L.lane, l = L.w * 32 + lane;
     const uint32_t piece = t * (uint32_t)p.tile_pieces + (uint32_t)l;
     const bool live = l < p.tile_pieces && piece < p.pieces;
@@ -659,8 +618,8 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
     RowQuant Q;
     Q.magic = 12584968.0f;                // 1.5 * 2^23 + 8 * 257: two nibbles of the sum are codes + 8
     float m[4] = {0.0f, 0.0f, 0.0f, 0.0f};                         // largest magnitude of each chunk of 32 columns
-    float inv = 0.0f, lm = 0.0f, slack = 0.0f, per_ref = 0.0f, thr_hi = 0.0f, thr_lo = 0.0f;
-    uint32_t cmask = 0u;                                           // per token: chunks with candidates for the row's extremes
+    float inv = 0.0f, lm = 0.0f, slack = 0.0f, per_ref = 0.0f, thr = 0.0f;
+    uint32_t cmask = 0u;                                           // per token: chunks with candidates for the row's maximum
     bool many_max = false, many = false;                           // more candidates, doubtful elements than are worth a note each
     unsigned long long aux = 0ull;                                 // exact maximum (ranges)
 
@@ -678,7 +637,7 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
                          fmaxf(fmaxf(qm[8 * c + 4], qm[8 * c + 5]), fmaxf(qm[8 * c + 6], qm[8 * c + 7])));
         }
         lm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
-        const float thr = lm - 2.0f * err * lm - lm * 2.4e-7f;
+        thr = lm - 2.0f * err * lm - lm * 2.4e-7f;
         uint32_t want = 0u;
 #pragma unroll
         for (int j = 0; j < 32; ++j) want |= (qm[j] >= thr) ? (1u << j) : 0u;
@@ -708,101 +667,37 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
         slack = 2.0e-7f;
     } else if (TOK || LOG2B >= 6) {
         // ---- fp32 maxima of the chunks, then of the rows (MX inside longer blocks: the error reference)
-        float ch[4], cl[4], hi = -3.0e38f, lo = 3.0e38f;
-        auto extremes = [&](const f32x2 (&u)[16], int c) {
-            if (MODE == ROW_ASYM) {
-                ch[c] = u[0].x;
-                cl[c] = u[0].x;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) { ch[c] = fmaxf(fmaxf(ch[c], u[k].x), u[k].y); cl[c] = fminf(fminf(cl[c], u[k].x), u[k].y); }
-                m[c] = fmaxf(fabsf(ch[c]), fabsf(cl[c]));
-                hi = fmaxf(hi, ch[c]);
-                lo = fminf(lo, cl[c]);
-            } else {
-                m[c] = tile_max(u);
-            }
-        };
 #pragma unroll
         for (int c = 0; c < 4; c += 2) {
             tmem_wait(ua);
             tmem_issue32(tmem + 32 * (c + 1), ub);
-            extremes(ua, c);
+            m[c] = tile_max(ua);
             tmem_wait(ub);
             tmem_issue32(tmem + (c ? 0 : 64), ua);                    // (in the end: the first chunk again, for the quantiser)
-            extremes(ub, c + 1);
+            m[c + 1] = tile_max(ub);
         }
         lm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
         if (TOK) {
-            float hr, lr = 0.0f;                                      // the row's extremes, or its largest magnitude
-            if (!live) { hi = -3.0e38f; lo = 3.0e38f; }
-            hr = MODE == ROW_ASYM ? hi : live ? lm : 0.0f;
+            float hr = live ? lm : 0.0f;                              // the row's largest magnitude
             if (!L.coupled && p.row_pieces == 32) {
                 hr = warp_max_f32(hr);
-                if (MODE == ROW_ASYM) lr = warp_min_f32(lo);
             } else if (!L.coupled) {
-                lr = lo;
-                for (int o = 1; o < p.row_pieces; o <<= 1) {
-                    hr = fmaxf(hr, __shfl_xor_sync(0xffffffffu, hr, o));
-                    if (MODE == ROW_ASYM) lr = fminf(lr, __shfl_xor_sync(0xffffffffu, lr, o));
-                }
+                for (int o = 1; o < p.row_pieces; o <<= 1) hr = fmaxf(hr, __shfl_xor_sync(0xffffffffu, hr, o));
             } else {
-                if (L.whole) {
-                    hr = warp_max_f32(hr);
-                    if (MODE == ROW_ASYM) lo = warp_min_f32(lo);
-                }
-                if (L.whole ? lane == 0 : live) {
-                    atomicMax(&rows->mx[par][L.ri], MODE == ROW_ASYM ? order_key32(hr) : __float_as_uint(hr));
-                    if (MODE == ROW_ASYM) atomicMin(&rows->mn[par][L.ri], order_key32(lo));
-                }
+                if (L.whole) hr = warp_max_f32(hr);
+                if (L.whole ? lane == 0 : live) atomicMax(&rows->mx[par][L.ri], __float_as_uint(hr));
                 named_barrier(bar, 128);
-                hr = MODE == ROW_ASYM ? order_value32(rows->mx[par][L.ri]) : __uint_as_float(rows->mx[par][L.ri]);
-                if (MODE == ROW_ASYM) lr = order_value32(rows->mn[par][L.ri]);
-                if (L.first) {                                        // (the other tile's words: everybody has left that tile)
-                    rows->mx[par ^ 1u][L.ri] = 0u;
-                    rows->mn[par ^ 1u][L.ri] = 0xffffffffu;
-                }
+                hr = __uint_as_float(rows->mx[par][L.ri]);
+                if (L.first) rows->mx[par ^ 1u][L.ri] = 0u;           // (the other tile's word: everybody has left that tile)
             }
-            if (MODE == ROW_ASYM) {
-                const float a_row = fmaxf(fabsf(hr), fabsf(lr)), e_abs = a_row * (2.0f * err + 2.4e-7f);
-                const bool some = live && a_row > 0.0f, flat = !(hr > lr);
-                thr_hi = hr - e_abs;
-                thr_lo = lr + e_abs;
+            thr = hr - hr * (2.0f * err + 2.4e-7f);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) cmask |= (ch[c] >= thr_hi || cl[c] <= thr_lo) ? (1u << c) : 0u;
-                if (!some) cmask = 0u;
-                float z;
-                const bool near = tile_zero_point(hr, lr, err, inv, z, slack, per_ref) && some;
-                if (!some) inv = z = per_ref = slack = 0.0f;
-                else if (flat) per_ref = 3.0e38f;                     // (equal in fp32: everything is in doubt)
-                // the zero point of a row of the tile is in doubt: its exact extremes now (the four warps agree on this)
-                // (from the row words alone: warps that share the tile but not the row must not miss the barrier)
-                bool doubt = false;
-                if (L.coupled) {
-                    const uint32_t khi = rows->mx[par][lane], klo = rows->mn[par][lane];
-                    float f[4];
-                    if (khi >= klo) {
-                        const float h = order_value32(khi), l0 = order_value32(klo);
-                        doubt = fmaxf(fabsf(h), fabsf(l0)) > 0.0f && tile_zero_point(h, l0, err, f[0], f[1], f[2], f[3]);
-                    }
-                }
-                if (L.coupled ? __any_sync(0xffffffffu, doubt) : __any_sync(0xffffffffu, near)) {
-                    tmem_wait(ua);
-                    tile_put_extremes<LOG2B, MODE>(p, tmem, piece, near ? cmask : 0u, thr_hi, thr_lo, notes, L.ri);
-                    if (L.coupled) named_barrier(bar, 128); else __syncwarp();
-                    if (near) z = (float)tile_scale_asym(p, order_value(notes->ex_hi[L.ri]), order_value(notes->ex_lo[L.ri])).z64;
-                    tmem_issue32(tmem, ua);
-                }
-                Q.magic = 12582912.0f - z;
-            } else {
-                thr_hi = hr - hr * (2.0f * err + 2.4e-7f);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) cmask |= (m[c] >= thr_hi) ? (1u << c) : 0u;
-                if (!live || !(hr > 0.0f)) cmask = 0u;
-                inv = row_inverse(hr);
-                // the element's error and the multiplier's (the maximum's, three roundings); integers: the distance's own
-                per_ref = (2.0f * err + 5.0e-7f) * inv;
-                slack = MODE == ROW_FP4 ? 0.0f : 2.0e-7f;
-            }
+            for (int c = 0; c < 4; ++c) cmask |= (m[c] >= thr) ? (1u << c) : 0u;
+            if (!live || !(hr > 0.0f)) cmask = 0u;
+            inv = row_inverse(hr);
+            // the element's error and the multiplier's (the maximum's, three roundings); integers: the distance's own
+            per_ref = (2.0f * err + 5.0e-7f) * inv;
+            slack = MODE == ROW_FP4 ? 0.0f : 2.0e-7f;
         }
     }
 
@@ -865,10 +760,10 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
                 Q.tau = per_ref * ref + slack;
             }
             const uint32_t place = (uint32_t)(64 * h + 32 * k) << 7 | (uint32_t)l;
-            if (TOK) {                                        // candidates for the row's extremes
+            if (TOK) {                                        // candidates for the row's maximum
                 const bool cand = (cmask >> (2 * h + k)) & 1u;
                 if (__any_sync(0xffffffffu, cand)) {
-                    uint32_t quads = cand ? tile_candidates<MODE>(u, thr_hi, thr_lo) : 0u;
+                    uint32_t quads = cand ? tile_candidates(u, thr) : 0u;
                     if (__popc(quads) > 2) { many_max = true; quads = 0u; }
                     while (quads) {
                         const uint32_t j = (uint32_t)__ffs(quads) - 1u;
@@ -910,7 +805,7 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
             named_barrier(bar, 128);
             codes = (*reinterpret_cast<volatile uint32_t *>(&notes->flat) & FLAT_CODES) != 0u;
         }
-        if (ext || codes) tile_put_extremes<LOG2B, MODE>(p, tmem, piece, many_max || codes ? cmask : 0u, thr_hi, thr_lo, notes, L.ri);
+        if (ext || codes) tile_put_maximum<LOG2B>(p, tmem, piece, many_max || codes ? cmask : 0u, thr, notes, L.ri);
         if (codes && L.coupled) named_barrier(bar, 128);
     }
     if (codes) tile_requantise<LOG2B, MODE>(p, tmem, piece, many, aux, notes, L.w, L.ri);
@@ -922,7 +817,7 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
 template <int LOG2B, int MODE>
 __device__ __forceinline__ void tile_settle_records(const TileParams &p, const TileRecord *list, int n, int lane)
 {
-    constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4 || MODE == ROW_ASYM;
+    constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4;
     if (lane >= n) return;
     const TileRecord rec = list[lane];
     const uint32_t c = (rec.job >> 7) & 127u;
@@ -933,24 +828,12 @@ __device__ __forceinline__ void tile_settle_records(const TileParams &p, const T
         tile_sums_global<LOG2B>(p, rec.piece, c, S);
         u = tile_output_of(S, c);
     }
-    if (TOK) {                                     // the row's extremes, from the quads that hold them
-        double a = 0.0, hi = -1.7976931348623157e308, lo = 1.7976931348623157e308;
-#pragma unroll 1
-        for (int k = 0; k < (MODE == ROW_ASYM ? 4 : 2); k += 2) {
-            if (rec.aux[k] == TILE_NONE) break;
-            double o[4];
-            tile_sums_global<LOG2B>(p, rec.aux[k], rec.aux[k + 1], S);
-            tile_quad_of(S, rec.aux[k + 1], o);
-            a = fmax(a, tile_abs_max(o));
-            hi = fmax(hi, tile_max_of(o));
-            lo = fmin(lo, tile_min_of(o));
-        }
-        q = MODE == ROW_ASYM ? tile_scale_asym(p, hi, lo) : tile_scale_max<MODE>(p, a);
-        if (!tie) {
-            const uint32_t row = rec.piece / (uint32_t)p.row_pieces;
-            if (MODE == ROW_ASYM) reinterpret_cast<float2 *>(p.out_scales)[row] = make_float2((float)q.s64, (float)q.z64);
-            else reinterpret_cast<float *>(p.out_scales)[row] = row_scale(a, p.inv_7_sqrt_b, p.sqrt_b, 7.0);
-        }
+    if (TOK) {                                     // the row's maximum, from the quad that holds it
+        double o[4];
+        tile_sums_global<LOG2B>(p, rec.aux[0], rec.aux[1], S);
+        tile_quad_of(S, rec.aux[1], o);
+        q = tile_scale_max<MODE>(p, tile_abs_max(o));
+        if (!tie) reinterpret_cast<float *>(p.out_scales)[rec.piece / (uint32_t)p.row_pieces] = row_scale(q.a, p.inv_7_sqrt_b, p.sqrt_b, 7.0);
     } else if (MODE == ROW_MX) {
         q = tile_scale_mx(p, rec.aux[0] >> (8 * (c >> 5)) & 0xffu);
     } else {
@@ -983,12 +866,12 @@ struct TileCollector {
     __device__ __forceinline__ void make_room() { if (n > TILE_RECORDS - 32) hand_over(0u); }
 };
 
-// The notes of a tile, by a warp.  Most become records; token rows with several candidates, or with extremes that have no note,
-// are settled here: their exact extremes and scales, then the doubtful codes.
+// The notes of a tile, by a warp.  Most become records; token rows with several candidates, or with maxima that have no note,
+// are settled here: their exact maxima and scales, then the doubtful codes.
 template <int LOG2B, int MODE>
 __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, TileNotes *notes, TileCollector &to, int lane)
 {
-    constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4 || MODE == ROW_ASYM;
+    constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4;
     const uint32_t piece0 = t * (uint32_t)p.tile_pieces, rp = (uint32_t)p.row_pieces;
     const uint32_t n = min(*reinterpret_cast<volatile uint32_t *>(&notes->count), (uint32_t)TILE_JOBS);
     if (!TOK && n == 0u) return;
@@ -1000,28 +883,20 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
         const unsigned cands = __ballot_sync(0xffffffffu, cand);
         const unsigned mates = __match_any_sync(0xffffffffu, has ? row : 0x100u + (uint32_t)lane) & cands;      // its row's candidates
         const bool my_row = (uint32_t)lane * rp < here;
-        const bool bad = has && (__popc(mates) > (MODE == ROW_ASYM ? 2 : 1) || mates == 0u);
+        const bool bad = has && __popc(mates) != 1;
         if (!__any_sync(0xffffffffu, bad)) {
             // rows without a candidate are rows of zeros
             const uint32_t rows = __reduce_or_sync(0xffffffffu, cand ? 1u << row : 0u);
-            if (my_row && !((rows >> lane) & 1u)) {
-                const size_t r = (size_t)(piece0 / rp) + lane;
-                if (MODE == ROW_ASYM) reinterpret_cast<float2 *>(p.out_scales)[r] = make_float2(0.0f, 0.0f);
-                else reinterpret_cast<float *>(p.out_scales)[r] = 0.0f;
-            }
-            const int c0 = mates ? __ffs(mates) - 1 : lane, c1 = mates ? 31 - __clz(mates) : lane;
-            const uint32_t j0 = __shfl_sync(0xffffffffu, j, c0), j1 = __shfl_sync(0xffffffffu, j, c1);
-            const bool mine = has && (!cand || c0 == lane);       // (one record for two candidates of a row)
-            const unsigned who = __ballot_sync(0xffffffffu, mine);
+            if (my_row && !((rows >> lane) & 1u)) reinterpret_cast<float *>(p.out_scales)[(size_t)(piece0 / rp) + lane] = 0.0f;
+            const uint32_t j0 = __shfl_sync(0xffffffffu, j, mates ? __ffs(mates) - 1 : lane);
+            const unsigned who = __ballot_sync(0xffffffffu, has);
             to.make_room();
-            if (mine) {
+            if (has) {
                 TileRecord rec;
                 rec.job = j;
                 rec.piece = piece0 + (j & 127u);
                 rec.aux[0] = piece0 + (j0 & 127u);
                 rec.aux[1] = (j0 >> 7) & 127u;
-                rec.aux[2] = c1 != c0 ? piece0 + (j1 & 127u) : TILE_NONE;
-                rec.aux[3] = (j1 >> 7) & 127u;
                 to.list()[to.n + __popc(who & ((1u << lane) - 1u))] = rec;
             }
             to.n += __popc(who);
@@ -1035,27 +910,13 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
                 double S[8], o[4];
                 tile_sums_global<LOG2B>(p, piece0 + (j & 127u), c, S);
                 tile_quad_of(S, c, o);
-                if (MODE == ROW_ASYM) {
-                    atomicMax(&notes->ex_hi[row], order_key(tile_max_of(o)));
-                    atomicMin(&notes->ex_lo[row], order_key(tile_min_of(o)));
-                } else {
-                    atomicMax(&notes->ex_hi[row], (unsigned long long)__double_as_longlong(tile_abs_max(o)));
-                }
+                atomicMax(&notes->ex[row], (unsigned long long)__double_as_longlong(tile_abs_max(o)));
             }
         }
         __syncwarp();
         // ---- scales: a row per lane
-        const bool mine = (uint32_t)lane * rp < here;
-        const size_t row = (size_t)(piece0 / rp) + lane;
-        if (MODE == ROW_ASYM) {
-            if (mine) {
-                if (notes->ex_hi[lane] == 0ull) notes->ex_hi[lane] = notes->ex_lo[lane] = order_key(0.0);      // (no candidates: a row of zeros)
-                const TileScale q = tile_scale_asym(p, order_value(notes->ex_hi[lane]), order_value(notes->ex_lo[lane]));
-                reinterpret_cast<float2 *>(p.out_scales)[row] = make_float2((float)q.s64, (float)q.z64);
-            }
-        } else if (mine) {
-            reinterpret_cast<float *>(p.out_scales)[row] = row_scale(__longlong_as_double((long long)notes->ex_hi[lane]), p.inv_7_sqrt_b, p.sqrt_b, 7.0);
-        }
+        if ((uint32_t)lane * rp < here)
+            reinterpret_cast<float *>(p.out_scales)[(size_t)(piece0 / rp) + lane] = row_scale(__longlong_as_double((long long)notes->ex[lane]), p.inv_7_sqrt_b, p.sqrt_b, 7.0);
         __syncwarp();
     }
     // ---- doubtful codes
@@ -1067,9 +928,7 @@ __device__ __forceinline__ void tile_settle(const TileParams &p, uint32_t t, Til
             if (tie) {
                 double S[8];
                 tile_sums_global<LOG2B>(p, piece0 + r, c, S);
-                const uint32_t row = (j >> 20) & 31u;
-                const TileScale q = MODE == ROW_ASYM ? tile_scale_asym(p, order_value(notes->ex_hi[row]), order_value(notes->ex_lo[row]))
-                                                     : tile_scale_max<MODE>(p, __longlong_as_double((long long)notes->ex_hi[row]));
+                const TileScale q = tile_scale_max<MODE>(p, __longlong_as_double((long long)notes->ex[(j >> 20) & 31u]));
                 tile_mend(p, piece0 + r, j, tile_code<MODE>(p, tile_output_of(S, c), q));
             }
         } else {
@@ -1118,8 +977,7 @@ static_assert(sizeof(TileNotes) % 8 == 0 && sizeof(TileBatches) % 8 == 0 && Tile
 // The words of a tile's notes as they are before it.
 __device__ __forceinline__ void tile_clear_notes(TileNotes *notes, int lane)
 {
-    notes->ex_hi[lane] = 0ull;
-    notes->ex_lo[lane] = ~0ull;
+    notes->ex[lane] = 0ull;
     if (lane < 4) notes->settled[lane] = 0u;
     if (lane == 0) notes->flat = notes->count = 0u;
 }
@@ -1146,7 +1004,6 @@ __global__ void __maxnreg__(TILE_REGS) perq_tile_kernel(const __grid_constant__ 
     if (warp < TILE_WGS) {
         TileRows *rows = reinterpret_cast<TileRows *>(smem + TileSmem::rows) + warp;
         rows->mx[0][lane] = rows->mx[1][lane] = 0u;
-        rows->mn[0][lane] = rows->mn[1][lane] = 0xffffffffu;
     }
     tile_write_hadamard<LOG2B>(smem + TileSmem::had, tid, TILE_THREADS);
     fence_async_smem();                       // (the operand was written by ordinary stores)

@@ -83,6 +83,8 @@ int launch_tile_b(int log2b, const CUtensorMap &map, const perq::TileParams &p, 
 //   FP4, 1 (16): 4096, b = 32 9.4 / 8.0 (21 / 15), b = 64 10.9 / 8.8 (25 / 18), at 200 161 / 142, 154 / 161; 2048, b = 32 at 32 29.9 / 23.6, at 64
 //     51 / 45, 48 / 48, b = 64 at 24 27 / 25, at 48 45 / 50; b = 128, 4096, 64: 60 / 71
 //     other widths, 8: b = 32 3072 11.8 / 11.2, 14336 12.5 / 11.7; 16: b = 64 6144 20 / 19, 3072 at 64 56 / 62; b = 128 12288 27 / 23, 6144 25.2 / 24.6 (73 / 81)
+// Asymmetric rows are not taken: a zero point in doubt has to be settled while its tile waits, 10 us for the first one; 4096 channels,
+// b = 16 at 64 53 / 70, 9728 at 4 12 / 21.
 bool tile_is_better(int mode, int d, int b, long long pieces)
 {
     const long long M = 8192;                                // pieces of 2^20 elements
@@ -94,10 +96,9 @@ bool tile_is_better(int mode, int d, int b, long long pieces)
     case perq::ROW_TOKEN:
         if (lean) return d >= 4096 && b == 64 && pieces >= 8 * M;
         return b >= 64 ? d >= (b == 128 ? 12288 : 3072) && pieces >= 16 * M : d > (b == 16 ? 12288 : 2048) && pieces >= 32 * M;
-    case perq::ROW_FP4:
+    default:
         if (lean) return b <= 64 && pieces >= M && pieces <= (d == 2048 ? b == 64 ? 24 : 32 : d == 4096 && b == 64 ? 128 : 1 << 17) * M;
         return b >= 64 ? d >= (b == 128 ? 12288 : 6144) && pieces >= 16 * M : d >= 3072 && pieces >= 8 * M;
-    default: return d >= 3072 && (b >= 32 || !lean) && pieces >= 16 * M;
     }
 }
 
@@ -109,7 +110,6 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     int mode;
     if (fmt == PERQ_FMT_MXFP4) mode = perq::ROW_MX;
     else if (fmt == PERQ_FMT_FP4) mode = perq::ROW_FP4;
-    else if (fmt == PERQ_FMT_INT4_ASYM) mode = perq::ROW_ASYM;
     else if (fmt == PERQ_FMT_INT4 && g == 128) mode = perq::ROW_GROUP;
     else if (fmt == PERQ_FMT_INT4 && g == d) mode = perq::ROW_TOKEN;
     else return -1;
@@ -142,7 +142,6 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     switch (mode) {
     case perq::ROW_MX: return launch_tile_b<perq::ROW_MX>(log2b, map, p, grid, st);
     case perq::ROW_FP4: return launch_tile_b<perq::ROW_FP4>(log2b, map, p, grid, st);
-    case perq::ROW_ASYM: return launch_tile_b<perq::ROW_ASYM>(log2b, map, p, grid, st);
     case perq::ROW_GROUP: return launch_tile_b<perq::ROW_GROUP>(log2b, map, p, grid, st);
     default: return launch_tile_b<perq::ROW_TOKEN>(log2b, map, p, grid, st);
     }
