@@ -116,3 +116,37 @@ def test_flat_rows(B, oracle, d, T, fmt, group):
     # nearly every piece has more candidates or ties than are noted: lanes settle them, with exact fp32 outputs and without
     for b in (16, 128):
         check(B, oracle, T, d, b, fmt, group, 33000 + d + b, make=flat_rows)
+
+
+def zero_blocks(d, seed):
+    """Blocks of 16 zeros beside blocks that are not, and channels of zeros at the end."""
+    x = base_rows(d, seed)
+    x[:, 16::64] = 0
+    x[:, 32:48] = 0
+    x[:, d - 80:] = 0
+    return x
+
+
+def pass_us(B, make, T, d, b, fmt, group, seed):
+    x = torch.from_numpy(make(d, seed).view(np.int16)).cuda()[20:120].repeat(-(-T // 100), 1)[:T].view(torch.bfloat16).contiguous()
+    codes, scales = B.alloc_outputs(T, d, FMT[fmt], group, "cuda")
+    best = float("inf")
+    for _ in range(5):
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        torch.cuda.synchronize()
+        e[0].record()
+        for _ in range(10):
+            B.perq_rotate_quantize(x, None, b, FMT[fmt], group, codes, scales)
+        e[1].record()
+        torch.cuda.synchronize()
+        best = min(best, e[0].elapsed_time(e[1]) * 100)
+    return best
+
+
+@pytest.mark.parametrize("fmt,group,d,T", [("fp4", 0, 4096, 4096), ("fp4", 0, 9728, 2048), ("mxfp4", 32, 9728, 2048)])
+def test_blocks_of_zeros_beside_others(B, oracle, fmt, group, d, T):
+    """The signs of their outputs are not in doubt: a call with some takes no longer than one without."""
+    check(B, oracle, T, d, 16, fmt, group, 34000 + d, make=zero_blocks)
+    dense, zeros = pass_us(B, base_rows, T, d, 16, fmt, group, 34001), pass_us(B, zero_blocks, T, d, 16, fmt, group, 34001)
+    print("%s %d x %d: dense %.1f us, blocks of zeros %.1f us" % (fmt, T, d, dense, zeros))
+    assert zeros < 2 * dense
