@@ -529,6 +529,9 @@ __device__ __noinline__ void tile_requantise(const TileParams &p, uint32_t tmem,
             q = tile_scale_mx(p, (uint32_t)Eb);
             Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - LOG2B / 2, 1), 254) << 23) * ((LOG2B & 1) ? 0.70710678118654752f : 1.0f);
             Q.tau = Eb == 0 ? 3.0e38f : err * ref * Q.mul + 2.0e-6f;          // (the lowest exponent: perhaps a group of zeros)
+            // exact, and so is the product with a power of two: the conversion rounds ties to even (2048 x 9728 of integers, b = 16: 869 us
+            // with every tie evaluated in fp64, 270)
+            if ((LOG2B & 1) == 0 && exact) Q.tau = 0.0f;
         }
         uint32_t cw[4];
         const bool fl = tile_quantise<MODE>(u, Q, cw) && mine;

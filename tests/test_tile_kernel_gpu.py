@@ -150,3 +150,19 @@ def test_blocks_of_zeros_beside_others(B, oracle, fmt, group, d, T):
     dense, zeros = pass_us(B, base_rows, T, d, 16, fmt, group, 34001), pass_us(B, zero_blocks, T, d, 16, fmt, group, 34001)
     print("%s %d x %d: dense %.1f us, blocks of zeros %.1f us" % (fmt, T, d, dense, zeros))
     assert zeros < 2 * dense
+
+
+def few_bits(d, seed):
+    """Integers, and values of four significant bits: with b = 16 and 64 many outputs lie on E2M1 midpoints."""
+    rng = np.random.default_rng(seed)
+    x = rng.integers(-3, 4, (BASE, d)).astype(np.float64)
+    x[BASE // 2:] = rng.integers(-15, 16, (BASE - BASE // 2, d)) * np.exp2(rng.integers(-3, 2, (BASE - BASE // 2, d)))
+    return bf16(x)
+
+
+@pytest.mark.parametrize("b,d,T", [(16, 9728, 2048), (64, 9728, 2048), (64, 4096, 4096)])
+def test_many_midpoints(B, oracle, b, d, T):
+    check(B, oracle, T, d, b, "mxfp4", 32, 35000 + b, make=few_bits)
+    dense, ties = pass_us(B, base_rows, T, d, b, "mxfp4", 32, 35001), pass_us(B, few_bits, T, d, b, "mxfp4", 32, 35001)
+    print("b = %d, %d x %d: dense %.1f us, midpoints %.1f us" % (b, T, d, dense, ties))
+    assert ties < 18 * dense
