@@ -3,7 +3,8 @@
 // A tile is 128 pieces of 128 adjacent channels.  Its rotation is one contraction, D[piece][column] = X H: the tile
 // lies in shared memory as the K-major operand with 128-byte swizzle, H_64 beside it as the other operand (its
 // leading 16 and 32 rows and columns are H_16 and H_32; H_128 is four H_64, one of them negated), the fp32 result in
-// tensor memory.  Every product is a bf16 value times +-1.
+// tensor memory.  The operand holds +-1/2, so that everything below is in halves of the unnormalised outputs: the sum of
+// some inputs of a block can be 1.75 times its largest output, which may lie just below 2^128.
 //
 // What follows the rotation has a piece per lane: a warp reads 32 columns of its 32 pieces with one load, so that the
 // maxima of MX groups and of ranges of 128, the rounding, the packing of 32 codes and the test for doubtful elements
@@ -47,7 +48,7 @@ struct TileParams {
     int row_pieces;          // d / 128
     int wide_store;          // codes are 32-byte aligned
     float err;
-    double sqrt_b, inv_sqrt_b, inv_7_sqrt_b;
+    double sqrt_b, inv_sqrt_b, inv_7_sqrt_b;         // (tile kernel: sqrt(b) / 2, what its halved outputs are divided by)
 };
 
 // fp32 maxima (bits) of token rows that lie in several warps; two tiles' worth, used in turn.
@@ -160,7 +161,7 @@ __device__ __forceinline__ void tile_store32(uint8_t *dst, const uint32_t (&w)[8
     }
 }
 
-// H_64 (or smaller), and for blocks of 128 its negative, as operands at h and h + TILE_H_BYTES.
+// H_64 / 2 (or smaller), and for blocks of 128 its negative, as operands at h and h + TILE_H_BYTES.
 template <int LOG2B>
 __device__ __forceinline__ void tile_write_hadamard(unsigned char *h, int tid, int nthr)
 {
@@ -168,7 +169,7 @@ __device__ __forceinline__ void tile_write_hadamard(unsigned char *h, int tid, i
     for (int e = tid; e < N * N / 2; e += nthr) {
         const int n = e / (N / 2), k = 2 * (e - n * (N / 2));
         const uint32_t at = (uint32_t)(n * 128 + (((k >> 3) ^ (n & 7)) << 4) + (k & 7) * 2);
-        const uint32_t w = hadamard_bf16(n, k) | (hadamard_bf16(n, k + 1) << 16);
+        const uint32_t w = (hadamard_bf16(n, k) | (hadamard_bf16(n, k + 1) << 16)) - 0x00800080u;
         *reinterpret_cast<uint32_t *>(h + at) = w;
         if (LOG2B == 7) *reinterpret_cast<uint32_t *>(h + TILE_H_BYTES + at) = w ^ 0x80008000u;
     }
@@ -217,7 +218,7 @@ __device__ __forceinline__ void tile_sums(uint32_t c, F load, double (&S)[8])
     for (uint32_t k = 0; k < B; k += 8) {
         const uint4 v = load(k);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        const double f = __hiloint2double(((__popc(i & k) & 1) ? (int)0x80000000 : 0) | 0x77f00000, 0);          // +-2^896
+        const double f = __hiloint2double(((__popc(i & k) & 1) ? (int)0x80000000 : 0) | 0x77e00000, 0);          // +-2^896 / 2
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             S[2 * j] = fma(bf16_raw_f64(w[j] << 16), f, S[2 * j]);
@@ -256,7 +257,7 @@ __device__ __forceinline__ void tile_butterfly(uint32_t w0, uint32_t w1, int lan
 {
     const double x0 = bf16_raw_f64(w0 << 16), x1 = bf16_raw_f64(w0), x2 = bf16_raw_f64(w1 << 16), x3 = bf16_raw_f64(w1);
     const double a0 = x0 + x1, a1 = x0 - x1, a2 = x2 + x3, a3 = x2 - x3;
-    o[0] = (a0 + a2) * 0x1p896; o[1] = (a1 + a3) * 0x1p896; o[2] = (a0 - a2) * 0x1p896; o[3] = (a1 - a3) * 0x1p896;
+    o[0] = (a0 + a2) * 0x1p895; o[1] = (a1 + a3) * 0x1p895; o[2] = (a0 - a2) * 0x1p895; o[3] = (a1 - a3) * 0x1p895;
 #pragma unroll
     for (int t = 0; t < LOG2B - 2; ++t) {
         const double sg = ((lane >> t) & 1) ? -1.0 : 1.0;
@@ -527,7 +528,7 @@ __device__ __noinline__ void tile_requantise(const TileParams &p, uint32_t tmem,
         if (MODE == ROW_MX) {
             const int Eb = (int)(((uint32_t)aux >> (8 * c)) & 0xffu);
             q = tile_scale_mx(p, (uint32_t)Eb);
-            Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - LOG2B / 2, 1), 254) << 23) * ((LOG2B & 1) ? 0.70710678118654752f : 1.0f);
+            Q.mul = __uint_as_float((uint32_t)min(max(255 - Eb - LOG2B / 2, 1), 254) << 23) * ((LOG2B & 1) ? 0.70710678118654752f : 1.0f);
             Q.tau = Eb == 0 ? 3.0e38f : err * ref * Q.mul + 2.0e-6f;          // (the lowest exponent: perhaps a group of zeros)
             // exact, and so is the product with a power of two: the conversion rounds ties to even (2048 x 9728 of integers, b = 16: 869 us
             // with every tie evaluated in fp64, 270)
@@ -730,17 +731,17 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
                 if (LOG2B == 4) { tile_half_max(u, hm[0], hm[1]); gm = fmaxf(hm[0], hm[1]); }
                 else gm = tile_max(u);
                 const float ref = LOG2B <= 5 ? gm : LOG2B == 6 ? (h ? fmaxf(m[2], m[3]) : fmaxf(m[0], m[1])) : lm;
-                // E + 127 with E = floor(log2(a / sqrt(b))) - 2; the distance of a to a value where the floor changes
+                // E + 127 with E = floor(log2(2 a / sqrt(b))) - 2; the distance of a to a value where the floor changes
                 const uint32_t bits = __float_as_uint(gm);
                 const int e8 = (int)(bits >> 23);
                 float dist;
                 if ((LOG2B & 1) == 0) {
                     const float lower = __uint_as_float(bits & 0x7f800000u);
                     dist = fminf(gm - lower, 2.0f * lower - gm);
-                    Eb = e8 - LOG2B / 2 - 2;
+                    Eb = e8 - LOG2B / 2 - 1;
                 } else {
                     dist = fabsf(gm - __uint_as_float((bits & 0x7f800000u) | 0x3504f3u));
-                    Eb = e8 - (LOG2B - 1) / 2 - 3 + ((bits & 0x7fffffu) >= 0x3504f4u ? 1 : 0);
+                    Eb = e8 - (LOG2B - 1) / 2 - 2 + ((bits & 0x7fffffu) >= 0x3504f4u ? 1 : 0);
                 }
                 const float tol = 2.0f * err * ref + gm * 4.8e-7f;
                 const bool near = live && gm > 0.0f && (dist <= tol || e8 == 0);
@@ -767,8 +768,8 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
                     }
                 }
                 Eb = min(max(Eb, 0), 254);
-                if ((LOG2B & 1) == 0) Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - LOG2B / 2, 1), 254) << 23);
-                else Q.mul = __uint_as_float((uint32_t)min(max(254 - Eb - (LOG2B - 1) / 2, 1), 254) << 23) * 0.70710678118654752f;
+                if ((LOG2B & 1) == 0) Q.mul = __uint_as_float((uint32_t)min(max(255 - Eb - LOG2B / 2, 1), 254) << 23);
+                else Q.mul = __uint_as_float((uint32_t)min(max(255 - Eb - (LOG2B - 1) / 2, 1), 254) << 23) * 0.70710678118654752f;
                 if (zero) { Eb = 0; Q.mul = 0.0f; }
                 Q.tau = (ref > 0.0f && !(near && zero)) ? err * ref * Q.mul + 2.0e-6f : 0.0f;        // (the multiplier's and the product's rounding)
                 exps |= (uint32_t)Eb << (16 * h + 8 * k);

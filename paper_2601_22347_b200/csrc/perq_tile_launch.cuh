@@ -131,7 +131,7 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     p.wide_store = (reinterpret_cast<uintptr_t>(out_codes) & 31u) == 0;
     const int log2b = ilog2(b);
     p.err = perq::tile_err(log2b);
-    p.sqrt_b = std::sqrt((double)b);
+    p.sqrt_b = 0.5 * std::sqrt((double)b);
     p.inv_sqrt_b = 1.0 / p.sqrt_b;
     p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);
     const int sms = sm_count();

@@ -136,6 +136,40 @@ def test_blocks(B, oracle, b, fmt, group):
     run(B, oracle, block_rows(1152, b, 42000 + b), 16 * 2 ** 20 // 1152 + 3, b, fmt, group)
 
 
+def upper_end_rows(oracle, d, b, seed):
+    """Largest unnormalised outputs in (2^125.98, 2^127.98]; and blocks in which the sum of the first inputs passes 2^128 although
+    no output does."""
+    rng = np.random.default_rng(seed)
+    x = to_bf16(rng.standard_normal((48, d)) + 0.2)
+    u = np.abs(oracle.rotate(bits(x), None, b)).max(axis=1) * np.sqrt(b)
+    x *= np.exp2(np.floor(126.98 + np.arange(48) % 2 - np.log2(u)))[:, None]
+    n = min(b, 128)
+    if n >= 64:
+        k, a = np.arange(n), 1.5 * 2.0 ** (121 if n == 128 else 122)
+        for i in range(0, 48, 4):
+            m = int(rng.integers(n))
+            signs = 1.0 - 2.0 * (np.array([bin(v).count("1") for v in (k & m)]) & 1)
+            x[i] = 0.0
+            x[i, n * (i // 4 % (d // n)):][:n] = np.where(k < n - 16, a, -3 * a if n == 128 else -a) * signs
+            if i % 8:
+                x[i] += np.where(x[i] == 0, to_bf16(rng.standard_normal(d) * 2.0 ** 115), 0.0)
+    return bits(x)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("fp4", 0), ("mxfp4", 32)])
+@pytest.mark.parametrize("b", [16, 32, 64, 128])
+def test_blocks_at_the_upper_end_of_the_range(B, oracle, b, fmt, group):
+    run(B, oracle, upper_end_rows(oracle, 1152, b, 44000 + b), 16 * 2 ** 20 // 1152 + 3, b, fmt, group)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
+@pytest.mark.parametrize("d,T", [(4096, 8195), (2048, 16389)])
+def test_whole_rows_at_the_upper_end_of_the_range(B, oracle, d, T, fmt):
+    run(B, oracle, upper_end_rows(oracle, d, d, 45000 + d), T, d, fmt, 0)
+
+
 def test_tile_err_covers_the_model():
     """|u32 - u| of the model against the tile kernel's constants (16, 20, 45 and 103 * 2^-24 of the block's largest output)."""
     rng = np.random.default_rng(43000)
