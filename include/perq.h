@@ -320,8 +320,9 @@ int perq_massdiff_perm_device(const float *chan_abs_sum, int32_t d, int32_t b, i
  * perq_device_error -- reads (synchronously, cudaMemcpyFromSymbol) the library's device-side
  * error word on the current device into *flags_host.  0 = no error.  Bit 0 is set when a
  * bounded wait inside a kernel ran out (an asynchronous copy that never completed); the
- * kernel then stops early and its outputs are incomplete.  Kernels only ever set bits; the
- * word keeps them until perq_device_error_clear.
+ * kernel then stops early and its outputs are incomplete.  Bits 1 and 2: such a wait inside the
+ * permuted and grouped kernels, for an exact maximum (1) or a free buffer (2); bit 3: in the
+ * statistic.  Kernels only ever set bits; the word keeps them until perq_device_error_clear.
  *
  * perq_device_error_clear -- writes 0 to that word on the current device (synchronously,
  * cudaMemcpyToSymbol), so that a later read reports only what happened since.  Call it with no

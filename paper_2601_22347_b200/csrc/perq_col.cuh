@@ -297,7 +297,7 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(smem + ColSmem::slot);
     const uint32_t first = blockIdx.x, n = first < p.tiles ? (p.tiles - first + gridDim.x - 1) / gridDim.x : 0u;
     auto stage_at = [&](uint32_t s) { return base + ColSmem::stages + s * 2 * ColSmem::half; };
-    auto give_up = [&]() { if (lane == 0) atomicOr(&g_perq_device_error, 8u); };
+    auto give_up = [&]() { if (lane == 0) atomicOr(&g_perq_device_error, 1u); };
 
     // (a wait that runs out ends its warp's part; the others' waits run out too, and all meet at the end)
     if (warp >= COL_WGS * 4) {
@@ -359,9 +359,8 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
             const uint32_t s = j % COL_STAGES, b = j % COL_ACCS, tile = stage_at(s), acc = tmem + b * 128 + ((uint32_t)(w * 32) << 16);
             const uint32_t row0 = (first + j * gridDim.x) * R, rows = min((uint32_t)R, rows_all - row0);
             ColNotes *N = &G->notes[it & 1u];
-            // (a wait that runs out is the same for the four warps: they leave together)
-            if (!mbar_wait_fast(done + b * 8, (j / COL_ACCS) & 1u) || !mbar_wait_fast(full + s * 8, (j / COL_STAGES) & 1u) ||
-                !mbar_wait_fast(scanned + s * 8, (j / COL_STAGES) & 1u)) { give_up(); break; }
+            bool ok = mbar_wait_fast(done + b * 8, (j / COL_ACCS) & 1u) && mbar_wait_fast(full + s * 8, (j / COL_STAGES) & 1u) &&
+                      mbar_wait_fast(scanned + s * 8, (j / COL_STAGES) & 1u);
             tmem_fence_after();
             // this lane's extremes of row k of 32 columns (symmetric: the largest magnitude)
             auto extremes = [&](int k, float &hi, float &lo) {
@@ -384,7 +383,7 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
             };
             // ---- extremes of the rows (loops that are not unrolled: these kernels are short of instruction cache)
 #pragma unroll 1
-            for (int un = 0; un < 4; ++un) {
+            for (int un = 0; un < 4 && ok; ++un) {
                 tmem_load32(acc + 32 * un, u);
                 col_stages<LOG2C>(u);
                 tmem_store32(acc + 32 * un, u);                              // (kept for the codes)
@@ -398,7 +397,7 @@ __global__ void __maxnreg__(TILE_REGS) perq_col_kernel(const __grid_constant__ C
                     if (lane == 0) { N->hi[r][w] = wh; N->lo[r][w] = wl; }
                 }
             }
-            named_barrier(bar, 128);
+            if (!named_barrier_all(bar, 128, ok)) { give_up(); break; }             // (the four warps leave together)
             if (w == 0 && lane < COL_ROWS) G->notes[(it & 1u) ^ 1u].count[lane] = 0u;      // (everybody has left that tile)
             if (w == 1 && lane < R) {                                        // (much lost: the row again, in fp64)
                 const float4 h4 = *reinterpret_cast<const float4 *>(N->hi[lane]), l4 = *reinterpret_cast<const float4 *>(N->lo[lane]);

@@ -79,6 +79,16 @@ struct TileRecord {
 constexpr int TILE_RECORDS = 64;              // per batch
 constexpr uint32_t TILE_LAST = 1u << 30;
 
+// A barrier of `threads` threads at which they agree: whether it is ok for all of them.  (Each warp polls a bounded wait by itself,
+// so that one may have run out and another not: none may go on to a barrier that the others do not reach.)
+__device__ __forceinline__ bool named_barrier_all(int id, int threads, bool ok)
+{
+    uint32_t all;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %1, 0; bar.red.and.pred q, %2, %3, p; selp.u32 %0, 1, 0, q; }"
+                 : "=r"(all) : "r"((uint32_t)ok), "r"(id), "r"(threads) : "memory");
+    return all != 0u;
+}
+
 // -------------------------------------------------------------------------------------------- tensor core and TMA
 
 // Operand descriptor, low and high word: K-major, 128-byte swizzle, eight rows of 128 bytes to an atom, 1024 bytes from
@@ -619,9 +629,10 @@ struct TileLane {
     bool first, coupled, whole;      // first piece of its row; rows lie in several warps; the warp lies in one row
 };
 
-// A warp's 32 pieces of tile t.  tmem: its lanes of the accumulator; bar: the four warps' named barrier.
+// A warp's 32 pieces of tile t.  tmem: its lanes of the accumulator; bar: the four warps' named barrier.  false: another of the four
+// warps, which share rows, has given up.
 template <int LOG2B, int MODE>
-__device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLane &L, uint32_t tmem, uint32_t tile, uint32_t half, uint32_t t, TileRows *rows,
+__device__ __forceinline__ bool tile_epilogue(const TileParams &p, const TileLane &L, uint32_t tmem, uint32_t tile, uint32_t half, uint32_t t, TileRows *rows,
                                               uint32_t par, int bar, TileNotes *notes)
 {
     constexpr bool TOK = MODE == ROW_TOKEN || MODE == ROW_FP4;
@@ -702,7 +713,7 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
             } else {
                 if (L.whole) hr = warp_max_f32(hr);
                 if (L.whole ? lane == 0 : live) atomicMax(&rows->mx[par][L.ri], __float_as_uint(hr));
-                named_barrier(bar, 128);
+                if (!named_barrier_all(bar, 128, true)) { tmem_wait(ua); return false; }
                 hr = __uint_as_float(rows->mx[par][L.ri]);
                 if (L.first) rows->mx[par ^ 1u][L.ri] = 0u;           // (the other tile's word: everybody has left that tile)
             }
@@ -837,6 +848,7 @@ __device__ __forceinline__ void tile_epilogue(const TileParams &p, const TileLan
         if (codes && L.coupled) named_barrier(bar, 128);
     }
     if (codes) tile_requantise<LOG2B, MODE>(p, tmem, piece, many, aux, notes, L.w, L.ri);
+    return true;
 }
 
 // -------------------------------------------------------------------------------------------- notes
@@ -888,7 +900,7 @@ struct TileCollector {
         if (lane == 0) mbar_arrive(full + (turn & 1u) * 8);
         ++turn;
         n = 0;
-        if (turn >= 2u && !mbar_wait_fast(free + (turn & 1u) * 8, ((turn >> 1) - 1u) & 1u) && lane == 0) atomicOr(&g_perq_device_error, 8u);
+        if (turn >= 2u && !mbar_wait_fast(free + (turn & 1u) * 8, ((turn >> 1) - 1u) & 1u) && lane == 0) atomicOr(&g_perq_device_error, 1u);
     }
     // room for 32 more
     __device__ __forceinline__ void make_room() { if (n > TILE_RECORDS - 32) hand_over(0u); }
@@ -1044,7 +1056,7 @@ __global__ void __maxnreg__(TILE_REGS) perq_tile_kernel(const __grid_constant__ 
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(smem + TileSmem::slot);
     const uint32_t first = blockIdx.x, n = first < p.tiles ? (p.tiles - first + gridDim.x - 1) / gridDim.x : 0u;
     auto stage_at = [&](uint32_t s) { return base + TileSmem::stages + s * 2 * TileSmem::half; };
-    auto give_up = [&]() { if (lane == 0) atomicOr(&g_perq_device_error, 8u); };
+    auto give_up = [&]() { if (lane == 0) atomicOr(&g_perq_device_error, 1u); };
     auto load = [&](uint32_t j) {
         const uint32_t s = j % TILE_STAGES;
         mbar_expect_tx(full + s * 8, (uint32_t)p.tile_pieces * 256u);
@@ -1082,10 +1094,14 @@ __global__ void __maxnreg__(TILE_REGS) perq_tile_kernel(const __grid_constant__ 
         __syncwarp();
     } else if (warp == TILE_WGS * 4 + 1) {
         TileCollector to = {reinterpret_cast<TileBatches *>(smem + TileSmem::batches), bfull, bfree, 0u, 0, lane};
+        uint32_t loaded = min(n, (uint32_t)TILE_STAGES);       // tiles, of which the first are the other warp's
         for (uint32_t j = 0; j < n; ++j) {
             const uint32_t s = j % TILE_NOTES;
             if (!mbar_wait_fast(noted + s * 8, (j / TILE_NOTES) & 1u)) { give_up(); break; }
-            if (IN_PLACE && lane == 0 && j + TILE_STAGES < n) load(j + TILE_STAGES);      // (its four warps have left the tile)
+            if (IN_PLACE && loaded < n && j + TILE_STAGES == loaded) {                    // (its four warps have left the tile)
+                if (lane == 0) load(loaded);
+                ++loaded;
+            }
             tile_settle<LOG2B, MODE>(p, first + j * gridDim.x, notes + s, to, lane);
             __syncwarp();
             tile_clear_notes(notes + s, lane);
@@ -1096,7 +1112,7 @@ __global__ void __maxnreg__(TILE_REGS) perq_tile_kernel(const __grid_constant__ 
         to.hand_over(TILE_LAST);
         to.hand_over(TILE_LAST);
         if (IN_PLACE && lane == 0) {                           // (as above)
-            for (uint32_t k = n > TILE_STAGES ? n - TILE_STAGES : 0u; k < n; ++k) (void)mbar_wait_fast(full + (k % TILE_STAGES) * 8, (k / TILE_STAGES) & 1u);
+            for (uint32_t k = loaded > TILE_STAGES ? loaded - TILE_STAGES : 0u; k < loaded; ++k) (void)mbar_wait_fast(full + (k % TILE_STAGES) * 8, (k / TILE_STAGES) & 1u);
         }
         __syncwarp();
     } else if (warp > TILE_WGS * 4 + 1) {
@@ -1124,14 +1140,18 @@ __global__ void __maxnreg__(TILE_REGS) perq_tile_kernel(const __grid_constant__ 
         L.whole = (L.w * 32) / rp == (L.w * 32 + 31) / rp && L.w * 32 + 31 < p.tile_pieces;
         for (uint32_t j = (uint32_t)wg; j < n; j += TILE_WGS) {
             const uint32_t s = j % TILE_STAGES, b = j % TILE_ACCS, m = j % TILE_NOTES;
-            // (a wait that runs out is the same for the four warps: they leave together)
             bool ok = mbar_wait_fast(done + b * 8, (j / TILE_ACCS) & 1u);
             if (IN_PLACE) ok = mbar_wait_fast(full + s * 8, (j / TILE_STAGES) & 1u) && ok;
             if (j >= TILE_NOTES) ok = mbar_wait_fast(nfree + m * 8, ((j / TILE_NOTES) - 1u) & 1u) && ok;
-            if (!ok) { give_up(); break; }
+            if (!ok) {                                        // (warps that share rows leave together)
+                if (MODE != ROW_GROUP && MODE != ROW_MX && L.coupled) (void)named_barrier_all(1 + wg, 128, false);
+                give_up();
+                break;
+            }
             tmem_fence_after();
-            tile_epilogue<LOG2B, MODE>(p, L, tmem + b * 128 + ((uint32_t)(L.w * 32) << 16), stage_at(s), TileSmem::half, first + j * gridDim.x, rows,
-                                       (j / TILE_WGS) & 1u, 1 + wg, notes + m);
+            ok = tile_epilogue<LOG2B, MODE>(p, L, tmem + b * 128 + ((uint32_t)(L.w * 32) << 16), stage_at(s), TileSmem::half, first + j * gridDim.x, rows,
+                                            (j / TILE_WGS) & 1u, 1 + wg, notes + m);
+            if (!ok) { give_up(); break; }
             tmem_fence_before();
             __syncwarp();
             if (lane == 0) {
