@@ -4,8 +4,9 @@ reused, and the deferred scale records fill up and are served in the middle of t
 kernel's tail).  The GPU runs the whole call, the oracle a sample of rows including the first and last.
 
 The number of units a warp group sees follows from the launch arithmetic of the library, restated in
-`units_per_group` below; every case asserts that it is at least MIN_UNITS, so a later change of the grid
-cannot hollow these tests out unnoticed.
+`units_per_group` below; every case asserts that it is at least MIN_UNITS, and that the call is not one of those that the
+tile and column kernels take (dispatch.py; where they take it from some number of rows on, the case has as many units as
+there are below that), so a later change of the grid or of the dispatch cannot hollow these tests out unnoticed.
 """
 import numpy as np
 import pytest
@@ -13,6 +14,7 @@ import torch
 
 from paper_2601_22347_b200 import inputs
 
+from dispatch import kernel_of, most_rows
 from parity import compare_quantized
 
 pytestmark = pytest.mark.gpu
@@ -67,7 +69,7 @@ def rows_for(d, b, fmt, group, permuted, want=MIN_UNITS):
     T = 1024
     while units_per_group(T, d, b, fmt, group, permuted) < want:
         T += 1024
-    return T
+    return T if permuted else most_rows("other", fmt, group, d, b, T)
 
 
 def tiled(bits, T):
@@ -82,6 +84,7 @@ def check_sampled(B, oracle, name, bits, perm, b, fmt, group, seed, n_rows=48, w
     T, d = bits.shape
     upg = units_per_group(T, d, b, fmt, group, perm is not None)
     assert upg >= want, "only %d units per group" % upg
+    assert kernel_of(fmt, group, T, d, b, perm is not None) == "other"
     x = torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16)
     p = None if perm is None else torch.from_numpy(perm).cuda()
     codes, scales = B.perq_rotate_quantize(x, p, b, FMT[fmt], group)
@@ -156,14 +159,15 @@ def test_per_128_short_blocks_many_units_per_group(B, oracle, b):
     bits = base_rows("laplace", d, 14000 + b)
     bits[2, 128:640] = 0
     T = rows_for(d, b, "int4", 128, False)
-    check_sampled(B, oracle, "g128-short", tiled(bits, T), None, b, "int4", 128, 14001 + b)
+    # (from 2^24 values on these are the tile kernel's: the ring of four stages wraps, and six segments have 48 records)
+    check_sampled(B, oracle, "g128-short", tiled(bits, T), None, b, "int4", 128, 14001 + b, want=6)
 
 
 # ------------------------------------------------------------------ per-token INT4 / FP4: the 32-record flush
 
-@pytest.mark.parametrize("fmt", ["int4", "fp4"])
-@pytest.mark.parametrize("d,b,kind", [(4096, 32, "laplace"), (1024, 16, "laplace"), (2048, 128, "gauss"),
-                                      (14336, 64, "laplace")])
+@pytest.mark.parametrize("fmt,d,b,kind", [("int4", 4096, 32, "laplace"), ("fp4", 4096, 128, "laplace"), ("int4", 1024, 16, "laplace"),
+                                          ("int4", 2048, 128, "gauss"), ("fp4", 2048, 128, "gauss"), ("int4", 11264, 128, "laplace"),
+                                          ("fp4", 11264, 128, "laplace")])
 def test_per_token_many_rows_per_group(B, oracle, d, b, fmt, kind):
     bits = base_rows(kind, d, 15000 + d + b)
     bits[4] = 0
@@ -177,7 +181,8 @@ def test_full_vector_many_rows_per_group(B, oracle, fmt, group):
     bits = base_rows("laplace", d, 16000)
     bits[6] = 0
     T = rows_for(d, d, fmt, group, False)
-    check_sampled(B, oracle, "full-long", tiled(bits, T), None, d, fmt, group, 16001, n_rows=16)
+    # (INT4: the column kernel's from 8192 rows on)
+    check_sampled(B, oracle, "full-long", tiled(bits, T), None, d, fmt, group, 16001, n_rows=16, want=10 if fmt == "int4" else MIN_UNITS)
 
 
 # ------------------------------------------------------------------ the workloads at their stated sizes

@@ -1,10 +1,11 @@
-"""Parity of the row kernels with the oracle on calls in which every CTA serves at least six rows: the ring of two stages
+"""Parity of the row kernels with the oracle on calls in which every CTA serves at least five or six rows: the ring of two stages
 is refilled (a refilled stage is read from a CTA's third row on), the stage parities flip, the lists and reduction words
 of one row are those of the next.  The GPU runs the whole call, the oracle rows of every sixth of it.
 
 A CTA's rows are blockIdx.x, blockIdx.x + grid, ...: a grid of at most 148 SMs times the rows that an SM's warps hold at
 a time (ROW_SM_WARPS and ROW64_SM_WARPS of perq_row.cuh, a warp per 1024 channels or more).  Every case asserts the
-six rows from that bound, so a change of the grid does not hollow the tests out unnoticed.
+rows from that bound, and that the call is not the column kernel's, so a change of the grid or the dispatch does not hollow
+the tests out unnoticed.
 """
 import numpy as np
 import pytest
@@ -12,6 +13,7 @@ import torch
 
 from paper_2601_22347_b200 import inputs
 
+from dispatch import kernel_of
 from parity import compare_quantized
 
 pytestmark = pytest.mark.gpu
@@ -48,8 +50,11 @@ def rows_in_flight(d, fmt, group, b):
                                       (2048, 2048, False), (1152, 128, True), (3072, 1024, True)])
 def test_many_rows_per_cta(B, oracle, d, b, perm, fmt, group):
     flight = rows_in_flight(d, fmt, group, b)
-    T = MIN_ROWS * flight + 3
-    assert T // flight >= MIN_ROWS
+    rows_each = MIN_ROWS
+    if not perm and kernel_of(fmt, group, MIN_ROWS * flight + 3, d, b) != "other":
+        rows_each -= 1                                        # (more rows are the column kernel's)
+    T = rows_each * flight + 3
+    assert T // flight >= rows_each and kernel_of(fmt, group, T, d, b, perm) == "other"
     base = inputs.laplace_outliers(192, d, max(1, d // 2048), 100.0, 20000 + d + b)[0]
     base[5] = 0
     idx = (np.arange(T) + np.arange(T) // 192) % 192         # a base row meets different CTAs and stages
@@ -58,7 +63,7 @@ def test_many_rows_per_cta(B, oracle, d, b, perm, fmt, group):
     codes, scales = B.perq_rotate_quantize(x, None if p is None else torch.from_numpy(p).cuda(), b, FMT[fmt], group)
     torch.cuda.synchronize()
     rng = np.random.default_rng(20002)
-    rows = np.unique(np.r_[0, T - 1, (np.arange(MIN_ROWS)[:, None] * flight + rng.integers(0, flight, (MIN_ROWS, 3))).ravel()])
+    rows = np.unique(np.r_[0, T - 1, (np.arange(rows_each)[:, None] * flight + rng.integers(0, flight, (rows_each, 3))).ravel()])
     at = torch.from_numpy(rows).cuda()
     ora = oracle.rotate_quantize(base[idx[rows]], p, b, FMT[fmt], group, want_pre=True)
     compare_quantized(fmt, codes[at].cpu().numpy(), scales[at].cpu().numpy(), ora)

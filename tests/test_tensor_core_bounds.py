@@ -6,6 +6,7 @@ import torch
 
 from paper_2601_22347_b200 import inputs
 
+from dispatch import kernel_of
 from mma_rows import hadamard, chained_contraction, hidden_in_every_piece, hidden_maximum, hidden_side, hidden_step, outputs, to_bf16
 from parity import compare_quantized
 
@@ -63,8 +64,10 @@ def block_rows(d, b, seed):
 
 
 def run(B, oracle, base, T, b, fmt, group):
-    """T rows made of the base rows, each of which is compared, and the same bytes at every repetition."""
+    """T rows made of the base rows, each of which is compared, and the same bytes at every repetition; in the kernels that
+    rotate by chained steps."""
     n = len(base)
+    assert kernel_of(fmt, group, T, base.shape[1], b) == ("column" if b > 128 else "tile")
     idx = (np.arange(T) + np.arange(T) // n) % n
     idx_t = torch.from_numpy(idx).cuda()
     x = torch.from_numpy(base.view(np.int16)).cuda()[idx_t].view(torch.bfloat16)
@@ -186,3 +189,56 @@ def test_tile_err_covers_the_model():
             worst = max(worst, off.max() * 2 ** 24)
         assert worst < err
         assert worst > (3 if b == 16 else 6 if b == 32 else 24 if b == 64 else 56)
+
+
+# ------------------------------------------------------------------ the other attacks on the bounds, at these kernels' sizes
+
+LARGE = [(1152, 16 * 2 ** 20 // 1152 + 3, b, fmt, group) for b in (16, 32, 64, 128) for fmt, group in (("int4", 0), ("int4", 128), ("fp4", 0), ("mxfp4", 32))]
+LARGE += [(d, T, d, fmt, 0) for d, T in ((4096, 8195), (2048, 16389)) for fmt in ("int4", "fp4", "int4_asym")]
+
+
+def flat_spectrum_rows(d, b, seed):
+    """Signs whose rotation is as flat as it can be, times mantissas in [1, 2): the partial sums are as large as the outputs."""
+    k, s = np.arange(b), 0
+    for i in range(int(np.log2(b)) - 1):
+        s = s ^ (k >> i) & (k >> (i + 1)) & 1
+    rng = np.random.default_rng(seed)
+    x = (1.0 + rng.integers(0, 128, (48, d // b, b)) / 128.0) * (1.0 - 2.0 * s)
+    x *= np.exp2(rng.integers(-3, 4, (48, d // b, 1))) * rng.choice([-1.0, 1.0], (48, d // b, 1))
+    x = x.reshape(48, d)
+    x[::7] = to_bf16(rng.standard_normal((7, d)))
+    return bits(x)
+
+
+def small_and_shifted_rows(d, b, seed):
+    """Rows at the lower end of the range (largest output 2^-119 and more), and rows far from symmetric (zero points of some 100)."""
+    rng = np.random.default_rng(seed)
+    x = rng.standard_normal((48, d))
+    x[1::3, :: max(1, d // 8)] *= 100.0
+    x[2::3] += 40.0
+    x[::3] *= np.exp2(-rng.integers(112, 118, (16, 1)))
+    return bits(to_bf16(x))
+
+
+def cancelling_rows(d, b, seed):
+    """Blocks of four runs 3v, 4v, 5v, 4v: a quarter of the outputs is zero exactly, and fp32 leaves noise there."""
+    rng = np.random.default_rng(seed)
+    shape = (48, d // b, 1, b // 4)
+    v = rng.integers(1, 16, shape) * np.exp2(rng.integers(-14, 15, shape)) * rng.choice([-1.0, 1.0], shape)
+    return bits((v * np.array([3.0, 4.0, 5.0, 4.0])[None, None, :, None]).reshape(48, d))
+
+
+def wide_rows(d, b, seed):
+    """Inputs over 40 binades, and one large input with tiny ones of one sign."""
+    rng = np.random.default_rng(seed)
+    x = rng.standard_normal((48, d)) * np.exp2(-rng.integers(0, 40, (48, d)))
+    x[::2] = np.abs(rng.standard_normal((24, d))) * np.exp2(-rng.integers(16, 28, (24, 1)))
+    x[np.arange(0, 48, 2), rng.integers(0, d, 24)] = 1.5
+    return bits(to_bf16(x))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("make", [flat_spectrum_rows, small_and_shifted_rows, cancelling_rows, wide_rows])
+@pytest.mark.parametrize("d,T,b,fmt,group", LARGE)
+def test_large_calls(B, oracle, d, T, b, fmt, group, make):
+    run(B, oracle, make(d, b, 46000 + b), T, b, fmt, group)

@@ -3,8 +3,9 @@ every CTA serves several tiles (ring stages, accumulators and note slots are use
 runs the whole call, the oracle the base rows it is made of; every repetition of a base row has to give the same bytes.
 
 The base rows hold what each rule of these kernels meets: rows with outliers, rows without, zeros, one nonzero (every
-output of its block ties), small integers (true rounding ties), a row of them at the lowest and one at the highest
-exponents of bf16 that the formats take.
+output of its block ties), small integers (true rounding ties), a row near the lower end of the range that the formats
+take and one near the upper end (the ends themselves: test_tensor_core_bounds.py).  Every case asserts that the call is the
+kernel's.
 """
 import numpy as np
 import pytest
@@ -12,6 +13,7 @@ import torch
 
 from paper_2601_22347_b200 import inputs
 
+from dispatch import kernel_of
 from parity import compare_quantized
 
 pytestmark = pytest.mark.gpu
@@ -50,8 +52,8 @@ def base_rows(d, seed):
     x[9] = bf16(rng.integers(-3, 4, d))                                        # small integers
     x[10] = bf16(np.where(rng.random(d) < 8.0 / d, rng.integers(1, 9, d), 0))  # a few of them
     x[11] = bf16(np.ones(d))
-    x[12] = bf16(rng.standard_normal(d) * 2.0 ** -80)
-    x[13] = bf16(rng.standard_normal(d) * 2.0 ** 100)
+    x[12] = bf16(rng.standard_normal(d) * 2.0 ** -116)
+    x[13] = bf16(rng.standard_normal(d) * 2.0 ** 116)
     x[14, d // 2:] = 0
     return x
 
@@ -69,6 +71,7 @@ def flat_rows(d, seed):
 
 
 def check(B, oracle, T, d, b, fmt, group, seed, offset=0, make=base_rows):
+    assert kernel_of(fmt, group, T, d, b) == ("column" if b > 128 else "tile")
     base = make(d, seed)
     idx = (np.arange(T) + np.arange(T) // BASE) % BASE           # a base row meets different CTAs, warps and stages
     idx_t = torch.from_numpy(idx).cuda()
@@ -88,34 +91,53 @@ def check(B, oracle, T, d, b, fmt, group, seed, offset=0, make=base_rows):
     compare_quantized(fmt, codes[at].cpu().numpy(), scales[at].cpu().numpy(), ora)
 
 
-@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0), ("int4_asym", 0)])
+def rows_of(T, b, fmt, group):
+    """Blocks of 128 with a scale per token are the kernel's from four times as many rows on."""
+    return 4 * T + 1 if b == 128 and group == 0 else T
+
+
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0)])
 @pytest.mark.parametrize("b", [16, 32, 64, 128])
 def test_ragged_widths(B, oracle, b, fmt, group):
     # pieces per row: 6 (21 rows a tile), 76 and 111 (one), 9 (14, 126 of 128 lanes)
     for d, T in ((768, 6001), (9728, 691), (14208, 433), (1152, 5003)):
-        check(B, oracle, T, d, b, fmt, group, 30000 + d + b)
+        check(B, oracle, rows_of(T, b, fmt, group), d, b, fmt, group, 30000 + d + b)
 
 
-@pytest.mark.parametrize("fmt,group,b", [("int4", 0, 64), ("int4", 0, 128), ("int4", 128, 16), ("int4", 128, 128), ("mxfp4", 32, 32),
-                                         ("mxfp4", 32, 64), ("mxfp4", 32, 128), ("fp4", 0, 16), ("fp4", 0, 128), ("int4_asym", 0, 32),
-                                         ("int4_asym", 0, 128)])
-@pytest.mark.parametrize("d", [4096, 8192, 14336])
+@pytest.mark.parametrize("d,fmt,group,b", [(d, "fp4", 0, b) for d in (512, 2048) for b in (16, 32, 64)] + [(512, "fp4", 0, 128)] +
+                         [(512, "int4", 0, b) for b in (16, 32, 64, 128)])
+def test_rows_inside_a_warp(B, oracle, d, fmt, group, b):
+    """4 and 16 pieces per row: rows meet by shuffles, without a barrier, and settle by warps (512: all 32 rows of a tile)."""
+    for make in (base_rows, flat_rows):
+        check(B, oracle, rows_of(8195, b, fmt, group), d, b, fmt, group, 36000 + d + b, make=make)
+
+
+@pytest.mark.parametrize("d,fmt,group,b", [(d, f, g, b) for d in (4096, 8192, 14336)
+                                           for f, g, b in (("int4", 0, 64), ("int4", 128, 16), ("int4", 128, 128), ("mxfp4", 32, 32),
+                                                           ("mxfp4", 32, 64), ("fp4", 0, 16), ("fp4", 0, 64))] +
+                         [(14336, "int4", 0, 128), (14336, "fp4", 0, 128)])
 def test_whole_segments(B, oracle, d, fmt, group, b):
-    check(B, oracle, 17 * 2 ** 20 // d, d, b, fmt, group, 31000 + d + b, offset=16)
+    check(B, oracle, (25 if b == 128 else 17) * 2 ** 20 // d, d, b, fmt, group, 31000 + d + b, offset=16)
 
 
 @pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
-@pytest.mark.parametrize("d,T", [(4096, 4099), (2048, 16389)])
+@pytest.mark.parametrize("d,T", [(4096, 8195), (2048, 16389)])
 def test_whole_row_rotations(B, oracle, d, T, fmt):
     check(B, oracle, T, d, d, fmt, 0, 32000 + d)
 
 
-@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0), ("int4_asym", 0)])
+@pytest.mark.parametrize("fmt,group", [("int4", 0), ("int4", 128), ("mxfp4", 32), ("fp4", 0)])
 @pytest.mark.parametrize("d,T", [(1536, 3001), (9728, 691), (4096, 4096)])
 def test_flat_rows(B, oracle, d, T, fmt, group):
     # nearly every piece has more candidates or ties than are noted: lanes settle them, with exact fp32 outputs and without
-    for b in (16, 128):
-        check(B, oracle, T, d, b, fmt, group, 33000 + d + b, make=flat_rows)
+    for b in (16, 128) if d % 1024 else {"int4": (64,) if group == 0 else (16, 64), "mxfp4": (32, 64), "fp4": (16, 64)}[fmt]:
+        check(B, oracle, rows_of(T, b, fmt, group), d, b, fmt, group, 33000 + d + b, make=flat_rows)
+
+
+@pytest.mark.parametrize("fmt", ["int4", "fp4", "int4_asym"])
+@pytest.mark.parametrize("d,T", [(4096, 8195), (2048, 16389)])
+def test_flat_whole_rows(B, oracle, d, T, fmt):
+    check(B, oracle, T, d, d, fmt, 0, 33500 + d, make=flat_rows)
 
 
 def zero_blocks(d, seed):
