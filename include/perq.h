@@ -120,8 +120,8 @@ typedef enum {
  * Range limits: a token whose largest |y| lies below about 2^-120 (every input subnormal or nearly so) gets
  * the exact scale but all-zero INT4/FP4 codes from the tensor-core kernels, because the fp32 reciprocal of
  * such a scale overflows; the definition would give +-7 at the maximum.  At the other end sqrt(b) |y| has to stay
- * below 2^126 (d % 1024 == 0 with b <= 128, or unpermuted blocks of 256 to 1024: above it the codes come out 0) or
- * below 2^128 (all other shapes).  A scale range or MX group that is part of a Hadamard block and whose outputs all
+ * below 2^126 (d % 1024 == 0 with b <= 128, or unpermuted blocks of 256 to 1024: above it the codes come out 0, except in
+ * large unpermuted calls, whose kernel goes up to 2^128) or below 2^128 (all other shapes).  A scale range or MX group that is part of a Hadamard block and whose outputs all
  * cancel to zero in fp32 (below about 2^-24 of the block's largest) gets scale 0.
  */
 int perq_rotate_quantize(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t b,

@@ -5,7 +5,7 @@
 // columns of the result.  A lane of tensor memory then holds output i of every piece of a row in adjacent columns, so
 // that the remaining stages, over the pieces of the row, are butterflies on the 32 values that one load brings -- no trip
 // through shared memory and no shuffle.  The outputs go back to tensor memory until the row's maximum is known (forming
-// them again took 96 instructions of 880 per 1024 elements).  32 x 32 codes of a warp change places in ten shuffles.
+// them again took 96 instructions per 1024 elements).  32 x 32 codes of a warp change places in ten shuffles.
 //
 // The row kernel, which makes a trip through an fp32 tile, spends 1160 warp instructions on 1024 elements and five
 // barriers of a row's warps on a row; here two barriers serve four rows.
@@ -15,7 +15,7 @@
 // on inputs of 4 to 26 binades).  Beside a large input tiny ones can be lost in every piece, to the same side: a bound that
 // covers any inputs is 900 * 2^-24 of the row's largest output, and with it a row has six doubtful codes.  But only inputs
 // 2^16 below their piece's l1 norm can be lost, and few rows have many: four warps count them (col_lost) while the tile waits
-// for its group.  (16384 x 4096, INT4: 98 us; 129 with a bound of 208 * 2^-24 for all rows; 85 with one of 12 that some
+// for its group, 82 of 863 warp instructions on 1024 elements.  (16384 x 4096, INT4: 95 to 98 us; 129 with a bound of 208 * 2^-24 for all rows; 85 with one of 12 that some
 // rows exceed.)
 //
 // Exact maxima and doubtful codes: sums over the whole row.  They are listed while the rows are quantised, and then a warp

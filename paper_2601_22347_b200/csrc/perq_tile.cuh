@@ -9,7 +9,7 @@
 // What follows the rotation has a piece per lane: a warp reads 32 columns of its 32 pieces with one load, so that the
 // maxima of MX groups and of ranges of 128, the rounding, the packing of 32 codes and the test for doubtful elements
 // are all lane-local, without a shuffle; per-token scales meet once per tile.  The kernels that rotate in registers (a
-// lane holds four adjacent outputs of eight chunks) spend 270 to 750 warp instructions on 1024 elements, this one 150 to 400.
+// lane holds four adjacent outputs of eight chunks) spend 270 to 750 warp instructions on 1024 elements, this one 220 to 390.
 // 65536 x 4096, b = 32, MXFP4: 110 us (floor 105; 135 in registers).  What bounds calls of ordinary size is what they pay
 // once: 5 to 8 us of set-up, first load, last tile and last batch of records.
 //
