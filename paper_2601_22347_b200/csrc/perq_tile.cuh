@@ -755,7 +755,8 @@ __device__ __forceinline__ bool tile_epilogue(const TileParams &p, const TileLan
                     Eb = e8 - (LOG2B - 1) / 2 - 2 + ((bits & 0x7fffffu) >= 0x3504f4u ? 1 : 0);
                 }
                 const float tol = 2.0f * err * ref + gm * 4.8e-7f;
-                const bool near = live && gm > 0.0f && (dist <= tol || e8 == 0);
+                // (a group inside a longer block can be zero in fp32 and not in truth)
+                const bool near = live && (LOG2B <= 5 ? gm : ref) > 0.0f && (dist <= tol || e8 == 0);
                 bool zero = !(gm > 0.0f);
                 if (__any_sync(0xffffffffu, near)) {          // rare: the exact maximum of the group
                     uint32_t want = near ? row_reach(u, gm - tol) : 0u;

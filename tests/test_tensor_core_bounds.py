@@ -242,3 +242,23 @@ def wide_rows(d, b, seed):
 @pytest.mark.parametrize("d,T,b,fmt,group", LARGE)
 def test_large_calls(B, oracle, d, T, b, fmt, group, make):
     run(B, oracle, make(d, b, 46000 + b), T, b, fmt, group)
+
+
+def vanishing_groups(d, b, seed):
+    """Two large inputs that cancel in half of a block's outputs, and before the second one tiny inputs that fp32 loses
+    beside the first: whole MX groups that are zero in fp32 and not in truth."""
+    rng, k, h = np.random.default_rng(seed), np.arange(b), hadamard(b)
+    x = np.zeros((48, d // b, b))
+    for i in range(48):
+        for j in range(d // b):
+            tiny = (k > 0) & (k < b // 2) & (rng.random(b) < (1.0 if i % 3 else 0.2))
+            x[i, j] = np.where(tiny, h[int(rng.integers(b))] * 0.9921875 * 2.0 ** -25, 0.0)
+            x[i, j, 0] = x[i, j, b // 2] = 1.0
+            x[i, j] *= 2.0 ** int(rng.integers(-20, 20))
+    return bits(x.reshape(48, d))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("b", [64, 128])
+def test_groups_that_vanish_in_fp32(B, oracle, b):
+    run(B, oracle, vanishing_groups(1152, b, 47000 + b), 16 * 2 ** 20 // 1152 + 3, b, "mxfp4", 32)
