@@ -20,7 +20,8 @@
 // largest term and P the sum, a step loses 8 T + 2 P at most, in 2^-24 (the first, of 15 terms, 7.5 T + 2 P).  In units of the
 // block's largest output T is at most 1 for an input (Parseval) and P, after m steps, what the Walsh coefficients of the first
 // 16 m inputs' indicator add up to: 1, 1, 1.5, 1, 1.5, 1.5, 1.75, 1.  In all 9.5, 19.5, 44.5 and 102 for b = 16, 32, 64, 128
-// (tile_err).  Rows that lose 64 of the 102 are among the tests; gaussian and heavy-tailed rows lose 6 at most.
+// (tile_err).  Rows that lose 64 of the 102 are among the tests; gaussian and heavy-tailed ones lose 3, with one
+// input 1000 times the others 4, 20000 times 12 (4000 pieces each, by the model).
 // The warps that quantise only note these places (candidates for a row's maximum, doubtful elements).  One warp turns
 // the notes of a tile into records, two others settle records in batches, one per lane, from the inputs in global
 // memory: they store the rows' scales and mend codes.  With the sums inside the quantising warps a tile of token rows took
