@@ -74,13 +74,7 @@ __device__ __forceinline__ void col_rotate(uint32_t tmem, uint32_t tile, uint32_
         tile_mma(tmem, h + (s >> 2) * (ColSmem::half / 16) + 2 * (s & 3), x + (s >> 2) * (ColSmem::half / 16) + 2 * (s & 3), tile_idesc(128), s > 0);
 }
 
-// Bound of what the contraction loses in any output of piece r of a tile, by one lane.  With g = 2^(e-23) and 2^(e+1) above
-// the sum of the piece's magnitudes, inputs of 2^7 g and more are multiples of g, every term and sum is below 2^(e+1), and
-// all grids that a step cuts at divide g.  A step without smaller inputs only moves the accumulator's part below g, and only
-// where its grid is coarser than any before: between two steps that have some, by less than g in all.  A step with n of
-// them cuts these and the accumulator, by less than g / 4 each.
-// guess: biased e of the lane's piece of the previous tile, plus one.  Inputs are counted against it while they are added
-// up, zeros as well; again where it was too low, or there are many.
+// Inputs 8 c .. 8 c + 7 of a piece.
 __device__ __forceinline__ void col_words(uint32_t tile, uint32_t r, uint32_t c, uint32_t (&w)[4])
 {
     asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(tile + tile_at(ColSmem::half, r, 8u * c)));
@@ -114,6 +108,13 @@ __device__ __noinline__ float col_count(uint32_t tile, uint32_t r, uint32_t e)
     }
     return (float)(n / 16u);
 }
+// Bound of what the contraction loses in any output of piece r of a tile, by one lane.  With g = 2^(e-23) and 2^(e+1) above
+// the sum of the piece's magnitudes, inputs of 2^7 g and more are multiples of g, every term and sum is below 2^(e+1), and
+// all grids that a step cuts at divide g.  A step without smaller inputs only moves the accumulator's part below g, and only
+// where its grid is coarser than any before: between two steps that have some, by less than g in all.  A step with n of
+// them cuts these and the accumulator, by less than g / 4 each.
+// guess: biased e of the lane's piece of the previous tile, plus one.  Inputs are counted against it while they are added
+// up, zeros as well; again where it was too low, or there are many.
 __device__ __forceinline__ float col_lost(uint32_t tile, uint32_t r, uint32_t &guess)
 {
     constexpr float MANY = 12.0f;

@@ -115,7 +115,10 @@ def test_rows_inside_a_warp(B, oracle, d, fmt, group, b):
 @pytest.mark.parametrize("d,fmt,group,b", [(d, f, g, b) for d in (4096, 8192, 14336)
                                            for f, g, b in (("int4", 0, 64), ("int4", 128, 16), ("int4", 128, 128), ("mxfp4", 32, 32),
                                                            ("mxfp4", 32, 64), ("fp4", 0, 16), ("fp4", 0, 64))] +
-                         [(14336, "int4", 0, 128), (14336, "fp4", 0, 128)])
+                         [(14336, "int4", 0, 128), (14336, "fp4", 0, 128)] +
+                         # 128, 24 and 48 pieces per row: one row, five and two of a tile
+                         [(16384, "int4", 0, 64), (16384, "fp4", 0, 16), (3072, "int4", 0, 64), (3072, "fp4", 0, 32), (6144, "fp4", 0, 64),
+                          (1024, "int4", 128, 64), (32768, "mxfp4", 32, 64)])
 def test_whole_segments(B, oracle, d, fmt, group, b):
     check(B, oracle, (25 if b == 128 else 17) * 2 ** 20 // d, d, b, fmt, group, 31000 + d + b, offset=16)
 
