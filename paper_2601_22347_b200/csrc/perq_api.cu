@@ -27,6 +27,7 @@
 #include "perq_row.cuh"
 #include "perq_tile.cuh"
 #include "perq_col.cuh"
+#include "perq_perm.cuh"
 
 namespace {
 
@@ -608,6 +609,8 @@ int launch_any(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t
     if (is_pow2(b)) {
         int rc = b == d && b > 128 ? try_launch_col(x, perm, T, d, b, fmt, g, out_codes, out_scales, st)
                                    : try_launch_tile(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
+        if (rc >= 0) return rc;
+        rc = try_launch_perm(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
         if (rc >= 0) return rc;
         rc = try_launch_fast(x, perm, T, d, b, fmt, g, out_codes, out_scales, st);
         if (rc >= 0) return rc;

@@ -147,6 +147,81 @@ int try_launch_tile(const void *x, const int32_t *perm, int64_t T, int32_t d, in
     }
 }
 
+// x as boxes of eight rows by 512 channels: 64 channels, the rows, blocks of 64 channels.
+bool perm_tensor_map(CUtensorMap *map, const void *x, uint64_t T, int d)
+{
+    TensorMapEncode encode = tensor_map_encode();
+    if (encode == nullptr) return false;
+    const cuuint64_t dims[3] = {64, T, (cuuint64_t)d / 64}, strides[2] = {(cuuint64_t)d * 2, 128};
+    const cuuint32_t box[3] = {64, perq::PERM_ROWS, perq::PERM_BOX / 64}, step[3] = {1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(x), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int MODE>
+int launch_perm_b(int log2b, const CUtensorMap &map, const perq::PermParams &p, int grid, size_t smem, cudaStream_t st)
+{
+    constexpr int threads = perq::PERM_THREADS;
+    switch (log2b) {
+    case 4: return launch_with_map(perq::perq_perm_kernel<4, MODE>, grid, threads, smem, st, map, p);
+    case 5: return launch_with_map(perq::perq_perm_kernel<5, MODE>, grid, threads, smem, st, map, p);
+    case 6: return launch_with_map(perq::perq_perm_kernel<6, MODE>, grid, threads, smem, st, map, p);
+    default: return launch_with_map(perq::perq_perm_kernel<7, MODE>, grid, threads, smem, st, map, p);
+    }
+}
+
+// Where the kernel for many permuted rows is the better one: widths that are no multiple of 1024, whose permuted rows were the row kernel's
+// (us, others / this one; gaussian and, after a comma, swiglu values).  A set of eight rows to every second SM at least; fewer rows
+// at 9728 are better spread by the row kernel (148 rows, MXFP4 b = 32: 7.7 / 10.3; 300 rows, b = 128: 13.5 / 14.5).
+//   MXFP4, 9728: b = 16, 592 rows 24 / 17, 8192 rows 240 / 103; b = 32, 1200 rows 44 / 27, 33.5 / 23.1, 8192 rows 176 / 82; b = 128, 592 rows 20.4 / 18.0,
+//     8192 rows 195 / 121; 4736: b = 32, 592 rows 11.0 / 7.8, 2368 rows 25.5 / 17.4; 640 and 1152: 592 rows 6.1 .. 8.4 / 5.9 .. 6.5
+//   INT4 per 128, 9728: b = 16, 592 rows 22.9 / 15.5; b = 128, 1200 rows 50.7 / 27.6, 8192 rows 282 / 105; 1152: b = 128, 8192 rows 40 / 25
+//   2048 x 9728, one nonzero, integers, few nonzeros, equal values, zeros: 0.17 .. 0.95 of the row kernel's time (b = 128, MXFP4, equal values: 1.06)
+// Widths of 1024 k stay with the group kernel, which has no ragged segments: 4096 x 8192, MXFP4, b = 32 37.6 / 41.8; per 128, b = 128 48.0 / 49.9.
+// (Here a set's rows are interleaved while no unit is being rotated: a third of the time at 8192 channels, whose interleaved rows fill
+// half of the shared memory.)
+bool perm_is_better(int d, long long T) { return d % perq::SEG_ELEMS != 0 && T >= 592; }
+
+// Returns -1 if that kernel does not take the call.
+int try_launch_perm(const void *x, const int32_t *perm, int64_t T, int32_t d, int32_t b, int32_t fmt, int g, void *out_codes, void *out_scales,
+                    cudaStream_t st)
+{
+    if (perm == nullptr || d % 128 != 0 || !is_pow2(b) || b < 16 || b > 128) return -1;
+    int mode;
+    if (fmt == PERQ_FMT_MXFP4) mode = perq::ROW_MX;
+    else if (fmt == PERQ_FMT_INT4 && g == 128) mode = perq::ROW_GROUP;
+    else return -1;
+    if (T >= (1ll << 31) - perq::PERM_ROWS || !perm_is_better(d, T)) return -1;
+    const int boxes = (d + perq::PERM_BOX - 1) / perq::PERM_BOX;
+    const perq::PermLayout lay(d, boxes, (uint32_t)kMaxSmem);
+    if (lay.stages < 4) return -1;
+    perq::PermParams p;
+    std::memset(&p, 0, sizeof(p));
+    p.perm = perm;
+    p.out_codes = static_cast<uint8_t *>(out_codes);
+    p.out_scales = out_scales;
+    p.T = (uint32_t)T;
+    p.sets = (uint32_t)((T + perq::PERM_ROWS - 1) / perq::PERM_ROWS);
+    p.d = d;
+    p.units = d / 128;
+    p.boxes = boxes;
+    p.stages = lay.stages;
+    p.off_ring = lay.ring;
+    p.off_tab = lay.tab;
+    p.off_bars = lay.bars;
+    p.sqrt_b = std::sqrt((double)b);
+    p.inv_7_sqrt_b = 1.0 / (7.0 * p.sqrt_b);
+    const int sms = sm_count();
+    if (sms <= 0) return PERQ_ERR_CUDA;
+    CUtensorMap map;
+    if (!perm_tensor_map(&map, x, (uint64_t)T, d)) return -1;
+    const int tail = (int)(p.sets % (uint32_t)sms);
+    p.parts = tail > 0 ? std::min(sms / tail, (p.units + perq::PERM_WARPS - 1) / perq::PERM_WARPS) : 1;
+    const int grid = p.sets >= (uint32_t)sms ? sms : tail * p.parts;
+    return mode == perq::ROW_MX ? launch_perm_b<perq::ROW_MX>(ilog2(b), map, p, grid, lay.total, st)
+                                : launch_perm_b<perq::ROW_GROUP>(ilog2(b), map, p, grid, lay.total, st);
+}
+
 // Where the column kernel is better than the row kernel (us, CUDA graphs, row / column, laplace and swiglu values): 4096
 // channels, 2048 rows 18.4 / 21.9, 18.6 / 21.4, 4096 rows 31.3 / 30.0, 30.9 / 29.8, 8192 rows 58.5 / 53.0, 58.9 / 53.7, 16384 rows 113 / 98,
 // 113 / 99; FP4 62.0 / 56.1 and 117 / 99; asymmetric, 4096 rows 51 / 40, 16384 rows 191 / 134.  2048 channels, 8192 rows 30.8 / 31.6, 16384
