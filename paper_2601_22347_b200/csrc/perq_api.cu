@@ -1024,12 +1024,20 @@ int perq_massdiff_perm_device(const float *chan_abs_sum, int32_t d, int32_t b, i
     p.d = d;
     p.b = b;
     const int n = d / b;
-    const perq::MdSmem lay(n);
-    if (int rc = allow_smem(perq::perq_massdiff_greedy_kernel, lay.total)) return rc;
     const int ctas = (d + perq::MD_RANK_CHANNELS - 1) / perq::MD_RANK_CHANNELS;
-    const int threads = std::min(perq::MD_MAX_THREADS, (n + 31) / 32 * 64);      // two threads per list entry up to 512 blocks
+    // up to 256 blocks (8192 channels, b = 32: 103 us, the other one 175; 1024 .. 14336 channels in 16 .. 256 blocks: 0.5 .. 0.7 of its time;
+    // 448 and 512 blocks would gain on real statistics, 313 to 222 and 178 to 124, and lose on masses 1 / rank, 445 to 556)
+    const bool sorts = n <= perq::MD_SORT_BLOCKS;
+    void (*greedy)(perq::MassdiffParams) = !sorts  ? perq::perq_massdiff_greedy_kernel
+                                           : n <= 32 ? perq::perq_massdiff_sort_kernel<1>
+                                           : n <= 64 ? perq::perq_massdiff_sort_kernel<2>
+                                           : n <= 128 ? perq::perq_massdiff_sort_kernel<4>
+                                                      : perq::perq_massdiff_sort_kernel<8>;
+    const size_t smem = sorts ? perq::MdSortSmem(d).total : perq::MdSmem(n).total;
+    if (int rc = allow_smem(greedy, smem)) return rc;
+    const int threads = sorts ? perq::MD_SORT_THREADS : std::min(perq::MD_MAX_THREADS, (n + 31) / 32 * 64);      // (two threads per list entry up to 512 blocks)
     if (launch_overlapped(perq::perq_massdiff_rank_kernel, ctas, perq::MD_RANK_THREADS, 0, st, p) != cudaSuccess ||
-        launch_overlapped(perq::perq_massdiff_greedy_kernel, 1, threads, lay.total, st, p) != cudaSuccess) {
+        launch_overlapped(greedy, 1, threads, smem, st, p) != cudaSuccess) {
         (void)cudaGetLastError();
         return PERQ_ERR_CUDA;
     }

@@ -14,7 +14,8 @@
 //   at once, and its new sums are merged into the list.
 //
 // Sums differ by about one channel mass, so a batch serves most of the blocks: 66 batches for 8192 channels of a
-// real statistic in 256 blocks, 176 us (one channel at a time, one warp scanning all running sums: 2316 us).
+// real statistic in 256 blocks, 176 us (one channel at a time, one warp scanning all running sums: 2316 us).  Up to 256
+// blocks the batches are formed by another kernel (below).
 // Masses that fall steeply make small batches, and few blocks small ones anyway.  Channels are then served one by one by
 // one warp: 32 channels reach no more than the first 32 entries of the list, so a lane holds one entry in registers and a
 // channel costs three warp reductions; afterwards the entries are merged back like a batch.  (By all threads, a barrier
@@ -143,7 +144,7 @@ __device__ __forceinline__ bool md_less(unsigned long long s, int i, unsigned lo
 }
 
 // A batch costs as much as 16 channels one by one.  Below 6 channels it is followed by 32 of those, by two and four
-// times 32 if the next batches are small again; up to 16 blocks all channels go one by one.  (Whenever 32 blocks or
+// times 32 if the next batches are small again; up to 16 blocks (in the kernel below) all channels go one by one.  (Whenever 32 blocks or
 // fewer are open: 244 against 176 us for the 8192 channels above, whose last blocks fill in large batches.)
 constexpr int MD_FEW_BLOCKS = 16;
 constexpr int MD_SERIAL_K = 6;
@@ -204,14 +205,14 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             __syncthreads();
         }
         if (m == 1 || mass[s - w0] == 0.0f) break;          // one block or only zero masses are left: below
-        const bool one_by_one = n <= MD_FEW_BLOCKS || serial > 0;
+        const bool one_by_one = serial > 0;
         unsigned long long M;                     // the smallest new sum
         int M_id = MD_ID_MASK, K, q, steps, given;
         if (one_by_one) {
-            // ---- 32 channels (few blocks: the window) one by one: lane j of warp 0 has entry j
-            if (serial > 0) --serial;
+            // ---- 32 channels one by one: lane j of warp 0 has entry j
+            --serial;
             if (warp == 0) {
-                const int room = n <= MD_FEW_BLOCKS ? w1 - s : min(32, w1 - s);
+                const int room = min(32, w1 - s);
                 unsigned long long v = lane < m ? sum[lane] : ~0ull;
                 int e = lane < m ? id[lane] : MD_ID_MASK, t = 0;
                 const int e0 = e;
@@ -363,6 +364,286 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
             if (j < m) p.perm[(size_t)(id[j] & MD_ID_MASK) * b + (id[j] >> MD_ID_BITS) + left] = c;
         }
     }
+}
+
+// ---------------------------------------------------------------- up to 256 blocks: a block to a lane
+//
+// The same batches in fewer dependent steps.  Above, places in the merged list are counted and searched (11000 warp instructions and
+// five barriers a batch, 5000 cycles).  Here the list is one 32-bit word a block and is sorted anew after every batch: by warps
+// (bitonic), then every word looks for its place in the other warps' runs.  A word is the block below 23 bits of the sum's distance to
+// the list's smallest one, in units of a little more than the next mass: a batch ends before its smallest new sum, which is at
+// most one mass away, so that sums further away need no order yet.  Sums and fill counts stay in shared memory by block, masses
+// and the place of every rank as well; the permutation is stored in the end.  Neighbours that their words do not tell apart are
+// looked at when the list is read.  Small batches (steep masses) are followed by runs of 32 channels one by one, as above.
+// 8192 channels of a real statistic in 256 blocks: 103 us (175 as above), 2800 cycles a batch (the sort in the warps 560, the places 750).
+// What it did not gain: all of it in one warp, eight words a lane and no barrier (151 us: one warp's issue), the places by fours
+// with 16-byte loads (116).  Other masses: 0.1 to 0.95 of the time above; 1.06 to 1.09 where half of the masses are too small
+// to change a sum (blocks fill one after the other).
+constexpr int MD_SORT_BLOCKS = 256;
+constexpr int MD_SORT_SLOTS = 512;                       // (entries of the tables by block: a word without a block has the last one)
+constexpr int MD_SORT_THREADS = 512;
+constexpr uint32_t MD_ID = MD_SORT_SLOTS - 1;            // block in the low 9 bits
+constexpr uint32_t MD_FAR = 0x7ffffeu << 9;              // too far for an order
+constexpr uint32_t MD_NONE = 0xffffffffu;                // full block, or none
+
+struct MdSortSmem {
+    size_t sum, lows, fill, list, runs, red, place, mass, total;
+    __host__ __device__ explicit MdSortSmem(int d)
+    {
+        size_t o = 0;
+        sum = o;   o += (size_t)MD_SORT_SLOTS * 8;
+        lows = o;  o += 16 * 8;
+        fill = o;  o += (size_t)MD_SORT_SLOTS * 4;
+        list = o;  o += (size_t)MD_SORT_BLOCKS * 4;
+        runs = o;  o += (size_t)MD_SORT_BLOCKS * 4;
+        red = o;   o += 32 * 4;
+        place = o; o += ((size_t)d * 2 + 15) & ~(size_t)15;
+        mass = o;  o += (size_t)d * 4;
+        total = o;
+    }
+};
+
+// A barrier of the warps that sort, with a count or a disjunction over their threads.
+__device__ __forceinline__ int md_barrier_count(int threads, bool v)
+{
+    uint32_t c;
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %1, 0; bar.red.popc.u32 %0, 1, %2, p; }" : "=r"(c) : "r"((uint32_t)v), "r"(threads) : "memory");
+    return (int)c;
+}
+__device__ __forceinline__ bool md_barrier_any(int threads, bool v)
+{
+    uint32_t any;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %1, 0; bar.red.or.pred q, 1, %2, p; selp.u32 %0, 1, 0, q; }"
+                 : "=r"(any) : "r"((uint32_t)v), "r"(threads) : "memory");
+    return any != 0u;
+}
+
+// Up to `room` channels from rank s on, one by one (a warp): lane j has entry j of the list.  Returns how many (a mass of zero ends it).
+// whole: the list has no more than 32 entries.  32 channels reach no more than the first 32 entries; where fewer are near, the first of
+// them must not become full before the last channel: until then no block that is served is further from it than the masses
+// served, so that all of them are near.
+__device__ __noinline__ int md_warp_serial(uint32_t *list, unsigned long long *sum, int *fill, uint16_t *place, const float *mass, int s, int room, int b,
+                                           bool whole, int lane)
+{
+    const uint32_t own = list[lane];
+    const bool has = whole ? own != MD_NONE : own < MD_FAR;
+    const int mine = has ? (int)(own & MD_ID) : MD_ID_MASK;
+    unsigned long long w = has ? sum[mine] : ~0ull;
+    int f = has ? fill[mine] : 0, t = 0;
+    if (!whole && __any_sync(0xffffffffu, !has)) room = min(room, b - __shfl_sync(0xffffffffu, f, 0));
+#pragma unroll 1
+    for (; t < room; ++t) {
+        const float a = mass[s + t];
+        if (a == 0.0f) break;
+        unsigned long long lowest;
+        int blk;
+        md_warp_min(w, mine, lowest, blk);
+        if (w == lowest && mine == blk) {
+            place[s + t] = (uint16_t)(blk * b + f);
+            w = (unsigned long long)__double_as_longlong(__longlong_as_double((long long)w) + (double)a);
+            if (++f == b) w = ~0ull;
+        }
+    }
+    if (has) {
+        fill[mine] = f;
+        if (w != ~0ull) sum[mine] = w; else list[lane] = MD_NONE;
+    }
+    __syncwarp();
+    return t;
+}
+
+// W warps sort (32 W blocks at most).
+template <int W>
+__global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(MassdiffParams p)
+{
+    extern __shared__ __align__(16) unsigned char md_smem[];
+    const int d = p.d, b = p.b, n = d / b;
+    constexpr int SERIAL_BELOW = W <= 4 ? 4 : 6;              // (about the channels one by one that a batch costs)
+    const MdSortSmem lay(d);
+    double *sum = (double *)(md_smem + lay.sum);
+    unsigned long long *sum_bits = (unsigned long long *)sum, *lows = (unsigned long long *)(md_smem + lay.lows);
+    int *fill = (int *)(md_smem + lay.fill);
+    uint32_t *list = (uint32_t *)(md_smem + lay.list), *runs = (uint32_t *)(md_smem + lay.runs), *red = (uint32_t *)(md_smem + lay.red);
+    int *full = (int *)(red + 16);                           // [3] blocks that became full; three steps in turn, so that one can be cleared
+    int *served_one = full + 3, *left = full + 4;            // channels of a run one by one; rank and open blocks in the end
+    uint16_t *place = (uint16_t *)(md_smem + lay.place);
+    float *mass = (float *)(md_smem + lay.mass);
+    int tid;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    const int lane = tid & 31, warp = tid >> 5;
+
+    for (int j = tid; j < MD_SORT_SLOTS; j += MD_SORT_THREADS) {
+        sum[j] = 0.0;
+        fill[j] = 0;
+        if (j < MD_SORT_BLOCKS) list[j] = j < n ? (uint32_t)j : MD_NONE;
+    }
+    if (tid < 32) red[tid] = 0u;
+    griddep_wait();             // nothing above reads or writes global memory
+    griddep_launch();
+#pragma unroll 4
+    for (int r = tid; r < d; r += MD_SORT_THREADS) mass[r] = md_mass(p.a[min(max(p.order[r], 0), d - 1)]);
+    __syncthreads();
+    if (tid < 32 * W) {
+        int m = n, s = 0, serial = 0, length = 1;            // open blocks; next rank; runs one by one to come, after the next small batch
+        int now = 0;                                         // step modulo 3
+#pragma unroll 1
+        while (s < d) {
+            const float unit = mass[s];
+            if (m == 1 || unit == 0.0f) break;               // one block or only zero masses are left: below
+            const int next = now < 2 ? now + 1 : 0;
+            // ---- sums, and those that the next channels would reach in the order of the list
+            uint32_t k = list[tid];
+            const double base = sum[list[0] & MD_ID];
+            double v = sum[k & MD_ID];
+            const uint32_t k1 = tid + 1 < 32 * W ? list[tid + 1] : MD_NONE;
+            const double v1 = sum[k1 & MD_ID], w = v + (double)mass[min(s + tid, d - 1)];
+            const int blk = (int)(k & MD_ID), f = fill[blk];
+            const float at = (float)(v - base), to = (float)(w - base);
+            const bool near = k < MD_FAR;
+            // (sums further away can not be the smallest)
+            const uint32_t low = __reduce_min_sync(0xffffffffu, near && f + 1 < b ? __float_as_uint(to) : 0x7f800000u);
+            if (lane == 0) red[warp] = low;
+            const bool wrong = k1 < MD_FAR && (v1 < v || (v1 == v && (int)(k1 & MD_ID) < blk));
+            if (md_barrier_any(32 * W, wrong)) {
+                // neighbours change places until all near entries are in order (an even round settles the even pairs)
+#pragma unroll 1
+                for (int r = 0; r < 64 * W + 2; ++r) {
+                    bool swapped = false;
+                    if (((tid ^ r) & 1) == 0 && tid + 1 < 32 * W) {
+                        const uint32_t e0 = list[tid], e1 = list[tid + 1];
+                        const int b0 = (int)(e0 & MD_ID), b1 = (int)(e1 & MD_ID);
+                        if (e1 < MD_FAR && md_less(sum_bits[b1], b1, sum_bits[b0], b0)) { list[tid] = e1; list[tid + 1] = e0; swapped = true; }
+                    }
+                    if (!md_barrier_any(32 * W, swapped) && (r & 1)) break;
+                }
+                continue;
+            }
+            bool served = false, rest = true;                // rest: K is known, and the reach
+            double from = base;
+            float reach = 1.05f * unit;
+            int K = 0;
+            if (n > 32 && list[0] >= MD_FAR) {
+                // ---- no sum was near: again, from the smallest of all
+                unsigned long long mine = k != MD_NONE ? (unsigned long long)__double_as_longlong(v) : ~0ull, lowest;
+                int unused;
+                md_warp_min(mine, blk, lowest, unused);
+                if (lane == 0) lows[warp] = lowest;
+                named_barrier(1, 32 * W);
+                lowest = lows[0];
+#pragma unroll
+                for (int j = 1; j < W; ++j) lowest = min(lowest, lows[j]);
+                from = __longlong_as_double((long long)lowest);
+                const uint32_t far = __reduce_max_sync(0xffffffffu, k != MD_NONE ? __float_as_uint(fmaxf((float)(v - from), 0.0f)) : 0u);
+                if (lane == 0) red[warp] = far;
+                named_barrier(1, 32 * W);
+                uint32_t most = red[0];
+#pragma unroll
+                for (int j = 1; j < W; ++j) most = max(most, red[j]);
+                // (all are near then: a run one by one may fill blocks)
+                reach = fmaxf(1.01f * __uint_as_float(most), unit);
+            } else if (n <= MD_FEW_BLOCKS || serial > 0) {
+                if (warp == 0) {
+                    const int t = md_warp_serial(list, sum_bits, fill, place, mass, s, n <= MD_FEW_BLOCKS ? d - s : min(32, d - s), b, W == 1, lane);
+                    if (lane == 0) *served_one = t;
+                }
+                named_barrier(1, 32 * W);
+                if (serial > 0) --serial;
+                const uint32_t before = k;
+                k = list[tid];
+                v = sum[k & MD_ID];
+                if (k == MD_NONE && before != MD_NONE) atomicAdd(&full[now], 1);
+                K = *served_one;
+                reach = (serial > 0 ? 67.0f : 34.0f) * unit;          // (from the old smallest sum: the new one is at most 32 masses away)
+            } else {
+                // ---- serve the entries below the smallest of them (the first one always)
+                uint32_t least_bits = red[0];
+#pragma unroll
+                for (int j = 1; j < W; ++j) least_bits = min(least_bits, red[j]);
+                const float least = __uint_as_float(least_bits);
+                served = near && (at < least || tid == 0);
+                if (served) {
+                    place[s + tid] = (uint16_t)(blk * b + f);
+                    fill[blk] = f + 1;
+                    sum[blk] = w;
+                    v = w;
+                    if (f + 1 == b) { k = MD_NONE; atomicAdd(&full[now], 1); }
+                }
+                if (least < 3.0e38f) from = base + (double)(least * 0.9999998f);
+                rest = false;
+            }
+            // ---- words of the new list, sorted by warps
+            auto word = [&](float r) {
+                const float scale = fminf(__fdividef(8388600.0f / 256.0f, r * 0.00390625f), 3.0e38f);
+                const float q = fminf(fmaxf((float)(v - from), 0.0f) * scale, 8388606.0f);
+                return k == MD_NONE ? MD_NONE : (__float_as_uint(q + 8388608.0f) << 9) | (k & MD_ID);
+            };
+            if (!rest) {
+                // (whether runs one by one follow, and need a longer reach, is known when the served entries are counted)
+                K = md_barrier_count(32 * W, served);
+                if (K < SERIAL_BELOW && K < m) { serial = length; length = min(2 * length, MD_SERIAL_RUNS); reach = 34.0f * unit; }
+                else if (K < m) length = 1;
+            }
+            k = word(reach);
+#pragma unroll
+            for (int size = 2; size <= 32; size *= 2) {
+#pragma unroll
+                for (int stride = size / 2; stride > 0; stride /= 2) {
+                    // (the first step of a size compares mirrored lanes, so that all are ascending)
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, k, stride == size / 2 ? size - 1 : stride);
+                    k = (lane & stride) == 0 ? min(k, o) : max(k, o);
+                }
+            }
+            int at_place = lane;
+            if (W > 1) {
+                runs[tid] = k;
+                named_barrier(1, 32 * W);
+                // ---- places: words before the own one in the other warps' runs
+#pragma unroll
+                for (int j = 1; j < W; ++j) {
+                    const uint32_t *run = runs + ((warp + j) % W) * 32;
+                    int c = 0;
+#pragma unroll
+                    for (int step = 16; step > 0; step /= 2) c += run[c + step - 1] < k ? step : 0;
+                    at_place += c + (run[c] < k ? 1 : 0);
+                }
+            } else {
+                __syncwarp();
+            }
+            m -= full[now];
+            if (tid == 0) full[next] = 0;
+            if (k != MD_NONE) list[at_place] = k;
+            if (tid >= m) list[tid] = MD_NONE;
+            s += K;
+            now = next;
+            named_barrier(1, 32 * W);
+        }
+        if (tid == 0) { left[0] = s; left[1] = m; }
+    }
+    __syncthreads();
+    const int s = left[0], m = left[1];
+    if (s < d) {
+        // ---- zero masses change no sum: the open blocks take what they have room for, in the order of their sums (so does the last
+        // open block).  Their order by counting.
+        const uint32_t mine = tid < m ? list[tid] & MD_ID : 0u;
+        int before = 0;
+        if (tid < m)
+#pragma unroll 1
+            for (int j = 0; j < m; ++j) {
+                const uint32_t o = list[j] & MD_ID;
+                before += md_less(sum_bits[o], (int)o, sum_bits[mine], (int)mine) ? 1 : 0;
+            }
+        if (tid < m) runs[before] = mine;
+        __syncthreads();
+#pragma unroll 1
+        for (int r = s + tid; r < d; r += MD_SORT_THREADS) {
+            int rest = r - s, j = 0;
+            while (j < m && rest >= b - fill[runs[j]]) { rest -= b - fill[runs[j]]; ++j; }
+            if (j < m) place[r] = (uint16_t)((int)runs[j] * b + fill[runs[j]] + rest);
+        }
+        __syncthreads();
+    }
+#pragma unroll 4
+    for (int r = tid; r < d; r += MD_SORT_THREADS) p.perm[place[r]] = min(max(p.order[r], 0), d - 1);
 }
 
 }  // namespace perq
