@@ -691,29 +691,43 @@ HostPipe *host_pipe()
     return hp.ok ? &hp : nullptr;     // without it the call still works, on the caller's stream alone
 }
 
-template <int KC, int CL, bool WB>
-int launch_stats_inst(const perq::StatsParams &p, const StatsPlan &plan, cudaStream_t st)
+int launch_stats_kernel(void (*kernel)(perq::StatsParams), int grid, int threads, size_t smem, const perq::StatsParams &p, cudaStream_t st)
 {
-    if (int rc = allow_smem(perq::perq_stats_partial_kernel<KC, CL, WB>, plan.smem)) return rc;
-    perq::perq_stats_partial_kernel<KC, CL, WB><<<plan.n_cta, perq::ST_THREADS, plan.smem, st>>>(p);
-    return cudaGetLastError() == cudaSuccess ? PERQ_OK : PERQ_ERR_CUDA;
+    if (int rc = allow_smem(kernel, smem)) return rc;
+    if (launch_overlapped(kernel, grid, threads, smem, st, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return PERQ_ERR_CUDA;
+    }
+    return PERQ_OK;
+}
+
+// Unpermuted rows, blocks up to 256 channels.
+template <int KC>
+int launch_stats_rows(perq::StatsParams p, const StatsPlan &plan, cudaStream_t st)
+{
+    const size_t stage = (size_t)perq::stats_rows(KC) * p.d * 2, fixed = 2 * perq::ST_MAX_STAGES * 8 + perq::ST_MAX_STAGES * 4 * 4;
+    const long long batches = (plan.rows_per_cta + perq::stats_rows(KC) - 1) / perq::stats_rows(KC);
+    p.n_stages = (int)std::min<long long>({(long long)perq::ST_MAX_STAGES, (long long)((220 * 1024 - fixed) / stage), std::max(2ll, batches)});
+    const size_t smem = p.n_stages * stage + fixed;
+    constexpr int threads = perq::ST_THREADS + 32;
+    if (p.ws_block == nullptr && p.token_max == nullptr)
+        return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 0, false>, plan.n_cta, threads, smem, p, st);
+    switch (p.log2b) {
+    case 3: return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 0, true>, plan.n_cta, threads, smem, p, st);
+    case 4: return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 1, true>, plan.n_cta, threads, smem, p, st);
+    case 5: return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 2, true>, plan.n_cta, threads, smem, p, st);
+    case 6: return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 3, true>, plan.n_cta, threads, smem, p, st);
+    case 7: return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 4, true>, plan.n_cta, threads, smem, p, st);
+    default: return launch_stats_kernel(perq::perq_stats_rows_kernel<KC, 5, true>, plan.n_cta, threads, smem, p, st);
+    }
 }
 
 template <int KC>
 int launch_stats_partial(const perq::StatsParams &p, const StatsPlan &plan, cudaStream_t st)
 {
-    // specialised variants: unpermuted rows of exactly KC * 4096 channels, blocks of 16, 32 or 128
-    if (KC <= 4 && p.perm == nullptr && p.d == KC * 4096) {
-        const bool wb = p.ws_block != nullptr || p.token_max != nullptr;
-        if (!wb) return launch_stats_inst<KC, 2, false>(p, plan, st);
-        switch (p.log2b) {
-        case 4: return launch_stats_inst<KC, 1, true>(p, plan, st);
-        case 5: return launch_stats_inst<KC, 2, true>(p, plan, st);
-        case 7: return launch_stats_inst<KC, 4, true>(p, plan, st);
-        default: break;
-        }
-    }
-    return launch_stats_inst<KC, -1, false>(p, plan, st);
+    const bool wb = p.ws_block != nullptr || p.token_max != nullptr;
+    if (!wb || (p.perm == nullptr && p.log2b <= 8)) return launch_stats_rows<KC>(p, plan, st);
+    return launch_stats_kernel(perq::perq_stats_partial_kernel<KC>, plan.n_cta, perq::ST_THREADS, plan.smem, p, st);
 }
 
 }  // namespace
@@ -920,8 +934,18 @@ int perq_block_l1_stats(const void *x, const int32_t *perm, int64_t T, int32_t d
     }
     if (rc != PERQ_OK) return rc;
     if (chan_abs_sum || block_l1_mean) {
-        perq::perq_stats_reduce_kernel<<<(d + 63) / 64, 256, 0, st>>>(
-            p.ws_chan, p.ws_block, plan.n_cta, d, d / b, (float)(1.0 / (double)T), chan_abs_sum, block_l1_mean);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((chan_abs_sum ? (d + 63) / 64 : 0) + (block_l1_mean ? (d / b + 63) / 64 : 0)));
+        cfg.blockDim = dim3(256);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const float *ws_chan = p.ws_chan, *ws_block = p.ws_block;
+        (void)cudaLaunchKernelEx(&cfg, perq::perq_stats_reduce_kernel, ws_chan, ws_block, plan.n_cta, (int)d, (int)(d / b), (float)(1.0 / (double)T),
+                                 chan_abs_sum, block_l1_mean);
         if (cudaGetLastError() != cudaSuccess) return PERQ_ERR_CUDA;
     }
     return PERQ_OK;

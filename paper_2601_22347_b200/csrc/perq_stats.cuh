@@ -2,7 +2,7 @@
 // per-token max block l1 norm under an optional permutation.
 //
 // Phase 1: each CTA walks a contiguous slab of rows, 64 KB of rows at a time through a ring of
-// bulk-copied shared-memory stages, keeps
+// bulk-copied shared-memory stages (32 KB where no gather is needed), keeps
 // per-channel and per-block partial sums in registers (every thread owns fixed columns /
 // blocks), and writes them to its own slice of the workspace.  Rows go through shared memory
 // only when a block statistic needs the gather through the permutation.
@@ -38,15 +38,11 @@ __device__ __forceinline__ float abs_bf16(uint16_t h) { return __uint_as_float((
 // consecutive rows are contiguous in global memory: one elected thread fetches each with a single
 // cp.async.bulk into a ring of shared-memory stages (bulk copies are not limited by the load
 // queue of the SM the way per-thread loads are), everybody reads its columns from there.
-// CL >= 0 selects a specialised variant: rows of exactly KC * 4096 channels, no permutation, blocks of
-// 2^CL chunks (CL <= 5: summed by shuffles), block statistics wanted (WB) or not -- the flags the general
-// variant (CL = -1) tests at run time inside its unrolled loops are constants there.
-template <int KC, int CL, bool WB>
+// Permuted rows and blocks of more than 256 channels; the others have the kernel below.
+template <int KC>
 __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsParams p)
 {
     constexpr int R = 8 / KC;
-    constexpr bool FAST = CL >= 0;
-    static_assert(CL <= 5, "shuffle sums need a block inside a warp");
     const int NST = p.n_stages;                   // 3, or 2 where 3 stages would not fit
     extern __shared__ __align__(128) unsigned char smem[];
     const int d = p.d, L = p.log2b, nb = d >> L, nchunks = d >> 3;
@@ -58,6 +54,7 @@ __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsPar
     uint64_t *full = (uint64_t *)(red + 2 * R * 16);                     // [NST] mbarriers
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
+    griddep_wait();             // nothing above reads or writes global memory
     for (int i = tid; i < d; i += ST_THREADS) {
         int q = p.perm ? __ldg(p.perm + i) : i;
         sperm[i] = (uint16_t)min(max(q, 0), d - 1);
@@ -72,10 +69,10 @@ __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsPar
     }
     const long long t0 = (long long)blockIdx.x * p.rows_per_cta;
     const long long t1 = min(p.T, t0 + p.rows_per_cta);
-    const bool want_blocks = FAST ? WB : ((p.ws_block != nullptr) || (p.token_max != nullptr));
-    const bool use_perm = FAST ? false : (p.perm != nullptr);
-    const int cpb = FAST ? (1 << (CL < 0 ? 0 : CL)) : (1 << (L - 3));   // 16-byte chunks per block
-    const bool shuffle_blocks = FAST ? true : cpb <= 32;                // a block's chunks sit in adjacent lanes of one warp
+    const bool want_blocks = (p.ws_block != nullptr) || (p.token_max != nullptr);
+    const bool use_perm = p.perm != nullptr;
+    const int cpb = 1 << (L - 3);                            // 16-byte chunks per block
+    const bool shuffle_blocks = cpb <= 32;                   // a block's chunks sit in adjacent lanes of one warp
 
     auto fetch = [&](int stage, long long t) {      // one thread: rows t .. t+R-1 (those below t1) into a stage
         if (t < t1) {
@@ -110,7 +107,7 @@ __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsPar
             for (int k = 0; k < KC; ++k) {
                 const int c = tid + k * ST_THREADS;
                 float s = 0.0f;
-                if (live && (FAST || c < nchunks)) {
+                if (live && c < nchunks) {
                     const uint4 w = ((const uint4 *)(rows + (size_t)r * d))[c];
                     const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
                     float2 m[4];
@@ -201,6 +198,7 @@ __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsPar
         __syncthreads();                                 // cs may be overwritten by the next batch
     }
 
+    griddep_launch();
     if (p.ws_chan) {
         float4 *dst = (float4 *)(p.ws_chan + (size_t)blockIdx.x * d);
 #pragma unroll
@@ -225,43 +223,176 @@ __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsPar
     }
 }
 
-// 256 threads: 64 outputs, each summed by 4 threads over a quarter of the CTA slices, then
-// combined in a fixed order (deterministic).
+// Unpermuted rows, blocks of 2^CL chunks of eight channels (up to 256 channels).  The same sums in the same order, without a barrier:
+// a 17th warp loads rows (32 KB of them to a stage, as many stages as fit) and the others hand a stage back by an mbarrier.  The rows'
+// largest block sums meet in a word of the stage, which the loading warp stores and clears before it loads again.  With 64 KB to a batch and
+// a barrier for each, the first and the last batch and the barriers were in the open, and widths other than 4096, 8192 and 16384
+// and blocks of 64 had flags to test in every unrolled step.  Both passes, 4096 x 8192: b = 32 25.2 -> 22.7 us, b = 64 31.4 -> 24.0; 8192 x
+// 14336 78 -> 53; 4096 x 2048 23.0 -> 16.6.  What bounds it: 13.6 us are this pass (5 TB/s), 7.5 the second one, also when it has
+// next to nothing to add: the end of a grid, the start of the next, two trips to L2.
+constexpr int ST_MAX_STAGES = 8;
+__host__ __device__ constexpr int stats_rows(int kc) { return kc >= 4 ? 1 : 4 / kc; }       // rows of a stage
+
+template <int KC, int CL, bool WB>
+__global__ void __launch_bounds__(ST_THREADS + 32) perq_stats_rows_kernel(StatsParams p)
+{
+    constexpr int R = stats_rows(KC);
+    constexpr int cpb = 1 << CL;
+    static_assert(CL <= 5, "shuffle sums need a block inside a warp");
+    const int NST = p.n_stages;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int d = p.d, nchunks = d >> 3;
+    const uint32_t stage_bytes = (uint32_t)(R * d * 2);
+    const uint32_t bars = smem_u32(smem) + (uint32_t)NST * stage_bytes, empty = bars + ST_MAX_STAGES * 8;
+    uint32_t *top = reinterpret_cast<uint32_t *>(smem + (size_t)NST * stage_bytes + 2 * ST_MAX_STAGES * 8);        // [NST][R]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < ST_MAX_STAGES) {
+        mbar_init(bars + tid * 8, 1);
+        mbar_init(empty + tid * 8, ST_THREADS / 32);
+        mbar_init_fence();
+    }
+    if (tid < ST_MAX_STAGES * R) top[tid] = 0u;
+    __syncthreads();
+    griddep_wait();             // nothing above reads or writes global memory
+    griddep_launch();           // (the second pass waits beside this one: 22.7 us, launched after the last row 23.5)
+    const long long t0 = (long long)blockIdx.x * p.rows_per_cta, t1 = min(p.T, t0 + p.rows_per_cta);
+    const uint32_t n = t1 > t0 ? (uint32_t)((t1 - t0 + R - 1) / R) : 0u;
+
+    if (warp == ST_THREADS / 32) {
+        // ---- the loading warp: batch i into stage i % NST, once the batch before it is done with
+        if (lane == 0) {
+            uint32_t s = 0, turn = 0;                        // turn: batches of this stage so far
+            for (uint32_t i = 0; i < n + (uint32_t)NST; ++i) {
+                if (i >= (uint32_t)NST && i - (uint32_t)NST < n) {
+                    if (!mbar_wait_fast(empty + s * 8, (turn - 1u) & 1u)) { atomicOr(&g_perq_device_error, 8u); break; }
+                    if (WB && p.token_max) {
+                        const long long t = t0 + (long long)(i - (uint32_t)NST) * R;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            if (t + r < t1) p.token_max[t + r] = __uint_as_float(*reinterpret_cast<volatile uint32_t *>(&top[s * R + r]));
+                            top[s * R + r] = 0u;
+                        }
+                    }
+                }
+                if (i < n) {
+                    const long long t = t0 + (long long)i * R;
+                    const uint32_t bytes = (uint32_t)(min((long long)R, t1 - t) * d * 2);
+                    mbar_expect_tx(bars + s * 8, bytes);     // (releases the cleared words)
+                    bulk_load(smem_u32(smem) + s * stage_bytes, p.x + (size_t)t * d, bytes, bars + s * 8);
+                }
+                if (++s == (uint32_t)NST) { s = 0; ++turn; }
+            }
+        }
+        return;
+    }
+
+    float2 csum[KC][4];      // per-channel sums of |x|, as pairs for the packed fp32 add
+    float bsum[KC];
+    bool has[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        bsum[k] = 0.0f;
+        has[k] = tid + k * ST_THREADS < nchunks;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) csum[k][e] = make_float2(0.0f, 0.0f);
+    }
+    uint32_t s = 0, parity = 0;
+    for (uint32_t i = 0; i < n; ++i) {
+        if (!mbar_wait_fast(bars + s * 8, parity)) {
+            if (lane == 0) atomicOr(&g_perq_device_error, 8u);
+            return;
+        }
+        const unsigned char *rows = smem + (size_t)s * stage_bytes;
+        const int live = (int)min((long long)R, t1 - (t0 + (long long)i * R));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (r >= live) break;
+            float mx = 0.0f;
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                if (has[k]) w = reinterpret_cast<const uint4 *>(rows + (size_t)r * d * 2)[tid + k * ST_THREADS];
+                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+                float2 m[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t a = ww[e] & 0x7fff7fffu;                 // |.| of both halves
+                    m[e] = make_float2(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u));
+                    csum[k][e] = __fadd2_rn(csum[k][e], m[e]);
+                }
+                if (WB) {
+                    const float2 h = __fadd2_rn(__fadd2_rn(m[0], m[1]), __fadd2_rn(m[2], m[3]));
+                    float b = h.x + h.y;
+#pragma unroll
+                    for (int o = 1; o < cpb; o <<= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+                    bsum[k] += b;                            // (the block's first chunk's is used)
+                    mx = fmaxf(mx, b);
+                }
+            }
+            if (WB) {
+                mx = warp_max_f32(mx);
+                if (lane == 0) atomicMax(&top[s * R + r], __float_as_uint(mx));
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty + s * 8);
+        if (++s == (uint32_t)NST) { s = 0; parity ^= 1u; }
+    }
+    if (p.ws_chan) {
+        float4 *dst = (float4 *)(p.ws_chan + (size_t)blockIdx.x * d);
+#pragma unroll
+        for (int k = 0; k < KC; ++k) {
+            const int c = tid + k * ST_THREADS;
+            if (has[k]) {
+                dst[2 * c] = make_float4(csum[k][0].x, csum[k][0].y, csum[k][1].x, csum[k][1].y);
+                dst[2 * c + 1] = make_float4(csum[k][2].x, csum[k][2].y, csum[k][3].x, csum[k][3].y);
+            }
+        }
+    }
+    if (WB && p.ws_block) {
+#pragma unroll
+        for (int k = 0; k < KC; ++k) {
+            const int c = tid + k * ST_THREADS;
+            if (has[k] && (c & (cpb - 1)) == 0) p.ws_block[(size_t)blockIdx.x * (nchunks >> CL) + (c >> CL)] = bsum[k];
+        }
+    }
+}
+
+// 256 threads: 64 outputs (of the channels, in the CTAs after those of the blocks), each summed by 4 threads over a quarter of the CTA
+// slices, then combined in a fixed order (deterministic).  The loads of a quarter are all in flight (in rounds of eight they
+// took five trips to L2).
+constexpr int ST_QUARTER = 38;                       // slices of a quarter: 148 CTAs at most
 __global__ void __launch_bounds__(256) perq_stats_reduce_kernel(const float *ws_chan, const float *ws_block, int n_cta, int d,
                                                                 int nb, float inv_T, float *chan_abs_sum, float *block_l1_mean)
 {
-    __shared__ float part[2][4][64];
+    __shared__ float part[4][64];
+    griddep_wait();             // nothing above reads or writes global memory
+    griddep_launch();
+    const int chan_ctas = chan_abs_sum ? (d + 63) / 64 : 0;
+    const bool blocks = (int)blockIdx.x >= chan_ctas;
+    const int width = blocks ? nb : d;
+    const float *ws = blocks ? ws_block : ws_chan;
     const int o = threadIdx.x & 63, quarter = threadIdx.x >> 6;
-    const int i = blockIdx.x * 64 + o;
+    const int i = ((int)blockIdx.x - (blocks ? chan_ctas : 0)) * 64 + o;
     const int per = (n_cta + 3) / 4;
     const int c0 = quarter * per, c1 = min(n_cta, c0 + per);
-    float sc = 0.0f, sb = 0.0f;
-    // eight independent loads at a time, added in slice order (x + 0 is exact, so padding is harmless)
-    if (chan_abs_sum && i < d) {
-        for (int c = c0; c < c1; c += 8) {
-            float v[8];
+    float sum = 0.0f;
+    if (i < width) {
+        // independent loads, added in slice order (x + 0 is exact, so padding is harmless)
+        for (int c = c0; c < c1; c += ST_QUARTER) {
+            float v[ST_QUARTER];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = (c + j < c1) ? ws_chan[(size_t)(c + j) * d + i] : 0.0f;
+            for (int j = 0; j < ST_QUARTER; ++j) v[j] = (c + j < c1) ? ws[(size_t)(c + j) * width + i] : 0.0f;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) sc += v[j];
+            for (int j = 0; j < ST_QUARTER; ++j) sum += v[j];
         }
     }
-    if (block_l1_mean && i < nb) {
-        for (int c = c0; c < c1; c += 8) {
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = (c + j < c1) ? ws_block[(size_t)(c + j) * nb + i] : 0.0f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sb += v[j];
-        }
-    }
-    part[0][quarter][o] = sc;
-    part[1][quarter][o] = sb;
+    part[quarter][o] = sum;
     __syncthreads();
-    if (quarter == 0) {
-        if (chan_abs_sum && i < d) chan_abs_sum[i] = ((part[0][0][o] + part[0][1][o]) + part[0][2][o]) + part[0][3][o];
-        if (block_l1_mean && i < nb)
-            block_l1_mean[i] = (((part[1][0][o] + part[1][1][o]) + part[1][2][o]) + part[1][3][o]) * inv_T;
+    if (quarter == 0 && i < width) {
+        const float all = ((part[0][o] + part[1][o]) + part[2][o]) + part[3][o];
+        if (blocks) block_l1_mean[i] = all * inv_T;
+        else chan_abs_sum[i] = all;
     }
 }
 
