@@ -982,7 +982,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_fast_kernel(FastParams p
     if (tid < 2 * FAST_WARPS) { wacc[tid] = 0ull; wacc2[tid] = ~0ull; wcnt[tid] = 0u; wflag[tid] = 0u; }
     __syncthreads();
 
-    const uint32_t first = blockIdx.x * GROUPS + group;
+    const uint32_t first = blockIdx.x + group * gridDim.x;      // (few units: one to an SM before two)
     const uint32_t stride = gridDim.x * GROUPS;
     if (group >= GROUPS || first >= p.units_total) return;   // whole groups leave together (no barrier is shared across groups)
 

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_mx_kernel(FastParams p)
     griddep_launch();           // the stream's next kernel may be set up on every SM this grid has left (it waits like this one)
 
     // units of this warp: first, first + stride, ...
-    const uint32_t first = blockIdx.x * FAST_WARPS + warp;
+    const uint32_t first = blockIdx.x + warp * gridDim.x;      // (few units: one to an SM before two)
     const uint32_t stride = gridDim.x * FAST_WARPS;
     if (first >= p.units_total) return;
     const uint32_t n_units = (p.units_total - first + stride - 1) / stride;

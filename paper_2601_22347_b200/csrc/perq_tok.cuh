@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(FAST_THREADS, 1) perq_tok_kernel(FastParams p)
     griddep_wait();             // nothing above reads or writes global memory
     griddep_launch();           // the stream's next kernel may be set up on every SM this grid has left (it waits like this one)
 
-    const uint32_t first = blockIdx.x * GROUPS + group;
+    const uint32_t first = blockIdx.x + group * gridDim.x;      // (few units: one to an SM before two)
     const uint32_t stride = gridDim.x * GROUPS;
     if (first >= p.units_total) return;          // whole groups leave together
     const uint32_t n_units = (p.units_total - first + stride - 1) / stride;
