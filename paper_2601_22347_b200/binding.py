@@ -27,6 +27,7 @@ FMT_BY_NAME = {"int4": PERQ_FMT_INT4, "mxfp4": PERQ_FMT_MXFP4, "f32": PERQ_FMT_F
 PERQ_OK = 0
 
 _lib = None
+_rotate_quantize = _swiglu_rotate_quantize = None       # the calls of these two: perq_call.c, or ctypes where that is not built
 
 
 class PerqError(RuntimeError):
@@ -37,7 +38,7 @@ class PerqError(RuntimeError):
 
 def load() -> C.CDLL:
     """Load libperq.so from the package directory (never builds implicitly)."""
-    global _lib
+    global _lib, _rotate_quantize, _swiglu_rotate_quantize
     if _lib is None:
         path = _build.LIB_PATH
         if not os.path.exists(path):
@@ -75,6 +76,11 @@ def load() -> C.CDLL:
                      "perq_block_l1_stats_workspace_bytes",
                      "perq_token_diagnostics", "perq_validate_perm", "perq_massdiff_perm", "perq_massdiff_perm_device"):
             getattr(lib, name).restype = C.c_int
+        _rotate_quantize, _swiglu_rotate_quantize = lib.perq_rotate_quantize, lib.perq_swiglu_rotate_quantize
+        if os.path.exists(_build.CALL_PATH):
+            from . import _perq_call
+            _perq_call.bind(C.cast(lib.perq_rotate_quantize, vp).value, C.cast(lib.perq_swiglu_rotate_quantize, vp).value)
+            _rotate_quantize, _swiglu_rotate_quantize = _perq_call.rotate_quantize, _perq_call.swiglu_rotate_quantize
         _lib = lib
     return _lib
 
@@ -135,8 +141,13 @@ def perq_rotate_quantize(x: torch.Tensor, perm: Optional[torch.Tensor], b: int, 
     T, d = x.shape
     if out_codes is None:
         out_codes, out_scales = alloc_outputs(T, d, fmt, group, x.device)
-    rc = (_lib or load()).perq_rotate_quantize(x.data_ptr(), _ptr(perm), T, d, b, fmt, group, _ptr(out_codes),
-                                               _ptr(out_scales), _stream(stream))
+    if _lib is None:
+        load()
+    args = (x.data_ptr(), None if perm is None else perm.data_ptr(), T, d, b, fmt, group, _ptr(out_codes), _ptr(out_scales), _stream(stream))
+    try:
+        rc = _rotate_quantize(*args)
+    except TypeError:           # (not plain integers: what ctypes makes of them)
+        rc = _lib.perq_rotate_quantize(*args)
     if rc != PERQ_OK:
         _check(rc, "perq_rotate_quantize")
     return out_codes, out_scales
@@ -152,8 +163,13 @@ def perq_swiglu_rotate_quantize(gate: torch.Tensor, up: torch.Tensor, perm: Opti
     T, d = gate.shape
     if out_codes is None:
         out_codes, out_scales = alloc_outputs(T, d, fmt, group, gate.device)
-    rc = load().perq_swiglu_rotate_quantize(_ptr(gate), _ptr(up), _ptr(perm), T, d, b, fmt, group, _ptr(out_codes),
-                                            _ptr(out_scales), _stream(stream))
+    if _lib is None:
+        load()
+    args = (gate.data_ptr(), up.data_ptr(), _ptr(perm), T, d, b, fmt, group, _ptr(out_codes), _ptr(out_scales), _stream(stream))
+    try:
+        rc = _swiglu_rotate_quantize(*args)
+    except TypeError:           # (as above)
+        rc = _lib.perq_swiglu_rotate_quantize(*args)
     _check(rc, "perq_swiglu_rotate_quantize")
     return out_codes, out_scales
 

@@ -4,11 +4,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 _CSRC = os.path.join(_PKG, "csrc")
 LIB_PATH = os.path.join(_PKG, "libperq.so")
+CALL_PATH = os.path.join(_PKG, "_perq_call.so")
 
 
 def _sources():
@@ -16,7 +18,7 @@ def _sources():
 
 
 def _deps():
-    deps = [os.path.join(_CSRC, f) for f in os.listdir(_CSRC)]
+    deps = [os.path.join(_CSRC, f) for f in os.listdir(_CSRC) if not f.endswith(".c")]
     deps.append(os.path.join(_ROOT, "include", "perq.h"))
     return deps
 
@@ -28,8 +30,25 @@ def needs_build() -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def build_call(force: bool = False) -> bool:
+    """Compile the interpreter's direct entry to perq_rotate_quantize (calls go through ctypes where there are no headers for it)."""
+    src, include = os.path.join(_CSRC, "perq_call.c"), sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        return False
+    if force or not os.path.exists(CALL_PATH) or os.path.getmtime(src) > os.path.getmtime(CALL_PATH):
+        tmp = CALL_PATH + ".tmp.%d" % os.getpid()
+        out = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", include, "-o", tmp, src],
+                             stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        if out.returncode != 0:
+            sys.stderr.write(out.stdout)
+            raise RuntimeError("%s failed building _perq_call.so" % os.environ.get("CC", "gcc"))
+        os.replace(tmp, CALL_PATH)
+    return True
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into one shared library for sm_100a."""
+    """Compile every .cu under csrc/ into one shared library for sm_100a, and the interpreter's entry to it."""
+    build_call(force)
     if not force and not needs_build():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
