@@ -493,7 +493,8 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
             const int next = now < 2 ? now + 1 : 0;
             // ---- sums, and those that the next channels would reach in the order of the list
             uint32_t k = list[tid];
-            const double base = sum[list[0] & MD_ID];
+            const uint32_t head = list[0];                   // (once: after the next barrier warp 0 may empty it, and all have to take the same way)
+            const double base = sum[head & MD_ID];
             double v = sum[k & MD_ID];
             const uint32_t k1 = tid + 1 < 32 * W ? list[tid + 1] : MD_NONE;
             const double v1 = sum[k1 & MD_ID], w = v + (double)mass[min(s + tid, d - 1)];
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
             double from = base;
             float reach = 1.05f * unit;
             int K = 0;
-            if (n > 32 && list[0] >= MD_FAR) {
+            if (n > 32 && head >= MD_FAR) {
                 // ---- no sum was near: again, from the smallest of all
                 unsigned long long mine = k != MD_NONE ? (unsigned long long)__double_as_longlong(v) : ~0ull, lowest;
                 int unused;
