@@ -420,13 +420,13 @@ __device__ __forceinline__ bool md_barrier_any(int threads, bool v)
 
 // Up to `room` channels from rank s on, one by one (a warp): lane j has entry j of the list.  Returns how many (a mass of zero ends it).
 // whole: the list has no more than 32 entries.  32 channels reach no more than the first 32 entries; where fewer are near, the first of
-// them must not become full before the last channel: until then no block that is served is further from it than the masses
-// served, so that all of them are near.
+// them must not become full before the last channel: until then no block that is served is further from where the first one
+// was than the masses served, so that all of them are near if the list reaches 32 masses beyond its first entry.
 __device__ __noinline__ int md_warp_serial(uint32_t *list, unsigned long long *sum, int *fill, uint16_t *place, const float *mass, int s, int room, int b,
                                            bool whole, int lane)
 {
     const uint32_t own = list[lane];
-    const bool has = whole ? own != MD_NONE : own < MD_FAR;
+    const bool has = own != MD_NONE && (whole || lane == 0 || own < MD_FAR);      // (the first entry is near)
     const int mine = has ? (int)(own & MD_ID) : MD_ID_MASK;
     unsigned long long w = has ? sum[mine] : ~0ull;
     int f = has ? fill[mine] : 0, t = 0;
@@ -493,13 +493,13 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
             const int next = now < 2 ? now + 1 : 0;
             // ---- sums, and those that the next channels would reach in the order of the list
             uint32_t k = list[tid];
-            const uint32_t head = list[0];                   // (once: after the next barrier warp 0 may empty it, and all have to take the same way)
-            const double base = sum[head & MD_ID];
+            const double base = sum[list[0] & MD_ID];        // (the smallest)
             double v = sum[k & MD_ID];
             const uint32_t k1 = tid + 1 < 32 * W ? list[tid + 1] : MD_NONE;
             const double v1 = sum[k1 & MD_ID], w = v + (double)mass[min(s + tid, d - 1)];
             const int blk = (int)(k & MD_ID), f = fill[blk];
             const float at = (float)(v - base), to = (float)(w - base);
+            const float step = unit + (float)(base * 1.2e-16);               // what a channel adds at most: the sum is rounded
             const bool near = k < MD_FAR;
             // (sums further away can not be the smallest)
             const uint32_t low = __reduce_min_sync(0xffffffffu, near && f + 1 < b ? __float_as_uint(to) : 0x7f800000u);
@@ -519,30 +519,11 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 }
                 continue;
             }
-            bool served = false, rest = true;                // rest: K is known, and the reach
             double from = base;
-            float reach = 1.05f * unit;
-            int K = 0;
-            if (n > 32 && head >= MD_FAR) {
-                // ---- no sum was near: again, from the smallest of all
-                unsigned long long mine = k != MD_NONE ? (unsigned long long)__double_as_longlong(v) : ~0ull, lowest;
-                int unused;
-                md_warp_min(mine, blk, lowest, unused);
-                if (lane == 0) lows[warp] = lowest;
-                named_barrier(1, 32 * W);
-                lowest = lows[0];
-#pragma unroll
-                for (int j = 1; j < W; ++j) lowest = min(lowest, lows[j]);
-                from = __longlong_as_double((long long)lowest);
-                const uint32_t far = __reduce_max_sync(0xffffffffu, k != MD_NONE ? __float_as_uint(fmaxf((float)(v - from), 0.0f)) : 0u);
-                if (lane == 0) red[warp] = far;
-                named_barrier(1, 32 * W);
-                uint32_t most = red[0];
-#pragma unroll
-                for (int j = 1; j < W; ++j) most = max(most, red[j]);
-                // (all are near then: a run one by one may fill blocks)
-                reach = fmaxf(1.01f * __uint_as_float(most), unit);
-            } else if (n <= MD_FEW_BLOCKS || serial > 0) {
+            float reach;
+            int K;
+            bool anew;                                       // the new smallest sum may be anywhere: to be looked for
+            if (n <= MD_FEW_BLOCKS || serial > 0) {
                 if (warp == 0) {
                     const int t = md_warp_serial(list, sum_bits, fill, place, mass, s, n <= MD_FEW_BLOCKS ? d - s : min(32, d - s), b, W == 1, lane);
                     if (lane == 0) *served_one = t;
@@ -554,14 +535,16 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 v = sum[k & MD_ID];
                 if (k == MD_NONE && before != MD_NONE) atomicAdd(&full[now], 1);
                 K = *served_one;
-                reach = (serial > 0 ? 67.0f : 34.0f) * unit;          // (from the old smallest sum: the new one is at most 32 masses away)
+                // (while the first block is open, the smallest sum is at most 32 masses above the old one, from which distances count)
+                anew = list[0] == MD_NONE;
+                reach = (serial > 0 && !anew ? 67.0f : 34.0f) * step;
             } else {
                 // ---- serve the entries below the smallest of them (the first one always)
                 uint32_t least_bits = red[0];
 #pragma unroll
                 for (int j = 1; j < W; ++j) least_bits = min(least_bits, red[j]);
                 const float least = __uint_as_float(least_bits);
-                served = near && (at < least || tid == 0);
+                const bool served = tid == 0 || (near && at < least);
                 if (served) {
                     place[s + tid] = (uint16_t)(blk * b + f);
                     fill[blk] = f + 1;
@@ -569,8 +552,28 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                     v = w;
                     if (f + 1 == b) { k = MD_NONE; atomicAdd(&full[now], 1); }
                 }
-                if (least < 3.0e38f) from = base + (double)(least * 0.9999998f);
-                rest = false;
+                // (at most two masses away where the first block stays open)
+                anew = !(least < 3.0e38f && least <= 2.0f * unit);
+                if (!anew) from = base + (double)(least * 0.9999998f);
+                // (whether runs one by one follow, and need a longer reach, is known when the served entries are counted; the reach of the
+                // largest masses would leave fp32)
+                K = md_barrier_count(32 * W, served);
+                reach = 1.05f * unit;
+                if (K < SERIAL_BELOW && K < m && unit < 1.0e36f) { serial = length; length = min(2 * length, MD_SERIAL_RUNS); reach = 34.0f * step; }
+                else if (K < m) length = 1;
+            }
+            if (anew) {
+                // ---- the first block is full, and the next one may be anywhere: distances count from the smallest sum there is.  (From the old
+                // one, entries that a run one by one needs would lie beyond its reach.)
+                unsigned long long lowest;
+                int unused;
+                md_warp_min(k != MD_NONE ? (unsigned long long)__double_as_longlong(v) : ~0ull, blk, lowest, unused);
+                if (lane == 0) lows[warp] = lowest;
+                named_barrier(1, 32 * W);
+                lowest = lows[0];
+#pragma unroll
+                for (int j = 1; j < W; ++j) lowest = min(lowest, lows[j]);
+                from = __longlong_as_double((long long)lowest);
             }
             // ---- words of the new list, sorted by warps
             auto word = [&](float r) {
@@ -578,12 +581,6 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 const float q = fminf(fmaxf((float)(v - from), 0.0f) * scale, 8388606.0f);
                 return k == MD_NONE ? MD_NONE : (__float_as_uint(q + 8388608.0f) << 9) | (k & MD_ID);
             };
-            if (!rest) {
-                // (whether runs one by one follow, and need a longer reach, is known when the served entries are counted)
-                K = md_barrier_count(32 * W, served);
-                if (K < SERIAL_BELOW && K < m) { serial = length; length = min(2 * length, MD_SERIAL_RUNS); reach = 34.0f * unit; }
-                else if (K < m) length = 1;
-            }
             k = word(reach);
 #pragma unroll
             for (int size = 2; size <= 32; size *= 2) {

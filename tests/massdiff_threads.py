@@ -192,3 +192,30 @@ def massdiff(a, b, policy=FIRST):
     status = _lib().massdiff(a.ctypes.data_as(ctypes.c_void_p), order.ctypes.data_as(ctypes.c_void_p),
                              perm.ctypes.data_as(ctypes.c_void_p), d, b, policy)
     return status, perm
+
+
+KINDS = ("lognormal2", "lognormal3", "power", "outliers", "graded", "rounded", "largest")
+
+
+def far_apart(kind, n, b, seed):
+    """Masses after which the next block to be served is far from the one that has just become full: heavy tails; graded masses, one to a
+    block, above light ones; masses that a running sum rounds up to its last place; the upper end of fp32."""
+    d = n * b
+    rng = np.random.default_rng(seed)
+    if kind.startswith("lognormal"):
+        return rng.lognormal(0, int(kind[-1]), d).astype(np.float32)
+    if kind == "power":
+        a = rng.random(d) ** -3.0
+    elif kind == "outliers":
+        a = rng.random(d) * np.where(rng.random(d) < 0.01, 1e5, 1.0)
+    elif kind == "graded":
+        a = 1.0 + 10.0 ** -rng.integers(1, 9) * rng.random(d)
+        k = rng.integers(1, n)
+        a[:k] = rng.uniform(1, 4 * b, k)
+    elif kind == "rounded":
+        a = rng.uniform(0.3, 3, d) * 2.0 ** -53
+        a[:n] = 1 + rng.integers(0, 60, n) * 2.0 ** -23
+    else:
+        a = np.full(d, 3e36)
+        a[:n] = rng.uniform(0, 3.4e38, n)
+    return rng.permutation(a.astype(np.float32))

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+from massdiff_threads import KINDS, far_apart
 from test_massdiff_device_gpu import B, device_perm  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -22,3 +23,11 @@ def test_blocks_to_lanes(B, kind, n, b):                     # noqa: F811
          "zeros": rng.exponential(size=d) * (rng.random(d) < 0.6)}[kind]
     a = rng.permutation(a.astype(np.float32))
     assert np.array_equal(device_perm(B, a, b), B.perq_massdiff_perm(a, b))
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n,b", [(32, 16), (33, 128), (63, 32), (66, 16), (75, 128), (100, 32), (128, 16), (129, 48), (256, 16), (256, 32), (256, 128)])
+def test_blocks_far_apart(B, kind, n, b):                    # noqa: F811
+    for seed in range(30):
+        a = far_apart(kind, n, b, seed)
+        assert np.array_equal(device_perm(B, a, b), B.perq_massdiff_perm(a, b)), seed
