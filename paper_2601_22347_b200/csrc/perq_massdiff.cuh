@@ -374,16 +374,19 @@ __global__ void __launch_bounds__(MD_MAX_THREADS, 1) perq_massdiff_greedy_kernel
 // the list's smallest one, in units of a little more than the next mass: a batch ends before its smallest new sum, which is at
 // most one mass away, so that sums further away need no order yet.  Sums and fill counts stay in shared memory by block, masses
 // and the place of every rank as well; the permutation is stored in the end.  Neighbours that their words do not tell apart are
-// looked at when the list is read.  Small batches (steep masses) are followed by runs of 32 channels one by one, as above.
-// 8192 channels of a real statistic in 256 blocks: 103 us (175 as above), 2800 cycles a batch (the sort in the warps 560, the places 750).
+// looked at when the list is read.  Small batches (steep masses) are followed by runs of 32 channels one by one, as above; these need
+// the 32 smallest entries, for which the distances beyond that reach keep their leading bits (3 % of the words: with half of them 17 instead of 8 of
+// 75 steps found neighbours to put in order, 120 us instead of 106).  Without them a run ended with its first block wherever fewer than
+// 32 entries were within reach: 256 blocks of 16, lognormal(0, 2) masses 246 -> 172 us, u^-3 681 -> 519.
+// 8192 channels of a real statistic in 256 blocks: 106 us (175 as above), 2800 cycles a batch (the sort in the warps 560, the places 750).
 // What it did not gain: all of it in one warp, eight words a lane and no barrier (151 us: one warp's issue), the places by fours
-// with 16-byte loads (116).  Other masses: 0.1 to 0.95 of the time above; 1.06 to 1.09 where half of the masses are too small
-// to change a sum (blocks fill one after the other).
+// with 16-byte loads (116).  Other masses (heavy-tailed, steep, equal, subnormal, too small to change a sum; 20 to 256 blocks of 8 to 128
+// channels): 0.1 to 0.94 of the time above.
 constexpr int MD_SORT_BLOCKS = 256;
 constexpr int MD_SORT_SLOTS = 512;                       // (entries of the tables by block: a word without a block has the last one)
 constexpr int MD_SORT_THREADS = 512;
 constexpr uint32_t MD_ID = MD_SORT_SLOTS - 1;            // block in the low 9 bits
-constexpr uint32_t MD_FAR = 0x7ffffeu << 9;              // too far for an order
+constexpr uint32_t MD_FAR = 0x7c0000u << 9;              // far: in order by ten bits of the distance's mantissa
 constexpr uint32_t MD_NONE = 0xffffffffu;                // full block, or none
 
 struct MdSortSmem {
@@ -419,18 +422,21 @@ __device__ __forceinline__ bool md_barrier_any(int threads, bool v)
 }
 
 // Up to `room` channels from rank s on, one by one (a warp): lane j has entry j of the list.  Returns how many (a mass of zero ends it).
-// whole: the list has no more than 32 entries.  32 channels reach no more than the first 32 entries; where fewer are near, the first of
-// them must not become full before the last channel: until then no block that is served is further from where the first one
-// was than the masses served, so that all of them are near if the list reaches 32 masses beyond its first entry.
+// 32 channels reach no more than the 32 smallest entries.  These are the first ones of the list where all of them are near, where the next one's
+// word tells it apart from them, or where there is none.  Elsewhere only near entries are looked at, and the first one must not become
+// full before the last channel: until then no block that is served is further from where the first one was than the masses served,
+// so that all of them are near if the list reaches 32 masses beyond its first entry.
 __device__ __noinline__ int md_warp_serial(uint32_t *list, unsigned long long *sum, int *fill, uint16_t *place, const float *mass, int s, int room, int b,
-                                           bool whole, int lane)
+                                           uint32_t beyond, int lane)
 {
-    const uint32_t own = list[lane];
-    const bool has = own != MD_NONE && (whole || lane == 0 || own < MD_FAR);      // (the first entry is near)
+    const uint32_t own = list[lane], last = __shfl_sync(0xffffffffu, own, 31);
+    const bool known = last < MD_FAR || last == MD_NONE || (last >> 9) < (beyond >> 9);
+    const bool has = own != MD_NONE && (known || lane == 0 || own < MD_FAR);      // (the first entry is near)
     const int mine = has ? (int)(own & MD_ID) : MD_ID_MASK;
     unsigned long long w = has ? sum[mine] : ~0ull;
     int f = has ? fill[mine] : 0, t = 0;
-    if (!whole && __any_sync(0xffffffffu, !has)) room = min(room, b - __shfl_sync(0xffffffffu, f, 0));
+    const int first_room = b - __shfl_sync(0xffffffffu, f, 0);
+    if (!known) room = min(room, first_room);
 #pragma unroll 1
     for (; t < room; ++t) {
         const float a = mass[s + t];
@@ -520,12 +526,17 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 continue;
             }
             double from = base;
-            float reach;
+            float reach, lift, scale;
+            auto reach_to = [&](float r) {
+                lift = r < 0x1p-60f ? 0x1p64f : 1.0f;        // (the reach has an inverse in fp32)
+                reach = fminf(r * lift, 3.4e38f);
+                scale = __fdividef(8126400.0f / 256.0f, reach * 0.00390625f);
+            };
             int K;
             bool anew;                                       // the new smallest sum may be anywhere: to be looked for
             if (n <= MD_FEW_BLOCKS || serial > 0) {
                 if (warp == 0) {
-                    const int t = md_warp_serial(list, sum_bits, fill, place, mass, s, n <= MD_FEW_BLOCKS ? d - s : min(32, d - s), b, W == 1, lane);
+                    const int t = md_warp_serial(list, sum_bits, fill, place, mass, s, n <= MD_FEW_BLOCKS ? d - s : min(32, d - s), b, W > 1 ? list[32] : MD_NONE, lane);
                     if (lane == 0) *served_one = t;
                 }
                 named_barrier(1, 32 * W);
@@ -537,7 +548,7 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 K = *served_one;
                 // (while the first block is open, the smallest sum is at most 32 masses above the old one, from which distances count)
                 anew = list[0] == MD_NONE;
-                reach = (serial > 0 && !anew ? 67.0f : 34.0f) * step;
+                reach_to((serial > 0 && !anew ? 67.0f : 34.0f) * step);
             } else {
                 // ---- serve the entries below the smallest of them (the first one always)
                 uint32_t least_bits = red[0];
@@ -557,9 +568,9 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 if (!anew) from = base + (double)(least * 0.9999998f);
                 // (whether runs one by one follow, and need a longer reach, is known when the served entries are counted; the reach of the
                 // largest masses would leave fp32)
+                reach_to(1.05f * unit);
                 K = md_barrier_count(32 * W, served);
-                reach = 1.05f * unit;
-                if (K < SERIAL_BELOW && K < m && unit < 1.0e36f) { serial = length; length = min(2 * length, MD_SERIAL_RUNS); reach = 34.0f * step; }
+                if (K < SERIAL_BELOW && K < m && unit < 1.0e36f) { serial = length; length = min(2 * length, MD_SERIAL_RUNS); reach_to(34.0f * step); }
                 else if (K < m) length = 1;
             }
             if (anew) {
@@ -576,12 +587,9 @@ __global__ void __launch_bounds__(MD_SORT_THREADS, 1) perq_massdiff_sort_kernel(
                 from = __longlong_as_double((long long)lowest);
             }
             // ---- words of the new list, sorted by warps
-            auto word = [&](float r) {
-                const float scale = fminf(__fdividef(8388600.0f / 256.0f, r * 0.00390625f), 3.0e38f);
-                const float q = fminf(fmaxf((float)(v - from), 0.0f) * scale, 8388606.0f);
-                return k == MD_NONE ? MD_NONE : (__float_as_uint(q + 8388608.0f) << 9) | (k & MD_ID);
-            };
-            k = word(reach);
+            const float away = fmaxf((float)(v - from), 0.0f) * lift, q = fminf(away * scale, 8126463.0f);
+            const uint32_t beyond = MD_FAR + ((__float_as_uint(away) - __float_as_uint(reach)) >> 13 << 9);
+            k = k == MD_NONE ? MD_NONE : (away < reach ? __float_as_uint(q + 8388608.0f) << 9 : beyond) | (k & MD_ID);
 #pragma unroll
             for (int size = 2; size <= 32; size *= 2) {
 #pragma unroll
