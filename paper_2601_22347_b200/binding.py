@@ -8,6 +8,7 @@ loaded, importing this module's functions raises.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from typing import Optional
 
@@ -27,7 +28,7 @@ FMT_BY_NAME = {"int4": PERQ_FMT_INT4, "mxfp4": PERQ_FMT_MXFP4, "f32": PERQ_FMT_F
 PERQ_OK = 0
 
 _lib = None
-_rotate_quantize = _swiglu_rotate_quantize = None       # the calls of these two: perq_call.c, or ctypes where that is not built
+_rotate_quantize = _swiglu_rotate_quantize = None       # the calls of these two: perq_call.c, or ctypes where that is not built or cannot be loaded
 
 
 class PerqError(RuntimeError):
@@ -77,10 +78,14 @@ def load() -> C.CDLL:
                      "perq_token_diagnostics", "perq_validate_perm", "perq_massdiff_perm", "perq_massdiff_perm_device"):
             getattr(lib, name).restype = C.c_int
         _rotate_quantize, _swiglu_rotate_quantize = lib.perq_rotate_quantize, lib.perq_swiglu_rotate_quantize
-        if os.path.exists(_build.CALL_PATH):
-            from . import _perq_call
-            _perq_call.bind(C.cast(lib.perq_rotate_quantize, vp).value, C.cast(lib.perq_swiglu_rotate_quantize, vp).value)
-            _rotate_quantize, _swiglu_rotate_quantize = _perq_call.rotate_quantize, _perq_call.swiglu_rotate_quantize
+        try:
+            spec = importlib.util.spec_from_file_location(__package__ + "._perq_call", _build.CALL_PATH)
+            call = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(call)
+            call.bind(C.cast(lib.perq_rotate_quantize, vp).value, C.cast(lib.perq_swiglu_rotate_quantize, vp).value)
+            _rotate_quantize, _swiglu_rotate_quantize = call.rotate_quantize, call.swiglu_rotate_quantize
+        except ImportError:         # (no such file, or none that this interpreter can load)
+            pass
         _lib = lib
     return _lib
 

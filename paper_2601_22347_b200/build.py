@@ -10,7 +10,7 @@ _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 _CSRC = os.path.join(_PKG, "csrc")
 LIB_PATH = os.path.join(_PKG, "libperq.so")
-CALL_PATH = os.path.join(_PKG, "_perq_call.so")
+CALL_PATH = os.path.join(_PKG, "_perq_call" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))      # (another interpreter has another name)
 
 
 def _sources():
@@ -31,19 +31,27 @@ def needs_build() -> bool:
 
 
 def build_call(force: bool = False) -> bool:
-    """Compile the interpreter's direct entry to perq_rotate_quantize (calls go through ctypes where there are no headers for it)."""
+    """Compile the interpreter's direct entry to the two calls of the online path.  False where there are no headers for it or
+    no compiler: these calls then go through ctypes, and an older file is taken away."""
     src, include = os.path.join(_CSRC, "perq_call.c"), sysconfig.get_paths()["include"]
-    if not os.path.exists(os.path.join(include, "Python.h")):
-        return False
-    if force or not os.path.exists(CALL_PATH) or os.path.getmtime(src) > os.path.getmtime(CALL_PATH):
+    if not force and os.path.exists(CALL_PATH) and os.path.getmtime(src) <= os.path.getmtime(CALL_PATH):
+        return True
+    why, cc = "no Python.h", os.environ.get("CC", "gcc")
+    if os.path.exists(os.path.join(include, "Python.h")):
         tmp = CALL_PATH + ".tmp.%d" % os.getpid()
-        out = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", include, "-o", tmp, src],
-                             stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
-        if out.returncode != 0:
-            sys.stderr.write(out.stdout)
-            raise RuntimeError("%s failed building _perq_call.so" % os.environ.get("CC", "gcc"))
-        os.replace(tmp, CALL_PATH)
-    return True
+        try:
+            out = subprocess.run([cc, "-O2", "-shared", "-fPIC", "-I", include, "-o", tmp, src],
+                                 stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+            if out.returncode == 0:
+                os.replace(tmp, CALL_PATH)
+                return True
+            why = "%s failed\n%s" % (cc, out.stdout)
+        except OSError as error:
+            why = "%s: %s" % (cc, error)
+    if os.path.exists(CALL_PATH):
+        os.remove(CALL_PATH)
+    sys.stderr.write("perq: without the interpreter's own entry, calls go through ctypes (%s)\n" % why)
+    return False
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -35,3 +35,34 @@ def test_refusals(B, bad):
         B._rotate_quantize(None, None, 0)
     with pytest.raises(TypeError):
         B._swiglu_rotate_quantize(None, None, None, 0, 2048, bad, 0, 0, None, None, None)
+
+
+def ctypes_takes_the_calls(B, monkeypatch, path):
+    from paper_2601_22347_b200 import build
+    for name in ("_lib", "_rotate_quantize", "_swiglu_rotate_quantize"):
+        monkeypatch.setattr(B, name, None)
+    monkeypatch.setattr(build, "CALL_PATH", str(path))
+    lib = B.load()
+    return B._rotate_quantize is lib.perq_rotate_quantize and B._swiglu_rotate_quantize is lib.perq_swiglu_rotate_quantize
+
+
+@pytest.mark.parametrize("content", [None, b"", b"another machine's file", b"\x7fELF" + bytes(200)], ids=["missing", "empty", "text", "header"])
+def test_an_entry_that_cannot_be_loaded(B, monkeypatch, tmp_path, content):
+    path = tmp_path / "_perq_call.so"
+    if content is not None:
+        path.write_bytes(content)
+    assert ctypes_takes_the_calls(B, monkeypatch, path)
+    assert B._rotate_quantize(None, None, 4, 2048, 16, 0, 0, None, None, None) == 1      # PERQ_ERR_NULL
+
+
+@pytest.mark.parametrize("cc", ["/nowhere/cc", "false"])
+def test_a_compiler_that_is_missing_or_fails(B, monkeypatch, tmp_path, cc):
+    """The entry is left out, an older one taken away, and the library built as ever."""
+    from paper_2601_22347_b200 import build
+    path = tmp_path / "_perq_call.so"
+    path.write_bytes(b"older")
+    os.utime(path, (0, 0))
+    monkeypatch.setattr(build, "CALL_PATH", str(path))
+    monkeypatch.setenv("CC", cc)
+    assert build.build() == build.LIB_PATH
+    assert not path.exists()
