@@ -18,7 +18,12 @@
 // rotated, and the time in which rows are interleaved, 64 wavefronts for 512 channels each way, by warps that then wait for each
 // other.  8192 x 9728, permuted, MXFP4, b = 32: 82 us (row kernel 176), INT4 per 128, b = 128: 105 (282).
 //
-// Exactness rules and error model as in perq_fast.cuh (the arithmetic is the same: one tensor-core step, then fp32).
+// Exactness rules as in perq_fast.cuh, whose arithmetic this is: one tensor-core step for a chunk of 16, then fp32 stages over the C
+// chunks of a block.  What they lose, in 2^-24 of the block's largest output M: a step loses 7.5 T + 2 P (perq_tile.cuh; measured here
+// too: mma.sync gives the bits of that model), T the chunk's largest input, P its output.  Over the chunks both sum to sqrt(C) M
+// at most (Cauchy; Parseval: M is at least the 2-norm of the inputs, and of the chunks' outputs that meet in one).  The stages round to
+// nearest: sqrt(C/2) + sqrt(C/4) + .. + 1.  In all 9.5, 14.4, 21.4 and 31.3 for b = 16, 32, 64, 128 (perm_err; the worst rows found lose 17).
+// The model of perq_fast.cuh is 16, 20, 24 and 28, of which MXFP4 takes twice.
 #pragma once
 #include <cuda.h>
 
@@ -98,9 +103,10 @@ __device__ __forceinline__ void perm_gather(uint32_t rows, uint2 at, uint32_t (&
         x[4 * j] = r[0]; x[4 * j + 1] = r[1]; x[4 * j + 2] = r[2]; x[4 * j + 3] = r[3];
     }
 }
-// Rounding window of E2M1 codes in scaled units: ref the largest magnitude of the element's block, m the multiplier.  Blocks up to 32: the
-// error model's 16 and 20 units are a bound (a tensor-core step loses 9.5, see perq_tile.cuh, the sum of two rounds once), and the scaled
-// values are below 8: one window for all groups.
+// Error bound of an fp32 output, relative to the largest of its block.
+__host__ __device__ constexpr float perm_err(int log2b, bool ranges) { return (ranges && log2b == 7 ? 32.0f : 4.0f * log2b) * 0x1p-24f; }
+// Rounding window of E2M1 codes in scaled units: ref the largest magnitude of the element's block, m the multiplier.  Twice the model's error
+// in blocks of 64 and 128.  Blocks up to 32: once, and the scaled values are below 8: one window for all groups.
 template <int LOG2B>
 __device__ __forceinline__ float perm_window(float err, float ref, float m) { return LOG2B <= 5 ? 8.01f * err + 2.0e-6f : 2.0f * err * ref * m + 2.0e-6f; }
 // Columns of H_16 for a lane's four adjacent outputs: column n of contraction m is output 4 (n / 2) + n % 2 + 2 m.
@@ -338,7 +344,7 @@ __device__ __noinline__ double perm_group_max(uint32_t rows, const uint2 *at, bo
 template <int LOG2B, int MODE>
 __device__ __noinline__ uint4 perm_mend(uint32_t rows, const uint2 *at, uint4 codes, double sqrt_b, double a, float inv, float tau, uint32_t ex, int lane)
 {
-    const float err = FAST_ERR_K * (float)LOG2B * TWO_M24;
+    constexpr float err = perm_err(LOG2B, false);
     const int q = lane & 3;
     uint32_t x[16], hb[2][2];
     f32x2 v[8][2];
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__(PERM_THREADS, 1) perq_perm_kernel(const __grid
 {
     static_assert(MODE == ROW_MX || MODE == ROW_GROUP, "ranges inside a unit");
     constexpr int CB = LOG2B - 4;
-    const float err = FAST_ERR_K * (float)LOG2B * TWO_M24;
+    constexpr float err = perm_err(LOG2B, MODE == ROW_GROUP);
     extern __shared__ __align__(128) unsigned char psmem_raw[];
     unsigned char *smem = psmem_raw + ((1024u - (smem_u32(psmem_raw) & 1023u)) & 1023u);
     const uint32_t base = smem_u32(smem), ring = base + p.off_ring, full = base + p.off_bars;
@@ -552,7 +558,7 @@ __global__ void __launch_bounds__(PERM_THREADS, 1) perq_perm_kernel(const __grid
                 if (q == 0 && live) *scales = __float_as_uint(row_scale(a, p.inv_7_sqrt_b, p.sqrt_b, 7.0));
                 // ---- quantise: distance to the rounded value
                 const float inv = row_inverse((float)a);
-                const float tau = (err + 5.0e-7f) * inv * a32 + 2.0e-7f;       // the element's error and the multiplier's (three roundings); the distance's own
+                const float tau = (err + 5.0e-7f) * (inv * a32) + 2.0e-7f;       // the element's error and the multiplier's (three roundings); the distance's own
                 const f32x2 m2 = pack2(inv, inv), mg = pack2(12584968.0f, 12584968.0f), up = pack2(-256.0f, -256.0f);     // 1.5 * 2^23 + 8 * 257
                 float far0 = 0.0f, far1 = 0.0f;
 #pragma unroll

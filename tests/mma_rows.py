@@ -119,3 +119,30 @@ def hidden_in_every_piece(d, gap):
     for t in range(int(np.log2(c))):
         x[128 * 2 ** t + 2] = eps * w[2 ** t]
     return x
+
+
+def one_step_and_stages(x):
+    """Unnormalised outputs of blocks x[i]: a step for every 16 inputs, then fp32 sums and differences over the chunks."""
+    n, b = x.shape
+    c = b // 16
+    v = chained_contraction(x.reshape(-1, 16), hadamard(16)).reshape(n, c, 16).astype(np.float32)
+    k, t = np.arange(c), 1
+    while t < c:
+        low = v[:, k & ~t], v[:, k | t]
+        v = np.where((k & t == 0)[None, :, None], low[0] + low[1], low[0] - low[1])
+        t *= 2
+    return v.reshape(n, b).astype(np.float64)
+
+
+def losing_chunks(n, b, rng):
+    """A large input in every chunk of 16, their spectrum flat, and tiny ones that are lost with the sign of one output."""
+    c = b // 16
+    x = np.zeros((n, c, 16))
+    spectrum = np.abs(rng.choice([-1, 1], (n, c)) @ hadamard(c))
+    size = np.where(rng.random((n, 1)) < 0.5, np.exp2(rng.integers(-2, 1, (n, c))), np.maximum(spectrum, 0.125 * c) / c)
+    size = to_bf16(size * (1 + rng.integers(0, 2, (n, 1)) * 2.0 ** -7)).reshape(n, c)
+    at = np.where(rng.random((n, 1)) < 0.5, 0, rng.integers(0, 16, (n, c)))
+    np.put_along_axis(x, at[:, :, None], (rng.choice([-1, 1], (n, c)) * size)[:, :, None], 2)
+    signs = hadamard(b)[:, rng.integers(0, b, n)].T.reshape(n, c, 16) * rng.choice([-1, 1], (n, 1, 1))
+    tiny = 1.9921875 * np.exp2(np.floor(np.log2(size)) - 26)[:, :, None] * signs
+    return np.where(x == 0, tiny, x).reshape(n, b)

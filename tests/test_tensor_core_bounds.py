@@ -1,13 +1,17 @@
 """Error bounds of the kernels that rotate by chained tensor-core steps (tile and column kernel), against the oracle, on rows
 whose fp32 outputs are as wrong as that arithmetic allows: a maximum, and a side of a rounding boundary, that fp32 hides."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2601_22347_b200 import inputs
 
-from dispatch import kernel_of
-from mma_rows import hadamard, chained_contraction, hidden_in_every_piece, hidden_maximum, hidden_side, hidden_step, outputs, to_bf16
+from dispatch import LAUNCH, kernel_of
+from mma_rows import (hadamard, chained_contraction, hidden_in_every_piece, hidden_maximum, hidden_side, hidden_step, losing_chunks, one_step_and_stages,
+                      outputs, to_bf16)
 from parity import compare_quantized
 
 FMT = {"int4": 0, "mxfp4": 1, "fp4": 3, "int4_asym": 4}
@@ -262,3 +266,43 @@ def vanishing_groups(d, b, seed):
 @pytest.mark.parametrize("b", [64, 128])
 def test_groups_that_vanish_in_fp32(B, oracle, b):
     run(B, oracle, vanishing_groups(1152, b, 47000 + b), 16 * 2 ** 20 // 1152 + 3, b, "mxfp4", 32)
+
+
+def perm_err(b, ranges):
+    """The permuted kernel's bound in 2^-24 of the block's largest output, from its source."""
+    with open(os.path.join(os.path.dirname(LAUNCH), "perq_perm.cuh")) as f:
+        rule = re.search(r"constexpr float perm_err\(int log2b, bool ranges\) \{ return \(ranges && log2b == 7 \? ([0-9.]+)f : ([0-9.]+)f \* log2b\) \* 0x1p-24f; \}", f.read())
+    return float(rule.group(1)) if ranges and b == 128 else float(rule.group(2)) * np.log2(b)
+
+
+@pytest.mark.parametrize("b", [16, 32, 64, 128])
+def test_what_a_step_and_stages_lose(b):
+    """The bound covers what the steps and the stages can lose, and with it what the model loses."""
+    c = b // 16
+    proven = 9.5 * np.sqrt(c) + sum(np.sqrt(2.0 ** k) for k in range(int(np.log2(c))))
+    assert perm_err(b, True) >= proven and 2 * perm_err(b, False) >= proven
+    rng, worst = np.random.default_rng(43000 + b), 0.0
+    for make in [lambda: losing_chunks(512, b, rng)] * 20 + [lambda: rng.standard_normal((512, b)) * np.exp2(-rng.integers(0, 30, (512, b)))] * 5:
+        x = to_bf16(make()).reshape(-1, b)
+        u = x @ hadamard(b)
+        worst = max(worst, (np.abs(one_step_and_stages(x) - u).max(1) / np.abs(u).max(1)).max() * 2.0 ** 24)
+    assert 3 < worst <= proven
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fmt,group", [("int4", 128), ("mxfp4", 32)])
+@pytest.mark.parametrize("b", [16, 32, 64, 128])
+def test_permuted_rows_that_lose(B, oracle, b, fmt, group):
+    d, n = 1152, 160
+    rng = np.random.default_rng(44000 + b)
+    x = losing_chunks(n * d // b, b, rng).reshape(n, d) * np.exp2(rng.integers(-20, 20, (n, 1)))
+    perm = rng.permutation(d).astype(np.int32)
+    base = np.empty((n, d), np.uint16)
+    base[:, perm] = bits(x)
+    xt = torch.from_numpy(np.tile(base, (4, 1)).view(np.int16)).cuda().view(torch.bfloat16)
+    codes, scales = B.perq_rotate_quantize(xt, torch.from_numpy(perm).cuda(), b, FMT[fmt], group)
+    torch.cuda.synchronize()
+    ora = oracle.rotate_quantize(base, perm, b, FMT[fmt], group, want_pre=True)
+    for part in range(4):
+        rows = slice(n * part, n * part + n)
+        compare_quantized(fmt, codes[rows].cpu().numpy(), scales[rows].cpu().numpy(), ora)
