@@ -395,6 +395,21 @@ __device__ __noinline__ uint4 perm_mend(uint32_t rows, const uint2 *at, uint4 co
     if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) > 16u) {
         uint32_t own = perm_row_exact(x) ? flags : 0u;
         flags &= ~own;
+        if (MODE == ROW_MX) {                                 // zeros beside others, flagged for their sign: all at once (2048 x 9728, b = 128, equal values: 342 -> 113 us)
+            uint32_t zero = 0u;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) zero |= (((j & 1) ? v[j >> 2][(j >> 1) & 1].y : v[j >> 2][(j >> 1) & 1].x) == 0.0f) ? 1u << j : 0u;
+            zero &= own;
+            own &= ~zero;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                uint32_t m = (zero >> (8 * w)) & 0xffu;       // a bit to a nibble
+                m = (m | m << 12) & 0x000f000fu;
+                m = (m | m << 6) & 0x03030303u;
+                m = (m | m << 3) & 0x11111111u;
+                cw[w] &= ~(m * 15u);
+            }
+        }
 #pragma unroll 1
         while (own) {
             const int e = __ffs(own) - 1;
