@@ -254,7 +254,6 @@ __global__ void __launch_bounds__(ST_THREADS + 32) perq_stats_rows_kernel(StatsP
     if (tid < ST_MAX_STAGES * R) top[tid] = 0u;
     __syncthreads();
     griddep_wait();             // nothing above reads or writes global memory
-    griddep_launch();           // (the second pass waits beside this one: 22.7 us, launched after the last row 23.5)
     const long long t0 = (long long)blockIdx.x * p.rows_per_cta, t1 = min(p.T, t0 + p.rows_per_cta);
     const uint32_t n = t1 > t0 ? (uint32_t)((t1 - t0 + R - 1) / R) : 0u;
 
@@ -359,9 +358,8 @@ __global__ void __launch_bounds__(ST_THREADS + 32) perq_stats_rows_kernel(StatsP
 }
 
 // 256 threads: 64 outputs (of the channels, in the CTAs after those of the blocks), each summed by 4 threads over a quarter of the CTA
-// slices, then combined in a fixed order (deterministic).  The loads of a quarter are all in flight (in rounds of eight they
-// took five trips to L2).
-constexpr int ST_QUARTER = 38;                       // slices of a quarter: 148 CTAs at most
+// slices, then combined in a fixed order (deterministic).  Eight loads in flight: with all 38 of a quarter in one round the pass took 4 to 6 us more
+// (both passes, CUDA graph, 600 x 1024: 9.6 / 4.7 us; 4096 x 8192 20.1 / 15.4), 74 registers and a predicate a load.
 __global__ void __launch_bounds__(256) perq_stats_reduce_kernel(const float *ws_chan, const float *ws_block, int n_cta, int d,
                                                                 int nb, float inv_T, float *chan_abs_sum, float *block_l1_mean)
 {
@@ -378,13 +376,13 @@ __global__ void __launch_bounds__(256) perq_stats_reduce_kernel(const float *ws_
     const int c0 = quarter * per, c1 = min(n_cta, c0 + per);
     float sum = 0.0f;
     if (i < width) {
-        // independent loads, added in slice order (x + 0 is exact, so padding is harmless)
-        for (int c = c0; c < c1; c += ST_QUARTER) {
-            float v[ST_QUARTER];
+        // eight independent loads at a time, added in slice order (x + 0 is exact, so padding is harmless)
+        for (int c = c0; c < c1; c += 8) {
+            float v[8];
 #pragma unroll
-            for (int j = 0; j < ST_QUARTER; ++j) v[j] = (c + j < c1) ? ws[(size_t)(c + j) * width + i] : 0.0f;
+            for (int j = 0; j < 8; ++j) v[j] = (c + j < c1) ? ws[(size_t)(c + j) * width + i] : 0.0f;
 #pragma unroll
-            for (int j = 0; j < ST_QUARTER; ++j) sum += v[j];
+            for (int j = 0; j < 8; ++j) sum += v[j];
         }
     }
     part[quarter][o] = sum;
