@@ -1,12 +1,11 @@
 // Calibration statistic kernels: per-channel sum of |x|, per-block mean l1 norm and
 // per-token max block l1 norm under an optional permutation.
 //
-// Phase 1: each CTA walks a contiguous slab of rows, 64 KB of rows at a time through a ring of
-// bulk-copied shared-memory stages (32 KB where no gather is needed), keeps
+// Phase 1: each CTA walks a contiguous slab of rows through a ring of bulk-copied shared-memory stages (64 KB
+// of rows to a stage under a permutation or with blocks over 256 channels, 32 KB otherwise), keeps
 // per-channel and per-block partial sums in registers (every thread owns fixed columns /
-// blocks), and writes them to its own slice of the workspace.  Rows go through shared memory
-// only when a block statistic needs the gather through the permutation.
-// Phase 2: one thread per output adds the CTA slices in CTA order.  All additions happen
+// blocks), and writes them to its own slice of the workspace.
+// Phase 2: four threads per output add the CTA slices, a quarter each, and then the quarters.  All additions happen
 // in a fixed order, so the results are bit-identical from run to run.
 #pragma once
 #include <cuda_runtime.h>
@@ -225,11 +224,11 @@ __global__ void __launch_bounds__(ST_THREADS) perq_stats_partial_kernel(StatsPar
 
 // Unpermuted rows, blocks of 2^CL chunks of eight channels (up to 256 channels).  The same sums in the same order, without a barrier:
 // a 17th warp loads rows (32 KB of them to a stage, as many stages as fit) and the others hand a stage back by an mbarrier.  The rows'
-// largest block sums meet in a word of the stage, which the loading warp stores and clears before it loads again.  With 64 KB to a batch and
+// largest block sums meet in a word of the stage, which the loading warp stores and clears before it loads again (asked for or not, and a word at a time, they
+// made block sums alone 16384 x 4096 slower than with a barrier a batch: 30.4 / 28.2 us; now 26.5).  With 64 KB to a batch and
 // a barrier for each, the first and the last batch and the barriers were in the open, and widths other than 4096, 8192 and 16384
-// and blocks of 64 had flags to test in every unrolled step.  Both passes, 4096 x 8192: b = 32 25.2 -> 22.7 us, b = 64 31.4 -> 24.0; 8192 x
-// 14336 78 -> 53; 4096 x 2048 23.0 -> 16.6.  What bounds it: 13.6 us are this pass (5 TB/s), 7.5 the second one, also when it has
-// next to nothing to add: the end of a grid, the start of the next, two trips to L2.
+// and blocks of 64 had flags to test in every unrolled step.  All outputs, both passes, inputs not in L2: 4096 x 8192, b = 32 24.8 -> 18.3 us; 8192 x
+// 14336 78 -> 47; 4096 x 2048 22.8 -> 12.6.  What bounds it: the read (4096 x 8192 at 5 TB/s), then the ends of two grids.
 constexpr int ST_MAX_STAGES = 8;
 __host__ __device__ constexpr int stats_rows(int kc) { return kc >= 4 ? 1 : 4 / kc; }       // rows of a stage
 
@@ -295,6 +294,7 @@ __global__ void __launch_bounds__(ST_THREADS + 32) perq_stats_rows_kernel(StatsP
 #pragma unroll
         for (int e = 0; e < 4; ++e) csum[k][e] = make_float2(0.0f, 0.0f);
     }
+    const bool tokens = WB && p.token_max != nullptr;
     uint32_t s = 0, parity = 0;
     for (uint32_t i = 0; i < n; ++i) {
         if (!mbar_wait_fast(bars + s * 8, parity)) {
@@ -303,6 +303,7 @@ __global__ void __launch_bounds__(ST_THREADS + 32) perq_stats_rows_kernel(StatsP
         }
         const unsigned char *rows = smem + (size_t)s * stage_bytes;
         const int live = (int)min((long long)R, t1 - (t0 + (long long)i * R));
+        float row_max = 0.0f;                                // (lane r: of the batch's row r)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (r >= live) break;
@@ -328,11 +329,13 @@ __global__ void __launch_bounds__(ST_THREADS + 32) perq_stats_rows_kernel(StatsP
                     mx = fmaxf(mx, b);
                 }
             }
-            if (WB) {
+            if (tokens) {
                 mx = warp_max_f32(mx);
-                if (lane == 0) atomicMax(&top[s * R + r], __float_as_uint(mx));
+                if (R == 1 && lane == 0) atomicMax(&top[s], __float_as_uint(mx));
+                if (R > 1 && lane == r) row_max = mx;
             }
         }
+        if (R > 1 && tokens && lane < live) atomicMax(&top[s * R + lane], __float_as_uint(row_max));
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s * 8);
         if (++s == (uint32_t)NST) { s = 0; parity ^= 1u; }

@@ -31,3 +31,16 @@ def test_edges(B, T, d, b, perm):                            # noqa: F811
     np.testing.assert_allclose(block.cpu().numpy(), norms.mean(0), rtol=(b + rows + 42) * eps)
     np.testing.assert_allclose(token.cpu().numpy(), norms.max(1), rtol=b * eps)
     assert B.perq_device_error() == 0
+
+
+@pytest.mark.parametrize("T,d,b", [(149, 4096, 32), (300, 4128, 32), (1033, 8192, 128), (150, 16384, 8), (9, 32768, 64)])
+def test_outputs_alone(B, T, d, b):                          # noqa: F811
+    """An output that is asked for alone has the bits that it has among all."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(9400 + T + d)
+    x = torch.randn(T, d, generator=gen, device="cuda").to(torch.bfloat16)
+    for perm in (None, torch.randperm(d, generator=gen, device="cuda").to(torch.int32)):
+        every = B.perq_block_l1_stats(x, perm, b)
+        for i, want in enumerate(("chan", "block", "token")):
+            alone = B.perq_block_l1_stats(x, perm, b, want=(want,))
+            assert torch.equal(alone[i], every[i]) and all(alone[k] is None for k in range(3) if k != i)
