@@ -309,7 +309,7 @@ int perq_zigzag_perm(const float *chan_abs_max_host, int32_t d, int32_t b, int32
  *   stream           cudaStream_t (0 = default); two kernels are enqueued, nothing is synchronised
  *
  * b >= 1, d % b == 0, d <= PERQ_MAX_D and at most 4096 blocks (d / b).  One CTA serves the channels in batches,
- * about 0.18 ms for a statistic of d = 8192, b = 32; masses that fall steeply are served one by one (about 1 ms
+ * about 0.11 ms for a statistic of d = 8192, b = 32; masses that fall steeply are served one by one (about 1.2 ms
  * there).  NaN and negative masses count as 0, infinity as the largest float.
  * Errors: NULL, SHAPE, BLOCK (also: too many blocks), WORKSPACE, ALIGN, CUDA.
  */

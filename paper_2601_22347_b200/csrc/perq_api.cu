@@ -1051,7 +1051,7 @@ int perq_massdiff_perm_device(const float *chan_abs_sum, int32_t d, int32_t b, i
     p.b = b;
     const int n = d / b;
     const int ctas = (d + perq::MD_RANK_CHANNELS - 1) / perq::MD_RANK_CHANNELS;
-    // up to 256 blocks (8192 channels, b = 32: 106 us, the other one 175; 256 .. 16384 channels in 16 .. 256 blocks: 0.57 .. 0.71 of its time, heavy-tailed masses up to 0.94;
+    // up to 256 blocks (8192 channels, b = 32: 106 us, the other one 175; 256 .. 16384 channels in 20 .. 256 blocks: 0.57 .. 0.71 of its time, heavy-tailed masses up to 0.94, 16 blocks 0.93;
     // 448 and 512 blocks would gain on real statistics, 313 to 222 and 178 to 124, and lose on masses 1 / rank, 445 to 556)
     const bool sorts = n <= perq::MD_SORT_BLOCKS;
     void (*greedy)(perq::MassdiffParams) = !sorts  ? perq::perq_massdiff_greedy_kernel

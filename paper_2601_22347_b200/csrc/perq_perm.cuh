@@ -14,9 +14,9 @@
 // A CTA per SM, 16 warps.  A set: the rows come in TMA boxes of eight rows by 512 channels (128-byte swizzle), a stage of the ring to a
 // warp, which interleaves a box and loads the next one into its place; a barrier; units of 128 positions in turn; a barrier.
 //
-// What bounds it: 360 (MXFP4, b = 32) to 640 (per 128, b = 128) instructions a unit of 1024 elements at 60 % of the issue slots while units are
-// rotated, and the time in which rows are interleaved, 64 wavefronts for 512 channels each way, by warps that then wait for each
-// other.  8192 x 9728, permuted, MXFP4, b = 32: 82 us (row kernel 176), INT4 per 128, b = 128: 105 (282).
+// What bounds it: 325 (MXFP4, b = 32) to 617 (per 128, b = 128) instructions and 100 wavefronts a segment of 1024 at 31 to 45 % of the issue slots, and
+// the time in which rows are interleaved, 64 wavefronts for 512 channels each way, by warps that then wait for each other (barriers are its
+// largest stall).  8192 x 9728, permuted, MXFP4, b = 32: 82 us (row kernel 176), INT4 per 128, b = 128: 106 (282).
 //
 // Exactness rules as in perq_fast.cuh, whose arithmetic this is: one tensor-core step for a chunk of 16, then fp32 stages over the C
 // chunks of a block.  What they lose, in 2^-24 of the block's largest output M: a step loses 7.5 T + 2 P (perq_tile.cuh; measured here

@@ -175,7 +175,7 @@ int launch_perm_b(int log2b, const CUtensorMap &map, const perq::PermParams &p, 
 // at 9728 are better spread by the row kernel (148 rows, MXFP4 b = 32: 7.7 / 10.3; 300 rows, b = 128: 13.5 / 14.5).
 //   MXFP4, 9728: b = 16, 592 rows 24 / 17, 8192 rows 240 / 103; b = 32, 1200 rows 44 / 27, 33.5 / 23.1, 8192 rows 176 / 82; b = 128, 592 rows 20.4 / 18.0,
 //     8192 rows 195 / 121; 4736: b = 32, 592 rows 11.0 / 7.8, 2368 rows 25.5 / 17.4; 640 and 1152: 592 rows 6.1 .. 8.4 / 5.9 .. 6.5
-//   INT4 per 128, 9728: b = 16, 592 rows 22.9 / 15.5; b = 128, 1200 rows 50.7 / 27.6, 8192 rows 282 / 105; 1152: b = 128, 8192 rows 40 / 25
+//   INT4 per 128, 9728: b = 16, 592 rows 22.9 / 15.5; b = 128, 1200 rows 50.7 / 27.6, 8192 rows 282 / 106; 1152: b = 128, 8192 rows 40 / 25
 //   One nonzero, integers, few nonzeros, equal values, zeros, eight shapes from 592 x 640 to 2368 x 4736: 0.07 .. 1.0 of the row kernel's time, but up to
 //     1.2 for small integers and 2 % of nonzeros in MXFP4, b = 16 .. 64 (592 x 640, 2 % of nonzeros, b = 64: 1.7)
 // Widths of 1024 k stay with the group kernel, which has no ragged segments: 4096 x 8192, MXFP4, b = 32 37.6 / 41.8; per 128, b = 128 48.0 / 49.9.
